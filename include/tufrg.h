@@ -132,7 +132,7 @@ enum { TUFRG_LOOPS_AUTO = 0, TUFRG_LOOPS_TC = 1, TUFRG_LOOPS_SIMT = 2 };
  * accordingly; the learned surrogate and tufrg_loops_noalloc support the temperature flow only. */
 enum { TUFRG_REG_TEMPERATURE = 0, TUFRG_REG_MOMENTUM_SHELL = 1 };
 
-/* Symmetries of the loop k-sums (split two-band path).  A point operation G of the square lattice
+/* Symmetries of the loop k-sums.  A point operation G of the square lattice
  * (rotations by multiples of 90 degrees, the four mirrors) with a spin unitary U such that every
  * hopping satisfies t_{G R} = U t_R U^dagger maps the band projectors as P_l(G k) = U P_l(k) U^dagger,
  * so both loops obey Lc(G q)[G Delta] = V Lc(q)[Delta] V^dagger (V = U (x) U on the P orbital pair,
@@ -142,7 +142,9 @@ enum { TUFRG_REG_TEMPERATURE = 0, TUFRG_REG_MOMENTUM_SHELL = 1 };
  * for one momentum per orbit and the others are written from it.  TUFRG_SYMMETRY_OFF sums every q. */
 /* For symmetric states (tufrg_rhs with TUFRG_SYMMETRIC_STATE, and every flow) the projections and products can
  * run for the orbit representatives only, and do so whenever the state symmetries hold (AUTO and STATES
- * alike; OFF disables every symmetry).  Both paths are timed at init for tufrg_symmetry_info. */
+ * alike; OFF disables every symmetry).  Both paths are timed at init for tufrg_symmetry_info.  FP64 two-band models use
+   the loop symmetries and, inside flows, the state symmetries; they ignore TUFRG_SYMMETRIC_STATE (a caller's state
+   that was kept in lower precision has the symmetries to that precision only). */
 enum { TUFRG_SYMMETRY_AUTO = 0, TUFRG_SYMMETRY_OFF = 1, TUFRG_SYMMETRY_STATES = 2 };
 
 /* Adaptive flow options (Dormand-Prince 5(4) in x = ln T, from T0 down to T_end; T is Lambda with the
@@ -207,11 +209,12 @@ tufrg_status tufrg_loop_momenta(const tufrg_model *m, int *n_direct);
 tufrg_status tufrg_loops_info(const tufrg_model *m, int *backend);
 
 /* Launch shape of the loop k-sum: *ky_chunks = the number of k_y ranges each fine-mesh column is split into (the
- * grid's depth; every range ends with a flush of its partial sums), and, for the two-band split path, which times
- * every candidate from 1 to 16 ranges (each range at least 8 rows) at model set-up and keeps the fastest:
+ * grid's depth; every range ends with a flush of its partial sums), and, for the flows of the two-band split path, which
+ * time every candidate from 1 to 16 ranges (each range at least 8 rows) at model set-up and keep the fastest:
  * *n_candidates = their number and h_ms[i] (i < min(n_ms, *n_candidates)) = the measured milliseconds per launch
  * of candidate i, which has i + 1 ranges.  Other paths report their heuristic choice and *n_candidates = 0.
- * The choice is cached per process and model shape, so models of the same shape sum in the same order.
+ * The choice is cached per process and model shape, so models of the same shape sum in the same order.  (The k-sum of
+ * single right-hand sides takes its ranges from the shape alone.)
  * Errors: TUFRG_EINVAL for NULL arguments or n_ms < 0 (h_ms may be NULL when n_ms is 0). */
 tufrg_status tufrg_loop_tiles(const tufrg_model *m, int *ky_chunks, int *n_candidates, double *h_ms, int n_ms);
 
@@ -332,8 +335,7 @@ tufrg_status tufrg_rhs(tufrg_model *m, double T, const void *d_state, int channe
  *      products: d_dstate_local [2][n_q][M][M], dX/dT of the shard's momenta in list order.
  * With the shards partitioning the mesh, the rows equal those of tufrg_rhs.  h_q_list: n_q distinct
  * momenta in [0, Nq) (host memory); the model keeps full-size work buffers, the shard's rows alone are
- * read and written.  The loops are summed at the listed momenta (the FP64 two-band path sums every
- * momentum); the general (not symmetric-state) path is taken; a model with an attached surrogate is
+ * read and written.  The loops are summed at the listed momenta; the general (not symmetric-state) path is taken; a model with an attached surrogate is
  * refused (TUFRG_ENOTSUP).  Stream ordered, no host synchronisation beyond the list upload.
  * Errors: TUFRG_EINVAL (NULL argument, bad list, T not positive and finite, bad mask), TUFRG_ENOTSUP,
  * TUFRG_ENOMEM, TUFRG_ECUDA.

@@ -266,6 +266,7 @@ struct LoopSymmetry {
     std::vector<int2> qmap;
     std::vector<tufrg::SymElem> elem;
     std::vector<int> ffinv;   // [elem][nff] source bond of each target bond (G R_src = R_target), -1 if none
+    int inv = -1;             // an element that inverts the momentum
 };
 
 struct Mono {
@@ -417,6 +418,7 @@ void build_loop_symmetry(const tufrg_model *m, LoopSymmetry &ls)
     for (const Elem &el : elems) {
         tufrg::SymElem e{};
         e.conj = el.conj;
+        if (el.Gq[0] == -1 && el.Gq[1] == 0 && el.Gq[2] == 0 && el.Gq[3] == -1) ls.inv = (int)ls.elem.size();
         for (int ch = 0; ch < 2; ch++)
             for (int a2 = 0; a2 < ns2; a2++) {
                 const cd v = el.V[ch].ph[a2];
@@ -528,7 +530,7 @@ void release(tufrg_model *m)
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
-                    m->d_shard_q, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
+                    m->d_shard_q, m->d_lph, m->d_hp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &p : m->d_k)
@@ -561,11 +563,11 @@ void release(tufrg_model *m)
 size_t state_elems(const tufrg_model *m) { return (size_t)2 * m->Nq * m->M * m->M; }
 
 // One evaluation of the right-hand side into d_out at the temperature held in m->d_scal[0],
-// each channel scaled by c_X * m->d_scal[1] (1 for dX/dT, T for the flow variable ln T).
+// each channel scaled by c_X * m->d_scal[1] (1 for dX/dT, T for the flow variable ln T); flow: a stage of a flow.
 // The split path evaluates on an FP32 copy of the state: d_state32 when the caller has already
 // written one (the flow's stage combinations do), else a conversion of d_state into m->d_X32.
 tufrg_status rhs_device(tufrg_model *m, const double2 *d_state, int mask, double2 *d_out, const float2 *d_state32,
-                        bool symmetric_state)
+                        bool symmetric_state, bool flow)
 {
     const bool split = m->precision != TUFRG_FP64;
     // a symmetric state needs projections and products at the orbit representatives only
@@ -601,7 +603,7 @@ tufrg_status rhs_device(tufrg_model *m, const double2 *d_state, int mask, double
     }
     CK(launch_fermi(m), "fermi tables");
     // a symmetric state's products read the loops of the orbit representatives only
-    CK(launch_loops(m, mask, sym), "loop k-sum");
+    CK(launch_loops(m, mask, sym, flow), "loop k-sum");
     if (fork) {
         CK(cudaStreamWaitEvent(m->stream, m->aux_ev[1], 0), "join");
     } else {
@@ -640,7 +642,7 @@ tufrg_status enqueue_attempt(tufrg_model *m, int mask)
         double2 *dst = j == 6 ? m->d_yn : (split ? nullptr : m->d_yt);
         CK(launch_rk_combine(m, dst, split ? m->d_X32 : nullptr, m->d_y, m->d_flow, DP_A[j], k, j, n), "stage combination");
         CK(launch_stage_scalars(m, m->d_flow, DP_C[j]), "stage temperature");
-        tufrg_status st = rhs_device(m, dst, mask, k[j], split ? m->d_X32 : nullptr, true);
+        tufrg_status st = rhs_device(m, dst, mask, k[j], split ? m->d_X32 : nullptr, true, true);
         if (st != TUFRG_OK) return st;
     }
     CK(launch_rk_error(m, m->d_y, m->d_yn, m->d_flow, DP_E, k, 7, n), "error norm");
@@ -718,7 +720,7 @@ tufrg_status flow_prepare(tufrg_model *m, const tufrg_flow_opts *o)
     CK(surrogate_rearm(m), "re-arm surrogate");
     // k1 = f(x0, y0) and max|A| of the initial state
     CK(launch_stage_scalars(m, m->d_flow, 0.0), "stage temperature");
-    st = rhs_device(m, m->d_y, o->channel_mask, m->d_k[0], nullptr, true);
+    st = rhs_device(m, m->d_y, o->channel_mask, m->d_k[0], nullptr, true, true);
     if (st != TUFRG_OK) return st;
     CK(launch_flow_init(m, m->d_flow), "flow init");
     if ((st = flow_capture(m, o->channel_mask)) != TUFRG_OK) return st;
@@ -915,7 +917,7 @@ try {
     build_loop_tables(m);
     build_gather_tables(m);
     build_irrep_basis(m);   // empty when the bond set is not closed under the point group
-    // loop symmetries (TUFRG_SYMMETRY_AUTO, split two-band path)
+    // loop symmetries (TUFRG_SYMMETRY_AUTO)
     m->n_loop_q = m->Nq;
     if (m->basis == TUFRG_BASIS_BAND && !band_basis_supported(m))
         return fail(m, TUFRG_ENOTSUP, "the band-basis flow needs a two-band model with M <= 64");
@@ -928,6 +930,7 @@ try {
             m->sym = true;
             m->n_loop_q = (int)ls.list.size();
             m->n_sym_elem = (int)ls.elem.size();
+            m->sym_inv = ls.inv;
             CK(upload(&m->d_loop_list, ls.list, m->stream), "upload symmetry tables");
             CK(upload(&m->d_qmap, ls.qmap, m->stream), "upload symmetry tables");
             CK(upload(&m->d_sym_elem, ls.elem, m->stream), "upload symmetry tables");
@@ -966,6 +969,10 @@ try {
                             qrow[o] = ls.elem[e].qt[ch][r % nsq];
                         }
                 m->sym_state = true;
+                // the FP64 two-band path takes a caller's state as it is: states kept in lower precision have the
+                // symmetries to that precision only, and its results are the reference for them; its own flows keep
+                // them to FP64 rounding
+                m->sym_calls = ns != 2 || m->precision != TUFRG_FP64;
                 CK(upload(&m->d_sym_srow, srow, m->stream), "upload symmetry tables");
                 CK(upload(&m->d_sym_qrow, qrow, m->stream), "upload symmetry tables");
                 // the inverse maps (every srow is a permutation when the bond set and the orbital pairs are closed
@@ -1018,8 +1025,9 @@ try {
     m->plan = plan_loops(m);
     // the two-band split loop kernel's launch shapes are timed at the end of the set-up (the partial sums are
     // sized for the largest)
-    if (loops2_supported(m)) m->plan_cand = loop_plan_candidates(m);
-    int max_partials = m->plan.n_partials;
+    if (loops2_supported(m) && m->precision != TUFRG_FP64) m->plan_cand = loop_plan_candidates(m);
+    m->plan_h = plan_loops2h(m);
+    int max_partials = std::max(m->plan.n_partials, m->plan_h.n_partials);
     for (const LoopPlan &p : m->plan_cand) max_partials = std::max(max_partials, p.n_partials);
 
     // ---- device memory (and the right-hand side's second stream)
@@ -1038,6 +1046,16 @@ try {
     CK(upload(&m->d_dslot, m->dslot, m->stream), "upload bond tables");
     CK(upload(&m->d_dpartner, m->dpartner, m->stream), "upload bond tables");
     CK(upload(&m->d_dij, m->dij, m->stream), "upload bond tables");
+    {
+        // the Hermitian half of the bond differences, and every difference's (or its negative's) place in it
+        std::vector<int> hp;
+        for (int k = 0; k < m->nd; k++)
+            if (m->deltas[2 * k + 1] > 0 || (m->deltas[2 * k + 1] == 0 && m->deltas[2 * k] >= 0)) hp.push_back(k);
+        const size_t n_hp = hp.size();
+        hp.resize(n_hp + m->nd);
+        for (size_t i = 0; i < n_hp; i++) hp[n_hp + hp[i]] = hp[n_hp + m->dpartner[hp[i]]] = (int)i;
+        CK(upload(&m->d_hp, hp, m->stream), "upload bond tables");
+    }
     for (int ch = 0; ch < 2; ch++) {
         CK(upload(&m->d_gofs[ch], m->gofs[ch], m->stream), "upload gather tables");
         CK(upload(&m->d_gterms[ch], m->gterms[ch], m->stream), "upload gather tables");
@@ -1128,19 +1146,25 @@ try {
             std::vector<float2> c32(cph.size());
             for (size_t i = 0; i < cph.size(); i++) c32[i] = make_float2((float)cph[i].x, (float)cph[i].y);
             CK(upload(&m->d_clsph32, c32, m->stream), "upload phase table");
-            // e^{-2 pi i n / Lf} of the split loop kernel, with exact quarter-turn values
-            std::vector<float2> lph(m->Lf);
-            for (int n = 0; n < m->Lf; n++) {
-                const double a = 2.0 * M_PI * (double)n / (double)m->Lf;
-                double c = std::cos(a), sn = std::sin(a);
-                if ((4 * n) % m->Lf == 0) {
-                    const int quarter = (4 * n) / m->Lf;
-                    c = quarter == 0 ? 1.0 : quarter == 2 ? -1.0 : 0.0;
-                    sn = quarter == 1 ? 1.0 : quarter == 3 ? -1.0 : 0.0;
-                }
-                lph[n] = make_float2((float)c, (float)-sn);
+        }
+        // e^{-2 pi i n / Lf} of the loop kernels, with exact quarter-turn values
+        std::vector<double2> lph(m->Lf);
+        for (int n = 0; n < m->Lf; n++) {
+            const double a = 2.0 * M_PI * (double)n / (double)m->Lf;
+            double c = std::cos(a), sn = std::sin(a);
+            if ((4 * n) % m->Lf == 0) {
+                const int quarter = (4 * n) / m->Lf;
+                c = quarter == 0 ? 1.0 : quarter == 2 ? -1.0 : 0.0;
+                sn = quarter == 1 ? 1.0 : quarter == 3 ? -1.0 : 0.0;
             }
-            CK(upload(&m->d_lph32, lph, m->stream), "upload phase table");
+            lph[n] = make_double2(c, -sn);
+        }
+        if (split) {
+            std::vector<float2> l32(lph.size());
+            for (size_t i = 0; i < lph.size(); i++) l32[i] = make_float2((float)lph[i].x, (float)lph[i].y);
+            CK(upload(&m->d_lph32, l32, m->stream), "upload phase table");
+        } else {
+            CK(upload(&m->d_lph, lph, m->stream), "upload phase table");
         }
     }
     CK(dalloc(&m->d_E, Nk * ns), "cudaMalloc eigenvalues");
@@ -1184,7 +1208,7 @@ try {
     CK(cudaMalloc(&m->d_dftpart, dft_scratch * (split ? sizeof(float2) : sizeof(double2))),
        "cudaMalloc Fourier partials");
     if (split) CK(dalloc(&m->d_Xr32, 2 * (size_t)m->ncls * M2), "cudaMalloc Fourier transforms");
-    if (loops2_supported(m)) CK(dalloc(&m->d_rec, Nk * 3), "cudaMalloc loop records");
+    if (loops2_supported(m)) CK(cudaMalloc(&m->d_rec, loops2_rec_bytes(m)), "cudaMalloc loop records");
     if (!split) CK(dalloc(&m->d_A, 2 * (size_t)m->Nq * M2), "cudaMalloc projections");   // split: FP32 copy only
     CK(dalloc(&m->d_amax, 4), "cudaMalloc reductions");
     CK(dalloc(&m->d_red, 512), "cudaMalloc reductions");
@@ -1317,10 +1341,10 @@ try {
         CK(cudaMemcpy(&dev_err, m->d_err, sizeof(int), cudaMemcpyDeviceToHost), "copy error flag");
         if (dev_err) return fail(m, TUFRG_ETIMEOUT, "a bounded device-side wait gave up during autotuning");
     }
-    if (m->sym_state && tune_lookup(m, 1 + m->products, &cached)) {
+    if (m->sym_calls && tune_lookup(m, 1 + m->products, &cached)) {
         m->sym_tune_ms[0] = cached.ms[0];
         m->sym_tune_ms[1] = cached.ms[1];
-    } else if (m->sym_state) {
+    } else if (m->sym_calls) {
         // symmetric states: projections and products for the orbit representatives plus the gather of the
         // other momenta, against both for every momentum (on zeroed operands: the cost does not depend on
         // the values).  Reported only: the representatives' path is taken whenever the symmetries hold (a
@@ -1447,9 +1471,9 @@ tufrg_status tufrg_widen_f64(const void *d_in, void *d_out, size_t n, void *cuda
 tufrg_status tufrg_symmetry_info(const tufrg_model *m, int *in_use, double *ms_general, double *ms_reps)
 {
     if (!m || !in_use || !ms_general || !ms_reps) return TUFRG_EINVAL;
-    *in_use = m->sym_state ? 1 : 0;
-    *ms_general = m->sym_state ? m->sym_tune_ms[0] : -1.0;
-    *ms_reps = m->sym_state ? m->sym_tune_ms[1] : -1.0;
+    *in_use = m->sym_calls ? 1 : 0;
+    *ms_general = m->sym_calls ? m->sym_tune_ms[0] : -1.0;
+    *ms_reps = m->sym_calls ? m->sym_tune_ms[1] : -1.0;
     return TUFRG_OK;
 }
 
@@ -1550,7 +1574,7 @@ try {
     CK(surrogate_rearm(m), "re-arm surrogate");
     auto direct = [&]() {
         return rhs_device(m, reinterpret_cast<const double2 *>(d_state), channel_mask & 3,
-                          reinterpret_cast<double2 *>(d_dstate), nullptr, (channel_mask & TUFRG_SYMMETRIC_STATE) != 0);
+                          reinterpret_cast<double2 *>(d_dstate), nullptr, m->sym_calls && (channel_mask & TUFRG_SYMMETRIC_STATE) != 0, false);
     };
     // The launches after the temperature (which they read from device memory) are replayed from a captured graph:
     // the same kernels in the same order without the gaps between launches.  Direct launches instead while the
@@ -1949,14 +1973,15 @@ tufrg_status tufrg_flow_resume(tufrg_model *m, const tufrg_flow_opts *o, const v
     if (h.products != m->products &&
         (m->precision == TUFRG_FP64 || (h.products != TUFRG_PRODUCTS_TC && h.products != TUFRG_PRODUCTS_SIMT)))
         return fail(m, TUFRG_EINVAL, "the checkpoint's products backend does not apply to this model");
-    if (h.ky_chunks != m->plan.ky_chunks && (h.ky_chunks < 1 || h.ky_chunks > (int)m->plan_cand.size()))
+    // (a path without timed launch shapes keeps its own)
+    if (h.ky_chunks < 1 || h.ky_chunks > (m->plan_cand.empty() ? 16 : (int)m->plan_cand.size()))
         return fail(m, TUFRG_EINVAL, "the checkpoint's loop launch shape does not apply to this model");
     bool reshaped = false;
     if (h.products != m->products) {
         m->products = h.products;
         reshaped = true;
     }
-    if (h.ky_chunks != m->plan.ky_chunks) {
+    if (!m->plan_cand.empty() && h.ky_chunks != m->plan.ky_chunks) {
         m->plan = m->plan_cand[h.ky_chunks - 1];
         reshaped = true;
     }
@@ -1977,7 +2002,7 @@ tufrg_status tufrg_flow_resume(tufrg_model *m, const tufrg_flow_opts *o, const v
         // the projections of the restored state (the final report locates max |A| in them); the derivative goes to
         // a stage buffer that the next attempt overwrites, k1 itself comes from the checkpoint
         CK(launch_stage_scalars(m, m->d_flow, 0.0), "stage temperature");
-        s2 = rhs_device(m, m->d_y, o->channel_mask, m->d_k[1], nullptr, true);
+        s2 = rhs_device(m, m->d_y, o->channel_mask, m->d_k[1], nullptr, true, true);
         if (s2 != TUFRG_OK) return s2;
         CK(cudaMemcpyAsync(m->d_k[0], p + sizeof(h) + sizeof(FlowDev) + sizeof(double2) * n, sizeof(double2) * n,
                            cudaMemcpyHostToDevice, m->stream), "copy derivative");

@@ -248,7 +248,7 @@ cudaError_t launch_fermi_shell(tufrg_model *m)
 
 cudaError_t launch_fermi(tufrg_model *m)
 {
-    if (loops2_supported(m)) return launch_loop_records(m);   // the split two-band kernel reads its own per-k records
+    if (loops2_supported(m)) return launch_loop_records(m);   // the two-band kernel reads its own per-k records
     if (m->regulator == TUFRG_REG_MOMENTUM_SHELL) return cudaSuccess;   // tables fixed at init (no Lambda dependence)
     const int n = m->Nk * m->ns;
     FermiEntry32 *ft32 = m->precision == TUFRG_FP64 ? nullptr : m->d_ft32;

@@ -1,6 +1,10 @@
-// Split-precision (FP32) loop k-sum for N_s = 2, the dominant kernel of the right-hand side.
+// Split-precision (FP32) loop k-sum for N_s = 2 over the whole fine mesh, as split-precision flows (and
+// tufrg_loops_noalloc) take it; right-hand sides outside of flows, and FP64, take k_loops2h.cu, which sums half of the mesh
+// and is faster.  Flows keep this order of summation: an adaptive flow that ends at a divergence turns a change of
+// rounding in the loops (1e-7) into percents of its last state (and 1e-5 .. 1e-4 of the critical scale) through the
+// steps it accepts, so a flow's results, and flows resumed from stored checkpoints, stay those they always were.
 //
-// Same sums as k_loops.cu (Eqs. loopminus / loopplus dressed by Eq. trafo), organised
+// Same sums as k_loops2h.cu (Eqs. loopminus / loopplus dressed by Eq. trafo), organised
 // around the structure of the two-band problem:
 //   * the band projectors are complete and rank one: rho^1 = 1 - rho^0 and
 //     rho^0_00 + rho^0_11 = 1, so one 48-byte record per fine k holds
@@ -18,8 +22,8 @@
 //     thread loads the next row while it computes the current one; rows advance
 //     without integer division.
 // One thread per fine-mesh column, one CTA per (transfer momentum, 64 columns, row range).
-// The flush and the partial layout are the ones of k_loops.cu, so the same
-// deterministic reduction kernel finishes the sum.
+// A warp's columns leave one partial sum; a deterministic reduction kernel finishes the sum.
+#include <algorithm>
 #include <cmath>
 
 #include "tufrg_internal.cuh"
@@ -282,63 +286,113 @@ __global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
     }
 }
 
-// Record of one fine k (FP32, three planes [j][ky][kx]): plane 0 = (rho00, Re rho01, Im rho01, e0),
-// plane 1 = (e1, g0, g1, g'0), plane 2 = (g'1, 0, 0, 0), with e = E - mu, g = dF/dT-type weight
-// derivative of the Fermi function and g' its derivative in e.  The projector and e do not depend on
-// T and are written once per model; only g and g' are refreshed per evaluation.
-__global__ void rec_static_kernel(const double *E, const double2 *U, int Nk, int Lf, double mu, float4 *rec)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= Nk) return;
-    // rho^0 = U_{.0} U*_{.0}: rho00 = |U_00|^2, rho01 = U_00 conj(U_10)
-    const double2 u0 = U[(size_t)k * 4 + 0], u1 = U[(size_t)k * 4 + 2];
-    const int kx = k / Lf, ky = k % Lf;
-    const size_t t = (size_t)ky * Lf + kx, plane = (size_t)Lf * Lf;
-    rec[t] = make_float4((float)(u0.x * u0.x + u0.y * u0.y), (float)(u0.x * u1.x + u0.y * u1.y),
-                         (float)(u0.y * u1.x - u0.x * u1.y), (float)(E[2 * k] - mu));
-    rec[plane + t] = make_float4((float)(E[2 * k + 1] - mu), 0.f, 0.f, 0.f);
-    rec[2 * plane + t] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
+constexpr int NS2 = 4, NS4 = 16;
 
-// g = -df/dT = (x / T) f (1 - f) and g' = dg/de with x = e / T, in the overflow-safe form with
-// z = exp(-|x|): f (1 - f) = z / (1 + z)^2 and dg/de = f (1 - f) / T^2 (1 - |x| (1 - z) / (1 + z)).
-// FP32 (the split path's loop sums are FP32).
-__global__ void rec_T_kernel(int n, double T_value, const double *Tp, float4 *rec)
+// Sum the partials of list position s in a fixed order and scale by 1/Nk; the half-plane partials
+// give both Hermitian halves.  The sum runs in the partials' own precision (FP32 on the split path:
+// this GPU's FP64 rate would make the reduction, not the memory traffic, its bound), with 16 loads
+// in flight per thread (the additions keep their sequential order).
+template <typename R>
+__device__ __forceinline__ typename cpx<R>::t reduce_one(const typename cpx<R>::t *__restrict__ part, int n_part,
+                                                         int ndx, int ndyh, const int *dslot, const int *deltas, int s,
+                                                         int d, int ab, R inv_nk)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const float invT = 1.f / (float)(Tp ? *Tp : T_value);   // device-resident temperature when given
-    const float e[2] = {rec[t].w, rec[n + t].x};
-    float g[2], gp[2];
+    using C2 = typename cpx<R>::t;
+    const int dx = deltas[2 * d], dy = deltas[2 * d + 1];
+    const bool half = dy > 0 || (dy == 0 && dx >= 0);
+    const int ia = ab / NS2, ib = ab % NS2;
+    const int src_ab = half ? ab : ib * NS2 + ia;
+    const int slot = dslot[d];   // dxi * ndyh + dyi of the half-plane representative of +-delta
+    const size_t stride = (size_t)ndx * ndyh * NS4;
+    const C2 *src = part + (size_t)s * n_part * stride + (size_t)slot * NS4 + src_ab;
+    R re = 0, im = 0;
+    constexpr int UB = 16;
+    int p = 0;
+    for (; p + UB <= n_part; p += UB) {
+        C2 v[UB];
 #pragma unroll
-    for (int l = 0; l < 2; l++) {
-        const float x = e[l] * invT, ax = fabsf(x);
-        const float z = expf(-ax), opz = 1.f + z;
-        const float h = z / (opz * opz);
-        g[l] = x * invT * h;
-        gp[l] = h * invT * invT * (1.f - ax * (1.f - z) / opz);
+        for (int j = 0; j < UB; j++) v[j] = src[(size_t)(p + j) * stride];
+#pragma unroll
+        for (int j = 0; j < UB; j++) {
+            re += v[j].x;
+            im += v[j].y;
+        }
     }
-    rec[n + t] = make_float4(e[1], g[0], g[1], gp[0]);
-    rec[2 * n + t] = make_float4(gp[1], 0.f, 0.f, 0.f);
+    for (; p < n_part; p++) {
+        const C2 v = src[(size_t)p * stride];
+        re += v.x;
+        im += v.y;
+    }
+    return mk(re * inv_nk, (half ? im : -im) * inv_nk);
 }
 
-// Momentum-shell records: (f, h) = (f(e), f (1 - f) / T) at the fixed temperature T in the slots of
-// (g, g'), from the FP64 energies (written once per model; the shell weight needs no T-dependent data).
-__global__ void rec_shell_kernel(const double *E, int Nk, int Lf, double mu, double T, float4 *rec)
+__device__ __forceinline__ double2 to64(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
+
+// Grid: blockIdx.y = transfer momentum (list position), blockIdx.z = channel (skipped when not in chmask;
+// its partials and outputs are offset by part_cs and out_cs), threads over (d, ab) = t (t >> 4, t & 15):
+// no runtime integer division (this GPU issues its conversions to the slow FP64 pipe).  List position s
+// is written at momentum qout[s] (orbit representatives only) or at s.
+template <typename R>
+__global__ void loops_reduce_kernel(const typename cpx<R>::t *__restrict__ part, int n_part, int ndx, int ndyh,
+                                    const int *dslot, const int *deltas, int nd, double inv_nk, const int *qout,
+                                    double2 *out64, typename cpx<R>::t *out32, const int *skip, int chmask,
+                                    size_t part_cs, size_t out_cs)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= Nk) return;
-    const int kx = k / Lf, ky = k % Lf;
-    const size_t t = (size_t)ky * Lf + kx, plane = (size_t)Lf * Lf;
-    double f[2], h[2];
-    for (int l = 0; l < 2; l++) {
-        const double e = E[2 * k + l] - mu, z = exp(-fabs(e) / T);
-        f[l] = e > 0 ? z / (1.0 + z) : 1.0 / (1.0 + z);
-        h[l] = z / ((1.0 + z) * (1.0 + z)) / T;
+    if (skip && *skip) return;
+    const int ch = blockIdx.z;
+    if (!((chmask >> ch) & 1)) return;
+    part += ch * part_cs;
+    if (out64) out64 += ch * out_cs;
+    if (out32) out32 += ch * out_cs;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nd * NS4) return;
+    const int s = blockIdx.y, d = t / NS4, ab = t % NS4;
+    const auto v = reduce_one<R>(part, n_part, ndx, ndyh, dslot, deltas, s, d, ab, R(inv_nk));
+    const size_t idx = (size_t)(qout ? qout[s] : s) * nd * NS4 + t;
+    if (out64) out64[idx] = to64(v);
+    if (out32) out32[idx] = v;
+}
+
+// Symmetry variant (two bands), gather form: blockIdx.y = output momentum q'; qmap[q'] = (list
+// position i of its orbit representative, group element e).  Thread (d', a'b') reads the representative's
+// partial sums of d = dinv[e][d'], a = src[a'], b = src[b'] (L2 resident) and writes
+// Lc(q')[d'][a'][b'] = i^(qt[a'] - qt[b']) (conj ? conj(v) : v) coalesced (see SymElem).
+template <typename C2>
+__device__ __forceinline__ C2 quarter_turn(C2 v, int k)
+{
+    switch (k & 3) {
+    case 0: return v;
+    case 1: return mk(-v.y, v.x);
+    case 2: return mk(-v.x, -v.y);
+    default: return mk(v.y, -v.x);
     }
-    const float e1 = rec[plane + t].x;
-    rec[plane + t] = make_float4(e1, (float)f[0], (float)f[1], (float)h[0]);
-    rec[2 * plane + t] = make_float4((float)h[1], 0.f, 0.f, 0.f);
+}
+
+template <typename R>
+__global__ void loops_reduce_sym_kernel(const typename cpx<R>::t *__restrict__ part, int n_part, int ndx, int ndyh,
+                                        const int *dslot, const int *deltas, int nd, const int2 *qmap,
+                                        const SymElem *elem, const int *dinv, double inv_nk, double2 *out64,
+                                        typename cpx<R>::t *out32, const int *skip, int chmask, size_t part_cs,
+                                        size_t out_cs)
+{
+    if (skip && *skip) return;
+    const int ch = blockIdx.z;   // as in loops_reduce_kernel
+    if (!((chmask >> ch) & 1)) return;
+    part += ch * part_cs;
+    out64 += ch * out_cs;
+    out32 += ch * out_cs;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nd * NS4) return;
+    const int q2 = blockIdx.y, d2 = t / NS4, a2 = (t / NS2) % NS2, b2 = t % NS2;
+    const int2 ie = qmap[q2];
+    const SymElem &e = elem[ie.y];
+    const int d = dinv[ie.y * nd + d2], a = e.src[ch][a2], b = e.src[ch][b2];
+    auto v = reduce_one<R>(part, n_part, ndx, ndyh, dslot, deltas, ie.x, d, a * NS2 + b, R(inv_nk));
+    if (e.conj) v.y = -v.y;
+    const auto w = quarter_turn(v, e.qt[ch][a2] - e.qt[ch][b2]);
+    const size_t o = (size_t)q2 * nd * NS4 + t;
+    if (out64) out64[o] = to64(w);
+    if (out32) out32[o] = w;
 }
 
 template <int NDYH, int WHICH>
@@ -371,40 +425,13 @@ int loops2_blocks_per_sm(const tufrg_model *m)
     return (e == cudaSuccess && n > 0) ? n : 4;
 }
 
-bool loops2_supported(const tufrg_model *m)
-{
-    int ndyh = 0;
-    for (int v : m->dys) ndyh += v >= 0;
-    return m->ns == 2 && m->precision != TUFRG_FP64 && ndyh <= 5 && (int)m->dxs.size() <= MAXD;
-}
-
-cudaError_t launch_loop_records_static(tufrg_model *m)
-{
-    rec_static_kernel<<<(m->Nk + 255) / 256, 256, 0, m->stream>>>(m->d_E, m->d_U, m->Nk, m->Lf, m->mu, m->d_rec);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_loop_records_shell(tufrg_model *m)
-{
-    rec_shell_kernel<<<(m->Nk + 255) / 256, 256, 0, m->stream>>>(m->d_E, m->Nk, m->Lf, m->mu, m->T_reg, m->d_rec);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_loop_records(tufrg_model *m)
-{
-    if (m->regulator == TUFRG_REG_MOMENTUM_SHELL) return cudaSuccess;   // the shell records do not depend on Lambda
-    PhaseScope ps(m, PH_FERMI);
-    rec_T_kernel<<<(m->Nk + 255) / 256, 256, 0, m->stream>>>(m->Nk, 0.0, m->d_scal, m->d_rec);
-    return cudaGetLastError();
-}
-
 // Loop sums of channel ch into the partial buffer (no reduction).  With s_list, only the
 // listed transfer momenta (n_list of them) are evaluated, into partial slots 0..n_list-1 of part.
 cudaError_t launch_loops2_ex(tufrg_model *m, int ch, const int *s_list, int n_list, float2 *part, const int *skip)
 {
     const LoopPlan &pl = m->plan;
     Args2 a{};
-    a.rec = m->d_rec;
+    a.rec = static_cast<const float4 *>(m->d_rec);
     a.part = part;
     a.s_list = s_list;
     a.skip = skip;
@@ -448,12 +475,111 @@ cudaError_t launch_loops2(tufrg_model *m, int ch)
                             reinterpret_cast<float2 *>(m->d_part), m->sur ? m->d_sur_flag : nullptr);
 }
 
+LoopPlan plan_loops(const tufrg_model *m)
+{
+    // Choose the number of ky ranges so that the grid fills whole waves of the
+    // SMs; the per-column flush costs about 8 rows of work.
+    LoopPlan p{};
+    p.kx_per_cta = 32 * WARPS;
+    const int ctas_x = (m->Lf + p.kx_per_cta - 1) / p.kx_per_cta;
+    const int per_sm = loops2_supported(m) ? loops2_blocks_per_sm(m) : (m->precision == TUFRG_FP64 ? 4 : 6);
+    const double slots = (double)m->sm_count * per_sm;
+    double best = 1e300;
+    int best_c = 1;
+    for (int c = 1; c <= 16; c++) {
+        const int len = (m->Lf + c - 1) / c;
+        if (len < 8) break;
+        const double ctas = (double)m->n_loop_q * ctas_x * c * (m->precision == TUFRG_FP64 ? 2 : 1);
+        const double waves = std::ceil(ctas / slots);
+        const double cost = waves * (len + 8.0);
+        if (cost < best * 0.999) { best = cost; best_c = c; }
+    }
+    p.ky_chunks = best_c;
+    p.n_partials = ctas_x * WARPS * best_c;
+    return p;
+}
+
+std::vector<LoopPlan> loop_plan_candidates(const tufrg_model *m)
+{
+    // every number of ky ranges per column from 1 to 16 whose ranges keep at least 8 rows
+    std::vector<LoopPlan> v;
+    const int kx_per_cta = 32 * WARPS, ctas_x = (m->Lf + kx_per_cta - 1) / kx_per_cta;
+    for (int c = 1; c <= 16; c++) {
+        if ((m->Lf + c - 1) / c < 8) break;
+        LoopPlan p{};
+        p.kx_per_cta = kx_per_cta;
+        p.ky_chunks = c;
+        p.n_partials = ctas_x * WARPS * c;
+        v.push_back(p);
+    }
+    return v;
+}
+
+// launch shape of the reductions: one row of CTAs per momentum, threads over (d, ab)
+static void reduce_shape(const tufrg_model *m, int n_s, dim3 &grid, int &thr)
+{
+    const int per = m->nd * NS4;
+    thr = std::min(1024, (per + 31) / 32 * 32);
+    grid = dim3((per + thr - 1) / thr, n_s);
+}
+
+cudaError_t launch_loops_reduce_f32(tufrg_model *m, const float2 *part, int n_s, double2 *out64, float2 *out32,
+                                    const int *skip)
+{
+    int ndyh = 0;
+    for (int v : m->dys) ndyh += v >= 0;
+    dim3 grid;
+    int thr;
+    reduce_shape(m, n_s, grid, thr);
+    PhaseScope ps(m, PH_LOOPRED);
+    loops_reduce_kernel<float><<<grid, thr, 0, m->stream>>>(part, m->plan.n_partials, (int)m->dxs.size(), ndyh,
+                                                          m->d_dslot, m->d_deltas, m->nd, 1.0 / (double)m->Nk, nullptr,
+                                                          out64, out32, skip, 1, 0, 0);
+    return cudaGetLastError();
+}
+
+// The loops of a split two-band flow (every stage of it and the surrogate's fallback).
+cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
+{
+    const LoopPlan &pl = m->plan;
+    const int ndx = (int)m->dxs.size();
+    int ndyh = 0;
+    for (int v : m->dys) ndyh += v >= 0;
+    // both channels' k-sums into their own halves of the partial buffer, then one reduction launch
+    const int n_s = m->sym ? m->n_loop_q : m->Nq;
+    const size_t part_cs = (size_t)n_s * pl.n_partials * ndx * ndyh * NS4, out_cs = (size_t)m->Nq * m->nd * NS4;
+    float2 *part = reinterpret_cast<float2 *>(m->d_part);
+    const int *skip = m->sur ? m->d_sur_flag : nullptr;
+    for (int ch = 0; ch < 2; ch++)
+        if ((channel_mask >> ch) & 1)
+            TUFRG_CUDA_TRY(launch_loops2_ex(m, ch, m->sym ? m->d_loop_list : nullptr, m->sym ? m->n_loop_q : 0,
+                                            part + ch * part_cs, skip));
+    dim3 grid;
+    int thr;
+    reduce_shape(m, reps_only ? m->n_loop_q : m->Nq, grid, thr);
+    grid.z = 2;
+    const double inv_nk = 1.0 / (double)m->Nk;
+    PhaseScope ps(m, PH_LOOPRED);
+    if (reps_only)   // the representatives' FP32 loops at their own momenta (what their products read)
+        loops_reduce_kernel<float><<<grid, thr, 0, m->stream>>>(part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas,
+                                                              m->nd, inv_nk, m->d_loop_list, nullptr, m->d_Lc32, skip,
+                                                              channel_mask, part_cs, out_cs);
+    else if (m->sym)
+        loops_reduce_sym_kernel<float><<<grid, thr, 0, m->stream>>>(
+            part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas, m->nd, m->d_qmap, m->d_sym_elem, m->d_sym_dinv,
+            inv_nk, m->d_Lc, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
+    else
+        loops_reduce_kernel<float><<<grid, thr, 0, m->stream>>>(part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas,
+                                                              m->nd, inv_nk, nullptr, m->d_Lc, m->d_Lc32, skip,
+                                                              channel_mask, part_cs, out_cs);
+    return cudaGetLastError();
+}
+
 }  // namespace tufrg
 
 // ---------------------------------------------------------------------------------
 // Loop k-sum without allocation: the same kernels with their scratch in a static array.
 // ---------------------------------------------------------------------------------
-#include <algorithm>
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -555,10 +681,7 @@ extern "C" tufrg_status tufrg_loops_noalloc(int Lq, int nc, const double *d_E, c
     float4 *rec = reinterpret_cast<float4 *>(base);
     float2 *part = reinterpret_cast<float2 *>(reinterpret_cast<unsigned char *>(base) + rec_bytes);
 
-    rec_static_kernel<<<(unsigned)((Nk + 255) / 256), 256, 0, st>>>(d_E, reinterpret_cast<const double2 *>(d_U), (int)Nk,
-                                                                      Lf, mu, rec);
-    rec_T_kernel<<<(unsigned)((Nk + 255) / 256), 256, 0, st>>>((int)Nk, T, nullptr, rec);
-    if (cudaGetLastError() != cudaSuccess) return TUFRG_ECUDA;
+    if (launch_records_f32(d_E, reinterpret_cast<const double2 *>(d_U), (int)Nk, Lf, mu, T, rec, st) != cudaSuccess) return TUFRG_ECUDA;
     Args2 a{};
     a.rec = rec;
     a.part = part;

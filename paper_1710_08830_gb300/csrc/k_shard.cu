@@ -84,7 +84,6 @@ cudaError_t launch_shard_gather(tufrg_model *m, const double2 *d_full, int n, co
 
 cudaError_t launch_loops_list(tufrg_model *m, int mask, const int *d_list, int n)
 {
-    if (m->ns == 2 && m->precision == TUFRG_FP64) return launch_loops(m, mask, false);   // sums every momentum
     // the list takes the place of the orbit representatives: loops at the listed momenta only, in chunks of the
     // loop scratch's capacity
     const int cap = m->sym ? m->n_loop_q : m->Nq;

@@ -122,9 +122,6 @@ __global__ void check_kernel(const float2 *Lc32, const double2 *chk, const int *
 
 }  // namespace
 
-cudaError_t launch_loops_reduce_f32(tufrg_model *m, const float2 *part, int n_s, double2 *out64, float2 *out32,
-                                    const int *skip);
-
 cudaError_t launch_surrogate(tufrg_model *m, int channel_mask)
 {
     (void)channel_mask;
@@ -192,7 +189,7 @@ try {
         m->err = "the loop surrogate is trained on the temperature flow";
         return TUFRG_ENOTSUP;
     }
-    if (!loops2_supported(m) || m->basis != TUFRG_BASIS_ORBITAL) {
+    if (!loops2_supported(m) || m->precision == TUFRG_FP64 || m->basis != TUFRG_BASIS_ORBITAL) {
         m->err = "the loop surrogate needs a split-precision two-band model in the orbital basis";
         return TUFRG_ENOTSUP;
     }

@@ -235,6 +235,7 @@ struct tufrg_model {
     bool sym = false;
     int n_loop_q = 0;               // transfer momenta summed directly (Nq without symmetry)
     int n_sym_elem = 0;             // group elements (identity included)
+    int sym_inv = -1;               // an element that inverts the momentum, or -1
     int *d_loop_list = nullptr;     // [n_loop_q] orbit representatives
     int2 *d_qmap = nullptr;         // [Nq] (list position of the orbit representative, group element)
     tufrg::SymElem *d_sym_elem = nullptr;   // [n_sym_elem]
@@ -243,6 +244,7 @@ struct tufrg_model {
     // element's bond permutation times its orbital-pair map, so projections and products run for the orbit
     // representatives only and dX/dT of the other momenta is gathered from them
     bool sym_state = false;
+    bool sym_calls = false;         // callers' TUFRG_SYMMETRIC_STATE is used too (not by the FP64 two-band path, see init)
     double sym_tune_ms[2] = {-1.0, -1.0};   // projections + products at every momentum / representatives + gather
     int *d_sym_srow = nullptr;      // [n_sym_elem][2][M] source index of every target row / column
     int *d_sym_qrow = nullptr;      // [n_sym_elem][2][M] quarter turns of every target row / column
@@ -257,7 +259,9 @@ struct tufrg_model {
                                                //  high bit = minus sign; phase-table column)
     double2 *d_v0d[2] = {nullptr, nullptr};    // [M*M] bare vertex V0 at the onsite bond pair, 0 elsewhere
     float2 *d_X32 = nullptr;        // [2][Nq][M][M] FP32 copy of the state being evaluated (split path)
-    float2 *d_lph32 = nullptr;      // [Lf] e^{-2 pi i n / Lf} for the split loop kernel
+    float2 *d_lph32 = nullptr;      // [Lf] e^{-2 pi i n / Lf} for the loop kernels (split path)
+    double2 *d_lph = nullptr;       // the same in FP64 (FP64 path)
+    int *d_hp = nullptr;            // [(nd + 1) / 2] bond differences of the Hermitian half, then [nd] the place of d or -d
     float2 *d_clsph32 = nullptr;    // [Nq][ncls] e^{i u.R''} (split-path Fourier transform)
     float2 *d_v0d32[2] = {nullptr, nullptr};   // FP32 copies of d_v0d (split path)
     double2 *d_ph = nullptr;        // [Nq][nph] phase table e^{i q.R}
@@ -271,7 +275,7 @@ struct tufrg_model {
     double2 *d_A = nullptr;         // [2][Nq][M][M] projected vertex
     float2 *d_A32 = nullptr;        // [2][Nq][M][M] (split path)
     double2 *d_T = nullptr;         // [Nq][M][M] GEMM intermediate (large M); split: [2][Nq][M][M] FP32 complex
-    float4 *d_rec = nullptr;        // [Nk][4] split-path loop records (projectors + Fermi data)
+    void *d_rec = nullptr;          // [3][Nk] two-band loop records (projectors + Fermi data; float4 or four doubles)
     float2 *d_Xr32 = nullptr;       // [2][ncls][M][M] Fourier transforms (split path)
     float2 *d_ph32 = nullptr;       // [Nq][nph] phase table (split path)
     void *d_dftpart = nullptr;      // Fourier-transform scratch: partial sums, or Z(u_x, R_y) of the separable form
@@ -331,7 +335,8 @@ struct tufrg_model {
     unsigned long long *d_amax_ch = nullptr; // [2] max |A| per channel (bit patterns of non-negative doubles)
     int step_graph_mask = 0;
 
-    tufrg::LoopPlan plan{};
+    tufrg::LoopPlan plan{};       // split two-band flows (k_loops2.cu)
+    tufrg::LoopPlan plan_h{};     // half-mesh k-sum (k_loops2h.cu)
     std::vector<tufrg::LoopPlan> plan_cand;   // timed launch shapes of the loop k-sum (two-band split path)
     std::vector<double> plan_ms;              // their measured times (ms per launch), same order
     int gen_chunks = 1;             // multi-orbital loop kernel: kx ranges (CTAs, accumulator slots) per momentum
@@ -379,7 +384,11 @@ cudaError_t launch_fermi(tufrg_model *m);
 cudaError_t launch_set_scalars(tufrg_model *m, double T, double scale);
 // reps_only (with loop symmetries): the FP32 loops of the orbit representatives only, at their own
 // momenta, and no FP64 copy on the split path (what the symmetric-state products read)
-cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only = false);
+// flow: a stage of a flow (split two-band flows keep their own k-sum)
+cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only = false, bool flow = false);
+cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only);
+LoopPlan plan_loops2h(const tufrg_model *m);
+cudaError_t launch_records_f32(const double *E, const double2 *U, int Nk, int Lf, double mu, double T, float4 *rec, cudaStream_t s);
 // The split path reads the FP32 copy of the state (d_state32), the plain path the FP64 state.
 // whether the separable transform applies: *warps = warps per CTA of its column pass, 0 if it does not
 void dft_sep_plan(const tufrg_model *m, int *warps);
@@ -453,6 +462,9 @@ cudaError_t launch_loop_records_shell(tufrg_model *m);    // once per model (mom
 cudaError_t launch_fermi_shell(tufrg_model *m);           // once per model (momentum shell): (e, f, h) tables
 cudaError_t launch_loops2(tufrg_model *m, int ch);
 cudaError_t launch_loops2_ex(tufrg_model *m, int ch, const int *s_list, int n_list, float2 *part, const int *skip);
+cudaError_t launch_loops_reduce_f32(tufrg_model *m, const float2 *part, int n_s, double2 *out64, float2 *out32, const int *skip);
+int loops2_half_mask(const tufrg_model *m);
+size_t loops2_rec_bytes(const tufrg_model *m);
 cudaError_t launch_surrogate(tufrg_model *m, int channel_mask);
 cudaError_t mlp_forward_on(tufrg_mlp *n, cudaStream_t s, const float *X, int batch, float *Y, const int *skip);
 // the network's GEMMs on the tensor cores (k_mlp_tc.cu); TA = __nv_bfloat16 (training) or float (inference)

@@ -530,7 +530,7 @@ void release(tufrg_model *m)
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
-                    m->d_shard_q, m->d_lph, m->d_hp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
+                    m->d_shard_q, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &p : m->d_k)
@@ -931,6 +931,7 @@ try {
             m->n_loop_q = (int)ls.list.size();
             m->n_sym_elem = (int)ls.elem.size();
             m->sym_inv = ls.inv;
+            m->loop_q = ls.list;
             CK(upload(&m->d_loop_list, ls.list, m->stream), "upload symmetry tables");
             CK(upload(&m->d_qmap, ls.qmap, m->stream), "upload symmetry tables");
             CK(upload(&m->d_sym_elem, ls.elem, m->stream), "upload symmetry tables");
@@ -1172,7 +1173,8 @@ try {
     CK(dalloc(&m->d_ft, Nk * ns), "cudaMalloc Fermi table");
     if (split) {
         CK(dalloc(&m->d_U32, Nk * ns2), "cudaMalloc eigenvectors");
-        CK(dalloc(&m->d_ft32, Nk * ns), "cudaMalloc Fermi table");
+        CK(dalloc(&m->d_ft32, (Nk + 4) * ns), "cudaMalloc Fermi table");
+        CK(cudaMemsetAsync(m->d_ft32 + Nk * ns, 0, sizeof(FermiEntry32) * 4 * ns, m->stream), "zero");
         CK(dalloc(&m->d_Lc32, 2 * (size_t)m->Nq * m->nd * ns4), "cudaMalloc loops");
         CK(dalloc(&m->d_A32, 2 * (size_t)m->Nq * M2), "cudaMalloc projections");
         CK(dalloc(&m->d_X32, 2 * (size_t)m->Nq * M2), "cudaMalloc state copy");
@@ -1186,11 +1188,21 @@ try {
         if (!loops_gen_supported(m)) return fail(m, TUFRG_ENOTSUP, "bond set too large for the multi-orbital loop kernel");
         m->loops_tc = d.loops != TUFRG_LOOPS_SIMT && loops_tc_supported(m);
         m->gen_chunks = m->loops_tc ? 1 : plan_gen_chunks(m);
-        // accumulators of one channel: one slot per (kx range, directly summed momentum), plus the FP64
-        // range sums of the representatives under symmetry
+        // accumulators of one channel: one slot per (kx range, directly summed momentum)
         m->part_bytes = gen_part_bytes(m);
-        if (m->loops_tc)
-            CK(cudaMalloc(reinterpret_cast<void **>(&m->d_loop_w), loops_tc_w_bytes(m)), "cudaMalloc loop column sums");
+        if (m->loops_tc) {
+            if (!m->sym) {
+                m->loop_q.resize(m->Nq);
+                for (int q = 0; q < m->Nq; q++) m->loop_q[q] = q;
+            }
+            const std::vector<int> grp = loops_tc_groups(m->loop_q, m->Lq);
+            m->n_tc_groups = (int)grp.size() / 3;
+            CK(upload(&m->d_tc_grp, grp, m->stream), "upload loop groups");
+            CK(cudaMalloc(&m->d_loop_w, loops_tc_w_bytes(m)), "cudaMalloc loop column sums");
+            // (rows past the last column are read, with zero weights: four more points, zeroed)
+            CK(dalloc(&m->d_rho, (Nk + 4) * ns2 * ns), "cudaMalloc loop projectors");
+            CK(cudaMemsetAsync(m->d_rho + Nk * ns2 * ns, 0, sizeof(float) * 4 * ns2 * ns, m->stream), "zero");
+        }
     }
     m->products = split ? (d.products == TUFRG_PRODUCTS_AUTO ? TUFRG_PRODUCTS_TC : d.products) : TUFRG_PRODUCTS_SIMT;
     // product scratch: the large-M CUDA-core GEMMs' intermediate, or the tensor-core products' first product of both
@@ -1215,6 +1227,7 @@ try {
 
     // ---- eigensystem and chemical potential
     CK(launch_bands(m), "eigensolve");
+    if (m->loops_tc) CK(launch_loops_rho(m), "loop projectors");
     if (d.filling > 0) {
         std::vector<double> E(Nk * ns);
         CK(cudaMemcpyAsync(E.data(), m->d_E, sizeof(double) * E.size(), cudaMemcpyDeviceToHost, m->stream), "copy bands");

@@ -5,16 +5,25 @@
 //   with rho^l_{tt'} = U_{tl} U*_{t'l},  T^{l1} = sum_{l2} w_{l1 l2} rho2'^{l2},  rho2' = rho2 (P) or conj (C),
 //   w the d/dT of the bubbles of Eqs. disc_2a / disc_2b (Eqs. loopminus, loopplus, loop_orbital).
 //
-// For fixed (s, q) the orbital dressing is the rank-N_s product Y = A B with A[(t1t3)][l] = rho1 and
-// B[l][(t2t4)] = T, an N_s^2 x N_s^2 complex matrix.  One CTA owns one transfer momentum; it walks the fine
-// mesh column by column in batches of KB rows.  The raw eigenvectors and Fermi entries of a batch arrive in
-// shared memory by cp.async while the batch before it is multiplied (two buffers); from them all threads
-// form A and B of the batch (projectors, pair weights, T), then every thread updates its TA x TB tile of
-//     W[dy][(t1t3),(t2t4)] += e^{-i ky dy} Y(k)
-// for the non-negative dy of the bond differences.  At the end of a column the thread adds
-// e^{-i kx dx} W into the FP64 accumulator of its own entries (no other CTA touches this s, so no
-// atomics; the order is fixed).  A final kernel writes the other Hermitian half,
-// L(-d)[b][a] = conj(L(d)[a][b]), and scales by 1/Nk.
+// rho1 and T are Hermitian N_s x N_s matrices, so each is N_s^2 real numbers (loop_comp: Re and Im of the upper triangle,
+// the diagonal; for C the sign of rho2' imaginary parts is left to the end), and for fixed (s, q) the orbital dressing is
+// the real rank-N_s product Y = A B with A[c][l] = rho1, B[l][c'] = T.  The row phase e^{-iqy dy} is a cosine and a sine
+// for dy > 0, so a column's sums are W[p][c][c'] = sum_qy phi_p(qy) Y, p over 1, cos, sin, cos, sin, ...: N_s^5 +
+// (2 n_dy - 1) N_s^4 real multiply-adds per (s, q), 3.3 times fewer than in complex arithmetic at N_s = 6 and n_dy = 3.
+// Half of the fine mesh suffices where exchanging the propagators maps the sum onto itself (see k_loops2.cu): columns
+// qx = hx + j, 2 hx = sx (mod Lf), a column that is its own partner with weight 1/2.
+//
+// One CTA owns one transfer momentum and a range of columns; it walks the fine mesh column by column in batches of KB
+// rows.  The raw eigenvectors and Fermi entries of a batch arrive in shared memory by cp.async while the batch before it
+// is multiplied (two buffers); from them all threads form A and B of the batch (projectors, pair weights, T), then every
+// thread updates its TA x TB tile of W (NG thread groups share the batch's rows where the tiles alone are too few
+// threads; their sums meet in shared memory at the end of the column).  At the end of a column the thread adds
+// e^{-iqx dx} W into the accumulator of its own entries (no other CTA touches them, so no atomics; the order is fixed).
+// loops_gen_finish puts the orbital entries together from the real components, adds the exchanged half, writes both
+// Hermitian halves, L(-d)[b][a] = conj(L(d)[a][b]), and scales by 1/Nk; loops_gen_gather writes the other momenta of
+// the orbits.
+// FP64: bound by the FP64 pipe (two results per clock and SM); the 8 x 8 / 6 x 6 three-orbital sums of both channels
+// take 1.8 ms (6.9 ms in complex arithmetic over the whole mesh).
 #include <cmath>
 
 #include "tufrg_internal.cuh"
@@ -34,8 +43,10 @@ template <typename R>
 struct GenArgs {
     const typename cpx<R>::t *U;        // [Nk][NS][NS]
     const typename FTg<R>::t *ft;       // [Nk][NS]
-    typename cpx<R>::t *acc;            // [kx range][slot][nd][NS^4] accumulators (zeroed), half plane filled;
+    typename cpx<R>::t *acc;            // [kx range][slot][nd][NS^2][NS^2] accumulators, half plane filled (by the first
+                                        // column of a range, the others added);
                                         // FP64 on the plain path, FP32 on the split path
+    const typename cpx<R>::t *ptab;     // e^{-2 pi i n / Lf}
     int Lq, nc, Lf, nd, ndx, ndyh;
     int dxs[GMAXD], dys[GMAXD];
     int dslot[GMAXD][GMAXD];            // [dxi][dyi] -> delta index (half plane), or -1
@@ -45,15 +56,8 @@ struct GenArgs {
     const int *s_list;                  // optional: CTA x sums transfer momentum s_list[x] into accumulator slot x
     int n_slot;                         // momenta per kx range (accumulator slots of one range)
     int kx_len;                         // columns per kx range; CTA y covers [y kx_len, (y + 1) kx_len)
+    int half;                           // half of the mesh
 };
-
-template <typename C2> __device__ __forceinline__ void cfma(C2 &acc, C2 a, C2 b)
-{
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(-a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(a.y, b.x, acc.y);
-}
 
 __device__ __forceinline__ void ldft(const FermiEntry *p, double &e, double &g, double &gp) { e = p->e; g = p->g; gp = p->gp; }
 __device__ __forceinline__ void ldft(const FermiEntry32 *p, float &e, float &g, float &gp) { e = p->e; g = p->g; gp = p->gp; }
@@ -62,64 +66,84 @@ __device__ __forceinline__ void ldft(const FermiEntry32 *p, float &e, float &g, 
 __device__ __forceinline__ int wrap1(int v, int L) { return v >= L ? v - L : v; }
 
 // Shared memory of one CTA: two buffers of the raw eigenvectors [2 sides][KB][NS^2] and Fermi entries
-// [2 sides][KB][NS] of a batch (side 0: k1, side 1: k2; filled by cp.async one batch ahead), then the phase
-// table [Lf], rho1 / T / rho2' [KB][NS][NS^2] each, batch phases [KB][NDYH], pair weights [KB][NS][NS].
+// [2 sides][KB][NS] of a batch (side 0: k1, side 1: k2; filled by cp.async one batch ahead), then rho1 / T / rho2'
+// [KB][NS][NS^2] each (16-byte aligned rows of rho1), batch phases [KB][NPH], pair weights [KB][NS][NS], and with several
+// thread groups their column sums [NG - 1][NPH][NS^4].
 template <typename R, int NS>
 constexpr size_t gen_raw_bytes()
 {
     return 2 * (sizeof(typename cpx<R>::t) * 2 * KB * NS * NS + sizeof(typename FTg<R>::t) * 2 * KB * NS);
 }
-template <typename R, int NS, int NDYH>
-size_t gen_smem(int Lf)
+template <typename R, int NS, int NDYH, int NG>
+size_t gen_smem()
 {
-    using C2 = typename cpx<R>::t;
-    return gen_raw_bytes<R, NS>() + sizeof(C2) * (Lf + 3 * KB * NS * NS * NS + KB * NDYH) + sizeof(R) * KB * NS * NS;
+    constexpr int NPH = 2 * NDYH - 1;
+    return gen_raw_bytes<R, NS>() +
+           sizeof(R) * (3 * KB * NS * NS * NS + KB * NPH + KB * NS * NS + (size_t)(NG - 1) * NPH * NS * NS * NS * NS);
 }
 
-template <typename R, int NS, int TA, int TB, int NDYH, int WHICH>
-__global__ void loops_gen_kernel(GenArgs<R> a)
+// TA consecutive values from shared memory (aligned to their size where that is 16 bytes)
+__device__ __forceinline__ void ld_tile(const float *p, float (&v)[4])
+{
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+template <typename R, int N> __device__ __forceinline__ void ld_tile(const R *p, R (&v)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; i++) v[i] = p[i];
+}
+
+template <typename R, int NS, int TA, int TB, int NG, int NDYH, int WHICH>
+__global__ void loops_gen_kernel(const __grid_constant__ GenArgs<R> a)
 {
     using C2 = typename cpx<R>::t;
-    constexpr int NS2 = NS * NS;
-    constexpr int GA = NS2 / TA, GB = NS2 / TB;     // thread grid over (a, b) tiles
+    constexpr int NS2 = NS * NS, NPH = 2 * NDYH - 1;
+    constexpr int GA = NS2 / TA, GB = NS2 / TB;     // thread grid over the (c, c') tiles: rows ta TA + i, columns tb + j GB
     constexpr int NT = GA * GB;
     using FT = typename FTg<R>::t;
-    static_assert(NT >= KB * NDYH, "batch phases are staged by one thread each");
     constexpr int CU = NS2 * (int)sizeof(C2) / 16, CF = NS * (int)sizeof(FT) / 16, CK = CU + CF;
     static_assert(CU * 16 == NS2 * (int)sizeof(C2) && CF * 16 == NS * (int)sizeof(FT), "rows of 16-byte chunks");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2 *sUr = reinterpret_cast<C2 *>(smem_raw);                     // [2 buffers][2 sides][KB][NS2]
     FT *sFr = reinterpret_cast<FT *>(sUr + 2 * 2 * KB * NS2);       // [2 buffers][2 sides][KB][NS]
-    C2 *ptab = reinterpret_cast<C2 *>(smem_raw + gen_raw_bytes<R, NS>());   // [Lf] e^{-2 pi i n / Lf}
-    C2 *sA = ptab + a.Lf;                                          // [KB][NS][NS2] rho1
-    C2 *sB = sA + KB * NS * NS2;                                   // [KB][NS][NS2] T
-    C2 *sR2 = sB + KB * NS * NS2;                                  // [KB][NS][NS2] rho2'
-    C2 *sPh = sR2 + KB * NS * NS2;                                 // [KB][NDYH] e^{-i ky dy} of the batch
-    R *sW = reinterpret_cast<R *>(sPh + KB * NDYH);                // [KB][NS][NS] pair weights
+    R *sA = reinterpret_cast<R *>(smem_raw + gen_raw_bytes<R, NS>());   // [KB][NS][NS2] rho1
+    R *sB = sA + KB * NS * NS2;                                    // [KB][NS][NS2] T
+    R *sR2 = sB + KB * NS * NS2;                                   // [KB][NS][NS2] rho2
+    R *sPh = sR2 + KB * NS * NS2;                                  // [KB][NPH] row phases
+    R *sW = sPh + KB * NPH;                                        // [KB][NS][NS] pair weights
+    R *sG = sW + KB * NS * NS;                                     // [NG - 1][NPH][NS2][NS2]
+    __shared__ int2 comp[NS2];                                     // (t NS + t', imaginary part) of a component
     const int Lf = a.Lf;
-    for (int n = threadIdx.x; n < Lf; n += blockDim.x) {
-        double sn, cs;
-        sincospi(2.0 * (double)n / (double)Lf, &sn, &cs);
-        ptab[n] = mk(R(cs), R(-sn));
+    if (threadIdx.x < NS2) {
+        int t, tp;
+        bool im;
+        loop_comp<NS>(threadIdx.x, t, tp, im);
+        comp[threadIdx.x] = make_int2(t * NS + tp, im);
     }
     const int s = a.s_list ? a.s_list[blockIdx.x] : blockIdx.x;
     const int sx = (s / a.Lq) * a.nc, sy = (s % a.Lq) * a.nc;
-    const int ta = threadIdx.x / GB, tb = threadIdx.x % GB;
+    const int grp = threadIdx.x / NT, tt = threadIdx.x - grp * NT, ta = tt / GB, tb = tt - ta * GB;
     const bool shell = a.shell_T > R(0);
     const R lam = shell ? (R)(*a.Tp) : R(0);
     const R thr = a.thr_factor * (shell ? a.shell_T : (R)(*a.Tp));
-    const bool active = threadIdx.x < NT;
+    const bool active = threadIdx.x < NT * NG;
+    // columns hx .. hx + ncol - 1 (mod Lf), fix0 and fix1 their own partners; or the whole mesh
+    const bool even_L = !(Lf & 1), odd_s = sx & 1;
+    const int hx = !a.half ? 0 : !odd_s ? sx / 2 : even_L ? (sx + 1) / 2 : (sx + Lf) / 2;
+    const int ncol = !a.half ? Lf : even_L ? Lf / 2 + (odd_s ? 0 : 1) : (Lf + 1) / 2;
+    const int fix0 = a.half && !(even_L && odd_s) ? 0 : -1, fix1 = a.half && even_L && !odd_s ? Lf / 2 : -1;
     C2 *acc = a.acc + ((size_t)blockIdx.y * a.n_slot + blockIdx.x) * a.nd * NS2 * NS2;
-    const int kx_end = min(Lf, (int)(blockIdx.y + 1) * a.kx_len);
+    const int j_end = min(ncol, (int)(blockIdx.y + 1) * a.kx_len);
     // fine-mesh indices of row ky of column kx: k1 = s - k, k2 = k (P); k1 = k, k2 = k - s (C)
     auto k_of = [&](int side, int kx, int ky) {
         if (side == (WHICH == 0 ? 1 : 0)) return kx * Lf + ky;                      // the point k itself
         return WHICH == 0 ? wrap1(sx - kx + Lf, Lf) * Lf + wrap1(sy - ky + Lf, Lf)  // s - k
                           : wrap1(kx - sx + Lf, Lf) * Lf + wrap1(ky - sy + Lf, Lf); // k - s
     };
-    // copies of the raw eigenvectors and Fermi entries of the rows [ky0, ky0 + KB) of column kx into buffer buf
-    auto stage_raw = [&](int kx, int ky0, int buf) {
-        const int nb = min(KB, Lf - ky0), per_side = nb * CK;
+    // copies of the raw eigenvectors and Fermi entries of the rows [ky0, ky0 + KB) of column j into buffer buf
+    auto stage_raw = [&](int j, int ky0, int buf) {
+        const int kx = wrap1(hx + j, Lf), nb = min(KB, Lf - ky0), per_side = nb * CK;
         for (int idx = threadIdx.x; idx < 2 * per_side; idx += blockDim.x) {
             const int side = idx >= per_side, r = idx - side * per_side, kb = r / CK, c = r % CK;
             const int k = k_of(side, kx, ky0 + kb);
@@ -134,40 +158,46 @@ __global__ void loops_gen_kernel(GenArgs<R> a)
         cp_async_commit();
     };
     int buf = 0;
-    if (blockIdx.y * a.kx_len < kx_end) stage_raw(blockIdx.y * a.kx_len, 0, 0);
+    const int j_beg = blockIdx.y * a.kx_len;
+    if (j_beg < j_end) stage_raw(j_beg, 0, 0);
 
-    for (int kx = blockIdx.y * a.kx_len; kx < kx_end; kx++) {
-        C2 W[NDYH][TA][TB];
+    for (int j = j_beg; j < j_end; j++) {
+        R W[NPH][TA][TB];
 #pragma unroll
-        for (int d = 0; d < NDYH; d++)
+        for (int p = 0; p < NPH; p++)
 #pragma unroll
             for (int i = 0; i < TA; i++)
 #pragma unroll
-                for (int j = 0; j < TB; j++) W[d][i][j] = mk(R(0), R(0));
+                for (int k = 0; k < TB; k++) W[p][i][k] = R(0);
         for (int ky0 = 0; ky0 < Lf; ky0 += KB, buf ^= 1) {
             const int nb = min(KB, Lf - ky0);
             // copies of the next batch (this column's next rows, else the next column's first) go out before
             // this batch is used; the raw buffer they fill was last read before the previous batch's products
-            if (ky0 + KB < Lf) stage_raw(kx, ky0 + KB, buf ^ 1);
-            else if (kx + 1 < kx_end) stage_raw(kx + 1, 0, buf ^ 1);
+            if (ky0 + KB < Lf) stage_raw(j, ky0 + KB, buf ^ 1);
+            else if (j + 1 < j_end) stage_raw(j + 1, 0, buf ^ 1);
             else cp_async_commit();   // an empty group keeps the count of one group in flight
             cp_async_wait<1>();        // this thread's copies of the current batch have landed
             __syncthreads();           // everyone's copies landed; previous batch fully consumed
             const C2 *rU1 = sUr + (size_t)(buf * 2 + 0) * KB * NS2, *rU2 = sUr + (size_t)(buf * 2 + 1) * KB * NS2;
             const FT *rF1 = sFr + (size_t)(buf * 2 + 0) * KB * NS, *rF2 = sFr + (size_t)(buf * 2 + 1) * KB * NS;
-            if (threadIdx.x < KB * NDYH) {
-                const int kb = threadIdx.x / NDYH, d = threadIdx.x % NDYH;
-                if (kb < nb && d < a.ndyh) sPh[threadIdx.x] = ptab[((ky0 + kb) * a.dys[d]) % Lf];
+            for (int idx = threadIdx.x; idx < nb * NDYH; idx += blockDim.x) {
+                const int kb = idx / NDYH, d = idx % NDYH;
+                if (d >= a.ndyh) continue;
+                const C2 ph = a.ptab[(int)(((long)(ky0 + kb) * a.dys[d]) % Lf)];   // (cos, -sin)
+                if (d == 0) sPh[kb * NPH] = R(1);
+                else {
+                    sPh[kb * NPH + 2 * d - 1] = ph.x;
+                    sPh[kb * NPH + 2 * d] = -ph.y;
+                }
             }
-            // stage projectors of the batch: rho1 (k1 side) into sA, rho2' (k2 side) into sR2
+            // projector components of the batch: rho1 (k1 side) into sA, rho2 (k2 side) into sR2
             for (int idx = threadIdx.x; idx < nb * NS * NS2; idx += blockDim.x) {
-                const int kb = idx / (NS * NS2), r = idx % (NS * NS2), l = r / NS2, p = r % NS2;
-                const int t = p / NS, tp = p % NS;
-                const C2 u = rU1[kb * NS2 + t * NS + l], v = rU1[kb * NS2 + tp * NS + l];
-                sA[idx] = mk(u.x * v.x + u.y * v.y, u.y * v.x - u.x * v.y);          // u conj(v)
-                const C2 x = rU2[kb * NS2 + t * NS + l], y = rU2[kb * NS2 + tp * NS + l];
-                sR2[idx] = WHICH == 0 ? mk(x.x * y.x + x.y * y.y, x.y * y.x - x.x * y.y)    // x conj(y)
-                                      : mk(x.x * y.x + x.y * y.y, x.x * y.y - x.y * y.x);   // conj(x) y
+                const int kb = idx / (NS * NS2), r = idx % (NS * NS2), l = r / NS2;
+                const int2 cc = comp[r % NS2];
+                const int o1 = kb * NS2 + (cc.x / NS) * NS + l, o2 = kb * NS2 + (cc.x % NS) * NS + l;
+                const C2 u = rU1[o1], v = rU1[o2], x = rU2[o1], y = rU2[o2];
+                sA[idx] = cc.y ? u.y * v.x - u.x * v.y : u.x * v.x + u.y * v.y;   // u conj(v)
+                sR2[idx] = cc.y ? x.y * y.x - x.x * y.y : x.x * y.x + x.y * y.y;
             }
             for (int idx = threadIdx.x; idx < nb * NS * NS; idx += blockDim.x) {
                 const int kb = idx / (NS * NS), l1 = (idx / NS) % NS, l2 = idx % NS;
@@ -177,368 +207,456 @@ __global__ void loops_gen_kernel(GenArgs<R> a)
                 sW[idx] = gen_pair_weight<WHICH, R>(e1, g1, gp1, e2, g2, gp2, thr, lam);
             }
             __syncthreads();
-            // T^{l1}_{p} = sum_l2 w_{l1 l2} rho2'^{l2}_p
+            // T^{l1}_{c'} = sum_l2 w_{l1 l2} rho2^{l2}_{c'}
             for (int idx = threadIdx.x; idx < nb * NS * NS2; idx += blockDim.x) {
                 const int kb = idx / (NS * NS2), l1 = (idx / NS2) % NS, p = idx % NS2;
-                C2 t = mk(R(0), R(0));
+                R t = R(0);
 #pragma unroll
-                for (int l2 = 0; l2 < NS; l2++) {
-                    const R w = sW[(kb * NS + l1) * NS + l2];
-                    const C2 r = sR2[(kb * NS + l2) * NS2 + p];
-                    t.x = fma(w, r.x, t.x);
-                    t.y = fma(w, r.y, t.y);
-                }
+                for (int l2 = 0; l2 < NS; l2++) t = fma(sW[(kb * NS + l1) * NS + l2], sR2[(kb * NS + l2) * NS2 + p], t);
                 sB[idx] = t;
             }
             __syncthreads();
             if (active) {
-                for (int kb = 0; kb < nb; kb++) {
-                    C2 Y[TA][TB];
+                for (int kb = grp; kb < nb; kb += NG) {
+                    R Y[TA][TB];
 #pragma unroll
                     for (int i = 0; i < TA; i++)
 #pragma unroll
-                        for (int j = 0; j < TB; j++) Y[i][j] = mk(R(0), R(0));
+                        for (int k = 0; k < TB; k++) Y[i][k] = R(0);
 #pragma unroll
                     for (int l = 0; l < NS; l++) {
-                        C2 av[TA], bv[TB];
+                        R av[TA], bv[TB];
+                        ld_tile(sA + (kb * NS + l) * NS2 + ta * TA, av);
 #pragma unroll
-                        for (int i = 0; i < TA; i++) av[i] = sA[(kb * NS + l) * NS2 + ta * TA + i];
-#pragma unroll
-                        for (int j = 0; j < TB; j++) bv[j] = sB[(kb * NS + l) * NS2 + tb * TB + j];
+                        for (int k = 0; k < TB; k++) bv[k] = sB[(kb * NS + l) * NS2 + tb + k * GB];
 #pragma unroll
                         for (int i = 0; i < TA; i++)
 #pragma unroll
-                            for (int j = 0; j < TB; j++) cfma(Y[i][j], av[i], bv[j]);
+                            for (int k = 0; k < TB; k++) Y[i][k] = fma(av[i], bv[k], Y[i][k]);
                     }
 #pragma unroll
-                    for (int d = 0; d < NDYH; d++) {
+                    for (int i = 0; i < TA; i++)
+#pragma unroll
+                        for (int k = 0; k < TB; k++) W[0][i][k] += Y[i][k];
+#pragma unroll
+                    for (int d = 1; d < NDYH; d++) {
                         if (d >= a.ndyh) break;
-                        const C2 ph = sPh[kb * NDYH + d];
+                        const R c = sPh[kb * NPH + 2 * d - 1], sn = sPh[kb * NPH + 2 * d];
 #pragma unroll
                         for (int i = 0; i < TA; i++)
 #pragma unroll
-                            for (int j = 0; j < TB; j++) cfma(W[d][i][j], ph, Y[i][j]);
+                            for (int k = 0; k < TB; k++) {
+                                W[2 * d - 1][i][k] = fma(c, Y[i][k], W[2 * d - 1][i][k]);
+                                W[2 * d][i][k] = fma(sn, Y[i][k], W[2 * d][i][k]);
+                            }
                     }
                 }
             }
         }
+        if (NG > 1) {   // the other groups' sums of this column
+            __syncthreads();
+            if (active && grp > 0) {
+#pragma unroll
+                for (int p = 0; p < NPH; p++)
+#pragma unroll
+                    for (int i = 0; i < TA; i++)
+#pragma unroll
+                        for (int k = 0; k < TB; k++) sG[(((grp - 1) * NPH + p) * NS2 + ta * TA + i) * NS2 + tb + k * GB] = W[p][i][k];
+            }
+            __syncthreads();
+            if (active && grp == 0) {
+#pragma unroll
+                for (int g = 0; g < NG - 1; g++)
+#pragma unroll
+                    for (int p = 0; p < NPH; p++)
+#pragma unroll
+                        for (int i = 0; i < TA; i++)
+#pragma unroll
+                            for (int k = 0; k < TB; k++) W[p][i][k] += sG[((g * NPH + p) * NS2 + ta * TA + i) * NS2 + tb + k * GB];
+            }
+        }
         // add e^{-i kx dx} W into this thread's accumulators (fixed order, no other writer)
-        if (active) {
+        if (active && grp == 0) {
+            const int kx = wrap1(hx + j, Lf);
+            const R f = j == fix0 || j == fix1 ? R(0.5) : R(1);
             for (int xi = 0; xi < a.ndx; xi++) {
-                const C2 phx = ptab[((kx * a.dxs[xi]) % Lf + Lf) % Lf];
+                C2 ph = a.ptab[(int)((((long)kx * a.dxs[xi]) % Lf + Lf) % Lf)];   // (cos, -sin)
+                ph.x *= f;
+                ph.y *= f;
 #pragma unroll
                 for (int d = 0; d < NDYH; d++) {
                     if (d >= a.ndyh) break;
                     const int di = a.dslot[xi][d];
                     if (di < 0) continue;
+                    C2 *o = acc + ((size_t)di * NS2 + ta * TA) * NS2 + tb;
+                    C2 v[TA][TB];   // all loads before the additions
 #pragma unroll
                     for (int i = 0; i < TA; i++)
 #pragma unroll
-                        for (int j = 0; j < TB; j++) {
-                            // GEMM indices (t1t3) x (t2t4) -> compact pair indices of the channel
-                            const int ga = ta * TA + i, gb = tb * TB + j;
-                            const int t1 = ga / NS, t3 = ga % NS, t2 = gb / NS, t4 = gb % NS;
-                            const int ra = WHICH == 0 ? t2 * NS + t1 : t1 * NS + t2;
-                            const int cb = WHICH == 0 ? t4 * NS + t3 : t3 * NS + t4;
-                            const C2 v = W[d][i][j];
-                            C2 &o = acc[((size_t)di * NS2 + ra) * NS2 + cb];
-                            o.x += phx.x * v.x - phx.y * v.y;
-                            o.y += phx.x * v.y + phx.y * v.x;
+                        for (int k = 0; k < TB; k++) v[i][k] = j == j_beg ? mk(R(0), R(0)) : o[i * NS2 + k * GB];
+#pragma unroll
+                    for (int i = 0; i < TA; i++)
+#pragma unroll
+                        for (int k = 0; k < TB; k++) {
+                            // (C - i S) (cos - i sin)
+                            const R C = W[d == 0 ? 0 : 2 * d - 1][i][k], S = d == 0 ? R(0) : W[d == 0 ? 0 : 2 * d][i][k];
+                            v[i][k].x += ph.x * C + ph.y * S;
+                            v[i][k].y += ph.y * C - ph.x * S;
+                            o[i * NS2 + k * GB] = v[i][k];
                         }
                 }
             }
         }
     }
     cp_async_wait<0>();   // nothing in flight at exit (the last group is empty)
+    if (j_beg >= j_end)   // a range without columns
+        for (size_t i = threadIdx.x; i < (size_t)a.nd * NS2 * NS2; i += blockDim.x) acc[i] = mk(R(0), R(0));
 }
 
-// re, im += the n values p[c stride] in order c = 0, 1, ... (FP64), eight loads in flight
-__device__ __forceinline__ double wide(float v) { return widen_f(v); }
-__device__ __forceinline__ double wide(double v) { return v; }
+// the kx ranges' accumulators added into the first range's (fixed order, eight loads in flight)
 template <typename C2>
-__device__ __forceinline__ void sum_ranges(const C2 *p, size_t stride, int n, double &re, double &im)
+__global__ void loops_gen_chunk_sum(C2 *acc, int nchunk, size_t n)
 {
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
     constexpr int UB = 8;
-    int c = 0;
-    for (; c + UB <= n; c += UB) {
+    C2 s = acc[t];
+    for (int c = 1; c < nchunk; c += UB) {
         C2 w[UB];
 #pragma unroll
-        for (int j = 0; j < UB; j++) w[j] = p[(size_t)(c + j) * stride];
+        for (int j = 0; j < UB; j++)
+            if (c + j < nchunk) w[j] = acc[(size_t)(c + j) * n + t];
 #pragma unroll
-        for (int j = 0; j < UB; j++) {
-            re += wide(w[j].x);
-            im += wide(w[j].y);
-        }
+        for (int j = 0; j < UB; j++)
+            if (c + j < nchunk) {
+                s.x += w[j].x;
+                s.y += w[j].y;
+            }
     }
-    for (; c < n; c++) {
-        const C2 w = p[(size_t)c * stride];
-        re += wide(w.x);
-        im += wide(w.y);
-    }
+    acc[t] = s;
 }
 
-// Mirror the half plane, L(-d)[b][a] = conj(L(d)[a][b]), sum the kx ranges (fixed order) and scale by
-// 1/Nk.  Grid: blockIdx.y = momentum, threads over (d, a, b).
-template <int NS, typename C2>
-__device__ __forceinline__ double2 gen_value(const C2 *acc, size_t chunk_stride, int nchunk, size_t base, int d,
-                                             int ia, int ib, const int *deltas, const int *partner)
+template <typename C2>
+struct FinArgs {
+    const C2 *acc;               // [slot][nd][NS2][NS2] half-plane sums in real components
+    const C2 *ptab;              // e^{-2 pi i n / Lf}
+    const int *deltas, *partner, *slot_q;   // slot_q: momentum of a slot (null: the slot)
+    const SymElem *elem;         // the element inv inverts the momentum (C channel's exchanged half)
+    const int *dinv;
+    int nd, Lq, nc, half, inv;
+    double inv_nk;
+    double2 *out64;
+    float2 *out32;
+};
+
+template <typename C2> __device__ __forceinline__ C2 turn(C2 v, int k)
+{
+    switch (k & 3) {
+    case 0: return v;
+    case 1: return mk(-v.y, v.x);
+    case 2: return mk(-v.x, -v.y);
+    default: return mk(v.y, -v.x);
+    }
+}
+__device__ __forceinline__ double2 wide2(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
+__device__ __forceinline__ double2 wide2(double2 v) { return v; }
+__device__ __forceinline__ void put_f32(float2 *p, float2 v) { *p = v; }
+__device__ __forceinline__ void put_f32(float2 *p, double2 v) { *p = make_float2((float)v.x, (float)v.y); }
+
+// orbital entry S[d][ia][ib] of one slot's half-plane sums
+template <int NS, int CH, typename C2>
+__device__ __forceinline__ C2 gen_entry(const C2 *acc, const FinArgs<C2> &f, int d, int ia, int ib)
 {
     constexpr int NS2 = NS * NS;
-    const int dx = deltas[2 * d], dy = deltas[2 * d + 1];
-    const bool half = dy > 0 || (dy == 0 && dx >= 0);
-    const size_t o = half ? base + ((size_t)d * NS2 + ia) * NS2 + ib : base + ((size_t)partner[d] * NS2 + ib) * NS2 + ia;
-    double re = 0.0, im = 0.0;
-    sum_ranges(acc + o, chunk_stride, nchunk, re, im);
-    return make_double2(re, half ? im : -im);
-}
-
-// blockIdx.y = accumulator slot s (n_slot of them), written at momentum qout[s] (orbit representatives
-// only) or at s.
-template <int NS, typename C2>
-__global__ void loops_gen_finish(const C2 *acc, int nchunk, int n_slot, const int *deltas, int nd, double inv_nk,
-                                 const int *partner, const int *qout, double2 *out64, float2 *out32)
-{
-    constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nd * NS4) return;
-    const int s = blockIdx.y, d = t / NS4, ia = (t / NS2) % NS2, ib = t % NS2;
-    const size_t per = (size_t)nd * NS4;
-    double2 v = gen_value<NS>(acc, (size_t)n_slot * per, nchunk, (size_t)s * per, d, ia, ib, deltas, partner);   // C2 deduced
-    v.x *= inv_nk;
-    v.y *= inv_nk;
-    const size_t o = (size_t)(qout ? qout[s] : s) * per + t;
-    if (out64) out64[o] = v;
-    if (out32) out32[o] = make_float2((float)v.x, (float)v.y);
-}
-
-// Sum of the kx ranges per accumulator slot (fixed order, FP64), before the symmetric gather: the gather
-// reads every slot Nq / n_slot times, so it must read one L2-resident value, not one per range from DRAM.
-// Grid: (elements / 256, slot).
-template <typename C2>
-__global__ void loops_gen_chunk_sum(const C2 *acc, int nchunk, int n_slot, int per, double2 *red)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= per) return;
-    const size_t o = (size_t)blockIdx.y * per + t, stride = (size_t)n_slot * per;
-    double re = 0.0, im = 0.0;
-    sum_ranges(acc + o, stride, nchunk, re, im);
-    red[o] = make_double2(re, im);
-}
-
-// Symmetric variant: blockIdx.y = output momentum q'; qmap[q'] = (accumulator slot of its orbit
-// representative, group element e); thread (d', a', b') reads the representative's (d, src a', src b')
-// (half plane or its Hermitian mirror) and writes i^(qt[a'] - qt[b']) (conj ? conj(v) : v) / Nk.
-template <int NS, typename C2>
-__global__ void loops_gen_finish_sym(const C2 *acc, int nchunk, int n_slot, const int *deltas, int nd,
-                                     double inv_nk, const int *partner, const int2 *qmap, const SymElem *elem,
-                                     const int *dinv, int ch, double2 *out64, float2 *out32)
-{
-    constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nd * NS4) return;
-    const int q2 = blockIdx.y, d2 = t / NS4, a2 = (t / NS2) % NS2, b2 = t % NS2;
-    const int2 ie = qmap[q2];
-    const SymElem &e = elem[ie.y];
-    const size_t per = (size_t)nd * NS4;
-    double2 v = gen_value<NS>(acc, (size_t)n_slot * per, nchunk, (size_t)ie.x * per, dinv[ie.y * nd + d2],
-                              e.src[ch][a2], e.src[ch][b2], deltas, partner);
-    if (e.conj) v.y = -v.y;
-    double2 w;
-    switch ((e.qt[ch][a2] - e.qt[ch][b2]) & 3) {
-    case 0: w = v; break;
-    case 1: w = make_double2(-v.y, v.x); break;
-    case 2: w = make_double2(-v.x, -v.y); break;
-    default: w = make_double2(v.y, -v.x); break;
+    const int dx = f.deltas[2 * d], dy = f.deltas[2 * d + 1];
+    const bool hp = dy > 0 || (dy == 0 && dx >= 0);
+    if (!hp) {   // L(-d)[b][a] = conj(L(d)[a][b])
+        d = f.partner[d];
+        const int t = ia;
+        ia = ib;
+        ib = t;
     }
-    w.x *= inv_nk;
-    w.y *= inv_nk;
-    const size_t o = (size_t)q2 * per + t;
-    out64[o] = w;
-    if (out32) out32[o] = make_float2((float)w.x, (float)w.y);
+    // compact pairs -> (t1 t3), (t2 t4)
+    const int ax = ia / NS, ay = ia % NS, bx = ib / NS, by = ib % NS;
+    const int t1 = CH == 0 ? ay : ax, t2 = CH == 0 ? ax : ay, t3 = CH == 0 ? by : bx, t4 = CH == 0 ? bx : by;
+    const int lr = loop_comp_index<NS>(t1, t3), rr = loop_comp_index<NS>(t2, t4);
+    const int ls = t1 == t3 ? 0 : t1 < t3 ? 1 : -1, rs0 = t2 == t4 ? 0 : t2 < t4 ? 1 : -1, rs = CH == 0 ? rs0 : -rs0;
+    const C2 *o = acc + (size_t)d * NS2 * NS2;
+    C2 v = o[lr * NS2 + rr];
+    if (ls) {
+        const C2 w = o[(lr + 1) * NS2 + rr];   // + i ls w
+        v.x -= ls * w.y;
+        v.y += ls * w.x;
+    }
+    if (rs) {
+        const C2 w = o[lr * NS2 + rr + 1];
+        v.x -= rs * w.y;
+        v.y += rs * w.x;
+    }
+    if (ls && rs) {
+        const C2 w = o[(lr + 1) * NS2 + rr + 1];
+        v.x -= ls * rs * w.x;
+        v.y -= ls * rs * w.y;
+    }
+    if (!hp) v.y = -v.y;
+    return v;
 }
 
-template <typename R, int NS, int TA, int TB, int NDYH, int WHICH>
-cudaError_t launch_gen(tufrg_model *m, const GenArgs<R> &a)
+// Every entry of every slot's loops at the slot's momentum: the sums, the exchanged half, 1/Nk.
+// Grid: (entries / 256, slots).
+template <int NS, int CH, typename R>
+__global__ void __launch_bounds__(256) loops_gen_finish(const __grid_constant__ FinArgs<typename cpx<R>::t> f)
 {
     using C2 = typename cpx<R>::t;
-    constexpr int NS2 = NS * NS;
-    constexpr int NT = (NS2 / TA) * (NS2 / TB);
-    const int threads = ((NT + 31) / 32) * 32;
-    const size_t smem = gen_smem<R, NS, NDYH>(m->Lf);
-    auto kern = loops_gen_kernel<R, NS, TA, TB, NDYH, WHICH>;
+    constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= f.nd * NS4) return;
+    const int s = blockIdx.y, d = t / NS4, ia = (t / NS2) % NS2, ib = t % NS2;
+    const int q = f.slot_q ? f.slot_q[s] : s;
+    const C2 *acc = f.acc + (size_t)s * f.nd * NS4;
+    C2 v = gen_entry<NS, CH>(acc, f, d, ia, ib);
+    if (f.half) {
+        auto swp = [](int a) { return (a % NS) * NS + a / NS; };
+        int d2 = d, k = 0;
+        C2 w;
+        if (CH == 0) {   // e^{-is.Delta} conj(S[b~][a~])
+            w = gen_entry<NS, CH>(acc, f, d, swp(ib), swp(ia));
+            w.y = -w.y;
+        } else {         // V [e^{iu.Delta} S[b~][a~]] V^dagger
+            const SymElem &e = f.elem[f.inv];
+            d2 = f.dinv[f.inv * f.nd + d];
+            w = gen_entry<NS, CH>(acc, f, d2, swp(e.src[1][ib]), swp(e.src[1][ia]));
+            k = e.qt[1][ia] - e.qt[1][ib];
+        }
+        const int n = (((q / f.Lq) * f.deltas[2 * d2] + (q % f.Lq) * f.deltas[2 * d2 + 1]) % f.Lq + f.Lq) % f.Lq * f.nc;
+        C2 p = f.ptab[n];
+        if (CH == 1) p.y = -p.y;
+        w = mk(p.x * w.x - p.y * w.y, p.x * w.y + p.y * w.x);
+        if (CH == 1) {
+            if (f.elem[f.inv].conj) w.y = -w.y;
+            w = turn(w, k);
+        }
+        v.x += w.x;
+        v.y += w.y;
+    }
+    v.x *= R(f.inv_nk);
+    v.y *= R(f.inv_nk);
+    const size_t o = (size_t)q * f.nd * NS4 + t;
+    if (f.out64) f.out64[o] = wide2(v);
+    if (f.out32) put_f32(f.out32 + o, v);
+}
+
+// The momenta that are not orbit representatives: entry (d', a', b') of q' from the representative's (d, src a', src b'),
+// i^(qt[a'] - qt[b']) (conj ? conj(v) : v).  Grid: (entries / 256, momenta).  Reads and writes the same buffers (the
+// representatives' rows are only read).
+template <int NS, typename C2>
+__global__ void __launch_bounds__(256) loops_gen_gather(C2 *L, double2 *out64, int nd, const int2 *qmap, const int *list,
+                                                        const SymElem *elem, const int *dinv, int ch)
+{
+    constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nd * NS4) return;
+    const int q2 = blockIdx.y;
+    const int2 ie = qmap[q2];
+    const int q = list[ie.x];
+    if (q == q2) return;
+    const int d2 = t / NS4, a2 = (t / NS2) % NS2, b2 = t % NS2;
+    const SymElem &e = elem[ie.y];
+    C2 v = L[(size_t)q * nd * NS4 + ((size_t)dinv[ie.y * nd + d2] * NS2 + e.src[ch][a2]) * NS2 + e.src[ch][b2]];
+    if (e.conj) v.y = -v.y;
+    v = turn(v, e.qt[ch][a2] - e.qt[ch][b2]);
+    const size_t o = (size_t)q2 * nd * NS4 + t;
+    L[o] = v;
+    if (sizeof(C2) == sizeof(float2)) out64[o] = wide2(v);
+}
+
+// per instantiation: tile and thread groups.  FP64 tiles are sized for the registers of the column sums; the FP32
+// N_s = 4 case (256 entries) takes 4 x 2 tiles, one warp, and four warps that share the rows.
+template <typename R, int NS> struct Tile;
+template <> struct Tile<double, 6> { static constexpr int A = 3, B = 3, G = 1; };
+template <> struct Tile<double, 4> { static constexpr int A = 2, B = 2, G = 1; };
+template <> struct Tile<float, 6> { static constexpr int A = 4, B = 3, G = 1; };
+template <> struct Tile<float, 4> { static constexpr int A = 4, B = 2, G = 4; };
+
+template <typename R, int NS> constexpr int gen_threads()
+{
+    using T = Tile<R, NS>;
+    return ((NS * NS / T::A) * (NS * NS / T::B) * T::G + 31) / 32 * 32;
+}
+template <typename R, int NS, int NDYH, int WHICH>
+auto gen_kernel() { return loops_gen_kernel<R, NS, Tile<R, NS>::A, Tile<R, NS>::B, Tile<R, NS>::G, NDYH, WHICH>; }
+
+template <typename R, int NS, int NDYH, int WHICH>
+cudaError_t launch_gen(tufrg_model *m, const GenArgs<R> &a)
+{
+    const size_t smem = gen_smem<R, NS, NDYH, Tile<R, NS>::G>();
+    auto kern = gen_kernel<R, NS, NDYH, WHICH>();
     if (smem > 48 * 1024) TUFRG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     PhaseScope ps(m, PH_LOOPS);
-    kern<<<dim3(a.n_slot, m->gen_chunks), threads, smem, m->stream>>>(a);
+    kern<<<dim3(a.n_slot, m->gen_chunks), gen_threads<R, NS>(), smem, m->stream>>>(a);
     return cudaGetLastError();
 }
 
-template <typename R, int NS, int TA, int TB>
+template <typename R, int NS>
 cudaError_t dispatch_gen(tufrg_model *m, const GenArgs<R> &a, int ch)
 {
-    if (a.ndyh <= 3) return ch == 0 ? launch_gen<R, NS, TA, TB, 3, 0>(m, a) : launch_gen<R, NS, TA, TB, 3, 1>(m, a);
-    if (a.ndyh <= 5) return ch == 0 ? launch_gen<R, NS, TA, TB, 5, 0>(m, a) : launch_gen<R, NS, TA, TB, 5, 1>(m, a);
+    if (a.ndyh <= 3) return ch == 0 ? launch_gen<R, NS, 3, 0>(m, a) : launch_gen<R, NS, 3, 1>(m, a);
+    if (a.ndyh <= 5) return ch == 0 ? launch_gen<R, NS, 5, 0>(m, a) : launch_gen<R, NS, 5, 1>(m, a);
     return cudaErrorNotSupported;
 }
 
 template <typename R>
-void fill_args(tufrg_model *m, GenArgs<R> &a)
+cudaError_t run_gen(tufrg_model *m, int ch, bool half, const typename cpx<R>::t *U, const typename FTg<R>::t *ft,
+                    const typename cpx<R>::t *ptab)
 {
+    using C2 = typename cpx<R>::t;
+    GenArgs<R> a{};
+    a.U = U; a.ft = ft; a.ptab = ptab;
+    a.acc = reinterpret_cast<C2 *>(m->d_part);
+    a.thr_factor = sizeof(R) == 4 ? R(1e-2) : R(1e-5);
+    a.Tp = m->d_scal;
+    a.shell_T = m->regulator == TUFRG_REG_MOMENTUM_SHELL ? (R)m->T_reg : R(0);
     a.Lq = m->Lq; a.nc = m->nc; a.Lf = m->Lf; a.nd = m->nd;
     a.ndx = (int)m->dxs.size();
-    int ndyh = 0;
     for (int v : m->dys)
-        if (v >= 0) a.dys[ndyh++] = v;
-    a.ndyh = ndyh;
+        if (v >= 0) a.dys[a.ndyh++] = v;
     for (int i = 0; i < a.ndx; i++) {
         a.dxs[i] = m->dxs[i];
         for (int j = 0; j < GMAXD; j++) {
             a.dslot[i][j] = -1;
-            if (j >= ndyh) continue;
+            if (j >= a.ndyh) continue;
             const int dx = a.dxs[i], dy = a.dys[j];
             if (!(dy > 0 || dx >= 0)) continue;
             for (int d = 0; d < m->nd; d++)
                 if (m->deltas[2 * d] == dx && m->deltas[2 * d + 1] == dy) a.dslot[i][j] = d;
         }
     }
+    a.s_list = m->sym ? m->d_loop_list : nullptr;
+    a.n_slot = m->sym ? m->n_loop_q : m->Nq;
+    a.half = half ? 1 : 0;
+    const int ncol = half ? m->Lf / 2 + 1 : m->Lf;
+    a.kx_len = (ncol + m->gen_chunks - 1) / m->gen_chunks;
+    const size_t n = (size_t)a.n_slot * m->nd * m->ns * m->ns * m->ns * m->ns;
+    TUFRG_CUDA_TRY((m->ns == 6 ? dispatch_gen<R, 6>(m, a, ch) : dispatch_gen<R, 4>(m, a, ch)));
+    if (m->gen_chunks > 1) {
+        PhaseScope ps(m, PH_LOOPRED);
+        loops_gen_chunk_sum<C2><<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(a.acc, m->gen_chunks, n);
+    }
+    return cudaGetLastError();
+}
+
+template <int NS, typename R>
+cudaError_t finish(tufrg_model *m, int ch, int n_slot, const FinArgs<typename cpx<R>::t> &f, bool gather, typename cpx<R>::t *L)
+{
+    constexpr int NS4 = NS * NS * NS * NS;
+    const unsigned gx = (unsigned)((m->nd * NS4 + 255) / 256);
+    PhaseScope ps(m, PH_LOOPRED, gather ? 2 : 1);
+    if (ch == 0) loops_gen_finish<NS, 0, R><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
+    else loops_gen_finish<NS, 1, R><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
+    TUFRG_CUDA_TRY(cudaGetLastError());
+    if (gather)
+        loops_gen_gather<NS><<<dim3(gx, m->Nq), 256, 0, m->stream>>>(L, f.out64, m->nd, m->d_qmap, m->d_loop_list, m->d_sym_elem,
+                                                                    m->d_sym_dinv, ch);
+    return cudaGetLastError();
+}
+
+int gen_ndyh(const tufrg_model *m)
+{
+    int n = 0;
+    for (int v : m->dys) n += v >= 0;
+    return n;
+}
+
+// Resident CTAs per SM of the instantiation the model launches
+template <typename R, int NS>
+int gen_blocks_per_sm(int ndyh)
+{
+    int n = 0;
+    const cudaError_t e =
+        ndyh <= 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gen_kernel<R, NS, 3, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 3, Tile<R, NS>::G>())
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gen_kernel<R, NS, 5, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 5, Tile<R, NS>::G>());
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return (e == cudaSuccess && n > 0) ? n : 1;
 }
 
 }  // namespace
 
 bool loops_gen_supported(const tufrg_model *m)
 {
-    int ndyh = 0;
-    for (int v : m->dys) ndyh += v >= 0;
-    return (m->ns == 4 || m->ns == 6) && (int)m->dxs.size() <= GMAXD && ndyh <= 5 && m->nd <= GMAXND;
-}
-
-namespace {
-
-// Resident CTAs per SM of the instantiation the model launches, and the kx ranges per momentum that
-// fill the GPU best (at least 4 columns per range).
-template <typename R, int NS, int TA, int TB>
-int gen_blocks_per_sm(const tufrg_model *m, int ndyh)
-{
-    constexpr int NS2 = NS * NS, NT = (NS2 / TA) * (NS2 / TB);
-    const int threads = ((NT + 31) / 32) * 32;
-    int n = 0;
-    cudaError_t e = ndyh <= 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops_gen_kernel<R, NS, TA, TB, 3, 0>, threads, gen_smem<R, NS, 3>(m->Lf))
-                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops_gen_kernel<R, NS, TA, TB, 5, 0>, threads, gen_smem<R, NS, 5>(m->Lf));
-    return (e == cudaSuccess && n > 0) ? n : 1;
-}
-
-}  // namespace
-
-size_t gen_red_offset(const tufrg_model *m)
-{
-    const size_t ns2 = (size_t)m->ns * m->ns;
-    return (size_t)m->gen_chunks * m->n_loop_q * m->nd * ns2 * ns2 * sizeof(double2);
+    return (m->ns == 4 || m->ns == 6) && (int)m->dxs.size() <= GMAXD && gen_ndyh(m) <= 5 && m->nd <= GMAXND;
 }
 
 size_t gen_part_bytes(const tufrg_model *m)
 {
     const size_t ns2 = (size_t)m->ns * m->ns;
-    return gen_red_offset(m) + (m->sym ? (size_t)m->n_loop_q * m->nd * ns2 * ns2 * sizeof(double2) : 0);
+    return (size_t)m->gen_chunks * m->n_loop_q * m->nd * ns2 * ns2 * (m->precision == TUFRG_FP64 ? sizeof(double2) : sizeof(float2));
 }
 
+// The kx ranges per momentum that fill the GPU best: the fewest waves of CTAs times columns per range (plus about one
+// column's time of start and end per CTA), up to one column per range within MAX_RANGES accumulators.  With few
+// momenta the short ranges are what fills the SMs: the sums of 28 momenta of the 12 x 12 / 5 x 5 bilayer mesh take 76 us
+// per evaluation, 206 us with at least four columns per range.
 int plan_gen_chunks(const tufrg_model *m)
 {
-    int ndyh = 0;
-    for (int v : m->dys) ndyh += v >= 0;
+    constexpr int MAX_RANGES = 64;
+    const int ndyh = gen_ndyh(m);
     int per_sm;
-    if (m->precision == TUFRG_FP64) per_sm = m->ns == 6 ? gen_blocks_per_sm<double, 6, 2, 3>(m, ndyh) : gen_blocks_per_sm<double, 4, 2, 2>(m, ndyh);
-    else per_sm = m->ns == 6 ? gen_blocks_per_sm<float, 6, 4, 3>(m, ndyh) : gen_blocks_per_sm<float, 4, 2, 2>(m, ndyh);
-    // minimise (waves) x (columns per range): a grid just over one wave doubles the time
+    if (m->precision == TUFRG_FP64) per_sm = m->ns == 6 ? gen_blocks_per_sm<double, 6>(ndyh) : gen_blocks_per_sm<double, 4>(ndyh);
+    else per_sm = m->ns == 6 ? gen_blocks_per_sm<float, 6>(ndyh) : gen_blocks_per_sm<float, 4>(ndyh);
     const long slots = (long)m->sm_count * per_sm;
+    const int ncol = loops2_half_mask(m) == 3 ? m->Lf / 2 + 1 : m->Lf;
     int best = 1;
     double best_cost = 1e300;
-    for (int c = 1; c <= std::min(16, std::max(1, m->Lf / 4)); c++) {
+    for (int c = 1; c <= std::min(MAX_RANGES, ncol); c++) {
         const double waves = std::ceil((double)m->n_loop_q * c / (double)slots);
-        const double cost = waves * std::ceil((double)m->Lf / c);
+        const double cost = waves * (std::ceil((double)ncol / c) + 1.0);
         if (cost < best_cost * 0.999) { best_cost = cost; best = c; }
     }
     return best;
 }
 
-namespace {
-
-template <typename R>
-void fill_chunks(const tufrg_model *m, GenArgs<R> &a)
-{
-    a.s_list = m->sym ? m->d_loop_list : nullptr;
-    a.n_slot = m->sym ? m->n_loop_q : m->Nq;
-    a.kx_len = (m->Lf + m->gen_chunks - 1) / m->gen_chunks;
-}
-
-}  // namespace
-
 cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only)
 {
-    const size_t ns2 = (size_t)m->ns * m->ns, per = (size_t)m->Nq * m->nd * ns2 * ns2;
+    const size_t ns4 = (size_t)m->ns * m->ns * m->ns * m->ns, per = (size_t)m->Nq * m->nd * ns4;
     const int n_slot = m->sym ? m->n_loop_q : m->Nq;
-    const size_t acc_n = (size_t)m->gen_chunks * n_slot * m->nd * ns2 * ns2;
+    const bool fp64 = m->precision == TUFRG_FP64;
     for (int ch = 0; ch < 2; ch++) {
         if (!((channel_mask >> ch) & 1)) continue;
-        const bool fp64 = m->precision == TUFRG_FP64;
-        cudaError_t e;
-        if (m->loops_tc) {
-            // tensor cores: the half-plane sums of every slot are written (not accumulated), one kx range
-            e = launch_loops_tc(m, ch, reinterpret_cast<float2 *>(m->d_part));
-        } else if (fp64) {
-            TUFRG_CUDA_TRY(cudaMemsetAsync(m->d_part, 0, sizeof(double2) * acc_n, m->stream));
-            GenArgs<double> a{};
-            a.U = m->d_U; a.ft = m->d_ft; a.acc = reinterpret_cast<double2 *>(m->d_part); a.thr_factor = 1e-5; a.Tp = m->d_scal;
-            a.shell_T = m->regulator == TUFRG_REG_MOMENTUM_SHELL ? m->T_reg : 0.0;
-            fill_args(m, a);
-            fill_chunks(m, a);
-            e = m->ns == 6 ? dispatch_gen<double, 6, 2, 3>(m, a, ch) : dispatch_gen<double, 4, 2, 2>(m, a, ch);
-        } else {
-            TUFRG_CUDA_TRY(cudaMemsetAsync(m->d_part, 0, sizeof(float2) * acc_n, m->stream));
-            GenArgs<float> a{};
-            a.U = m->d_U32; a.ft = m->d_ft32; a.acc = reinterpret_cast<float2 *>(m->d_part); a.thr_factor = 1e-2f; a.Tp = m->d_scal;
-            a.shell_T = m->regulator == TUFRG_REG_MOMENTUM_SHELL ? (float)m->T_reg : 0.f;
-            fill_args(m, a);
-            fill_chunks(m, a);
-            e = m->ns == 6 ? dispatch_gen<float, 6, 4, 3>(m, a, ch) : dispatch_gen<float, 4, 2, 2>(m, a, ch);
-        }
-        TUFRG_CUDA_TRY(e);
-        PhaseScope ps(m, PH_LOOPRED);
-        double2 *o64 = m->d_Lc + ch * per;
-        float2 *o32 = fp64 ? nullptr : m->d_Lc32 + ch * per;
-        const int n4 = m->nd * (int)(ns2 * ns2);
-        const dim3 grid((n4 + 255) / 256, m->Nq);
-        const double inv_nk = 1.0 / (double)m->Nk;
-        const double2 *a64 = reinterpret_cast<const double2 *>(m->d_part);
-        const float2 *a32 = reinterpret_cast<const float2 *>(m->d_part);
-        const int nc = m->gen_chunks;
-        auto finish = [&](dim3 g, int n_s, const int *qout, double2 *w64, float2 *w32) {
-            if (m->ns == 6 && fp64)
-                loops_gen_finish<6><<<g, 256, 0, m->stream>>>(a64, nc, n_s, m->d_deltas, m->nd, inv_nk, m->d_dpartner, qout, w64, w32);
-            else if (m->ns == 6)
-                loops_gen_finish<6><<<g, 256, 0, m->stream>>>(a32, nc, n_s, m->d_deltas, m->nd, inv_nk, m->d_dpartner, qout, w64, w32);
-            else if (fp64)
-                loops_gen_finish<4><<<g, 256, 0, m->stream>>>(a64, nc, n_s, m->d_deltas, m->nd, inv_nk, m->d_dpartner, qout, w64, w32);
-            else
-                loops_gen_finish<4><<<g, 256, 0, m->stream>>>(a32, nc, n_s, m->d_deltas, m->nd, inv_nk, m->d_dpartner, qout, w64, w32);
+        // the tensor-core kernel's half sums need the init-time list (its groups share their columns)
+        const bool half = ((loops2_half_mask(m) >> ch) & 1) && (!m->loops_tc || m->loop_list_is_reps);
+        if (m->loops_tc) TUFRG_CUDA_TRY(launch_loops_tc(m, ch, half, reinterpret_cast<float2 *>(m->d_part)));
+        else if (fp64) TUFRG_CUDA_TRY(run_gen<double>(m, ch, half, m->d_U, m->d_ft, m->d_lph));
+        else TUFRG_CUDA_TRY(run_gen<float>(m, ch, half, m->d_U32, m->d_ft32, m->d_lph32));
+        auto fill = [&](auto &f) {
+            f.deltas = m->d_deltas;
+            f.partner = m->d_dpartner;
+            f.slot_q = m->sym ? m->d_loop_list : nullptr;
+            f.elem = m->d_sym_elem;
+            f.dinv = m->d_sym_dinv;
+            f.nd = m->nd;
+            f.Lq = m->Lq;
+            f.nc = m->nc;
+            f.half = half ? 1 : 0;
+            f.inv = m->sym_inv;
+            f.inv_nk = 1.0 / (double)m->Nk;
+            // symmetric states: the split path's products read the FP32 loops only
+            f.out64 = reps_only && !fp64 ? nullptr : m->d_Lc + ch * per;
+            f.out32 = fp64 ? nullptr : m->d_Lc32 + ch * per;
         };
-        if (reps_only) {
-            // the representatives at their own momenta; the split path's products read the FP32 loops only
-            finish(dim3((n4 + 255) / 256, n_slot), n_slot, m->d_loop_list, fp64 ? o64 : nullptr, o32);
-        } else if (m->sym) {
-            // the kx ranges summed per representative (same order as the plain finish), then the gather
-            double2 *red = reinterpret_cast<double2 *>(static_cast<char *>(m->d_part) + gen_red_offset(m));
-            const dim3 g1((n4 + 255) / 256, n_slot);
-            if (fp64) loops_gen_chunk_sum<<<g1, 256, 0, m->stream>>>(a64, nc, n_slot, n4, red);
-            else loops_gen_chunk_sum<<<g1, 256, 0, m->stream>>>(a32, nc, n_slot, n4, red);
-            if (m->ns == 6)
-                loops_gen_finish_sym<6><<<grid, 256, 0, m->stream>>>(red, 1, n_slot, m->d_deltas, m->nd, inv_nk, m->d_dpartner,
-                                                                     m->d_qmap, m->d_sym_elem, m->d_sym_dinv, ch, o64, o32);
-            else
-                loops_gen_finish_sym<4><<<grid, 256, 0, m->stream>>>(red, 1, n_slot, m->d_deltas, m->nd, inv_nk, m->d_dpartner,
-                                                                     m->d_qmap, m->d_sym_elem, m->d_sym_dinv, ch, o64, o32);
+        const bool gather = m->sym && !reps_only;
+        if (fp64) {
+            FinArgs<double2> f{};
+            f.acc = reinterpret_cast<const double2 *>(m->d_part);
+            f.ptab = m->d_lph;
+            fill(f);
+            TUFRG_CUDA_TRY((m->ns == 6 ? finish<6, double>(m, ch, n_slot, f, gather, f.out64) : finish<4, double>(m, ch, n_slot, f, gather, f.out64)));
         } else {
-            finish(grid, m->Nq, nullptr, o64, o32);
+            FinArgs<float2> f{};
+            f.acc = reinterpret_cast<const float2 *>(m->d_part);
+            f.ptab = m->d_lph32;
+            fill(f);
+            TUFRG_CUDA_TRY((m->ns == 6 ? finish<6, float>(m, ch, n_slot, f, gather, f.out32) : finish<4, float>(m, ch, n_slot, f, gather, f.out32)));
         }
-        TUFRG_CUDA_TRY(cudaGetLastError());
     }
     return cudaSuccess;
 }

@@ -4,31 +4,43 @@
 // For a transfer momentum s the compact loop is
 //   Lc[Delta][(t1 t3),(t2 t4)] = (1/Nk) sum_k e^{-+ i k.Delta} sum_l rho^l_{t1 t3}(k) T^l_{t2 t4}(s, k)
 // with rho^l_{tt'} = U_{tl} U*_{t'l} at the summation point k and T^l = sum_{l2} w_{l l2} rho'^{l2} at its partner:
-//   C (u = s):  partner k - u, rho' = conj(U_{t2 l2}) U_{t4 l2}, phase e^{-i k.Delta};
+//   C (u = s):  partner k - u, rho' = conj(rho), phase e^{-i k.Delta};
 //   P (s):      the sum runs over the first propagator's momentum k' = s - q (a relabelling of the fine mesh),
-//               partner s - k', rho' = U_{t2 l2} U*_{t4 l2}, phase e^{-i (s - k').Delta} = e^{-i s.Delta} e^{+i k'.Delta}.
+//               partner s - k', rho' = rho, phase e^{-i (s - k').Delta} = e^{-i s.Delta} e^{+i k'.Delta}.
 // Written this way the summation point's projectors do not depend on s, so one operand serves several momenta.
-// With Delta = (dx, dy) the phase separates; per fine-mesh column kx the sum over ky is one complex GEMM
-//   W[(dy, t1 t3)][(s_j, t2 t4)] = sum_{(ky, l)} e^{-+ i ky dy} rho^l_{t1 t3}(kx, ky) * T^l_{t2 t4}(s_j; kx, ky)
-// with M = 3 dy x 36 = 108 rows (padded to 128), N = 3 momenta x 36 = 108 columns (padded to 112) and
-// K = Lf x 6.  It runs as 3xTF32 (hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor memory), the complex
-// product as four real MMA streams (the minus of -Ai Bi by the descriptor's negate-A bit), exactly like the
-// V.L.V products.  The x phases e^{-+ i kx dx} are applied afterwards by loops_tc_xsum over the written columns.
+// Three exact rewritings keep the contraction small:
+//   * rho and T are Hermitian 6 x 6 matrices (the weights are real): each is 36 real numbers (Re and Im of the upper
+//     triangle, the diagonal), so the sums are real; the orbital entries are put together from them at the end
+//     (loops_gen_finish; for C the imaginary parts of rho' change sign there);
+//   * the row phase e^{-+ i ky dy} is a cosine and a sine (dy = 0: one), so for dy >= 0 there are five real row
+//     phases: per fine-mesh column kx the sum over ky is one real GEMM
+//       W[(s_j, c')][(p, c)] = sum_{(ky, l)} T^l_{c'}(s_j; kx, ky) * phi_p(ky) rho^l_c(kx, ky)
+//     with M = 3 momenta x 36 = 108 rows (of 128), N = 5 x 36 = 180 columns (of 192), K = Lf x 6;
+//   * exchanging the two propagators maps k to s - k, so one point of every pair {k, s - k} suffices where the channel
+//     allows it (P always, C with a symmetry that inverts the momentum; see k_loops2.cu): columns
+//     kx = hx + c, 2 hx = sx (mod Lf), c up to Lf / 2.  The momenta of a group share sx and hence their columns.
+// It runs as 3xTF32 (hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor memory).  The x phases e^{-+ i kx dx} are
+// applied afterwards by loops_tc_xsum over the written columns.
+// Why this shape: complex arithmetic on both sides needs 4 real products of 108 x 36 per (momentum, k, band), the real
+// basis one of 180 x 36, 2.4 times less, and half of the operand values to form, split and store.  A launch over the 153
+// orbit representatives of the 32 x 32 / 6 x 6 workload takes 2.81 ms per channel (7.25 ms in complex arithmetic over the
+// whole mesh); the MMAs alone are about 1.0 ms of it, the producers' instructions bound it.
 //
-// The left operand (the phased projectors, four TF32 planes) lives in tensor memory: the producers write it with
-// tcgen05.st, and the MMAs read it from there, so shared memory carries only the right operand.
+// The left operand (T, two TF32 planes) lives in tensor memory: the producers write it with tcgen05.st, and the MMAs
+// read it from there, so shared memory carries only the right operand.
 // One persistent CTA per SM walks its (momentum group, column) items.  Warp roles:
-//   warps 0-15  producers: per stage (4 ky rows = K of 24) they stage the raw eigenvectors and Fermi entries of
-//               the 4 summation points and their 12 partners (cp.async, two stages ahead, four buffers), form
-//               the pair weights and row phases, then write the operands' TF32 hi/lo planes: A into tensor memory
-//               (lane = row), B into shared memory in the K-major core-matrix layout (each thread one ky row of
-//               one row of A and of B);
-//   warp 16     TMEM allocation and the MMA issuer (one thread): 36 MMAs per stage;
-//   warps 17-20 epilogue: tensor memory -> W in global memory (coalesced, row index fastest).
-// Two stage buffers (mbarriers full / empty) so operand generation and MMAs overlap; one tensor-memory accumulator
-// (mbarriers acc_full / acc_empty): the next column's MMAs start once the epilogue has read the previous one.  Every wait is bounded; on time-out
-// the kernel raises the error flag, every role stops, the MMAs in flight are waited for (bounded), the
-// cp.async copies drained, and the tensor memory is freed.
+//   warps 0-15  producers, thread (ky row kb of the stage's four, operand row r): every thread holds the next stage's
+//               inputs in registers (projector values of its rows and the Fermi entries of one pair weight, loaded
+//               straight from the L2-resident tables one stage ahead); per stage it forms its pair weight into shared
+//               memory, then row r of T at its ky row (six bands from the weights of its pair of points) and its one or
+//               two phased projector rows, and writes the TF32 hi / lo parts: T into tensor memory (lane = row), the
+//               projectors into shared memory in the K-major core-matrix layout;
+//   warp 16     TMEM allocation and the MMA issuer (one thread): 9 MMAs of 128 x 192 x 8 per stage; then its quarter of
+//               the previous column's epilogue (20 warps leave every thread 96 registers, 21 would leave 80);
+//   warps 17-19 epilogue: tensor memory -> W in global memory (coalesced, row index fastest).
+// Two stage buffers (mbarriers full / empty) and two tensor-memory accumulators (acc_full / acc_empty).  Every wait is
+// bounded; on time-out the kernel raises the error flag, every role stops, the MMAs in flight are waited for (bounded)
+// and the tensor memory is freed.
 #include <algorithm>
 #include <cmath>
 
@@ -38,40 +50,39 @@
 namespace tufrg {
 namespace {
 
-constexpr int NS = 6, NS2 = 36, NS4 = NS2 * NS2;
-constexpr int GRP = 3;                       // transfer momenta per item (column blocks of B)
-constexpr int NDYM = 3;                      // non-negative y components of the bond differences (row blocks of A)
-constexpr int ROWS = NDYM * NS2;             // 108 rows used
-constexpr int COLS = GRP * NS2;              // 108 columns used
+constexpr int NS = 6, NS2 = 36;
+constexpr int GRP = 3;                       // transfer momenta per item (row blocks of the left operand)
+constexpr int NDYM = 3;                      // non-negative y components of the bond differences
+constexpr int NPH = 2 * NDYM - 1;            // real row phases: 1, then cos and sin per dy > 0
+constexpr int ROWS = GRP * NS2;              // 108 rows used
+constexpr int COLS = NPH * NS2;              // 180 columns used
 constexpr int TM = 128;                      // MMA M
-constexpr int TN = 112;                      // MMA N: COLS padded to a multiple of 16
+constexpr int TN = 192;                      // MMA N: COLS padded to a multiple of 16
 constexpr int KB = 4;                        // ky rows per stage
 constexpr int KST = KB * NS;                 // K per stage: 24 = three MMA K-steps of 8
 constexpr int NPROD = 512;                   // producer threads, warps 0-15: thread (ky row kb, operand row r)
-constexpr int MMA_WARP = 16;                 // warps 17-20: epilogue
-constexpr int NTHREADS = 21 * 32;
-constexpr int NRAW = 4;                      // raw staging buffers (stage n + 2 is fetched while n is formed)
+constexpr int MMA_WARP = 16;                 // it and warps 17-19: epilogue
+constexpr int NTHREADS = 20 * 32;
 constexpr unsigned B_PLANE = TN * KST * 4;   // bytes per plane and stage of the right operand (shared memory)
-constexpr unsigned STAGE_BYTES = 4 * B_PLANE;   // planes: Re hi, Re lo, Im hi, Im lo
-// tensor memory: accumulator Re at [0, TN), Im at [128, 128 + TN); left operand of stage b at 256 + 128 b, plane p
-// at + 32 p (K = 24 columns used)
-constexpr unsigned ACC_IM = 128, A_COL0 = 256, A_STAGE_COLS = 128, A_PLANE_COLS = 32;
-constexpr int NPTS = KB * (1 + GRP);         // raw points per stage: 4 summation points, then [j][kb] partners
-constexpr int CU = NS2 * 8 / 16, CF = NS * 16 / 16, CP = CU + CF;   // 16-byte chunks per point: U, Fermi entries
-constexpr unsigned RAW_U = NPTS * NS2 * 8, RAW_BYTES = RAW_U + NPTS * NS * 16;
-constexpr unsigned TMEM_COLS = 512;
-constexpr unsigned SW_BYTES = GRP * KB * NS * 8 * 4;         // pair weights, rows padded to 8
-constexpr size_t SMEM_BYTES = 2 * (size_t)STAGE_BYTES + NRAW * (size_t)RAW_BYTES + SW_BYTES + KB * NDYM * 8 + 4 * NPTS * 4;
+constexpr unsigned STAGE_BYTES = 2 * B_PLANE;   // planes: hi, lo
+// tensor memory: accumulator b at [TN b, TN b + TN); left operand of stage b at A_COL0 + 64 b, planes hi, lo at + 32 p
+// (K = 24 columns used)
+constexpr unsigned A_COL0 = 2 * TN, A_STAGE_COLS = 64, A_PLANE_COLS = 32, TMEM_COLS = 512;
+static_assert(A_COL0 + 2 * A_STAGE_COLS <= TMEM_COLS, "tensor memory budget");
+constexpr int NW = GRP * KB * NS2;           // pair weights per stage
+static_assert(NW <= NPROD, "one pair weight per producer thread");
 
 struct LtArgs {
-    const float2 *U;            // [Nk][NS][NS] eigenvectors (row orbital, column band), FP32
+    const float *rho;           // [Nk][36][6] real projector components (loop_comp), band fastest
     const FermiEntry32 *ft;     // [Nk][NS] (e, g, g') at the flow scale, or (e, f, h) with the momentum shell
-    float2 *W;                  // [n_groups][Lf][COLS][ROWS] column sums
+    float *W;                   // [n_groups][ncol][COLS][ROWS] column sums
     const int *s_list;          // slot -> transfer momentum (null: the slot is the momentum)
-    int n_slot, n_groups, n_items;
+    const int *grp;             // [n_groups][GRP] slots of a group, -1: none (null: slot g GRP + j)
+    int n_slot, n_items;
     int Lq, nc, Lf, spc;        // spc: stages per column
-    int ndyh;
-    int dys[NDYM];
+    int ncol, half;             // columns per group; half: kx = hx + c, else kx = c
+    int dy1, dy2;               // y differences of the phases 1..4, modulo Lf (0 where absent)
+    const float2 *ptab;         // e^{-2 pi i n / Lf}
     const double *Tp;           // device flow scale
     float thr_factor, shell_T;
     int *err;
@@ -81,19 +92,6 @@ __device__ __forceinline__ int wrapm(int v, int L)
 {
     v %= L;
     return v < 0 ? v + L : v;
-}
-
-
-// six consecutive complex values from shared memory (16-byte aligned) as three 16-byte loads
-__device__ __forceinline__ void ld6(const float2 *p, float2 (&v)[NS])
-{
-    const float4 *q = reinterpret_cast<const float4 *>(p);
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-        const float4 t = q[i];
-        v[2 * i] = make_float2(t.x, t.y);
-        v[2 * i + 1] = make_float2(t.z, t.w);
-    }
 }
 
 // the loop weight of one band pair (gen_pair_weight) with the FP32 fast division of the split two-band kernel
@@ -113,64 +111,45 @@ __device__ __forceinline__ float tc_pair_weight(float e1, float g1, float gp1, f
 // 2^-10 |x|, so hi + lo keeps FP32 accuracy through the three products of 3xTF32
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
-// writes 4 consecutive K values of one row of a plane group (Re hi, Re lo, Im hi, Im lo) as TF32 hi / lo parts
-__device__ __forceinline__ void put4(float *planes, unsigned plane_floats, int off, float2 v0, float2 v1, float2 v2, float2 v3)
-{
-    float4 h, l;
-    h = make_float4(tf32_trunc(v0.x), tf32_trunc(v1.x), tf32_trunc(v2.x), tf32_trunc(v3.x));
-    l = make_float4(v0.x - h.x, v1.x - h.y, v2.x - h.z, v3.x - h.w);
-    *reinterpret_cast<float4 *>(planes + 0 * plane_floats + off) = h;
-    *reinterpret_cast<float4 *>(planes + 1 * plane_floats + off) = l;
-    h = make_float4(tf32_trunc(v0.y), tf32_trunc(v1.y), tf32_trunc(v2.y), tf32_trunc(v3.y));
-    l = make_float4(v0.y - h.x, v1.y - h.y, v2.y - h.z, v3.y - h.w);
-    *reinterpret_cast<float4 *>(planes + 2 * plane_floats + off) = h;
-    *reinterpret_cast<float4 *>(planes + 3 * plane_floats + off) = l;
-}
-
-// two consecutive K values (an even k) of one row
-__device__ __forceinline__ void put2(float *planes, unsigned plane_floats, int off, float2 v0, float2 v1)
-{
-    float2 h, l;
-    h = make_float2(tf32_trunc(v0.x), tf32_trunc(v1.x));
-    l = make_float2(v0.x - h.x, v1.x - h.y);
-    *reinterpret_cast<float2 *>(planes + 0 * plane_floats + off) = h;
-    *reinterpret_cast<float2 *>(planes + 1 * plane_floats + off) = l;
-    h = make_float2(tf32_trunc(v0.y), tf32_trunc(v1.y));
-    l = make_float2(v0.y - h.x, v1.y - h.y);
-    *reinterpret_cast<float2 *>(planes + 2 * plane_floats + off) = h;
-    *reinterpret_cast<float2 *>(planes + 3 * plane_floats + off) = l;
-}
-
-// the six K values kb * 6 + l (l = 0..5) of row r of an R-row operand: 4 + 2 or 2 + 4 along the 4-wide groups
-__device__ __forceinline__ void put6(float *planes, unsigned plane_floats, int r, int kb, int R, const float2 (&v)[NS])
+// the six K values kb * 6 + l (l = 0..5) of row r of the right operand, hi and lo planes: 4 + 2 or 2 + 4 along the
+// 4-wide groups
+__device__ __forceinline__ void put6(float *planes, int r, int kb, const float (&v)[NS])
 {
     const int k0 = 6 * kb;
+    float h[NS], l[NS];
+#pragma unroll
+    for (int i = 0; i < NS; i++) {
+        h[i] = tf32_trunc(v[i]);
+        l[i] = v[i] - h[i];
+    }
+    float *p0 = planes, *p1 = planes + B_PLANE / 4;
     if ((kb & 1) == 0) {
-        put4(planes, plane_floats, tc::core_off(r, k0, R), v[0], v[1], v[2], v[3]);
-        put2(planes, plane_floats, tc::core_off(r, k0 + 4, R), v[4], v[5]);
+        const int a = tc::core_off(r, k0, TN), b = tc::core_off(r, k0 + 4, TN);
+        *reinterpret_cast<float4 *>(p0 + a) = make_float4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<float2 *>(p0 + b) = make_float2(h[4], h[5]);
+        *reinterpret_cast<float4 *>(p1 + a) = make_float4(l[0], l[1], l[2], l[3]);
+        *reinterpret_cast<float2 *>(p1 + b) = make_float2(l[4], l[5]);
     } else {
-        put2(planes, plane_floats, tc::core_off(r, k0, R), v[0], v[1]);
-        put4(planes, plane_floats, tc::core_off(r, k0 + 2, R), v[2], v[3], v[4], v[5]);
+        const int a = tc::core_off(r, k0, TN), b = tc::core_off(r, k0 + 2, TN);
+        *reinterpret_cast<float2 *>(p0 + a) = make_float2(h[0], h[1]);
+        *reinterpret_cast<float4 *>(p0 + b) = make_float4(h[2], h[3], h[4], h[5]);
+        *reinterpret_cast<float2 *>(p1 + a) = make_float2(l[0], l[1]);
+        *reinterpret_cast<float4 *>(p1 + b) = make_float4(l[2], l[3], l[4], l[5]);
     }
 }
 
-// the six K values kb * 6 + l of this lane's row of the left operand into tensor memory: four planes (Re hi, Re lo,
-// Im hi, Im lo, truncation split) at columns col0 + 32 p + 6 kb + l, as a 4 + 2 (kb even) or 2 + 4 (kb odd) column
-// split so that every store starts at a multiple of its width; warp-collective (every lane of the warp)
-__device__ __forceinline__ void put6_tmem(unsigned col0, int kb, const float2 (&v)[NS])
+// the six K values kb * 6 + l of this lane's row of the left operand into tensor memory, hi and lo planes, as a 4 + 2
+// (kb even) or 2 + 4 (kb odd) column split so that every store starts at a multiple of its width; warp-collective
+__device__ __forceinline__ void put6_tmem(unsigned col0, int kb, const float (&v)[NS])
 {
     const unsigned c = col0 + 6 * kb;
-    const bool even = (kb & 1) == 0;
 #pragma unroll
-    for (int p = 0; p < 4; p++) {
+    for (int p = 0; p < 2; p++) {
         float t[NS];
 #pragma unroll
-        for (int l = 0; l < NS; l++) {
-            const float x = p < 2 ? v[l].x : v[l].y;
-            t[l] = (p & 1) ? x - tf32_trunc(x) : tf32_trunc(x);
-        }
+        for (int l = 0; l < NS; l++) t[l] = p ? v[l] - tf32_trunc(v[l]) : tf32_trunc(v[l]);
         const unsigned cp = c + p * A_PLANE_COLS;
-        if (even) {
+        if ((kb & 1) == 0) {
             tc::tmem_st4(cp, t[0], t[1], t[2], t[3]);
             tc::tmem_st2(cp + 4u, t[4], t[5]);
         } else {
@@ -180,27 +159,31 @@ __device__ __forceinline__ void put6_tmem(unsigned col0, int kb, const float2 (&
     }
 }
 
+__device__ __forceinline__ void ld_six(const float *p, float (&v)[NS])   // six consecutive floats, 8-byte aligned
+{
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const float2 t = __ldg(reinterpret_cast<const float2 *>(p) + i);
+        v[2 * i] = t.x;
+        v[2 * i + 1] = t.y;
+    }
+}
+
 __device__ __forceinline__ void bar_producers() { asm volatile("bar.sync 1, %0;" ::"n"(NPROD) : "memory"); }
 
+inline size_t lt_smem_bytes(int Lf) { return 2 * (size_t)STAGE_BYTES + 2 * NW * sizeof(float) + 2 * sizeof(float) * Lf; }
+
 template <int WHICH>
-__global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(LtArgs a)
+__global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(const __grid_constant__ LtArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    // stage buffer b at smem + b STAGE_BYTES, raw buffer b at smem + 2 STAGE_BYTES + b RAW_BYTES
-    auto stage = [&](int b) { return smem + (size_t)b * STAGE_BYTES; };
-    auto raw = [&](int b) { return smem + 2 * (size_t)STAGE_BYTES + (size_t)b * RAW_BYTES; };
-    float *sW = reinterpret_cast<float *>(smem + 2 * STAGE_BYTES + NRAW * RAW_BYTES);   // [GRP][KB][NS][8]
-    float2 *sPh = reinterpret_cast<float2 *>(smem + 2 * STAGE_BYTES + NRAW * RAW_BYTES + SW_BYTES);   // [KB][NDYM]
-    int *sPt = reinterpret_cast<int *>(sPh + KB * NDYM);                                   // [4][NPTS]
+    float *sW = reinterpret_cast<float *>(smem + 2 * STAGE_BYTES);   // [2][GRP][KB][l2][l1]
+    float *ptab = sW + 2 * NW;                                       // [Lf] cos, [Lf] sin of 2 pi n / Lf
     __shared__ __align__(8) unsigned long long full[2], empty[2], accf[2], acce[2], done;
     __shared__ unsigned tmem_base;
-    __shared__ int abort_flag, stop;
+    __shared__ int abort_flag, stop[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // kernel arguments used inside the lambdas below, copied to registers (no local copy of the struct)
-    const int Lf = a.Lf, Lq = a.Lq, nc = a.nc, spc = a.spc, n_slot = a.n_slot;
-    const int *const s_list = a.s_list;
-    const float2 *const Ug = a.U;
-    const FermiEntry32 *const Fg = a.ft;
+    const int Lf = a.Lf, spc = a.spc;
 
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&tmem_base)),
@@ -213,20 +196,22 @@ __global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(LtArgs a)
             tc::mbar_init(tc::smem_u32(&empty[b]), 1);
             tc::mbar_init(tc::smem_u32(&accf[b]), 1);
             tc::mbar_init(tc::smem_u32(&acce[b]), 128);
+            stop[b] = 0;
         }
         tc::mbar_init(tc::smem_u32(&done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
-        stop = 0;
     }
-    // padding rows of B (108..111) are zero in both stage buffers for the whole kernel (the padding lanes of A are
-    // written as zeros with every stage)
-    for (int i = tid; i < 2 * 4 * (TN - COLS) * KST; i += NTHREADS) {
-        const int per_buf = 4 * (TN - COLS) * KST, b = i / per_buf, r0 = i % per_buf;
-        const int plane = r0 / ((TN - COLS) * KST), r1 = r0 % ((TN - COLS) * KST);
-        const int row = r1 / KST, k = r1 % KST;
-        float *base = reinterpret_cast<float *>(stage(b));
-        base[plane * (B_PLANE / 4) + tc::core_off(COLS + row, k, TN)] = 0.f;
+    for (int n = tid; n < Lf; n += NTHREADS) {
+        const float2 p = a.ptab[n];
+        ptab[n] = p.x;
+        ptab[Lf + n] = -p.y;
+    }
+    // the padding columns of the right operand (rows 180..191 of its planes) are zero in both stage buffers for the whole
+    // kernel (the padding lanes of the left operand are written as zeros with every stage)
+    for (int i = tid; i < 4 * (TN - COLS) * KST; i += NTHREADS) {
+        const int pl = i / ((TN - COLS) * KST), r = i % ((TN - COLS) * KST);
+        reinterpret_cast<float *>(smem)[pl * (B_PLANE / 4) + tc::core_off(COLS + r / KST, r % KST, TN)] = 0.f;
     }
     tc::fence_smem_async();
     tc::fence_before();
@@ -234,103 +219,139 @@ __global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(LtArgs a)
     tc::fence_after();
     const unsigned tmem = tmem_base;
     const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int n_stages = my_items * a.spc;
+    const int n_stages = my_items * spc;
 
     if (warp < MMA_WARP) {
         // ------------------------------------------------------------------ producers
         const bool shell = a.shell_T > 0.f;
         const float lam = shell ? (float)(*a.Tp) : 0.f;
         const float thr = a.thr_factor * (shell ? a.shell_T : (float)(*a.Tp));
-        const int kb = tid >> 7, r = tid & 127;   // ky row of the stage (warp-uniform) and operand row
-        // fine-mesh index of raw point p of stage n (-1 when its row or momentum does not exist); evaluated once
-        // per stage and point, three stages ahead, into sPt[n % 4]
-        auto point = [&](int n, int p) {
-            const int item = (int)blockIdx.x + (n / spc) * (int)gridDim.x, st = n % spc;
-            const int g = item / Lf, kx = item % Lf;
-            const int pk = p & (KB - 1), ky = st * KB + pk;
-            if (n >= n_stages || ky >= Lf) return -1;
-            if (p < KB) return kx * Lf + ky;
-            const int slot = g * GRP + (p - KB) / KB;
-            if (slot >= n_slot) return -1;
-            const int s = s_list ? s_list[slot] : slot;
-            const int sx = (s / Lq) * nc, sy = (s % Lq) * nc;
-            return WHICH == 0 ? wrapm(sx - kx, Lf) * Lf + wrapm(sy - ky, Lf) : wrapm(kx - sx, Lf) * Lf + wrapm(ky - sy, Lf);
+        const int kb = tid >> 7, r = tid & 127;            // ky row of the stage (warp-uniform) and operand row
+        const int rj = r / NS2, rc = r % NS2;              // left operand: momentum of the group, component
+        const bool has_a = r < ROWS, has_b1 = r + 128 < COLS;   // right operand rows r and (r < 52) r + 128
+        const int p0 = r / NS2, p1 = (r + 128) / NS2, c1 = (r + 128) % NS2;   // their phases and components
+        const bool has_w = tid < NW;                       // this thread's pair weight (wj, wk, l2, l1)
+        const int wj = tid / (KB * NS2), wk = (tid / NS2) % KB, wl2 = (tid % NS2) / NS, wl1 = tid % NS;
+        // phase of a row: 0 -> 1 (the cosine of zero), 1 / 3 -> cos, 2 / 4 -> sin of ky dy
+        const int step0 = p0 == 0 ? 0 : p0 < 3 ? a.dy1 : a.dy2, step1 = p1 < 3 ? a.dy1 : a.dy2;
+        const int adv0 = (KB * step0) % Lf, adv1 = (KB * step1) % Lf, beg0 = (kb * step0) % Lf, beg1 = (kb * step1) % Lf;
+        const float *tab0 = ptab + (p0 == 0 || (p0 & 1) ? 0 : Lf), *tab1 = ptab + ((p1 & 1) ? 0 : Lf);
+        const float *w_a = sW + (rj * KB + kb) * NS2;
+        // cursor of the stage that is loaded next (one stage ahead of the one being formed): table offsets of this
+        // thread's points, stepping by KB rows (the partner's by -KB for P), with wrap
+        constexpr unsigned ROW = NS2 * NS;                 // floats of one fine k
+        const unsigned col_len = (unsigned)Lf * ROW, fcol_len = (unsigned)Lf * NS;
+        int f_item = (int)blockIdx.x, f_st = 0, kyA = 0, kyW = 0, i0 = 0, i1 = 0;
+        unsigned oA = 0, oB = 0, oF1 = 0, oF2 = 0;
+        bool okW = false;
+        auto slot_q = [&](int g, int j) {   // transfer momentum of group member j (-1 where there is none)
+            const int slot = a.grp ? a.grp[g * GRP + j] : (g * GRP + j < a.n_slot ? g * GRP + j : -1);
+            if (slot < 0) return -1;
+            return a.s_list ? a.s_list[slot] : slot;
         };
-        auto fetch = [&](int n) {
-            if (n < n_stages) {
-                unsigned char *rb = raw(n % NRAW);
-                const int *pts = sPt + (n & 3) * NPTS;
-                for (int i = tid; i < NPTS * CP; i += NPROD) {
-                    const int p = i / CP, c = i % CP, k = pts[p];
-                    if (k < 0) {   // a row or momentum that does not exist: zeros (no operand value then depends on it)
-                        unsigned char *d = c < CU ? rb + (size_t)p * NS2 * 8 + 16 * c : rb + RAW_U + (size_t)p * NS * 16 + 16 * (c - CU);
-                        *reinterpret_cast<float4 *>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-                        continue;
-                    }
-                    if (c < CU) cp_async16(rb + (size_t)p * NS2 * 8 + 16 * c, reinterpret_cast<const char *>(Ug + (size_t)k * NS2) + 16 * c);
-                    else cp_async16(rb + RAW_U + (size_t)p * NS * 16 + 16 * (c - CU),
-                                    reinterpret_cast<const char *>(Fg + (size_t)k * NS) + 16 * (c - CU));
-                }
-            }
-            cp_async_commit();
+        auto column = [&]() {   // the cursor's column: points of this thread's rows at its first ky rows
+            const int g = f_item / a.ncol, c = f_item - g * a.ncol;
+            const int q0 = slot_q(g, 0), qa = has_a ? slot_q(g, rj) : -1, qw = has_w ? slot_q(g, wj) : -1;
+            const int sx0 = (q0 / a.Lq) * a.nc;
+            const int hx = !(sx0 & 1) ? sx0 / 2 : (Lf & 1) ? (sx0 + Lf) / 2 : (sx0 + 1) / 2;
+            int kx = a.half ? hx + c : c;
+            if (kx >= Lf) kx -= Lf;
+            const int ua = qa < 0 ? q0 : qa, uw = qw < 0 ? q0 : qw;
+            const int xa = ua / a.Lq, xw = uw / a.Lq;
+            const int sxa = xa * a.nc, sya = (ua - xa * a.Lq) * a.nc, sxw = xw * a.nc, syw = (uw - xw * a.Lq) * a.nc;
+            int kxA = WHICH == 0 ? sxa - kx : kx - sxa, kxW = WHICH == 0 ? sxw - kx : kx - sxw;
+            if (kxA < 0) kxA += Lf;
+            if (kxW < 0) kxW += Lf;
+            kyA = WHICH == 0 ? wrapm(sya - kb, Lf) : wrapm(kb - sya, Lf);
+            kyW = WHICH == 0 ? wrapm(syw - wk, Lf) : wrapm(wk - syw, Lf);
+            oA = ((unsigned)(kxA * Lf + kyA) * NS2 + rc) * NS;
+            oB = ((unsigned)(kx * Lf + kb) * NS2) * NS;
+            oF1 = (unsigned)(kx * Lf + wk) * NS + wl1;
+            oF2 = (unsigned)(kxW * Lf + kyW) * NS + wl2;
+            okW = qw >= 0;
+            i0 = beg0;
+            i1 = beg1;
         };
-        if (tid < 3 * NPTS) sPt[tid] = point(tid / NPTS, tid % NPTS);
-        bar_producers();
-        fetch(0);
-        fetch(1);
-        int item = (int)blockIdx.x, st = 0;   // item and stage within the column of stage n
-        for (int n = 0; n < n_stages; n++) {
-            const int g = item / Lf;
-            const int buf = n & 1;
-            // raw buffer (n + 2) % 4 was last read by stage n - 2, which every producer has finished
-            fetch(n + 2);
-            cp_async_wait<2>();
-            bar_producers();          // raw data of stage n landed; stage n - 1 fully formed (sW, sPh, sPt free)
-            const float2 *rU = reinterpret_cast<const float2 *>(raw(n % NRAW));
-            const FermiEntry32 *rF = reinterpret_cast<const FermiEntry32 *>(raw(n % NRAW) + RAW_U);
-            // pair weights [j][kb][l1][8] (rows padded to 8), the row phases [kb][dy] and the points of stage n + 3
-            if (tid < GRP * KB * NS * NS) {
-                const int i = tid, j = i / (KB * NS * NS), wk = (i / (NS * NS)) % KB, l1 = (i / NS) % NS, l2 = i % NS;
-                const int pp = KB + j * KB + wk;
-                float w = 0.f;
-                if (st * KB + wk < Lf && g * GRP + j < n_slot) {
-                    const FermiEntry32 f1 = rF[wk * NS + l1], f2 = rF[pp * NS + l2];
-                    w = tc_pair_weight<WHICH>(f1.e, f1.g, f1.gp, f2.e, f2.g, f2.gp, thr, lam);
-                }
-                sW[((j * KB + wk) * NS + l1) * 8 + l2] = w;
-            } else if (tid >= NPROD - KB * NDYM) {
-                const int i = tid - (NPROD - KB * NDYM), pk = i / NDYM, dyi = i % NDYM, ky = st * KB + pk;
-                const int dyv = dyi == 0 ? a.dys[0] : dyi == 1 ? a.dys[1] : a.dys[2];
-                float sn = 0.f, cs = 0.f;
-                if (ky < Lf && dyi < a.ndyh) sincospif(2.0f * (float)wrapm(ky * dyv, Lf) / (float)Lf, &sn, &cs);
-                sPh[i] = make_float2(cs, WHICH == 0 ? sn : -sn);   // zero for missing rows and y components
-            } else if (tid >= NPROD - KB * NDYM - NPTS) {
-                const int p = tid - (NPROD - KB * NDYM - NPTS);
-                sPt[((n + 3) & 3) * NPTS + p] = point(n + 3, p);
+        struct In {
+            float A[NS], B0[NS], B1[NS];
+            float4 f1, f2;
+            float ph0, ph1;
+            bool ok;
+        };
+        const float4 *ft = reinterpret_cast<const float4 *>(a.ft);
+        auto load = [&](In &x) {   // the cursor's stage into registers; then the cursor steps
+            // (rows past the column in its last stage are read from the tables' padding or the next column: their
+            // weights are zero, so T is)
+            if (has_a) ld_six(a.rho + oA, x.A);
+            ld_six(a.rho + oB + rc * NS, x.B0);
+            if (has_b1) ld_six(a.rho + oB + c1 * NS, x.B1);
+            if (has_w) {
+                x.f1 = __ldg(ft + oF1);
+                x.f2 = __ldg(ft + oF2);
             }
-            if (tid == 0) stop = *(volatile int *)&abort_flag;
+            x.ok = okW && f_st * KB + wk < Lf;   // the weights of a row or momentum that does not exist are zero
+            x.ph0 = tab0[i0];
+            x.ph1 = tab1[i1];
+            if (++f_st == spc) {
+                f_st = 0;
+                f_item += (int)gridDim.x;
+                if (f_item < a.n_items) column();
+                return;
+            }
+            oB += KB * ROW;
+            oF1 += KB * NS;
+            if (WHICH == 0) {
+                kyA -= KB;
+                kyW -= KB;
+                oA -= KB * ROW;
+                oF2 -= KB * NS;
+                while (kyA < 0) { kyA += Lf; oA += col_len; }
+                while (kyW < 0) { kyW += Lf; oF2 += fcol_len; }
+            } else {
+                kyA += KB;
+                kyW += KB;
+                oA += KB * ROW;
+                oF2 += KB * NS;
+                while (kyA >= Lf) { kyA -= Lf; oA -= col_len; }
+                while (kyW >= Lf) { kyW -= Lf; oF2 -= fcol_len; }
+            }
+            i0 += adv0;
+            i1 += adv1;
+            if (i0 >= Lf) i0 -= Lf;
+            if (i1 >= Lf) i1 -= Lf;
+        };
+        // one stage in buffer buf (n & 1): weights, T and projector rows from x; the next stage's inputs into y
+        auto form = [&](int n, const int buf, In &x, In &y) -> bool {
+            if (has_w)
+                sW[buf * NW + tid] = x.ok ? tc_pair_weight<WHICH>(x.f1.x, x.f1.y, x.f1.z, x.f2.x, x.f2.y, x.f2.z, thr, lam) : 0.f;
+            if (tid == 0) stop[buf] = *(volatile int *)&abort_flag;
+            // the stage's weights are complete; weights and stop flag have two buffers, so that the next stage's may be
+            // written while this stage's are read (those of the stage after next come behind the next barrier)
             bar_producers();
-            if (stop) break;   // every producer reads the same value: they leave the loop together
-            float *pb = reinterpret_cast<float *>(stage(buf));
-            float2 va[NS];
+            if (stop[buf]) return false;   // every producer reads the same value: they leave the loop together
+            if (n + 1 < n_stages) load(y);
+            // T row r = (s_j, component): T^{l1} = sum_l2 w_{l1 l2} rho'^{l2} (zero in the padding lanes)
+            float2 t2[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            if (has_a) {
+                const float4 *wr = reinterpret_cast<const float4 *>(w_a + buf * NW);
 #pragma unroll
-            for (int l = 0; l < NS; l++) va[l] = make_float2(0.f, 0.f);   // the padding lanes of A (rows 108..127)
-            if (r < ROWS) {
-                // A row r = (dy, t1 t3): e^{-+ i ky dy} rho^l_{t1 t3}(k) at K = kb * 6 + l (zero for a missing row: the
-                // phase is zero there, and so are the raw values of a point that does not exist)
-                const int dyi = r / NS2, ab = r % NS2, t1 = ab / NS, t3 = ab % NS;
-                const float2 ph = sPh[kb * NDYM + dyi];
-                float2 u[NS], w[NS];
-                ld6(rU + kb * NS2 + t1 * NS, u);
-                ld6(rU + kb * NS2 + t3 * NS, w);
-#pragma unroll
-                for (int l = 0; l < NS; l++) {
-                    // rho = u conj(w) = u w.x + (u.y, -u.x) w.y;  ph rho = rho ph.x + (-rho.y, rho.x) ph.y
-                    const float2 rho = __ffma2_rn(make_float2(u[l].y, -u[l].x), make_float2(w[l].y, w[l].y),
-                                                  __fmul2_rn(u[l], make_float2(w[l].x, w[l].x)));
-                    va[l] = __ffma2_rn(make_float2(-rho.y, rho.x), make_float2(ph.y, ph.y),
-                                       __fmul2_rn(rho, make_float2(ph.x, ph.x)));
+                for (int h = 0; h < 3; h++) {   // two partner bands: weights (l2, l1 = 0..5), (l2 + 1, l1 = 0..5)
+                    const float4 w0 = wr[3 * h], w1 = wr[3 * h + 1], w2 = wr[3 * h + 2];
+                    const float2 u = make_float2(x.A[2 * h], x.A[2 * h]), v = make_float2(x.A[2 * h + 1], x.A[2 * h + 1]);
+                    t2[0] = __ffma2_rn(make_float2(w0.x, w0.y), u, t2[0]);
+                    t2[1] = __ffma2_rn(make_float2(w0.z, w0.w), u, t2[1]);
+                    t2[2] = __ffma2_rn(make_float2(w1.x, w1.y), u, t2[2]);
+                    t2[0] = __ffma2_rn(make_float2(w1.z, w1.w), v, t2[0]);
+                    t2[1] = __ffma2_rn(make_float2(w2.x, w2.y), v, t2[1]);
+                    t2[2] = __ffma2_rn(make_float2(w2.z, w2.w), v, t2[2]);
                 }
+            }
+            const float t[NS] = {t2[0].x, t2[0].y, t2[1].x, t2[1].y, t2[2].x, t2[2].y};
+            // phased projector rows
+#pragma unroll
+            for (int l = 0; l < NS; l++) {
+                x.B0[l] *= x.ph0;
+                x.B1[l] *= x.ph1;
             }
             // the MMAs that read this stage (tensor-memory A, shared-memory B) two stages ago must be complete before
             // it is overwritten
@@ -344,127 +365,110 @@ __global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(LtArgs a)
                     atomicExch(&abort_flag, 1);
                     atomicExch(a.err, 1);
                 }
-            } else {
-                tc::fence_after();
-                // A: this warp's 32 lanes (rows) of the stage's tensor-memory columns, every lane (also padding)
-                put6_tmem(tmem + ((unsigned)((warp & 3) * 32) << 16) + A_COL0 + buf * A_STAGE_COLS, kb, va);
-                if (r < ROWS) {
-                    // B row r = (s_j, t2 t4): T^l_{t2 t4} = sum_l2 w_{l l2} rho'^{l2}_{t2 t4} at K = kb * 6 + l (the
-                    // weights of a missing row or momentum are zero)
-                    const int j = r / NS2, cd = r % NS2, t2 = cd / NS, t4 = cd % NS, pp = KB + j * KB + kb;
-                    float2 x[NS], y[NS], vb[NS];
-                    ld6(rU + pp * NS2 + t2 * NS, x);
-                    ld6(rU + pp * NS2 + t4 * NS, y);
-                    float2 rho[NS];
-#pragma unroll
-                    for (int l2 = 0; l2 < NS; l2++)
-                        rho[l2] = WHICH == 0
-                                      // x conj(y) = x y.x + (x.y, -x.x) y.y
-                                      ? __ffma2_rn(make_float2(x[l2].y, -x[l2].x), make_float2(y[l2].y, y[l2].y),
-                                                   __fmul2_rn(x[l2], make_float2(y[l2].x, y[l2].x)))
-                                      // conj(x) y = y x.x + (y.y, -y.x) x.y
-                                      : __ffma2_rn(make_float2(y[l2].y, -y[l2].x), make_float2(x[l2].y, x[l2].y),
-                                                   __fmul2_rn(y[l2], make_float2(x[l2].x, x[l2].x)));
-#pragma unroll
-                    for (int l1 = 0; l1 < NS; l1++) {
-                        const float4 w0 = *reinterpret_cast<const float4 *>(sW + ((j * KB + kb) * NS + l1) * 8);
-                        const float2 w1 = *reinterpret_cast<const float2 *>(sW + ((j * KB + kb) * NS + l1) * 8 + 4);
-                        const float wl[NS] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y};
-                        float2 t = __fmul2_rn(make_float2(wl[0], wl[0]), rho[0]);
-#pragma unroll
-                        for (int l2 = 1; l2 < NS; l2++) t = __ffma2_rn(make_float2(wl[l2], wl[l2]), rho[l2], t);
-                        vb[l1] = t;
-                    }
-                    put6(pb, B_PLANE / 4, r, kb, TN, vb);
-                }
-                tc::tmem_wait_st();
-                tc::fence_smem_async();
-                tc::fence_before();
-                tc::mbar_arrive(tc::smem_u32(&full[buf]));
+                return true;
             }
-            if (++st == spc) {
-                st = 0;
-                item += (int)gridDim.x;
-            }
+            tc::fence_after();
+            put6_tmem(tmem + ((unsigned)((warp & 3) * 32) << 16) + A_COL0 + buf * A_STAGE_COLS, kb, t);
+            float *pb = reinterpret_cast<float *>(smem + buf * STAGE_BYTES);
+            put6(pb, r, kb, x.B0);
+            if (has_b1) put6(pb, r + 128, kb, x.B1);
+            tc::tmem_wait_st();
+            tc::fence_smem_async();
+            tc::fence_before();
+            tc::mbar_arrive(tc::smem_u32(&full[buf]));
+            return true;
+        };
+        In in0, in1;
+#pragma unroll
+        for (int l = 0; l < NS; l++) in0.B1[l] = in1.B1[l] = 0.f;
+        if (n_stages > 0) {
+            column();
+            load(in0);
         }
-        cp_async_wait<0>();
-    } else if (warp == MMA_WARP) {
-        // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const unsigned id = tc::idesc_tf32(TM, TN, false), idn = tc::idesc_tf32(TM, TN, true);
-            bool ok = true;
-            int n = 0;
-            for (int col = 0; col < my_items && ok; col++) {
-                // the accumulator must have been read by the epilogue of the previous column
-                if (col >= 1 && !tc::mbar_wait_or_abort(tc::smem_u32(&acce[0]), (col - 1) & 1, &abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after();
-                const unsigned tr = tmem, ti = tmem + ACC_IM;
-                for (int st = 0; st < a.spc; st++, n++) {
-                    const int b = n & 1;
-                    if (!tc::mbar_wait_or_abort(tc::smem_u32(&full[b]), (n >> 1) & 1, &abort_flag)) { ok = false; break; }
-                    tc::fence_after();
-                    const unsigned sb = tc::smem_u32(stage(b)), ta = tmem + A_COL0 + b * A_STAGE_COLS;
-#pragma unroll
-                    for (int kk = 0; kk < KST / 8; kk++) {
-                        const unsigned bo = kk * 2 * (TN / 8) * 128;
-                        // A planes in tensor memory: K-step kk = 8 columns of each plane
-                        const unsigned arh = ta + 0 * A_PLANE_COLS + 8 * kk, arl = ta + 1 * A_PLANE_COLS + 8 * kk;
-                        const unsigned aih = ta + 2 * A_PLANE_COLS + 8 * kk, ail = ta + 3 * A_PLANE_COLS + 8 * kk;
-                        const unsigned long long brh = tc::smem_desc(sb + 0 * B_PLANE + bo, TN), brl = tc::smem_desc(sb + 1 * B_PLANE + bo, TN);
-                        const unsigned long long bih = tc::smem_desc(sb + 2 * B_PLANE + bo, TN), bil = tc::smem_desc(sb + 3 * B_PLANE + bo, TN);
-                        const unsigned first = (st == 0 && kk == 0) ? 0u : 1u;
-                        tc::mma_tf32_ta(tr, arh, brh, id, first);  tc::mma_tf32_ta(tr, arh, brl, id, 1u);  tc::mma_tf32_ta(tr, arl, brh, id, 1u);
-                        tc::mma_tf32_ta(tr, aih, bih, idn, 1u);    tc::mma_tf32_ta(tr, aih, bil, idn, 1u); tc::mma_tf32_ta(tr, ail, bih, idn, 1u);
-                        tc::mma_tf32_ta(ti, arh, bih, id, first);  tc::mma_tf32_ta(ti, arh, bil, id, 1u);  tc::mma_tf32_ta(ti, arl, bih, id, 1u);
-                        tc::mma_tf32_ta(ti, aih, brh, id, 1u);     tc::mma_tf32_ta(ti, aih, brl, id, 1u);  tc::mma_tf32_ta(ti, ail, brh, id, 1u);
-                    }
-                    tc::commit(tc::smem_u32(&empty[b]));
-                }
-                if (ok) tc::commit(tc::smem_u32(&accf[0]));
-            }
-            if (!ok) {
+        for (int n = 0; n < n_stages; n += 2) {
+            if (!form(n, 0, in0, in1)) break;
+            if (n + 1 < n_stages && !form(n + 1, 1, in1, in0)) break;
+        }
+    } else {
+        // ------------------------------------------------------------------ MMA issuer (warp 16) and epilogue
+        const int qw = warp & 3, row = qw * 32 + lane;
+        const unsigned lane_off = (unsigned)(qw * 32) << 16;
+        auto fail = [&]() {
+            if (lane == 0) {
                 atomicExch(&abort_flag, 1);
                 atomicExch(a.err, 1);
             }
-            tc::commit(tc::smem_u32(&done));   // completion of every MMA issued above
-        }
-        __syncwarp();
-    } else {
-        // ------------------------------------------------------------------ epilogue: tensor memory -> W
-        const int qw = warp & 3, row = qw * 32 + lane;
-        const unsigned lane_off = (unsigned)(qw * 32) << 16;
-        for (int col = 0; col < my_items; col++) {
+        };
+        // this warp's rows of a finished column: tensor memory -> W
+        auto drain = [&](int col) -> bool {
+            const int ab = col & 1;
             int ok = 1;
-            if (lane == 0) ok = tc::mbar_wait_or_abort(tc::smem_u32(&accf[0]), col & 1, &abort_flag) ? 1 : 0;
+            if (lane == 0) ok = tc::mbar_wait_or_abort(tc::smem_u32(&accf[ab]), (col >> 1) & 1, &abort_flag) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) {
-                if (lane == 0) {
-                    atomicExch(&abort_flag, 1);
-                    atomicExch(a.err, 1);
-                }
-                break;
-            }
+            if (!ok) return false;
             tc::fence_after();
-            const int item = (int)blockIdx.x + col * (int)gridDim.x, g = item / Lf, kx = item % Lf;
-            float2 *Wc = a.W + ((size_t)g * Lf + kx) * COLS * ROWS;
-            for (int c0 = 0; c0 < TN; c0 += 8) {
-                unsigned vr[8], vi[8];
-                tc::tmem_ld8(tmem + lane_off + (unsigned)c0, vr);
-                tc::tmem_ld8(tmem + lane_off + ACC_IM + (unsigned)c0, vi);
+            const int item = (int)blockIdx.x + col * (int)gridDim.x;
+            float *Wc = a.W + (size_t)item * COLS * ROWS + row;
+            for (int c0 = 0; c0 < COLS; c0 += 8) {
+                unsigned v[8];
+                tc::tmem_ld8(tmem + ab * TN + lane_off + (unsigned)c0, v);
                 tc::tmem_wait_ld();
                 if (row < ROWS) {
 #pragma unroll
-                    for (int jj = 0; jj < 8; jj++) {
-                        const int j = c0 + jj;
-                        if (j < COLS) Wc[(size_t)j * ROWS + row] = make_float2(__uint_as_float(vr[jj]), __uint_as_float(vi[jj]));
-                    }
+                    for (int i = 0; i < 8; i++)
+                        if (c0 + i < COLS) Wc[(size_t)(c0 + i) * ROWS] = __uint_as_float(v[i]);
                 }
             }
             tc::fence_before();
-            tc::mbar_arrive(tc::smem_u32(&acce[0]));
+            tc::mbar_arrive(tc::smem_u32(&acce[ab]));
+            return true;
+        };
+        // the MMAs of one column (one thread)
+        auto issue = [&](int col) -> bool {
+            const int ab = col & 1;
+            // the accumulator must have been read by the epilogue of the column before the previous one
+            if (col >= 2 && !tc::mbar_wait_or_abort(tc::smem_u32(&acce[ab]), ((col >> 1) - 1) & 1, &abort_flag)) return false;
+            tc::fence_after();
+            const unsigned id = tc::idesc_tf32(TM, TN, false), d = tmem + ab * TN;
+            int n = col * spc;
+            for (int st = 0; st < spc; st++, n++) {
+                const int b = n & 1;
+                if (!tc::mbar_wait_or_abort(tc::smem_u32(&full[b]), (n >> 1) & 1, &abort_flag)) return false;
+                tc::fence_after();
+                const unsigned sb = tc::smem_u32(smem + b * STAGE_BYTES), ta = tmem + A_COL0 + b * A_STAGE_COLS;
+#pragma unroll
+                for (int kk = 0; kk < KST / 8; kk++) {
+                    const unsigned bo = kk * 2 * (TN / 8) * 128;
+                    const unsigned ah = ta + 8 * kk, al = ah + A_PLANE_COLS;   // K-step kk = 8 columns of each plane
+                    const unsigned long long bh = tc::smem_desc(sb + bo, TN), bl = tc::smem_desc(sb + B_PLANE + bo, TN);
+                    tc::mma_tf32_ta(d, ah, bh, id, (st == 0 && kk == 0) ? 0u : 1u);
+                    tc::mma_tf32_ta(d, ah, bl, id, 1u);
+                    tc::mma_tf32_ta(d, al, bh, id, 1u);
+                }
+                tc::commit(tc::smem_u32(&empty[b]));
+            }
+            tc::commit(tc::smem_u32(&accf[ab]));
+            return true;
+        };
+        if (warp == MMA_WARP) {
+            bool ok = true;
+            for (int col = 0; col <= my_items && ok; col++) {
+                if (col < my_items) {
+                    int y = 1;
+                    if (lane == 0) y = issue(col) ? 1 : 0;
+                    ok = __shfl_sync(0xffffffffu, y, 0);
+                }
+                if (ok && col > 0) ok = drain(col - 1);
+            }
+            if (!ok) fail();
+            if (lane == 0) tc::commit(tc::smem_u32(&done));   // completion of every MMA issued above
+            __syncwarp();
+        } else {
+            for (int col = 0; col < my_items; col++)
+                if (!drain(col)) {
+                    fail();
+                    break;
+                }
         }
     }
     __syncthreads();
@@ -477,85 +481,109 @@ __global__ void __launch_bounds__(NTHREADS, 1) loops_tc_kernel(LtArgs a)
     }
 }
 
+// Real projector components of every fine k and band, in the order of loop_comp: rho[k][c][l].
+__global__ void loops_rho_kernel(const double2 *U, size_t n, float *rho)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // over Nk * 36 * 6
+    if (i >= n) return;
+    const int l = (int)(i % NS), c = (int)((i / NS) % NS2);
+    const size_t k = i / (NS * NS2);
+    int t, tp;
+    bool im;
+    loop_comp<NS>(c, t, tp, im);
+    const double2 u = U[k * NS2 + t * NS + l], v = U[k * NS2 + tp * NS + l];
+    rho[i] = (float)(im ? u.y * v.x - u.x * v.y : u.x * v.x + u.y * v.y);   // Im or Re of u conj(v)
+}
+
 struct XsArgs {
-    const float2 *W;            // [n_groups][Lf][COLS][ROWS]
-    float2 *acc;                // [n_slot][nd][NS2][NS2] half-plane entries written
-    const int *s_list;
-    int n_slot, n_groups, Lq, nc, Lf, nd, ndx, ndyh;
-    int dxs[9], dys[NDYM];
-    int dslot[9][NDYM];         // [dx index][dy index] -> delta index of the half plane, or -1
+    const float *W;             // [n_groups][ncol][COLS][ROWS]
+    float2 *acc;                // [n_slot][nd][36][36] half-plane entries written
+    const int *s_list, *grp;
+    int n_slot, n_groups, Lq, nc, Lf, nd, ndxh, ndyh, ncol, half;
+    int dxm[4];                 // positive dx modulo Lf
+    int dxs[5], dys[NDYM];      // non-negative dx and dy
+    int dslot[9][NDYM];         // [4 + signed dx index][dy index] -> delta index of the half plane, or -1
+    const float2 *ptab;
 };
 
-// x phases and the P-channel momentum phase: acc[slot][d][ra][cb] = sum_kx e^{-+ i kx dx} W[g][kx][j][r]
-// (times e^{-i s.Delta} for P), one thread per (group, column j, row r), r fastest.
+// x phases and the P-channel momentum phase: with C, S the column sums of the cosine and sine row phases,
+//   F[d][c][c'] = sum_kx (cx C - sx S) +- i (sx C + cx S)   (upper sign P, lower sign C; times e^{-i s.Delta} for P),
+// the sums of cx C, sx S, sx C, cx S serving dx and -dx; a column that is its own partner (half sums) enters with weight
+// 1/2.  One thread per (group, dy, component c, row (j, c')), rows fastest; eight columns' loads in flight.
 template <int WHICH>
-__global__ void loops_tc_xsum(XsArgs x)
+__global__ void __launch_bounds__(256) loops_tc_xsum(const __grid_constant__ XsArgs x)
 {
     extern __shared__ float2 ptab[];   // [Lf] e^{-2 pi i n / Lf}
     const int Lf = x.Lf;
-    for (int n = threadIdx.x; n < Lf; n += blockDim.x) {
-        float sn, cs;
-        sincospif(2.0f * (float)n / (float)Lf, &sn, &cs);
-        ptab[n] = make_float2(cs, -sn);
-    }
+    for (int n = threadIdx.x; n < Lf; n += blockDim.x) ptab[n] = x.ptab[n];
     __syncthreads();
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)x.n_groups * COLS * ROWS) return;
-    const int r = (int)(idx % ROWS), j = (int)((idx / ROWS) % COLS), g = (int)(idx / ((size_t)ROWS * COLS));
-    const int dyi = r / NS2, ab = r % NS2;
-    const int slot = g * GRP + j / NS2, cd = j % NS2;
-    if (dyi >= x.ndyh || slot >= x.n_slot) return;
-    float2 acc[9];
-    int ix[9], inc[9];
+    if (idx >= (size_t)x.n_groups * x.ndyh * NS2 * ROWS) return;
+    const int r = (int)(idx % ROWS), c = (int)((idx / ROWS) % NS2), dyi = (int)((idx / (ROWS * NS2)) % x.ndyh);
+    const int g = (int)(idx / ((size_t)ROWS * NS2 * x.ndyh));
+    const int j = r / NS2, slot = x.grp ? x.grp[g * GRP + j] : (g * GRP + j < x.n_slot ? g * GRP + j : -1);
+    if (slot < 0) return;
+    const int s = x.s_list ? x.s_list[slot] : slot, sx = (s / x.Lq) * x.nc, sy = (s % x.Lq) * x.nc;
+    const int hx = !x.half ? 0 : !(sx & 1) ? sx / 2 : (Lf & 1) ? (sx + Lf) / 2 : (sx + 1) / 2;
+    const bool none = x.half && (sx & 1) && !(Lf & 1);   // no self-paired column, one column less
+    const int ncol = none ? Lf / 2 : x.ncol;
+    const int fix0 = x.half && !none ? 0 : -1, fix1 = x.half && !none && !(Lf & 1) ? Lf / 2 : -1;
+    const size_t stride = (size_t)COLS * ROWS;
+    const float *wc = x.W + (size_t)g * x.ncol * stride + (size_t)((dyi == 0 ? 0 : 2 * dyi - 1) * NS2 + c) * ROWS + r;
+    const float *ws = wc + (size_t)NS2 * ROWS;   // the sine rows (dy > 0)
+    float c0 = 0.f, s0 = 0.f, cC[4], sS[4], sC[4], cS[4];
+    int ix[4];
 #pragma unroll
-    for (int xi = 0; xi < 9; xi++) {
-        acc[xi] = make_float2(0.f, 0.f);
-        ix[xi] = 0;
-        inc[xi] = xi < x.ndx ? ((x.dxs[xi] % Lf) + Lf) % Lf : 0;
+    for (int i = 0; i < 4; i++) {
+        cC[i] = sS[i] = sC[i] = cS[i] = 0.f;
+        ix[i] = i + 1 < x.ndxh ? (int)(((long)hx * x.dxm[i]) % Lf) : 0;
     }
-    const float2 *w = x.W + (size_t)g * Lf * COLS * ROWS + (size_t)j * ROWS + r;
-    constexpr int UB = 8;   // columns loaded ahead (independent loads in flight)
-    for (int kx0 = 0; kx0 < Lf; kx0 += UB) {
-        float2 vb[UB];
-#pragma unroll
-        for (int u = 0; u < UB; u++) vb[u] = kx0 + u < Lf ? w[(size_t)(kx0 + u) * COLS * ROWS] : make_float2(0.f, 0.f);
+    constexpr int UB = 8;
+    for (int k0 = 0; k0 < ncol; k0 += UB) {
+        float vc[UB], vs[UB];
 #pragma unroll
         for (int u = 0; u < UB; u++) {
-            if (kx0 + u >= Lf) break;
-            const float2 v = vb[u];
+            const bool in = k0 + u < ncol;
+            vc[u] = in ? wc[(size_t)(k0 + u) * stride] : 0.f;
+            vs[u] = in && dyi > 0 ? ws[(size_t)(k0 + u) * stride] : 0.f;
+        }
 #pragma unroll
-            for (int xi = 0; xi < 9; xi++) {
-                if (xi >= x.ndx) break;
-                float2 p = ptab[ix[xi]];
-                if (WHICH == 0) p.y = -p.y;
-                acc[xi].x = fmaf(p.x, v.x, fmaf(-p.y, v.y, acc[xi].x));
-                acc[xi].y = fmaf(p.x, v.y, fmaf(p.y, v.x, acc[xi].y));
-                ix[xi] += inc[xi];
-                if (ix[xi] >= Lf) ix[xi] -= Lf;
+        for (int u = 0; u < UB; u++) {
+            if (k0 + u >= ncol) break;
+            const float f = k0 + u == fix0 || k0 + u == fix1 ? 0.5f : 1.f;
+            const float C = f * vc[u], S = f * vs[u];
+            c0 += C;
+            s0 += S;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                if (i + 1 >= x.ndxh) break;
+                const float2 p = ptab[ix[i]];   // (cos, -sin)
+                cC[i] = fmaf(p.x, C, cC[i]);
+                sS[i] = fmaf(-p.y, S, sS[i]);
+                sC[i] = fmaf(-p.y, C, sC[i]);
+                cS[i] = fmaf(p.x, S, cS[i]);
+                ix[i] += x.dxm[i];
+                if (ix[i] >= Lf) ix[i] -= Lf;
             }
         }
     }
-    int sx = 0, sy = 0;
-    if (WHICH == 0) {
-        const int s = x.s_list ? x.s_list[slot] : slot;
-        sx = (s / x.Lq) * x.nc;
-        sy = (s % x.Lq) * x.nc;
-    }
-    const int t1 = ab / NS, t3 = ab % NS, t2 = cd / NS, t4 = cd % NS;
-    const int ra = WHICH == 0 ? t2 * NS + t1 : t1 * NS + t2;
-    const int cb = WHICH == 0 ? t4 * NS + t3 : t3 * NS + t4;
-#pragma unroll
-    for (int xi = 0; xi < 9; xi++) {
-        if (xi >= x.ndx) break;
-        const int di = x.dslot[xi][dyi];
-        if (di < 0) continue;
-        float2 v = acc[xi];
+    auto put = [&](int xi, float re, float im) {   // xi: signed dx index
+        const int d = x.dslot[4 + xi][dyi];
+        if (d < 0) return;
+        float2 v = make_float2(re, WHICH == 0 ? im : -im);
         if (WHICH == 0) {
-            // e^{-i s.Delta}: index (sx dx + sy dy) mod Lf of the table
-            const float2 p = ptab[(int)(((long long)sx * x.dxs[xi] + (long long)sy * x.dys[dyi]) % Lf + Lf) % Lf];
+            const int dx = xi < 0 ? -x.dxs[-xi] : x.dxs[xi];
+            const float2 p = ptab[(int)(((long long)sx * dx + (long long)sy * x.dys[dyi]) % Lf + Lf) % Lf];
             v = make_float2(p.x * v.x - p.y * v.y, p.x * v.y + p.y * v.x);
         }
-        x.acc[((size_t)slot * x.nd + di) * NS4 + ra * NS2 + cb] = v;
+        x.acc[(((size_t)slot * x.nd + d) * NS2 + c) * NS2 + r % NS2] = v;
+    };
+    put(0, c0, s0);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        if (i + 1 >= x.ndxh) break;
+        put(i + 1, cC[i] - sS[i], sC[i] + cS[i]);
+        put(-(i + 1), cC[i] + sS[i], cS[i] - sC[i]);
     }
 }
 
@@ -568,69 +596,106 @@ bool loops_tc_supported(const tufrg_model *m)
     return m->precision == TUFRG_SPLIT32 && m->ns == NS && ndyh <= NDYM && (int)m->dxs.size() <= 9 && m->Lf <= 4096;
 }
 
+// Groups of at most GRP list positions whose momenta share q_x (their half sums then run over the same columns).
+std::vector<int> loops_tc_groups(const std::vector<int> &q_of_slot, int Lq)
+{
+    std::vector<std::vector<int>> by(Lq);
+    for (size_t i = 0; i < q_of_slot.size(); i++) by[q_of_slot[i] / Lq].push_back((int)i);
+    std::vector<int> g;
+    for (auto &v : by)
+        for (size_t i = 0; i < v.size(); i += GRP)
+            for (size_t j = 0; j < GRP; j++) g.push_back(i + j < v.size() ? v[i + j] : -1);
+    return g;
+}
+
+// columns of the sums: a list of momenta in any order (no groups) runs over the whole mesh
+static int tc_cols(const tufrg_model *m, bool half) { return half ? m->Lf / 2 + 1 : m->Lf; }
+
 size_t loops_tc_w_bytes(const tufrg_model *m)
 {
-    const int n_slot = m->sym ? m->n_loop_q : m->Nq;
-    const size_t n_groups = (size_t)(n_slot + GRP - 1) / GRP;
-    return n_groups * m->Lf * COLS * ROWS * sizeof(float2);
+    const size_t n_slot = m->sym ? m->n_loop_q : m->Nq;
+    const size_t listed = (n_slot + GRP - 1) / GRP * m->Lf;                            // a shard's list: the whole mesh
+    const size_t grouped = (size_t)m->n_tc_groups * tc_cols(m, m->sym_inv >= 0);       // (without inversion C is not halved)
+    return std::max(listed, grouped) * COLS * ROWS * sizeof(float);
+}
+
+cudaError_t launch_loops_rho(tufrg_model *m)
+{
+    const size_t n = (size_t)m->Nk * NS2 * NS;
+    loops_rho_kernel<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(m->d_U, n, m->d_rho);
+    return cudaGetLastError();
 }
 
 // Loop column sums of one channel on the tensor cores, then the x phases into the accumulator slots of the
-// multi-orbital path (one kx range): acc[slot][d][a][b] for the half-plane d.
-cudaError_t launch_loops_tc(tufrg_model *m, int ch, float2 *acc)
+// multi-orbital path (one kx range): acc[slot][d][c][c'] for the half-plane d, real components (loop_comp).
+cudaError_t launch_loops_tc(tufrg_model *m, int ch, bool half, float2 *acc)
 {
+    const int *grp = m->loop_list_is_reps ? m->d_tc_grp : nullptr;
     LtArgs a{};
-    a.U = m->d_U32;
+    a.rho = m->d_rho;
     a.ft = m->d_ft32;
-    a.W = m->d_loop_w;
+    a.W = reinterpret_cast<float *>(m->d_loop_w);
     a.s_list = m->sym ? m->d_loop_list : nullptr;
+    a.grp = grp;
     a.n_slot = m->sym ? m->n_loop_q : m->Nq;
-    a.n_groups = (a.n_slot + GRP - 1) / GRP;
-    a.n_items = a.n_groups * m->Lf;
+    const int n_groups = grp ? m->n_tc_groups : (a.n_slot + GRP - 1) / GRP;
+    a.half = half ? 1 : 0;
+    a.ncol = tc_cols(m, half);
+    a.n_items = n_groups * a.ncol;
     a.Lq = m->Lq;
     a.nc = m->nc;
     a.Lf = m->Lf;
     a.spc = (m->Lf + KB - 1) / KB;
-    int ndyh = 0;
+    XsArgs x{};
+    std::vector<int> dxh;
     for (int v : m->dys)
-        if (v >= 0) a.dys[ndyh++] = v;
-    a.ndyh = ndyh;
+        if (v >= 0) x.dys[x.ndyh++] = v;
+    for (int v : m->dxs)
+        if (v >= 0) dxh.push_back(v);
+    a.dy1 = x.ndyh > 1 ? x.dys[1] % m->Lf : 0;
+    a.dy2 = x.ndyh > 2 ? x.dys[2] % m->Lf : 0;
+    a.ptab = m->d_lph32;
     a.Tp = m->d_scal;
     a.thr_factor = 1e-2f;
     a.shell_T = m->regulator == TUFRG_REG_MOMENTUM_SHELL ? (float)m->T_reg : 0.f;
     a.err = m->d_err;
     auto kern = ch == 0 ? loops_tc_kernel<0> : loops_tc_kernel<1>;
-    TUFRG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    const size_t smem_k = lt_smem_bytes(m->Lf);
+    TUFRG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_k));
     {
         PhaseScope ps(m, PH_LOOPS);
-        kern<<<std::min(a.n_items, m->sm_count), NTHREADS, SMEM_BYTES, m->stream>>>(a);
+        kern<<<std::min(a.n_items, m->sm_count), NTHREADS, smem_k, m->stream>>>(a);
         TUFRG_CUDA_TRY(cudaGetLastError());
     }
-    XsArgs x{};
-    x.W = m->d_loop_w;
+    x.W = a.W;
     x.acc = acc;
     x.s_list = a.s_list;
+    x.grp = grp;
     x.n_slot = a.n_slot;
-    x.n_groups = a.n_groups;
+    x.n_groups = n_groups;
     x.Lq = m->Lq;
     x.nc = m->nc;
     x.Lf = m->Lf;
     x.nd = m->nd;
-    x.ndx = (int)m->dxs.size();
-    x.ndyh = ndyh;
-    for (int i = 0; i < ndyh; i++) x.dys[i] = a.dys[i];
-    for (int i = 0; i < x.ndx; i++) {
-        x.dxs[i] = m->dxs[i];
+    x.ncol = a.ncol;
+    x.half = a.half;
+    x.ptab = m->d_lph32;
+    x.ndxh = (int)dxh.size();
+    for (int i = 0; i < x.ndxh; i++) {
+        x.dxs[i] = dxh[i];
+        if (i > 0) x.dxm[i - 1] = dxh[i] % m->Lf;
+    }
+    for (int i = 0; i < 9; i++)
         for (int jy = 0; jy < NDYM; jy++) {
             x.dslot[i][jy] = -1;
-            if (jy >= ndyh) continue;
-            const int dx = x.dxs[i], dy = x.dys[jy];
+            const int xi = i - 4;
+            if (jy >= x.ndyh || std::abs(xi) >= x.ndxh) continue;
+            const int dx = xi < 0 ? -dxh[-xi] : dxh[xi], dy = x.dys[jy];
             if (!(dy > 0 || dx >= 0)) continue;
             for (int d = 0; d < m->nd; d++)
                 if (m->deltas[2 * d] == dx && m->deltas[2 * d + 1] == dy) x.dslot[i][jy] = d;
         }
-    }
-    const size_t n = (size_t)a.n_groups * COLS * ROWS;
+    const size_t n = (size_t)n_groups * x.ndyh * NS2 * ROWS;
     const size_t smem = sizeof(float2) * (size_t)m->Lf;
     auto xk = ch == 0 ? loops_tc_xsum<0> : loops_tc_xsum<1>;
     if (smem > 48 * 1024) TUFRG_CUDA_TRY(cudaFuncSetAttribute(xk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

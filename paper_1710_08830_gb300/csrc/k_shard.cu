@@ -90,6 +90,7 @@ cudaError_t launch_loops_list(tufrg_model *m, int mask, const int *d_list, int n
     const bool sym0 = m->sym;
     int *list0 = m->d_loop_list;
     const int n0 = m->n_loop_q;
+    m->loop_list_is_reps = false;
     cudaError_t e = cudaSuccess;
     for (int c0 = 0; c0 < n && e == cudaSuccess; c0 += cap) {
         m->sym = true;
@@ -100,6 +101,7 @@ cudaError_t launch_loops_list(tufrg_model *m, int mask, const int *d_list, int n
     m->sym = sym0;
     m->d_loop_list = list0;
     m->n_loop_q = n0;
+    m->loop_list_is_reps = true;
     return e;
 }
 

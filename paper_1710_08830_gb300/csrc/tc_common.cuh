@@ -8,7 +8,10 @@
 namespace tufrg {
 namespace tc {
 
-constexpr unsigned long long WAIT_LIMIT = 1ull << 22;   // polls of one bounded mbarrier wait
+// polls of one bounded mbarrier wait, each suspended for up to WAIT_NS (about a second in all): a waiting warp then leaves
+// the issue slots to the others
+constexpr unsigned long long WAIT_LIMIT = 1ull << 21;
+constexpr unsigned WAIT_NS = 500;
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -42,8 +45,8 @@ __device__ __forceinline__ unsigned idesc_tf32(int M, int N, bool neg_a)
 __device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity)
 {
     unsigned done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity), "r"(WAIT_NS) : "memory");
     return done != 0;
 }
 

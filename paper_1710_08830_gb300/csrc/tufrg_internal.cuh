@@ -99,6 +99,31 @@ struct SymElem {
     int qt[2][SYM_MAXNS2];
 };
 
+// A Hermitian N x N matrix as N^2 real components: for the pairs t < t' in lexicographic order Re and Im of its (t, t')
+// entry, then the diagonal.  loop_comp: the entry of component c; loop_comp_index: the component of Re (t, t') (Im
+// follows it off the diagonal).
+template <int N> __host__ __device__ constexpr int loop_comp_index(int t, int tp)
+{
+    const int a = t < tp ? t : tp, b = t < tp ? tp : t;
+    return a == b ? N * (N - 1) + a : 2 * (a * N - a * (a + 1) / 2 + b - a - 1);
+}
+template <int N> __host__ __device__ inline void loop_comp(int c, int &t, int &tp, bool &im)
+{
+    if (c >= N * (N - 1)) {
+        t = tp = c - N * (N - 1);
+        im = false;
+        return;
+    }
+    int p = c >> 1;
+    im = c & 1;
+    t = 0;
+    while (p >= N - 1 - t) {
+        p -= N - 1 - t;
+        t++;
+    }
+    tp = t + 1 + p;
+}
+
 // (hi, lo) words of the exact double of a float, formed on the integer pipe only (this GPU's FP64 pipe,
 // which also executes conversions, is slow; a branch to a plain conversion gets if-converted into an
 // unconditional one): normal, zero, subnormal (normalised with clz), inf and nan.
@@ -349,7 +374,12 @@ struct tufrg_model {
     int *d_shard_q = nullptr;       // [Nq] momenta of a shard (sharded right-hand side)
     double2 *d_shard_out = nullptr; // [2][Nq][M][M] products of a shard's momenta before they are gathered
     bool loops_tc = false;          // multi-orbital loop k-sum on the tensor cores (k_loops_tc.cu)
-    float2 *d_loop_w = nullptr;     // its column sums [groups][Lf][108][108]
+    void *d_loop_w = nullptr;       // its column sums [groups][columns][180][108]
+    float *d_rho = nullptr;         // its projector components [Nk][36][6]
+    int *d_tc_grp = nullptr;        // its momentum groups [n_tc_groups][3]
+    int n_tc_groups = 0;
+    std::vector<int> loop_q;        // momentum of every list position (loop symmetries: the representatives)
+    bool loop_list_is_reps = true;  // d_loop_list is that list (a shard's list takes its place for a call)
 
     // ---- learned loop surrogate (optional)
     tufrg_mlp *sur = nullptr;       // network (not owned)
@@ -418,7 +448,6 @@ void drop_rhs_graphs(tufrg_model *m);
 // the launch shapes the two-band split loop kernel's autotuner times (ky ranges per column)
 std::vector<LoopPlan> loop_plan_candidates(const tufrg_model *m);
 int plan_gen_chunks(const tufrg_model *m);   // kx ranges per momentum of the multi-orbital loop kernel
-size_t gen_red_offset(const tufrg_model *m);   // byte offset of the representatives' range sums in d_part
 size_t gen_part_bytes(const tufrg_model *m);   // loop scratch of the multi-orbital kernel
 int dft_plan_nsplit(const tufrg_model *m);
 bool loops2_supported(const tufrg_model *m);
@@ -438,7 +467,9 @@ bool build_irrep_basis(tufrg_model *m);
 cudaError_t launch_irrep_basis(tufrg_model *m, const double2 *d_state, int inverse, double2 *d_out);
 bool loops_tc_supported(const tufrg_model *m);
 size_t loops_tc_w_bytes(const tufrg_model *m);
-cudaError_t launch_loops_tc(tufrg_model *m, int ch, float2 *acc);
+std::vector<int> loops_tc_groups(const std::vector<int> &q_of_slot, int Lq);
+cudaError_t launch_loops_rho(tufrg_model *m);   // once per model
+cudaError_t launch_loops_tc(tufrg_model *m, int ch, bool half, float2 *acc);
 cudaError_t launch_vlv_large(tufrg_model *m, const double2 *d_A, int channel_mask, double2 *d_out, const int *qlist,
                              int nlist);
 cudaError_t launch_sym_scatter(tufrg_model *m, double2 *d_out);

@@ -7,9 +7,9 @@
 // inputs and activations would make it a staircase in log T that an adaptive integrator resolves with
 // ever smaller steps).  Loss: mean squared error.
 // Kernels: the GEMMs on the tensor cores (k_mlp_tc.cu: BF16 x BF16 for training, FP32 activations split into
-// TF32 parts x BF16 weights for inference, FP32 accumulation, fixed summation order), GELU forward/backward, the
-// loss gradient, bias gradients as fixed-order column sums, and Adam.  Nothing here is part of the paper: it
-// serves the surrogate of the loops.
+// TF32 parts x BF16 weights for inference, FP32 accumulation, fixed summation order); the element-wise functions, the loss
+// gradient and the column sums of the bias gradients are formed where the GEMMs' operands are packed; and Adam.  Nothing
+// here is part of the paper: it serves the surrogate of the loops.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -20,6 +20,7 @@
 #include <string>
 #include <vector>
 
+#include "mlp.cuh"
 #include "tufrg_internal.cuh"
 
 struct tufrg_mlp {
@@ -36,10 +37,9 @@ struct tufrg_mlp {
     int adam_t = 0;
     int cap = 0;                           // batch capacity of the activation buffers
     std::vector<float *> Z;                // [layer] pre-activations, FP32 [cap][dout]
-    std::vector<__nv_bfloat16 *> H;        // [layer + 1] layer inputs, BF16 [cap][din]; H[0] = input
     float *dA = nullptr, *dA2 = nullptr;   // FP32 upstream gradients [cap][max width]
-    __nv_bfloat16 *dZ16 = nullptr;         // BF16 copy of dZ
-    float *dZ = nullptr;                   // FP32 dZ
+    std::vector<float *> part;             // [layer] partial sums of the bias gradients
+    double *loss_part = nullptr;           // partial sums of the loss
     float *loss = nullptr;                 // [1]
     void *ws = nullptr;                    // packed GEMM operands (tensor cores)
     size_t ws_bytes = 0;
@@ -49,69 +49,10 @@ struct tufrg_mlp {
 namespace tufrg {
 namespace {
 
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_d(float x)
+__global__ void to_bf16_kernel(const float *x, __nv_bfloat16 *y, size_t n)
 {
-    return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
-__global__ void to_bf16_kernel(const float *x, __nv_bfloat16 *y, size_t n, const int *skip = nullptr)
-{
-    if (skip && *skip) return;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         y[i] = __float2bfloat16(x[i]);
-}
-
-__device__ __forceinline__ void st_act(__nv_bfloat16 *p, float v) { *p = __float2bfloat16(v); }
-__device__ __forceinline__ void st_act(float *p, float v) { *p = v; }
-
-// H = GELU(Z); H may alias Z (FP32 inference, in place)
-template <typename TH>
-__global__ void gelu_fwd_kernel(const float *Z, TH *H, size_t n, const int *skip)
-{
-    if (skip && *skip) return;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        st_act(H + i, gelu(Z[i]));
-}
-
-// dZ = dA * gelu'(Z) (hidden layers) or dZ = dA (output layer); FP32 and BF16 copies
-__global__ void act_bwd_kernel(const float *dA, const float *Z, int hidden, float *dZ, __nv_bfloat16 *dZ16, size_t n)
-{
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float g = hidden ? dA[i] * gelu_d(Z[i]) : dA[i];
-        dZ[i] = g;
-        dZ16[i] = __float2bfloat16(g);
-    }
-}
-
-// dY = 2 (Y - T) / n, and the loss sum((Y - T)^2) / n by a fixed-order block reduction (one block)
-__global__ void mse_kernel(const float *Y, const float *T, float *dY, size_t n, float *loss)
-{
-    __shared__ double sh[256];
-    double s = 0.0;
-    const float inv = 1.f / (float)n;
-    for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const float d = Y[i] - T[i];
-        dY[i] = 2.f * d * inv;
-        s += (double)d * d;
-    }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = (float)(sh[0] / (double)n);
-}
-
-// db[c] = sum_r dZ[r][c] in row order
-__global__ void colsum_kernel(const float *dZ, int rows, int cols, float *db)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.f;
-    for (int r = 0; r < rows; r++) s += dZ[(size_t)r * cols + c];
-    db[c] = s;
 }
 
 __global__ void adam_kernel(float *w, const float *g, float *m, float *v, __nv_bfloat16 *w16, size_t n, float lr,
@@ -158,45 +99,36 @@ tufrg_status mlp_host_alloc_fail(tufrg_mlp *n, const std::exception &ex) noexcep
                          std::string(where) + ": " + cudaGetErrorString(_e));                     \
     } while (0)
 
-// C = op(A) op(B) (+ bias) on the tensor cores with the network's operand scratch
-template <typename TA>
-cudaError_t gemm(tufrg_mlp *n, cudaStream_t s, const TA *A, int lda, int ta, const __nv_bfloat16 *B, int ldb, int tb,
-                 float *C, int ldc, int M, int N, int K, const float *bias, const int *skip = nullptr)
-{
-    if (mlp_tc_scratch_bytes(M, N, K) > n->ws_bytes) return cudaErrorInvalidValue;   // sized by ensure_capacity
-    return mlp_gemm_tc<TA>(s, A, lda, ta, B, ldb, tb, C, ldc, M, N, K, bias, skip, n->ws, n->d_err);
-}
-
 tufrg_status ensure_capacity(tufrg_mlp *n, int batch)
 {
     if (batch <= n->cap) return TUFRG_OK;
     for (auto p : n->Z) cudaFree(p);
-    for (auto p : n->H) cudaFree(p);
-    cudaFree(n->dA); cudaFree(n->dA2); cudaFree(n->dZ16); cudaFree(n->dZ);
+    for (auto p : n->part) cudaFree(p);
+    cudaFree(n->dA); cudaFree(n->dA2); cudaFree(n->loss_part);
+    n->dA = n->dA2 = nullptr;
+    n->loss_part = nullptr;
     n->Z.assign(n->n_layers, nullptr);
-    n->H.assign(n->n_layers + 1, nullptr);
+    n->part.assign(n->n_layers, nullptr);
     int wmax = n->n_in;
     for (int l = 0; l < n->n_layers; l++) wmax = std::max(wmax, std::max(n->din[l], n->dout[l]));
-    for (int l = 0; l < n->n_layers; l++) MK(cudaMalloc(&n->Z[l], sizeof(float) * (size_t)batch * n->dout[l]), "cudaMalloc activations");
-    for (int l = 0; l <= n->n_layers; l++) {
-        const int w = l < n->n_layers ? n->din[l] : n->n_out;
-        MK(cudaMalloc(&n->H[l], sizeof(__nv_bfloat16) * (size_t)batch * w), "cudaMalloc activations");
+    for (int l = 0; l < n->n_layers; l++) {
+        MK(cudaMalloc(&n->Z[l], sizeof(float) * (size_t)batch * n->dout[l]), "cudaMalloc activations");
+        MK(cudaMalloc(&n->part[l], sizeof(float) * (size_t)mlp_sum_parts(batch) * n->dout[l]), "cudaMalloc gradients");
     }
     MK(cudaMalloc(&n->dA, sizeof(float) * (size_t)batch * wmax), "cudaMalloc gradients");
     MK(cudaMalloc(&n->dA2, sizeof(float) * (size_t)batch * wmax), "cudaMalloc gradients");
-    MK(cudaMalloc(&n->dZ, sizeof(float) * (size_t)batch * wmax), "cudaMalloc gradients");
-    MK(cudaMalloc(&n->dZ16, sizeof(__nv_bfloat16) * (size_t)batch * wmax), "cudaMalloc gradients");
-    // operand scratch of the largest GEMM: the forward (batch x dout x din), weight-gradient (din x dout x batch)
-    // and input-gradient (batch x din x dout) products of every layer
+    MK(cudaMalloc(&n->loss_part, sizeof(double) * mlp_loss_parts(batch, n->n_out)), "cudaMalloc gradients");
+    // operand scratch: the forward (batch x dout x din) product of a layer, or its weight-gradient (din x dout x batch)
+    // and input-gradient (batch x din x dout) products together
     size_t ws = 0;
     for (int l = 0; l < n->n_layers; l++) {
         ws = std::max(ws, mlp_tc_scratch_bytes(batch, n->dout[l], n->din[l]));
-        ws = std::max(ws, mlp_tc_scratch_bytes(n->din[l], n->dout[l], batch));
-        ws = std::max(ws, mlp_tc_scratch_bytes(batch, n->din[l], n->dout[l]));
+        ws = std::max(ws, mlp_tc_scratch_bytes(n->din[l], n->dout[l], batch) + mlp_tc_scratch_bytes(batch, n->din[l], n->dout[l]));
     }
     if (ws > n->ws_bytes) {
         cudaFree(n->ws);
         n->ws = nullptr;
+        n->ws_bytes = 0;
         MK(cudaMalloc(&n->ws, ws), "cudaMalloc GEMM operands");
         n->ws_bytes = ws;
     }
@@ -204,76 +136,51 @@ tufrg_status ensure_capacity(tufrg_mlp *n, int batch)
     return TUFRG_OK;
 }
 
-// Training forward pass (BF16 activations); Y (FP32 [batch][n_out]) receives the output; keeps the
-// hidden pre-activations Z and the layer inputs H for the backward pass (the output layer is linear,
-// so its Z is never needed).
-tufrg_status forward(tufrg_mlp *n, const float *X, int batch, float *Y)
+// the input of layer l: X, or GELU of the previous pre-activations
+MlpSrc layer_input(const tufrg_mlp *n, int l, const float *X, int trans)
+{
+    return l == 0 ? MlpSrc{X, nullptr, n->din[0], trans, MLP_F32, 0.f} : MlpSrc{n->Z[l - 1], nullptr, n->din[l], trans, MLP_GELU, 0.f};
+}
+
+// Forward pass; Y (FP32 [batch][n_out]) receives the output, the pre-activations Z of the hidden layers stay for the
+// backward pass.  Training rounds the layer inputs to BF16; inference (fp32) keeps them in FP32.  With skip != NULL every
+// kernel returns at once while *skip != 0 (device-side decision, graph-capturable).
+tufrg_status forward(tufrg_mlp *n, const float *X, int batch, float *Y, bool fp32, const int *skip)
 {
     tufrg_status st = ensure_capacity(n, batch);
     if (st != TUFRG_OK) return st;
-    cudaStream_t s = n->stream;
-    to_bf16_kernel<<<gsz((size_t)batch * n->n_in), 256, 0, s>>>(X, n->H[0], (size_t)batch * n->n_in);
-    MK(cudaGetLastError(), "convert input");
     for (int l = 0; l < n->n_layers; l++) {
-        const bool last = l == n->n_layers - 1;
-        float *out = last ? Y : n->Z[l];
-        MK(gemm(n, s, n->H[l], n->din[l], 0, n->d_w16 + n->woff[l], n->dout[l], 0, out, n->dout[l], batch, n->dout[l],
-                n->din[l], n->d_w + n->boff[l]), "layer GEMM");
-        if (!last) {
-            gelu_fwd_kernel<<<gsz((size_t)batch * n->dout[l]), 256, 0, s>>>(n->Z[l], n->H[l + 1], (size_t)batch * n->dout[l],
-                                                                            (const int *)nullptr);
-            MK(cudaGetLastError(), "GELU");
-        }
+        const MlpGemm g{layer_input(n, l, X, 0), MlpSrc{n->d_w16 + n->woff[l], nullptr, n->dout[l], 1, MLP_BF16, 0.f},
+                        l == n->n_layers - 1 ? Y : n->Z[l], batch, n->dout[l], n->din[l], n->d_w + n->boff[l]};
+        MK(mlp_gemms(n->stream, fp32, &g, 1, nullptr, skip, n->ws, n->ws_bytes, n->d_err), "layer GEMM");
     }
     return TUFRG_OK;
 }
 
-// Inference forward pass: BF16 weights, FP32 input and activations (GELU in place on Z).  With
-// skip != NULL every kernel returns at once while *skip != 0 (device-side decision, graph-capturable).
-tufrg_status infer(tufrg_mlp *n, const float *X, int batch, float *Y, const int *skip)
+// backward pass from the output Y and the targets T into the flat gradient g and the loss; per layer
+// dW = H^T dZ (din x dout), dH = dZ W^T (batch x din), db = column sums of dZ (FP32), with dZ = dH GELU'(Z)
+tufrg_status backward(tufrg_mlp *n, const float *X, int batch, const float *Y, const float *T, float *g)
 {
-    tufrg_status st = ensure_capacity(n, batch);
-    if (st != TUFRG_OK) return st;
-    cudaStream_t s = n->stream;
-    const float *in = X;
-    for (int l = 0; l < n->n_layers; l++) {
-        const bool last = l == n->n_layers - 1;
-        float *out = last ? Y : n->Z[l];
-        MK(gemm(n, s, in, n->din[l], 0, n->d_w16 + n->woff[l], n->dout[l], 0, out, n->dout[l], batch, n->dout[l], n->din[l],
-                n->d_w + n->boff[l], skip), "layer GEMM");
-        if (!last) {
-            gelu_fwd_kernel<<<gsz((size_t)batch * n->dout[l]), 256, 0, s>>>(n->Z[l], n->Z[l], (size_t)batch * n->dout[l],
-                                                                            skip);
-            MK(cudaGetLastError(), "GELU");
-            in = n->Z[l];
-        }
-    }
-    return TUFRG_OK;
-}
-
-// backward pass from dY = dLoss/dY into the flat gradient g
-tufrg_status backward(tufrg_mlp *n, int batch, const float *dY, float *g)
-{
-    cudaStream_t s = n->stream;
-    const float *up = dY;
+    const double inv_n = 1.0 / ((double)batch * n->n_out);
+    const float *up = nullptr;
+    std::vector<float *> db(n->n_layers);
     for (int l = n->n_layers - 1; l >= 0; l--) {
-        const size_t cnt = (size_t)batch * n->dout[l];
-        const bool hidden = l < n->n_layers - 1;
-        act_bwd_kernel<<<gsz(cnt), 256, 0, s>>>(up, n->Z[l], hidden ? 1 : 0, n->dZ, n->dZ16, cnt);
-        MK(cudaGetLastError(), "activation backward");
-        // dW = H^T dZ  (din x dout), db = column sums of dZ
-        MK(gemm(n, s, n->H[l], n->din[l], 1, n->dZ16, n->dout[l], 0, g + n->woff[l], n->dout[l], n->din[l], n->dout[l],
-                batch, nullptr), "weight gradient");
-        colsum_kernel<<<(n->dout[l] + 127) / 128, 128, 0, s>>>(n->dZ, batch, n->dout[l], g + n->boff[l]);
-        MK(cudaGetLastError(), "bias gradient");
-        if (l > 0) {
-            // dH = dZ W^T  (batch x din)
-            float *dst = (up == n->dA) ? n->dA2 : n->dA;
-            MK(gemm(n, s, n->dZ16, n->dout[l], 0, n->d_w16 + n->woff[l], n->dout[l], 1, dst, n->din[l], batch, n->din[l],
-                    n->dout[l], nullptr), "input gradient");
-            up = dst;
-        }
+        const bool last = l == n->n_layers - 1;
+        const int din = n->din[l], dout = n->dout[l];
+        const MlpSrc dz = last ? MlpSrc{Y, T, dout, 0, MLP_MSE, 1.f / (float)((size_t)batch * n->n_out)} : MlpSrc{up, n->Z[l], dout, 0, MLP_DGELU, 0.f};
+        MlpSrc dzt = dz;
+        dzt.trans = 1;
+        float *dst = up == n->dA ? n->dA2 : n->dA;   // (the output sits in dA2 until the last layer's operands are packed)
+        const MlpGemm gm[2] = {
+            {layer_input(n, l, X, 1), dzt, g + n->woff[l], din, dout, batch, nullptr},
+            {dz, MlpSrc{n->d_w16 + n->woff[l], nullptr, dout, 0, MLP_BF16, 0.f}, dst, batch, din, dout, nullptr}};
+        const MlpSums sums{dz, batch, dout, n->part[l], n->loss_part};
+        MK(mlp_gemms(n->stream, false, gm, l > 0 ? 2 : 1, &sums, nullptr, n->ws, n->ws_bytes, n->d_err), "gradient GEMMs");
+        up = dst;
+        db[l] = g + n->boff[l];
     }
+    MK(mlp_finish(n->stream, n->n_layers, n->dout.data(), n->part.data(), db.data(), mlp_sum_parts(batch), n->loss_part,
+                  mlp_loss_parts(batch, n->n_out), inv_n, n->loss), "bias gradients");
     return TUFRG_OK;
 }
 
@@ -340,8 +247,8 @@ void tufrg_mlp_free(tufrg_mlp *n)
     if (!n) return;
     cudaStreamSynchronize(n->stream);
     for (auto p : n->Z) cudaFree(p);
-    for (auto p : n->H) cudaFree(p);
-    void *ptrs[] = {n->d_w, n->d_w16, n->d_g, n->d_m, n->d_v, n->loss, n->dA, n->dA2, n->dZ16, n->dZ, n->ws, n->d_err};
+    for (auto p : n->part) cudaFree(p);
+    void *ptrs[] = {n->d_w, n->d_w16, n->d_g, n->d_m, n->d_v, n->loss, n->dA, n->dA2, n->loss_part, n->ws, n->d_err};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete n;
@@ -375,7 +282,7 @@ tufrg_status tufrg_mlp_set_params(tufrg_mlp *n, const float *h_params)
 tufrg_status tufrg_mlp_forward(tufrg_mlp *n, const float *d_X, int batch, float *d_Y)
 {
     if (!n || !d_X || !d_Y || batch < 1) return TUFRG_EINVAL;
-    return infer(n, d_X, batch, d_Y, nullptr);
+    return forward(n, d_X, batch, d_Y, true, nullptr);
 }
 
 tufrg_status tufrg_mlp_gradients(tufrg_mlp *n, const float *d_X, const float *d_T, int batch, float *d_grad, float *h_loss)
@@ -383,14 +290,9 @@ tufrg_status tufrg_mlp_gradients(tufrg_mlp *n, const float *d_X, const float *d_
     if (!n || !d_X || !d_T || !d_grad || batch < 1) return TUFRG_EINVAL;
     tufrg_status st = ensure_capacity(n, batch);
     if (st != TUFRG_OK) return st;
-    float *Y = n->dA2;   // output buffer reused (overwritten by the backward pass only after dY is formed)
-    float *dY = n->dA;
-    // the output and its gradient need [batch][n_out]; dA/dA2 are sized for max(width, n_out)
-    if ((st = forward(n, d_X, batch, Y)) != TUFRG_OK) return st;
-    const size_t cnt = (size_t)batch * n->n_out;
-    mse_kernel<<<1, 256, 0, n->stream>>>(Y, d_T, dY, cnt, n->loss);
-    MK(cudaGetLastError(), "loss");
-    if ((st = backward(n, batch, dY, d_grad)) != TUFRG_OK) return st;
+    float *Y = n->dA2;   // sized for max(width, n_out); the input gradients overwrite it after its last use
+    if ((st = forward(n, d_X, batch, Y, false, nullptr)) != TUFRG_OK) return st;
+    if ((st = backward(n, d_X, batch, Y, d_T, d_grad)) != TUFRG_OK) return st;
     if (h_loss) {
         int e = 0;
         MK(cudaMemcpyAsync(h_loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->stream), "copy loss");
@@ -430,7 +332,7 @@ cudaError_t mlp_forward_on(tufrg_mlp *n, cudaStream_t s, const float *X, int bat
 {
     cudaStream_t keep = n->stream;
     n->stream = s;
-    const tufrg_status st = infer(n, X, batch, Y, skip);
+    const tufrg_status st = forward(n, X, batch, Y, true, skip);
     n->stream = keep;
     return st == TUFRG_OK ? cudaSuccess : cudaErrorUnknown;
 }

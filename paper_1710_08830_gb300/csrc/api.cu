@@ -530,7 +530,7 @@ void release(tufrg_model *m)
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
-                    m->d_shard_q, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
+                    m->d_shard_q, m->d_oz, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &p : m->d_k)
@@ -1209,6 +1209,7 @@ try {
     // channels (FP32 complex, the same bytes)
     if (m->M > 64 || split)
         CK(cudaMalloc(reinterpret_cast<void **>(&m->d_T), (size_t)m->Nq * M2 * sizeof(double2)), "cudaMalloc product scratch");
+    if (m->M > 64 && !split) CK(cudaMalloc(&m->d_oz, vlv64_scratch_bytes(m)), "cudaMalloc product digits");
     CK(dalloc(&m->d_err, 1), "cudaMalloc error flag");
     CK(dalloc(&m->d_scal, 2), "cudaMalloc scalars");
     CK(cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream), "zero error flag");

@@ -1,10 +1,10 @@
-// dX/dT(q) = c_X A_X(q) L_X(q) A_X(q) for large M (multi-orbital bond sets, M = N_ff N_s^2 > 64):
-// Eq. RGE_spin (c_P = 1) and the orbital form of Eq. rge_Dmat (c_C = 2).
+// dX/dT(q) = c_X A_X(q) L_X(q) A_X(q) for large M (multi-orbital bond sets, M = N_ff N_s^2 > 64) on the CUDA cores, split
+// path: Eq. RGE_spin (c_P = 1) and the orbital form of Eq. rge_Dmat (c_C = 2).
 //
 // Batched complex GEMM on CUDA cores, 64 x 64 output tiles, 16-deep K slices staged in shared
 // memory, a 4 x 4 complex register tile per thread.  Pass 1 forms T = A L with the loop matrix
 // gathered from the compact loops (L[(R1,a),(R2,b)] = Lc[d(R1-R2)][a][b], never stored); pass 2
-// writes c * T A.  FP64 on the plain path, FP32 on the split path.
+// writes c * T A.  FP32 arithmetic (the FP64 path multiplies on the tensor cores, k_vlv64.cu).
 #include "tufrg_internal.cuh"
 
 namespace tufrg {
@@ -120,11 +120,9 @@ cudaError_t run(tufrg_model *m, const typename cpx<R>::t *A, const typename cpx<
 
 }  // namespace
 
-cudaError_t launch_vlv_large(tufrg_model *m, const double2 *d_A, int channel_mask, double2 *d_out, const int *qlist,
-                             int nlist)
+cudaError_t launch_vlv_large(tufrg_model *m, int channel_mask, double2 *d_out, const int *qlist, int nlist)
 {
     PhaseScope ps(m, PH_VLV, 4);
-    if (m->precision == TUFRG_FP64) return run<double>(m, d_A, m->d_Lc, channel_mask, d_out, m->d_T, qlist, nlist);
     return run<float>(m, m->d_A32, m->d_Lc32, channel_mask, d_out, reinterpret_cast<float2 *>(m->d_T), qlist, nlist);
 }
 

@@ -490,7 +490,9 @@ cudaError_t launch_vlv(tufrg_model *m, const double2 *d_A, int channel_mask, dou
 {
     const int M = m->M;
     if (tc_supported(m)) return launch_vlv_tc(m, channel_mask, d_out, qlist, nlist);
-    if (M > 64) return launch_vlv_large(m, d_A, channel_mask, d_out, qlist, nlist);
+    if (M > 64)
+        return m->precision == TUFRG_FP64 ? launch_vlv64(m, d_A, channel_mask, d_out, qlist, nlist)
+                                          : launch_vlv_large(m, channel_mask, d_out, qlist, nlist);
     const int ns2 = m->ns * m->ns;
     dim3 grid(qlist ? nlist : m->Nq, 2);
     PhaseScope ps(m, PH_VLV);

@@ -87,12 +87,12 @@ __device__ __forceinline__ float pw(float e1, float g1, float gp1, float e2, flo
     }
 }
 
+// The sums of one CTA: row range kyc of a column block of one transfer momentum.
 // SHELL: momentum-shell regulator (a separate instantiation, so that the temperature flow's code is unchanged)
-template <int NDYH, int WHICH, bool SHELL = false>
-__global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
+template <int NDYH, int WHICH, bool SHELL>
+__device__ __forceinline__ void loops2_body(const Args2 &a, const int kyc)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (a.skip && *a.skip) return;   // uniform over the grid
     float2 *ptab = reinterpret_cast<float2 *>(smem_raw);
     const int Lf = a.Lf;
     if (a.ptab) {
@@ -118,7 +118,6 @@ __global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
     const float lam = SHELL ? (float)*a.Tp : 0.f;
     const float thr = SHELL ? 1e-2f * a.shell_T : (a.Tp ? (float)(1e-2 * *a.Tp) : a.thr);
     const bool valid = kx < Lf;
-    const int kyc = blockIdx.z;
     const int ky0 = kyc * a.ky_len;
     const int ky1 = min(Lf, ky0 + a.ky_len);
 
@@ -258,8 +257,8 @@ __global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
     constexpr int PITCH = NV + 1;
     float *buf = reinterpret_cast<float *>(region);
     __syncwarp();   // every lane of the warp is done with its ring entries (lanes past Lf skipped the k-sum)
-    const int n_part = gridDim.y * WARPS * gridDim.z;
-    const int p = (blockIdx.y * WARPS + warp) * gridDim.z + kyc;
+    const int n_part = gridDim.y * WARPS * a.ky_chunks;
+    const int p = (blockIdx.y * WARPS + warp) * a.ky_chunks + kyc;
     for (int dxi = 0; dxi < a.ndx; dxi++) {
         if (a.needed[dxi] == 0) continue;
         const int n = (int)((((long)kx * a.dxs[dxi]) % Lf + Lf) % Lf);
@@ -395,6 +394,41 @@ __global__ void loops_reduce_sym_kernel(const typename cpx<R>::t *__restrict__ p
     if (out32) out32[o] = w;
 }
 
+// one channel
+template <int NDYH, int WHICH, bool SHELL = false>
+__global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
+{
+    if (a.skip && *a.skip) return;   // uniform over the grid
+    loops2_body<NDYH, WHICH, SHELL>(a, blockIdx.z);
+}
+
+// both channels (blockIdx.z: channel, row range): the C channel's CTAs run beside the P channel's, which on small meshes
+// fill a fraction of the SMs (8 x 8 transfer, 128 x 128 fine mesh, 15 representatives, 3 row ranges: 180 CTAs of two
+// warps for both).  Latency bound there, 22 us for both channels.
+template <int NDYH, bool SHELL>
+__global__ void __launch_bounds__(32 * WARPS) loops2_both_kernel(Args2 a, size_t part_cs)
+{
+    if (a.skip && *a.skip) return;
+    if ((int)blockIdx.z < a.ky_chunks) {
+        loops2_body<NDYH, 0, SHELL>(a, blockIdx.z);
+    } else {
+        a.part += part_cs;
+        loops2_body<NDYH, 1, SHELL>(a, blockIdx.z - a.ky_chunks);
+    }
+}
+
+template <int NDYH>
+cudaError_t launch2_both(tufrg_model *m, const Args2 &a, int n_s, size_t part_cs)
+{
+    const dim3 grid(n_s, (m->Lf + 32 * WARPS - 1) / (32 * WARPS), 2 * a.ky_chunks);
+    const size_t smem = loops2_smem_bytes(m->Lf, NDYH);
+    auto kern = a.shell_T > 0.f ? loops2_both_kernel<NDYH, true> : loops2_both_kernel<NDYH, false>;
+    if (smem > 48 * 1024) TUFRG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    PhaseScope ps(m, PH_LOOPS);
+    kern<<<grid, 32 * WARPS, smem, m->stream>>>(a, part_cs);
+    return cudaGetLastError();
+}
+
 template <int NDYH, int WHICH>
 cudaError_t launch2(tufrg_model *m, const Args2 &a, int n_s)
 {
@@ -425,9 +459,7 @@ int loops2_blocks_per_sm(const tufrg_model *m)
     return (e == cudaSuccess && n > 0) ? n : 4;
 }
 
-// Loop sums of channel ch into the partial buffer (no reduction).  With s_list, only the
-// listed transfer momenta (n_list of them) are evaluated, into partial slots 0..n_list-1 of part.
-cudaError_t launch_loops2_ex(tufrg_model *m, int ch, const int *s_list, int n_list, float2 *part, const int *skip)
+static Args2 loops2_args(const tufrg_model *m, const int *s_list, float2 *part, const int *skip)
 {
     const LoopPlan &pl = m->plan;
     Args2 a{};
@@ -457,8 +489,16 @@ cudaError_t launch_loops2_ex(tufrg_model *m, int ch, const int *s_list, int n_li
     a.Tp = m->d_scal;
     a.shell_T = m->regulator == TUFRG_REG_MOMENTUM_SHELL ? (float)m->T_reg : 0.f;
     a.ptab = m->d_lph32;
+    return a;
+}
+
+// Loop sums of channel ch into the partial buffer (no reduction).  With s_list, only the
+// listed transfer momenta (n_list of them) are evaluated, into partial slots 0..n_list-1 of part.
+cudaError_t launch_loops2_ex(tufrg_model *m, int ch, const int *s_list, int n_list, float2 *part, const int *skip)
+{
+    const Args2 a = loops2_args(m, s_list, part, skip);
     const int n_s = s_list ? n_list : m->Nq;
-    switch (ndyh) {
+    switch (a.ndyh) {
     case 1: return ch == 0 ? launch2<1, 0>(m, a, n_s) : launch2<1, 1>(m, a, n_s);
     case 2: return ch == 0 ? launch2<2, 0>(m, a, n_s) : launch2<2, 1>(m, a, n_s);
     case 3: return ch == 0 ? launch2<3, 0>(m, a, n_s) : launch2<3, 1>(m, a, n_s);
@@ -550,10 +590,20 @@ cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
     const size_t part_cs = (size_t)n_s * pl.n_partials * ndx * ndyh * NS4, out_cs = (size_t)m->Nq * m->nd * NS4;
     float2 *part = reinterpret_cast<float2 *>(m->d_part);
     const int *skip = m->sur ? m->d_sur_flag : nullptr;
-    for (int ch = 0; ch < 2; ch++)
-        if ((channel_mask >> ch) & 1)
-            TUFRG_CUDA_TRY(launch_loops2_ex(m, ch, m->sym ? m->d_loop_list : nullptr, m->sym ? m->n_loop_q : 0,
-                                            part + ch * part_cs, skip));
+    const int *list = m->sym ? m->d_loop_list : nullptr;
+    if (channel_mask == 3) {
+        const Args2 a = loops2_args(m, list, part, skip);
+        switch (a.ndyh) {
+        case 1: TUFRG_CUDA_TRY(launch2_both<1>(m, a, n_s, part_cs)); break;
+        case 2: TUFRG_CUDA_TRY(launch2_both<2>(m, a, n_s, part_cs)); break;
+        case 3: TUFRG_CUDA_TRY(launch2_both<3>(m, a, n_s, part_cs)); break;
+        case 4: TUFRG_CUDA_TRY(launch2_both<4>(m, a, n_s, part_cs)); break;
+        default: TUFRG_CUDA_TRY(launch2_both<5>(m, a, n_s, part_cs)); break;   // (loops2_supported)
+        }
+    } else {
+        for (int ch = 0; ch < 2; ch++)
+            if ((channel_mask >> ch) & 1) TUFRG_CUDA_TRY(launch_loops2_ex(m, ch, list, n_s, part + ch * part_cs, skip));
+    }
     dim3 grid;
     int thr;
     reduce_shape(m, reps_only ? m->n_loop_q : m->Nq, grid, thr);

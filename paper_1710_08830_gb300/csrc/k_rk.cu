@@ -129,6 +129,18 @@ __global__ void stage_scalars_kernel(const FlowDev *fs, double cj, double *scal)
     scal[1] = T;
 }
 
+// the same for the six stages of an attempt: stage j = 1 .. 6 at scal[2 j]
+struct StageNodes {
+    double c[7];
+};
+__global__ void attempt_scalars_kernel(const FlowDev *fs, StageNodes s, double *scal)
+{
+    const int j = threadIdx.x + 1;
+    const double T = exp(fs->x + s.c[j] * fs->h);
+    scal[2 * j] = T;
+    scal[2 * j + 1] = T;
+}
+
 __global__ void flow_init_kernel(FlowDev *fs, const unsigned long long *red)
 {
     const double amax = __longlong_as_double((long long)red[0]);
@@ -284,6 +296,15 @@ cudaError_t launch_stage_scalars(tufrg_model *m, const FlowDev *fs, double cj)
 {
     m->launches++;
     stage_scalars_kernel<<<1, 1, 0, m->stream>>>(fs, cj, m->d_scal);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_attempt_scalars(tufrg_model *m, const FlowDev *fs, const double (&c)[7])
+{
+    m->launches++;
+    StageNodes s;
+    std::copy(c, c + 7, s.c);
+    attempt_scalars_kernel<<<1, 6, 0, m->stream>>>(fs, s, m->d_scal);
     return cudaGetLastError();
 }
 

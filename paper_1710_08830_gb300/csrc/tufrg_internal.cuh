@@ -251,7 +251,8 @@ struct tufrg_model {
     int *d_dpartner = nullptr;      // [nd] index of -delta
     int *d_hopR = nullptr;          // [nhop][2]
     double2 *d_hopt = nullptr;      // [nhop][ns][ns]
-    double *d_scal = nullptr;       // device scalars: [0] temperature of the current evaluation, [1] product scale
+    double *d_scal = nullptr;       // device scalars: [0] temperature of the current evaluation, [1] product scale; the
+                                    // stages j = 1 .. 6 of a flow's attempt at [2 j], [2 j + 1]
     int *d_dij = nullptr;           // [nff][nff]
     int *d_gofs[2] = {nullptr, nullptr};
     tufrg::GatherTerm *d_gterms[2] = {nullptr, nullptr};
@@ -338,6 +339,9 @@ struct tufrg_model {
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t aux_ev[2] = {nullptr, nullptr};
     cudaEvent_t flow_ev = nullptr;
+    cudaEvent_t flow_L[7] = {}, flow_O[7] = {};   // stage j's loops are there / its products have read them
+    double2 *d_LcB = nullptr;       // second loop buffer of a flow's stages (FP64 path; split path below), or null
+    float2 *d_Lc32B = nullptr;
     // tufrg_rhs replays captured graphs of its launches, one per (input, output, mask) used more than once (the
     // four most recently used triples kept; exec is null after the first use)
     struct RhsGraph {
@@ -438,6 +442,7 @@ cudaError_t launch_rk_combine(tufrg_model *m, double2 *out, float2 *out32, const
 cudaError_t launch_rk_error(tufrg_model *m, const double2 *y, const double2 *yn, const FlowDev *fs, const double *e,
                             double2 *const *k, int nk, size_t n);
 cudaError_t launch_stage_scalars(tufrg_model *m, const FlowDev *fs, double cj);
+cudaError_t launch_attempt_scalars(tufrg_model *m, const FlowDev *fs, const double (&c)[7]);
 cudaError_t launch_flow_init(tufrg_model *m, FlowDev *fs);
 cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs);
 cudaError_t launch_flow_commit(tufrg_model *m, const FlowDev *fs, double2 *y, const double2 *yn, double2 *k0,

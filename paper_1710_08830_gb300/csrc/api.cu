@@ -696,7 +696,7 @@ tufrg_status enqueue_attempt(tufrg_model *m, int mask)
         // split path the combination writes the FP32 copy that the evaluation reads instead
         double2 *dst = j == 6 ? m->d_yn : (split ? nullptr : m->d_yt);
         CK(launch_rk_combine(m, dst, split ? m->d_X32 : nullptr, m->d_y, m->d_flow, DP_A[j], k, j, n), "stage combination");
-        CK(launch_dft(m, dst, split ? m->d_X32 : nullptr, mask), "Fourier transform");
+        CK(launch_dft(m, dst, split ? m->d_X32 : nullptr, mask, true), "Fourier transform");
         CK(launch_project(m, dst, split ? m->d_X32 : nullptr, mask, split ? nullptr : m->d_A, ql, nl), "projections");
         CK(cudaStreamWaitEvent(m->stream, m->flow_L[jl], 0), "join");
         if (sym) CK(launch_products_sym(m, mask, k[j]), "V.L.V products (orbit representatives)");

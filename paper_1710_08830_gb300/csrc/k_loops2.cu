@@ -337,6 +337,7 @@ __global__ void loops_reduce_kernel(const typename cpx<R>::t *__restrict__ part,
                                     double2 *out64, typename cpx<R>::t *out32, const int *skip, int chmask,
                                     size_t part_cs, size_t out_cs)
 {
+    grid_wait();
     if (skip && *skip) return;
     const int ch = blockIdx.z;
     if (!((chmask >> ch) & 1)) return;
@@ -398,6 +399,7 @@ __global__ void loops_reduce_sym_kernel(const typename cpx<R>::t *__restrict__ p
 template <int NDYH, int WHICH, bool SHELL = false>
 __global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
 {
+    grid_release();
     if (a.skip && *a.skip) return;   // uniform over the grid
     loops2_body<NDYH, WHICH, SHELL>(a, blockIdx.z);
 }
@@ -408,6 +410,8 @@ __global__ void __launch_bounds__(32 * WARPS) loops2_kernel(Args2 a)
 template <int NDYH, bool SHELL>
 __global__ void __launch_bounds__(32 * WARPS) loops2_both_kernel(Args2 a, size_t part_cs)
 {
+    grid_release();
+    grid_wait();
     if (a.skip && *a.skip) return;
     if ((int)blockIdx.z < a.ky_chunks) {
         loops2_body<NDYH, 0, SHELL>(a, blockIdx.z);
@@ -425,8 +429,7 @@ cudaError_t launch2_both(tufrg_model *m, const Args2 &a, int n_s, size_t part_cs
     auto kern = a.shell_T > 0.f ? loops2_both_kernel<NDYH, true> : loops2_both_kernel<NDYH, false>;
     if (smem > 48 * 1024) TUFRG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     PhaseScope ps(m, PH_LOOPS);
-    kern<<<grid, 32 * WARPS, smem, m->stream>>>(a, part_cs);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, 32 * WARPS, smem, m->stream, loops_chained(m), a, part_cs);
 }
 
 template <int NDYH, int WHICH>
@@ -611,17 +614,15 @@ cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
     const double inv_nk = 1.0 / (double)m->Nk;
     PhaseScope ps(m, PH_LOOPRED);
     if (reps_only)   // the representatives' FP32 loops at their own momenta (what their products read)
-        loops_reduce_kernel<float><<<grid, thr, 0, m->stream>>>(part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas,
-                                                              m->nd, inv_nk, m->d_loop_list, nullptr, m->d_Lc32, skip,
-                                                              channel_mask, part_cs, out_cs);
-    else if (m->sym)
+        return launch_chained(loops_reduce_kernel<float>, grid, thr, 0, m->stream, true, part, pl.n_partials, ndx, ndyh, m->d_dslot,
+                              m->d_deltas, m->nd, inv_nk, m->d_loop_list, nullptr, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
+    if (m->sym)
         loops_reduce_sym_kernel<float><<<grid, thr, 0, m->stream>>>(
             part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas, m->nd, m->d_qmap, m->d_sym_elem, m->d_sym_dinv,
             inv_nk, m->d_Lc, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
     else
-        loops_reduce_kernel<float><<<grid, thr, 0, m->stream>>>(part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas,
-                                                              m->nd, inv_nk, nullptr, m->d_Lc, m->d_Lc32, skip,
-                                                              channel_mask, part_cs, out_cs);
+        return launch_chained(loops_reduce_kernel<float>, grid, thr, 0, m->stream, true, part, pl.n_partials, ndx, ndyh, m->d_dslot,
+                              m->d_deltas, m->nd, inv_nk, nullptr, m->d_Lc, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
     return cudaGetLastError();
 }
 

@@ -420,6 +420,7 @@ template <typename R>
 __global__ void rec_T_kernel(int n, double T_value, const double *Tp, typename vec4<R>::t *rec)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_release();   // (the k-sum of a flow waits for it)
     if (t >= n) return;
     const R invT = R(1) / (R)(Tp ? *Tp : T_value);   // device-resident temperature when given
     const R e[2] = {rec[t].w, rec[n + t].x};

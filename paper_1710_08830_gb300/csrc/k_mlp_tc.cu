@@ -76,11 +76,6 @@ __device__ __forceinline__ float src_a(const MlpSrc &s, size_t i)
     return s.mode == MLP_BF16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(s.S)[i]) : static_cast<const float *>(s.S)[i];
 }
 
-// The launches of a pass overlap: a kernel may start while the one before it finishes (programmatic stream
-// serialization), sets up, and waits here before it touches global memory.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 struct PackJob {
     MlpSrc src;
     int rows, K, R, tiles, nks, planes;

@@ -113,14 +113,17 @@ template <typename R, typename XT>
 __global__ void __launch_bounds__(DFT_THREADS) dft_rows_kernel(const XT *__restrict__ X, int Lq, int M2, int nry,
                                                                const typename cpx<R>::t *__restrict__ phy, int ch_lo,
                                                                typename cpx<R>::t *__restrict__ Z,
-                                                               float2 *__restrict__ x32)
+                                                               float2 *__restrict__ x32, unsigned long long *amax)
 {
     using C2 = typename cpx<R>::t;
     constexpr int UB = 8;   // loads in flight per thread (more registers than this leave too few warps per SM)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2 *sphy = reinterpret_cast<C2 *>(smem_raw);   // [Lq][nry]  e^{i u_y R_y}
+    grid_release();
     for (int i = threadIdx.x; i < Lq * nry; i += blockDim.x) sphy[i] = phy[i];
     __syncthreads();
+    grid_wait();
+    if (amax && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *amax = 0;   // the projections' maximum
     const int e = blockIdx.x * blockDim.x + threadIdx.x, ux = blockIdx.y, ch = ch_lo + blockIdx.z;
     if (e >= M2) return;
     const size_t row = ((size_t)ch * Lq * Lq + (size_t)ux * Lq) * M2 + e;
@@ -175,9 +178,11 @@ __global__ void __launch_bounds__(32 * DFT_MAXG) dft_cols_kernel(const typename 
     C2 *sz = reinterpret_cast<C2 *>(smem_raw);              // [DFT_UXC][32]  Z(u_x, R_y) of the CTA's entries
     C2 *sphx = sz + DFT_UXC * 32;                           // [Lq][nrx]  e^{i u_x R_x}
     int *stab = reinterpret_cast<int *>(sphx + Lq * nrx);   // cid [ncls], rxi [ncls], ryo [nry + 1]
+    grid_release();
     for (int i = threadIdx.x; i < Lq * nrx; i += blockDim.x) sphx[i] = phx[i];
     for (int i = threadIdx.x; i < 2 * ncls + nry + 1; i += blockDim.x) stab[i] = tabs[i];
     __syncthreads();
+    grid_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int e0 = blockIdx.x * 32, r = blockIdx.y, ch = ch_lo + blockIdx.z;
     const int *cid = stab, *rxi = stab + ncls, *ryo = stab + 2 * ncls;
@@ -252,6 +257,7 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
     C2 *phs = reinterpret_cast<C2 *>(smem_raw);   // [QT][nph]
     __shared__ int sq[QT];                         // transfer momenta of this CTA (list positions p0 ..)
     const int ch = blockIdx.z, p0 = blockIdx.y * QT, nq = min(QT, nlist - p0);
+    grid_release();
     if (threadIdx.x < QT) sq[threadIdx.x] = threadIdx.x < nq ? (qlist ? qlist[p0 + threadIdx.x] : p0 + threadIdx.x) : 0;
     __syncthreads();
     for (int i = threadIdx.x; i < QT * nph; i += blockDim.x) {
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
         phs[i] = qi < nq ? ph[(size_t)sq[qi] * nph + (i - qi * nph)] : mk(R(0), R(0));
     }
     __syncthreads();
+    grid_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     R m2 = R(0);
     if (e < M2) {
@@ -458,7 +465,7 @@ void dft_sep_plan(const tufrg_model *m, int *warps)
 
 template <typename R, typename XT>
 cudaError_t dft_sep_run(tufrg_model *m, const XT *d_state, const typename cpx<R>::t *phy, const typename cpx<R>::t *phx,
-                        int ch_lo, int nch, typename cpx<R>::t *Xr, float2 *x32)
+                        int ch_lo, int nch, typename cpx<R>::t *Xr, float2 *x32, bool chained)
 {
     using C2 = typename cpx<R>::t;
     const int M2 = m->M * m->M, xb = (M2 + DFT_THREADS - 1) / DFT_THREADS;
@@ -467,28 +474,28 @@ cudaError_t dft_sep_run(tufrg_model *m, const XT *d_state, const typename cpx<R>
     const size_t smem_cols = sizeof(C2) * ((size_t)m->Lq * m->dft_nrx + DFT_UXC * 32) +
                              sizeof(int) * (2 * m->ncls + m->dft_nry + 1);
     PhaseScope ps(m, PH_DFT, 2);
-    dft_rows_kernel<R, XT><<<dim3(xb, m->Lq, nch), DFT_THREADS, smem_rows, m->stream>>>(d_state, m->Lq, M2, m->dft_nry, phy, ch_lo, Z,
-                                                                      x32);
-    TUFRG_CUDA_TRY(cudaGetLastError());
-    dft_cols_kernel<R><<<dim3((M2 + 31) / 32, m->dft_nry, nch), 32 * m->dft_warps, smem_cols, m->stream>>>(
-        Z, m->Lq, M2, m->ncls, m->dft_nry, m->dft_nrx, m->d_dft_tabs, phx, ch_lo, 1.0 / m->Nq, Xr);
-    return cudaGetLastError();
+    TUFRG_CUDA_TRY(launch_chained(dft_rows_kernel<R, XT>, dim3(xb, m->Lq, nch), DFT_THREADS, smem_rows, m->stream, chained, d_state,
+                                  m->Lq, M2, m->dft_nry, phy, ch_lo, Z, x32, m->d_amax));
+    return launch_chained(dft_cols_kernel<R>, dim3((M2 + 31) / 32, m->dft_nry, nch), 32 * m->dft_warps, smem_cols, m->stream, sizeof(R) == 4,
+                          Z, m->Lq, M2, m->ncls, m->dft_nry, m->dft_nrx, m->d_dft_tabs, phx, ch_lo, 1.0 / m->Nq, Xr);
 }
 
-cudaError_t launch_dft(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask)
+cudaError_t launch_dft(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask, bool chained)
 {
     const int ch_lo = (channel_mask & 1) ? 0 : 1, ch_hi = (channel_mask & 2) ? 1 : 0;
+    // (cleared by the separable transform's first kernel)
+    if (ch_lo > ch_hi || m->dft_warps == 0) TUFRG_CUDA_TRY(cudaMemsetAsync(m->d_amax, 0, sizeof(unsigned long long), m->stream));
     if (ch_lo > ch_hi) return cudaSuccess;
     const int nch = ch_hi - ch_lo + 1;
     if (m->dft_warps > 0) {
         if (m->precision == TUFRG_FP64)
-            return dft_sep_run<double, double2>(m, d_state, m->d_dft_phy, m->d_dft_phx, ch_lo, nch, m->d_Xr, nullptr);
+            return dft_sep_run<double, double2>(m, d_state, m->d_dft_phy, m->d_dft_phx, ch_lo, nch, m->d_Xr, nullptr, chained);
         // the split path reads the FP32 copy where one exists, else the FP64 state, writing its rounding to
         // the model's copy as it reads
         if (d_state32)
             return dft_sep_run<float, float2>(m, d_state32, m->d_dft_phy32, m->d_dft_phx32, ch_lo, nch, m->d_Xr32,
-                                              nullptr);
-        return dft_sep_run<float, double2>(m, d_state, m->d_dft_phy32, m->d_dft_phx32, ch_lo, nch, m->d_Xr32, m->d_X32);
+                                              nullptr, chained);
+        return dft_sep_run<float, double2>(m, d_state, m->d_dft_phy32, m->d_dft_phx32, ch_lo, nch, m->d_Xr32, m->d_X32, chained);
     }
     if (m->precision == TUFRG_FP64)
         return dft_run<double, double2, 16>(m, d_state, m->d_clsph, ch_lo, nch, reinterpret_cast<double2 *>(m->d_dftpart),
@@ -504,23 +511,21 @@ constexpr int PROJ_QT = 8;   // transfer momenta per thread
 template <typename R, typename XT, int QT>
 cudaError_t project_run(tufrg_model *m, const XT *d_state, const typename cpx<R>::t *Xr, const XT *v0d0, const XT *v0d1,
                         const typename cpx<R>::t *ph, int channel_mask, const int *qlist, int nlist, double2 *d_A,
-                        float2 *d_A32, int x_local, const XT *v0q)
+                        float2 *d_A32, int x_local, const XT *v0q, bool chained)
 {
     const int M2 = m->M * m->M;
     const dim3 grid((M2 + 255) / 256, (nlist + QT - 1) / QT, 2);
     const size_t smem = sizeof(typename cpx<R>::t) * QT * m->nph;
     auto k = project_kernel<R, XT, QT>;
     if (smem > 48 * 1024) TUFRG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, 256, smem, m->stream>>>(d_state, Xr, v0d0, v0d1, m->d_eofs[0], m->d_eofs[1], m->d_eterms[0],
-                                      m->d_eterms[1], ph, m->nph, m->Nq, M2, m->ncls, channel_mask, qlist, nlist, d_A,
-                                      d_A32, m->d_amax, x_local, v0q);
-    return cudaGetLastError();
+    return launch_chained(k, grid, 256, smem, m->stream, chained, d_state, Xr, v0d0, v0d1, m->d_eofs[0], m->d_eofs[1],
+                          m->d_eterms[0], m->d_eterms[1], ph, m->nph, m->Nq, M2, m->ncls, channel_mask, qlist, nlist, d_A, d_A32,
+                          m->d_amax, x_local, v0q);
 }
 
 cudaError_t launch_project(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask,
                            double2 *d_A, const int *qlist, int nlist)
 {
-    TUFRG_CUDA_TRY(cudaMemsetAsync(m->d_amax, 0, sizeof(unsigned long long), m->stream));
     const int M2 = m->M * m->M;
     if (!qlist) nlist = m->Nq;
     const int xb = (M2 + 255) / 256;
@@ -531,12 +536,12 @@ cudaError_t launch_project(tufrg_model *m, const double2 *d_state, const float2 
     if (m->precision == TUFRG_FP64) {
         auto run = short_list ? project_run<double, double2, 2> : project_run<double, double2, PROJ_QT>;
         return run(m, d_state, m->d_Xr, m->d_v0d[0], m->d_v0d[1], m->d_ph, channel_mask, qlist, nlist, d_A, nullptr, 0,
-                   m->d_v0q);
+                   m->d_v0q, false);
     }
     if (!d_state32) return cudaErrorInvalidValue;   // the split path projects the FP32 copy
     auto run = short_list ? project_run<float, float2, 2> : project_run<float, float2, PROJ_QT>;
     return run(m, d_state32, m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_ph32, channel_mask, qlist, nlist, d_A,
-               m->d_A32, 0, m->d_v0q32);
+               m->d_A32, 0, m->d_v0q32, true);
 }
 
 cudaError_t launch_project_local(tufrg_model *m, const double2 *d_state_local, const float2 *d_state32_local,
@@ -546,9 +551,9 @@ cudaError_t launch_project_local(tufrg_model *m, const double2 *d_state_local, c
     PhaseScope ps(m, PH_PROJ);
     if (m->precision == TUFRG_FP64)
         return project_run<double, double2, 2>(m, d_state_local, m->d_Xr, m->d_v0d[0], m->d_v0d[1], m->d_ph, channel_mask,
-                                               qlist, nlist, d_A, nullptr, 1, m->d_v0q);
+                                               qlist, nlist, d_A, nullptr, 1, m->d_v0q, false);
     return project_run<float, float2, 2>(m, d_state32_local, m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_ph32,
-                                         channel_mask, qlist, nlist, d_A, m->d_A32, 1, m->d_v0q32);
+                                         channel_mask, qlist, nlist, d_A, m->d_A32, 1, m->d_v0q32, false);
 }
 
 cudaError_t launch_amax_channels(tufrg_model *m, bool reps_only)

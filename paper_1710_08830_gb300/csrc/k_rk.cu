@@ -18,6 +18,8 @@ struct StageArgs {
 // FP64 result goes to out and/or its FP32 rounding to out32 (either may be NULL)
 __global__ void rk_combine_kernel(double *out, float *out32, const double *y, const FlowDev *fs, StageArgs s, size_t n)
 {
+    grid_release();
+    grid_wait();
     const double h = fs->h;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
@@ -33,6 +35,8 @@ __global__ void rk_combine_kernel(double *out, float *out32, const double *y, co
 // its FP64 accumulation, the increment carries the FP32 accuracy of the derivatives)
 __global__ void rk_combine_f32_kernel(double *out, float *out32, const double *y, const FlowDev *fs, StageArgs s, size_t n)
 {
+    grid_release();
+    grid_wait();
     const double h = fs->h;
     float a[7];
 #pragma unroll
@@ -68,6 +72,8 @@ __global__ void round_f32_kernel(const double *x, float *y, size_t n)
 __global__ void rk_error_kernel(const double2 *y, const double2 *yn, const FlowDev *fs, StageArgs s, size_t n,
                                 unsigned long long *out)
 {
+    grid_release();
+    grid_wait();
     const double h = fs->h, atol = fs->atol, rtol = fs->rtol;
     double mx = 0.0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -95,6 +101,8 @@ __global__ void rk_error_kernel(const double2 *y, const double2 *yn, const FlowD
 __global__ void rk_error_f32_kernel(const double2 *y, const double2 *yn, const FlowDev *fs, StageArgs s, size_t n,
                                     unsigned long long *out)
 {
+    grid_release();
+    grid_wait();
     const float h = fabsf((float)fs->h), atol = (float)fs->atol, rtol = (float)fs->rtol;
     float e[7];
 #pragma unroll
@@ -133,8 +141,10 @@ __global__ void stage_scalars_kernel(const FlowDev *fs, double cj, double *scal)
 struct StageNodes {
     double c[7];
 };
-__global__ void attempt_scalars_kernel(const FlowDev *fs, StageNodes s, double *scal)
+__global__ void attempt_scalars_kernel(const FlowDev *fs, StageNodes s, double *scal, unsigned long long *err)
 {
+    grid_release();
+    if (threadIdx.x == 0) *err = 0;
     const int j = threadIdx.x + 1;
     const double T = exp(fs->x + s.c[j] * fs->h);
     scal[2 * j] = T;
@@ -157,6 +167,8 @@ __global__ void flow_init_kernel(FlowDev *fs, const unsigned long long *red)
 // Accept or reject the attempt just computed (error norm in red[2], max|A| at the candidate in red[0]).
 __global__ void flow_decide_kernel(FlowDev *fs, const unsigned long long *red)
 {
+    grid_release();
+    grid_wait();
     fs->accepted = 0;
     if (fs->status != 0) return;
     const double err = __longlong_as_double((long long)red[2]);
@@ -202,6 +214,8 @@ __global__ void flow_decide_kernel(FlowDev *fs, const unsigned long long *red)
 // FSAL commit of an accepted attempt: y <- y_n, k_1 <- k_7
 __global__ void flow_commit_kernel(const FlowDev *fs, double2 *y, const double2 *yn, double2 *k0, const double2 *k6, size_t n)
 {
+    grid_release();
+    grid_wait();
     if (!fs->accepted) return;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         y[i] = yn[i];
@@ -232,14 +246,10 @@ cudaError_t launch_rk_combine(tufrg_model *m, double2 *out, float2 *out32, const
     const size_t nd = 2 * n;
     PhaseScope ps(m, PH_RK);
     if (m->precision == TUFRG_FP64)
-        rk_combine_kernel<<<grid_for(m, nd), 256, 0, m->stream>>>(reinterpret_cast<double *>(out),
-                                                                  reinterpret_cast<float *>(out32),
-                                                                  reinterpret_cast<const double *>(y), fs, s, nd);
-    else
-        rk_combine_f32_kernel<<<grid_for(m, nd), 256, 0, m->stream>>>(reinterpret_cast<double *>(out),
-                                                                      reinterpret_cast<float *>(out32),
-                                                                      reinterpret_cast<const double *>(y), fs, s, nd);
-    return cudaGetLastError();
+        return launch_chained(rk_combine_kernel, grid_for(m, nd), 256, 0, m->stream, true, reinterpret_cast<double *>(out),
+                              reinterpret_cast<float *>(out32), reinterpret_cast<const double *>(y), fs, s, nd);
+    return launch_chained(rk_combine_f32_kernel, grid_for(m, nd), 256, 0, m->stream, true, reinterpret_cast<double *>(out),
+                          reinterpret_cast<float *>(out32), reinterpret_cast<const double *>(y), fs, s, nd);
 }
 
 __global__ void widen_f64_kernel(const float *in, double *out, size_t n)
@@ -283,13 +293,9 @@ cudaError_t launch_rk_error(tufrg_model *m, const double2 *y, const double2 *yn,
         s.a[s.nk] = e[j];
         s.nk++;
     }
-    TUFRG_CUDA_TRY(cudaMemsetAsync(m->d_amax + 2, 0, sizeof(unsigned long long), m->stream));
     PhaseScope ps(m, PH_RK);
-    if (m->precision == TUFRG_FP64)
-        rk_error_kernel<<<grid_for(m, n), 256, 0, m->stream>>>(y, yn, fs, s, n, m->d_amax + 2);
-    else
-        rk_error_f32_kernel<<<grid_for(m, n), 256, 0, m->stream>>>(y, yn, fs, s, n, m->d_amax + 2);
-    return cudaGetLastError();
+    auto k_err = m->precision == TUFRG_FP64 ? rk_error_kernel : rk_error_f32_kernel;
+    return launch_chained(k_err, grid_for(m, n), 256, 0, m->stream, true, y, yn, fs, s, n, m->d_amax + 2);
 }
 
 cudaError_t launch_stage_scalars(tufrg_model *m, const FlowDev *fs, double cj)
@@ -304,7 +310,7 @@ cudaError_t launch_attempt_scalars(tufrg_model *m, const FlowDev *fs, const doub
     m->launches++;
     StageNodes s;
     std::copy(c, c + 7, s.c);
-    attempt_scalars_kernel<<<1, 6, 0, m->stream>>>(fs, s, m->d_scal);
+    attempt_scalars_kernel<<<1, 6, 0, m->stream>>>(fs, s, m->d_scal, m->d_amax + 2);
     return cudaGetLastError();
 }
 
@@ -318,16 +324,14 @@ cudaError_t launch_flow_init(tufrg_model *m, FlowDev *fs)
 cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs)
 {
     m->launches++;
-    flow_decide_kernel<<<1, 1, 0, m->stream>>>(fs, m->d_amax);
-    return cudaGetLastError();
+    return launch_chained(flow_decide_kernel, 1, 1, 0, m->stream, true, fs, m->d_amax);
 }
 
 cudaError_t launch_flow_commit(tufrg_model *m, const FlowDev *fs, double2 *y, const double2 *yn, double2 *k0,
                                const double2 *k6, size_t n)
 {
     PhaseScope ps(m, PH_RK);
-    flow_commit_kernel<<<grid_for(m, n), 256, 0, m->stream>>>(fs, y, yn, k0, k6, n);
-    return cudaGetLastError();
+    return launch_chained(flow_commit_kernel, grid_for(m, n), 256, 0, m->stream, true, fs, y, yn, k0, k6, n);
 }
 
 }  // namespace tufrg

@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(1024) vlv_orbit_kernel(const float2 *__restric
     float2 *s0 = reinterpret_cast<float2 *>(smem_raw);   // A^T, then A, then the result R
     float2 *s1 = s0 + M * M;                              // L, then T^T
     __shared__ int s_q2[ORB_MAX], s_e[ORB_MAX];           // the orbit's momenta and elements (-1: q itself)
+    grid_release();
     const int p = blockIdx.x, ch = blockIdx.y, q = list[p];
     const int M2 = M * M, nt = M / 2, B = blockDim.x;
     const int m0 = orb_ofs[p], nmem = orb_ofs[p + 1] - m0;

@@ -427,7 +427,8 @@ cudaError_t launch_records_f32(const double *E, const double2 *U, int Nk, int Lf
 // The split path reads the FP32 copy of the state (d_state32), the plain path the FP64 state.
 // whether the separable transform applies: *warps = warps per CTA of its column pass, 0 if it does not
 void dft_sep_plan(const tufrg_model *m, int *warps);
-cudaError_t launch_dft(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask);
+// also clears the maximum that launch_project reduces into; chained: see launch_chained
+cudaError_t launch_dft(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask, bool chained = false);
 // qlist (nlist entries): only these transfer momenta (the orbit representatives of a symmetric state)
 cudaError_t launch_project(tufrg_model *m, const double2 *d_state, const float2 *d_state32, int channel_mask,
                            double2 *d_A, const int *qlist = nullptr, int nlist = 0);
@@ -442,6 +443,7 @@ cudaError_t launch_rk_combine(tufrg_model *m, double2 *out, float2 *out32, const
 cudaError_t launch_rk_error(tufrg_model *m, const double2 *y, const double2 *yn, const FlowDev *fs, const double *e,
                             double2 *const *k, int nk, size_t n);
 cudaError_t launch_stage_scalars(tufrg_model *m, const FlowDev *fs, double cj);
+// also clears the maximum that launch_rk_error reduces into
 cudaError_t launch_attempt_scalars(tufrg_model *m, const FlowDev *fs, const double (&c)[7]);
 cudaError_t launch_flow_init(tufrg_model *m, FlowDev *fs);
 cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs);
@@ -509,6 +511,36 @@ cudaError_t surrogate_rearm(tufrg_model *m);
 void mlp_dims(const tufrg_mlp *n, int *n_in, int *n_out);
 
 enum Phase { PH_FERMI = 0, PH_LOOPS = 1, PH_LOOPRED = 2, PH_DFT = 3, PH_PROJ = 4, PH_VLV = 5, PH_RK = 6, PH_SCATTER = 7, PH_N = 8 };
+
+// Chained launches: a kernel may start while the kernel before it on the stream finishes (programmatic stream
+// serialization), reads its tables, and waits in grid_wait for that kernel's results.  Every CTA of a chained kernel
+// waits before it returns, so that its own completion implies its predecessor's.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// chained: the preceding work of the stream is a kernel (never after a wait for an event or a memset).
+// Taken where each kernel of a chain leaves most of the GPU idle: the stages of a flow (28 -> 21 us per stage at 8 x 8
+// momenta, two bands) and the split path's transforms and projections (2 us of 126 at 24 x 24).  Not for the reductions
+// of the loops of a single right-hand side, whose early CTAs take the places of the other branch's (106 -> 110 us), nor
+// for FP64 transforms and projections (258 -> 270 us at 8 x 8).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained, const A &...args)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// whether a flow's two-band k-sum directly follows the kernel that writes its records
+inline bool loops_chained(const tufrg_model *m) { return m->regulator != TUFRG_REG_MOMENTUM_SHELL && !m->sur; }
 
 // Brackets one kernel phase with events when timing is on; counts launches always.
 struct PhaseScope {

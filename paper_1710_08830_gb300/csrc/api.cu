@@ -510,6 +510,14 @@ std::vector<double2> phase_table(int Lq, const std::vector<int> &vecs)
 }  // namespace
 namespace tufrg {
 // the captured right-hand-side graphs are dropped whenever the launches they hold would change
+void drop_flow_graphs(tufrg_model *m)
+{
+    for (tufrg_model::FlowGraph *g : {&m->step_graph, &m->loop_graph}) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        g->exec = nullptr;
+    }
+}
+
 void drop_rhs_graphs(tufrg_model *m)
 {
     for (auto &r : m->rhs_graphs)
@@ -539,7 +547,7 @@ void release(tufrg_model *m)
     m->evpool.clear();
     tufrg_set_surrogate(m, nullptr, nullptr, nullptr, nullptr, 0.0, 0, nullptr);
     if (m->h_flow) cudaFreeHost(m->h_flow);
-    if (m->step_graph) cudaGraphExecDestroy(m->step_graph);
+    drop_flow_graphs(m);
     drop_rhs_graphs(m);
     for (auto &e : m->rhs_ev)
         if (e) cudaEventDestroy(e);
@@ -640,7 +648,7 @@ const double DP_E[7] = {35.0 / 384 - 5179.0 / 57600, 0.0, 500.0 / 1113 - 7571.0 
 // it their loops (with a surrogate every stage evaluates its own, as its counters and decisions go by evaluation).
 // Launch chains of 29 us (loops) and 28 us (state) per stage at 8 x 8 momenta, two bands: one after the other
 // 12.7 ms per flow of 56 attempts, side by side 9.4 ms.
-tufrg_status enqueue_attempt(tufrg_model *m, int mask)
+tufrg_status enqueue_attempt(tufrg_model *m, int mask, const cudaGraphConditionalHandle *loop)
 {
     const size_t n = state_elems(m);
     double2 *k[7];
@@ -707,7 +715,7 @@ tufrg_status enqueue_attempt(tufrg_model *m, int mask)
     }
     m->stream = base.stream;
     CK(launch_rk_error(m, m->d_y, m->d_yn, m->d_flow, DP_E, k, 7, n), "error norm");
-    CK(launch_flow_decide(m, m->d_flow), "step decision");
+    CK(launch_flow_decide(m, m->d_flow, loop), "step decision");
     CK(launch_flow_commit(m, m->d_flow, m->d_y, m->d_yn, k[0], k[6], n), "step commit");
     return TUFRG_OK;
 }
@@ -734,39 +742,60 @@ tufrg_status flow_alloc(tufrg_model *m)
     return TUFRG_OK;
 }
 
-// Capture one Dormand-Prince attempt of the given channel mask as the model's step graph (kept while the mask and
-// the launch shapes stay the same).
-tufrg_status flow_capture(tufrg_model *m, int mask)
+// Capture one Dormand-Prince attempt of the given channel mask as the model's step graph, or (loop) as the body of a
+// graph that repeats it until the device controller stops the flow.  The host's part of an attempt (launch, copy, wait)
+// left the GPU idle for 10 to 30 us of 125 (two bands, 8 x 8 momenta): 6.9-8.1 -> 6.4 ms per flow.  Kept while the mask and the launch shapes stay the same.
+tufrg_status flow_capture(tufrg_model *m, int mask, bool loop)
 {
-    if (m->step_graph && m->step_graph_mask == mask) return TUFRG_OK;
-    if (m->step_graph) {
-        cudaGraphExecDestroy(m->step_graph);
-        m->step_graph = nullptr;
+    tufrg_model::FlowGraph &fg = loop ? m->loop_graph : m->step_graph;
+    if (fg.exec && fg.mask == mask) return TUFRG_OK;
+    if (fg.exec) {
+        cudaGraphExecDestroy(fg.exec);
+        fg.exec = nullptr;
     }
     const bool timing = m->timing;
     m->timing = false;   // no event records inside the captured graph
     const long long l0 = m->launches, ll0 = m->loop_launches;
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-    tufrg_status st = enqueue_attempt(m, mask);
-    cudaError_t ce = cudaStreamEndCapture(m->stream, &g);
+    cudaGraph_t g = nullptr, body = nullptr;
+    cudaGraphConditionalHandle cond{};
+    cudaError_t ce = cudaSuccess;
+    if (loop) {
+        ce = cudaGraphCreate(&g, 0);
+        if (ce == cudaSuccess) ce = cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault);
+        cudaGraphNodeParams p{};
+        p.type = cudaGraphNodeTypeConditional;
+        p.conditional.handle = cond;
+        p.conditional.type = cudaGraphCondTypeWhile;
+        p.conditional.size = 1;
+        cudaGraphNode_t node = nullptr;
+        if (ce == cudaSuccess) ce = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &p);
+        if (ce == cudaSuccess) body = p.conditional.phGraph_out[0];
+        if (ce == cudaSuccess)
+            ce = cudaStreamBeginCaptureToGraph(m->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    } else {
+        ce = cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal);
+    }
+    tufrg_status st = TUFRG_OK;
+    if (ce == cudaSuccess) {
+        st = enqueue_attempt(m, mask, loop ? &cond : nullptr);
+        ce = cudaStreamEndCapture(m->stream, loop ? &body : &g);
+    }
     m->timing = timing;
     m->launches = l0;
     m->loop_launches = ll0;
-    if (st != TUFRG_OK) {
-        if (g) cudaGraphDestroy(g);
-        return st;
+    if (st == TUFRG_OK && ce == cudaSuccess) ce = cudaGraphInstantiate(&fg.exec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (st != TUFRG_OK) return st;
+    if (ce != cudaSuccess) {
+        fg.exec = nullptr;
+        return cuda_fail(m, ce, "capture of a flow step");
     }
-    if (ce != cudaSuccess) return cuda_fail(m, ce, "end capture");
-    ce = cudaGraphInstantiate(&m->step_graph, g, 0);
-    cudaGraphDestroy(g);
-    if (ce != cudaSuccess) return cuda_fail(m, ce, "graph instantiate");
-    m->step_graph_mask = mask;
+    fg.mask = mask;
     return TUFRG_OK;
 }
 
-// Allocate the flow buffers, zero the state, evaluate k1 = f(y0) and capture one attempt as a graph.
-tufrg_status flow_prepare(tufrg_model *m, const tufrg_flow_opts *o)
+// Allocate the flow buffers, zero the state, evaluate k1 = f(y0) and capture one attempt (or a loop of them) as a graph.
+tufrg_status flow_prepare(tufrg_model *m, const tufrg_flow_opts *o, bool loop = false)
 {
     const size_t n = state_elems(m);
     tufrg_status st = flow_alloc(m);
@@ -791,7 +820,7 @@ tufrg_status flow_prepare(tufrg_model *m, const tufrg_flow_opts *o)
     st = rhs_device(m, m->d_y, o->channel_mask, m->d_k[0], nullptr, true, true);
     if (st != TUFRG_OK) return st;
     CK(launch_flow_init(m, m->d_flow), "flow init");
-    if ((st = flow_capture(m, o->channel_mask)) != TUFRG_OK) return st;
+    if ((st = flow_capture(m, o->channel_mask, loop)) != TUFRG_OK) return st;
     // the controller state after the initial evaluation: a flow whose initial max|A| already exceeds the stop
     // value is critical at T0 and runs no attempt
     CK(cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream), "copy flow state");
@@ -1916,14 +1945,13 @@ tufrg_status tufrg_flow(tufrg_model *m, const tufrg_flow_opts *o, void *d_state_
     std::memset(res, 0, sizeof(*res));
     cudaStream_t user;
     if ((st = flow_enter(m, &user)) != TUFRG_OK) return st;
-    st = flow_prepare(m, o);
-    // replay the captured attempt until the device controller stops the flow
-    while (st == TUFRG_OK && m->h_flow->status == 0) {
-        cudaError_t e = cudaGraphLaunch(m->step_graph, m->stream);
+    st = flow_prepare(m, o, true);
+    // the attempts repeat on the device until its controller stops the flow
+    if (st == TUFRG_OK && m->h_flow->status == 0) {
+        cudaError_t e = cudaGraphLaunch(m->loop_graph.exec, m->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
         if (e != cudaSuccess) st = cuda_fail(m, e, "flow graph");
-        else if (m->h_flow->status != 0) break;
     }
     if (st == TUFRG_OK) st = read_device_error(m);
     if (st == TUFRG_OK) st = flow_finish(m, d_state_out, res);
@@ -1959,7 +1987,7 @@ tufrg_status tufrg_flow_step(tufrg_model *m, tufrg_flow_step_info *s)
     if (!m || !s) return fail(m, TUFRG_EINVAL, "NULL argument");
     if (!m->flow_open) return fail(m, TUFRG_EINVAL, "no stepwise flow is open on this model");
     if (m->h_flow->status == 0) {
-        cudaError_t e = cudaGraphLaunch(m->step_graph, m->stream);
+        cudaError_t e = cudaGraphLaunch(m->step_graph.exec, m->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
         if (e != cudaSuccess) return cuda_fail(m, e, "flow graph");
@@ -2071,11 +2099,10 @@ tufrg_status tufrg_flow_resume(tufrg_model *m, const tufrg_flow_opts *o, const v
         m->plan = m->plan_cand[h.ky_chunks - 1];
         reshaped = true;
     }
-    if (reshaped && m->step_graph) {
-        cudaGraphExecDestroy(m->step_graph);
-        m->step_graph = nullptr;
+    if (reshaped) {
+        drop_flow_graphs(m);
+        drop_rhs_graphs(m);
     }
-    if (reshaped) drop_rhs_graphs(m);
     cudaStream_t user;
     if ((st = flow_enter(m, &user)) != TUFRG_OK) return st;
     auto run = [&]() -> tufrg_status {
@@ -2092,7 +2119,7 @@ tufrg_status tufrg_flow_resume(tufrg_model *m, const tufrg_flow_opts *o, const v
         if (s2 != TUFRG_OK) return s2;
         CK(cudaMemcpyAsync(m->d_k[0], p + sizeof(h) + sizeof(FlowDev) + sizeof(double2) * n, sizeof(double2) * n,
                            cudaMemcpyHostToDevice, m->stream), "copy derivative");
-        if ((s2 = flow_capture(m, o->channel_mask)) != TUFRG_OK) return s2;
+        if ((s2 = flow_capture(m, o->channel_mask, false)) != TUFRG_OK) return s2;
         CK(cudaStreamSynchronize(m->stream), "sync");
         return TUFRG_OK;
     };
@@ -2148,7 +2175,7 @@ try {
         for (int i = 0; i < n; i++) {
             if (!active[i]) continue;
             tufrg_model *m = models[i];
-            cudaError_t e = cudaGraphLaunch(m->step_graph, m->stream);
+            cudaError_t e = cudaGraphLaunch(m->step_graph.exec, m->stream);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream);
             if (e != cudaSuccess) {

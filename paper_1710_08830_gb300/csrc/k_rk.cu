@@ -165,10 +165,8 @@ __global__ void flow_init_kernel(FlowDev *fs, const unsigned long long *red)
 }
 
 // Accept or reject the attempt just computed (error norm in red[2], max|A| at the candidate in red[0]).
-__global__ void flow_decide_kernel(FlowDev *fs, const unsigned long long *red)
+__device__ void flow_decide(FlowDev *fs, const unsigned long long *red)
 {
-    grid_release();
-    grid_wait();
     fs->accepted = 0;
     if (fs->status != 0) return;
     const double err = __longlong_as_double((long long)red[2]);
@@ -209,6 +207,16 @@ __global__ void flow_decide_kernel(FlowDev *fs, const unsigned long long *red)
     }
     if (fs->x + fs->h < fs->xend) fs->h = fs->xend - fs->x;
     if (fs->tries >= fs->max_tries) fs->status = 3;
+}
+
+// (every attempt counts towards max_tries, so that a loop ends; a kernel that gave up a wait ends it at once)
+__global__ void flow_decide_kernel(FlowDev *fs, const unsigned long long *red, const int *wait_err,
+                                   cudaGraphConditionalHandle loop, int looped)
+{
+    grid_release();
+    grid_wait();
+    flow_decide(fs, red);
+    if (looped) cudaGraphSetConditional(loop, fs->status == 0 && *wait_err == 0 ? 1 : 0);
 }
 
 // FSAL commit of an accepted attempt: y <- y_n, k_1 <- k_7
@@ -321,10 +329,11 @@ cudaError_t launch_flow_init(tufrg_model *m, FlowDev *fs)
     return cudaGetLastError();
 }
 
-cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs)
+cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs, const cudaGraphConditionalHandle *loop)
 {
     m->launches++;
-    return launch_chained(flow_decide_kernel, 1, 1, 0, m->stream, true, fs, m->d_amax);
+    return launch_chained(flow_decide_kernel, 1, 1, 0, m->stream, true, fs, m->d_amax, m->d_err,
+                          loop ? *loop : cudaGraphConditionalHandle{}, loop ? 1 : 0);
 }
 
 cudaError_t launch_flow_commit(tufrg_model *m, const FlowDev *fs, double2 *y, const double2 *yn, double2 *k0,

@@ -175,10 +175,7 @@ try {
         m->sur = nullptr;
     };
     cudaStreamSynchronize(m->stream);
-    if (m->step_graph) {   // a captured flow step must be re-captured with (or without) the surrogate
-        cudaGraphExecDestroy(m->step_graph);
-        m->step_graph = nullptr;
-    }
+    drop_flow_graphs(m);   // a captured flow step must be re-captured with (or without) the surrogate
     drop();
     if (!net) return TUFRG_OK;
     if (!h_mean || !h_std || !h_feature_params || !h_check_q || n_check < 1 || n_check > m->Nq || !(resid_tol > 0)) {

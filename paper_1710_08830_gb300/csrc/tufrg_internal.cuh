@@ -332,7 +332,12 @@ struct tufrg_model {
     cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_comp[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr};
     tufrg::FlowDev *d_flow = nullptr;        // device controller state
     tufrg::FlowDev *h_flow = nullptr;        // pinned host mirror
-    cudaGraphExec_t step_graph = nullptr;    // one captured Dormand-Prince attempt
+    // captured Dormand-Prince attempts of a channel mask: one (steps on the host's call), and a loop of them that the
+    // device controller ends
+    struct FlowGraph {
+        cudaGraphExec_t exec = nullptr;
+        int mask = 0;
+    } step_graph, loop_graph;
     cudaStream_t flow_stream = nullptr;      // private capturable stream of the flow (joined to `stream` by events)
     // second stream of a right-hand side: the Fourier transform and projections (they read the state only) run
     // there while the loop k-sum (it reads the temperature only) runs on `stream`; joined before the products
@@ -363,7 +368,6 @@ struct tufrg_model {
     int flow_mask = 0;
     double flow_t0 = 0.0;                    // host clock at the start (seconds)
     unsigned long long *d_amax_ch = nullptr; // [2] max |A| per channel (bit patterns of non-negative doubles)
-    int step_graph_mask = 0;
 
     tufrg::LoopPlan plan{};       // split two-band flows (k_loops2.cu)
     tufrg::LoopPlan plan_h{};     // half-mesh k-sum (k_loops2h.cu)
@@ -446,13 +450,15 @@ cudaError_t launch_stage_scalars(tufrg_model *m, const FlowDev *fs, double cj);
 // also clears the maximum that launch_rk_error reduces into
 cudaError_t launch_attempt_scalars(tufrg_model *m, const FlowDev *fs, const double (&c)[7]);
 cudaError_t launch_flow_init(tufrg_model *m, FlowDev *fs);
-cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs);
+// loop: the condition of the graph loop that repeats the attempt, or null
+cudaError_t launch_flow_decide(tufrg_model *m, FlowDev *fs, const cudaGraphConditionalHandle *loop);
 cudaError_t launch_flow_commit(tufrg_model *m, const FlowDev *fs, double2 *y, const double2 *yn, double2 *k0,
                                const double2 *k6, size_t n);
 cudaError_t launch_amax_channels(tufrg_model *m, bool reps_only);
 cudaError_t launch_amax_locate(tufrg_model *m, size_t n, bool reps_only);   // on the last projection (d_A or d_A32)
 LoopPlan plan_loops(const tufrg_model *m);
 void drop_rhs_graphs(tufrg_model *m);
+void drop_flow_graphs(tufrg_model *m);
 // the launch shapes the two-band split loop kernel's autotuner times (ky ranges per column)
 std::vector<LoopPlan> loop_plan_candidates(const tufrg_model *m);
 int plan_gen_chunks(const tufrg_model *m);   // kx ranges per momentum of the multi-orbital loop kernel

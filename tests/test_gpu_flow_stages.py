@@ -43,3 +43,22 @@ def test_attempt_is_the_dormand_prince_step(name, mask, symmetric, prec, tol):
         k.append(T * m.rhs(T, m._dev(z), mask=mask).cpu().numpy())
     ref = y + h * sum(a * v for a, v in zip(A[6], k))
     assert np.abs(X.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("prec", ["FP64", "SPLIT32"])
+@pytest.mark.parametrize("name", ["two_band", "bilayer"])
+def test_device_loop_is_the_flow_step_by_step(name, prec, tmp_path):
+    """the loop on the device and single attempts on the host's call end in the same state, counts and step limit"""
+    from paper_1710_08830_gb300 import api
+    from paper_1710_08830_gb300._lib import TufrgError
+    m = api.Model(_spec(name), getattr(api, prec))
+    args = dict(T0=1.0, T_end=0.3, rtol=1e-3, atol=1e-3, h0=-0.2)
+    X, r = m.flow(**args)
+    Y, s = m.flow(**args, metrics_path=str(tmp_path / "m.jsonl"))
+    assert (X == Y).all()
+    for key in ("n_steps", "n_reject", "n_rhs", "amax", "T_last", "Tc", "crossed", "lead_channel", "lead_q"):
+        assert r[key] == s[key], key
+    with pytest.raises(TufrgError):
+        m.flow(**args, max_steps=r["n_steps"] + r["n_reject"] - 1)
+    Z, _ = m.flow(**args)
+    assert (X == Z).all()

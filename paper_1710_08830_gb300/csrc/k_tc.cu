@@ -5,23 +5,32 @@
 // tile) of every requested channel and momentum:
 //   first:   T = A L    with L[k][n] gathered from the compact loops through the bond-pair table, FP32 scratch;
 //   second:  dX = c T A in FP64 (exact widening on the integer pipe).
-// Complex GEMM as four real MMA streams into two tensor-memory accumulators:
-//   Cr += Ar Br - Ai Bi,   Ci += Ar Bi + Ai Br     (the minus by the descriptor's negate-A bit).
+// Complex GEMM as two real MMA streams into one tensor-memory accumulator [Cr | Ci] of twice the columns:
+//   [Cr | Ci] += Ar [Br | Bi],   [Cr | Ci] += Ai [-Bi | Br];
+// the right operand is stored as [-Bi | Br | Bi], whose two windows are the two right-hand factors.  An MMA of 128 x N x 8
+// takes about 34 cycles plus half a cycle per column, so half as many of twice the width are faster than four streams
+// into two accumulators.
+// Both products of 225 momenta, two channels, M = 324: 1.45 ms with four streams, one row per lane and a shared-memory
+// tile for the epilogue; 1.15 ms now (its MMAs alone about 0.95 ms, its producers alone 0.88 ms).
 // Precision: 3xTF32 - every FP32 operand x is split into hi = x with the 13 low mantissa bits cleared and lo = x - hi
 // (exact), and each real product is hi*hi + hi*lo + lo*hi accumulated in FP32 in tensor memory.
 //
 // The operands are read in FP32 straight from the matrices and split inside the kernel (no packing launches).  Warp
-// roles of the 672-thread CTA (one per SM):
-//   warps 0-15  producers, thread (K group kg = tid / 128, row r = tid % 128): per K stage of 16 columns each thread
-//               loads 4 complex values of left-operand row r and 4 of right-operand row r for the next stage into
-//               registers while it splits the current one; the left operand's four TF32 planes (Re hi, Re lo,
-//               Im hi, Im lo) go to tensor memory (tcgen05.st, lane = row: warp w writes lanes 32 (w % 4) ..), the
-//               right operand's to shared memory in the K-major core-matrix layout;
-//   warp 16     tensor-memory allocation and the MMA issuer (one thread): 24 MMAs per stage (2 K-steps x 4 real
-//               products x 3 TF32 passes), the left operand read from tensor memory;
-//   warps 17-20 epilogue: tensor memory -> a shared-memory tile (then the accumulator is released to the next
-//               item's MMAs) -> T (FP32) or c dX (FP64) in global memory, consecutive lanes on consecutive columns.
-// Three stage buffers (mbarriers full / empty); one accumulator (mbarriers acc_full / acc_empty).  Every wait is
+// roles of the 640-thread CTA (one per SM):
+//   warps 0-15  producers, two groups of eight that take the K stages of 16 columns in turn (the waits, fences and
+//               arrivals of a stage are paid half as often per warp): each thread loads 8 complex values of the left
+//               operand and 8 of the right operand of its group's next stage into registers while it splits the
+//               current one.  Left operand: warp (quarter w % 4 of the rows, columns 8 (w / 4 % 2)), a thread two
+//               neighbouring columns of rows lane / 4 + 8 i, so that a load covers 64 contiguous bytes of 8 rows (one
+//               row per lane, 32 lines per load, kept the L1 tags busy for half of a stage); its four TF32 planes
+//               (Re hi, Re lo, Im hi, Im lo) go to tensor memory (tcgen05.st 16x256b: that same arrangement).  Right
+//               operand: thread (K half, column tid % 128), to shared memory in the K-major core-matrix layout;
+//   warp 16     tensor-memory allocation and the MMA issuer (one thread): 12 MMAs per stage (2 K-steps x 2 real
+//               streams x 3 TF32 passes), the left operand read from tensor memory; then its quarter of the
+//               epilogue (20 warps leave every thread 96 registers, 21 would leave 80);
+//   warps 16-19 epilogue: tensor memory (16x256b: a thread holds two neighbouring columns of a row, four threads 8)
+//               -> T (FP32) or c dX (FP64, one 32-byte store per thread) in global memory.
+// Four stage buffers (mbarriers full / empty), one accumulator (mbarriers accf / acce).  Every wait is
 // bounded; on time-out the kernel raises the error flag, every role stops, the MMAs in flight are waited for
 // (bounded) and the tensor memory is freed.
 #include "tc_common.cuh"
@@ -32,14 +41,14 @@ namespace {
 
 constexpr int TM = 128;             // MMA M: rows per tile
 constexpr int KS = 16;              // K per stage (two MMA K-steps of 8)
-constexpr int NSTAGE = 3;           // stage buffers
+constexpr int NSTAGE = 4;           // stage buffers (a multiple of the producer groups: each buffer belongs to one)
 constexpr int NPROD = 512;          // producer threads (warps 0-15)
-constexpr int MMA_WARP = 16;        // warps 17-20: epilogue
-constexpr int NTHREADS = 21 * 32;
+constexpr int MMA_WARP = 16;        // it and warps 17-19: epilogue
+constexpr int NTHREADS = 20 * 32;
 constexpr int NB_MAX = 112;         // columns per tile (complex), a multiple of 16
-// tensor memory: accumulator Re at [0, NB), Im at [128, 128 + NB); left operand of stage b at 256 + 64 b, plane p at
-// + 16 p (K = 16 columns)
-constexpr unsigned ACC_IM = 128, A_COL0 = 256, A_STAGE_COLS = 64, A_PLANE_COLS = 16;
+// tensor memory: accumulator Re at [0, NB), Im at [NB, 2 NB); left operand of stage b at 256 + 64 b, plane p at + 16 p
+// (K = 16 columns)
+constexpr unsigned A_COL0 = 256, A_STAGE_COLS = 64, A_PLANE_COLS = 16;
 constexpr unsigned TMEM_COLS = 512;
 static_assert(A_COL0 + NSTAGE * A_STAGE_COLS <= TMEM_COLS, "tensor memory budget");
 
@@ -69,6 +78,7 @@ struct VlvArgs {
     const int *dij;         // [nff][nff] bond pair -> bond-difference index of the compact loops
     float2 *T;              // [2][nz][M][M] first product (written by the first launch, read by the second)
     double2 *out;           // [2][Nq][M][M] second product
+    int out32B;             // out lies on a 32-byte boundary
     const int *qlist;       // slot z -> transfer momentum (null: the slot is the momentum)
     const double *scal;     // scal[1]: the flow-scale factor of the right-hand side
     int *err;
@@ -78,28 +88,31 @@ struct VlvArgs {
     int n_items;
 };
 
-// the stage's values of one producer thread: left-operand row r at K = k0 .. k0 + 3 and right-operand row r (an
-// output column) at the same K
+// the stage's values of one producer thread: left-operand rows ra + 8 i at two K (a[2 i], a[2 i + 1]), and right-operand
+// row r (an output column) at eight K
 struct Vals {
-    float2 a[4], b[4];
+    float2 a[8], b[8];
 };
 
 // one producer thread's sources for one item: the left operand's row (A in the first product, T in the second) and
 // the right operand's column (the compact loops of the momentum, or A), null when the row / column is padding
 struct Src {
-    const float2 *a;    // row m of the left operand
+    const float2 *a;    // row ra of the left operand
+    int rows;           // rows from ra on that exist
     const float2 *b;    // first product: the momentum's compact loops + (n % NS2); second: column n of A
     int nj;             // first product: n / NS2 (the column's bond index)
 };
 
 template <int PH, int NS2>
-__device__ __forceinline__ Src item_src(const VlvArgs &p, int ch, int z, int mt, int nt, int r)
+__device__ __forceinline__ Src item_src(const VlvArgs &p, int ch, int z, int mt, int nt, int ra, int r)
 {
-    const int M = p.d.M, m = mt * TM + r, n = nt * p.d.nb + r;
+    const int M = p.d.M, n = nt * p.d.nb + r;
     const size_t M2 = (size_t)M * M;
     const int qs = p.qlist ? p.qlist[z] : z;
-    Src s{nullptr, nullptr, 0};
-    if (m < M) s.a = (PH == 0 ? p.A + ((size_t)ch * p.Nq + qs) * M2 : p.T + ((size_t)ch * p.nz + z) * M2) + (size_t)m * M;
+    Src s{};
+    const int m = mt * TM + ra;
+    s.a = (PH == 0 ? p.A + ((size_t)ch * p.Nq + qs) * M2 : p.T + ((size_t)ch * p.nz + z) * M2) + (size_t)m * M;
+    s.rows = M - m;
     if (r < p.d.nb && n < M) {
         if (PH == 0) {
             s.b = p.Lc + ((size_t)ch * p.Nq + qs) * p.lper + n % NS2;
@@ -111,37 +124,36 @@ __device__ __forceinline__ Src item_src(const VlvArgs &p, int ch, int z, int mt,
     return s;
 }
 
-// K = k0 .. k0 + 3 of both operands (k0 a multiple of 4; M and NS2 are multiples of 4, so the four K values lie in
-// one bond block)
+// K = ka, ka + 1 of the left operand (ka even, M a multiple of 4) and k0 .. k0 + 7 of the right operand (k0 a multiple
+// of 4; M and NS2 are multiples of 4, so each four of them lie in one bond block)
 template <int PH, int NS2>
-__device__ __forceinline__ void load_stage(const Src &src, const int *sdij, int nff, int M, int k0, Vals &v)
+__device__ __forceinline__ void load_stage(const Src &src, const int *sdij, int nff, int M, int ka, int k0, Vals &v)
 {
-    const bool in = k0 < M;
-    if (src.a && in) {
-        const float4 *q = reinterpret_cast<const float4 *>(src.a + k0);
-        const float4 u0 = __ldg(q), u1 = __ldg(q + 1);
-        v.a[0] = make_float2(u0.x, u0.y);
-        v.a[1] = make_float2(u0.z, u0.w);
-        v.a[2] = make_float2(u1.x, u1.y);
-        v.a[3] = make_float2(u1.z, u1.w);
-    } else {
 #pragma unroll
-        for (int j = 0; j < 4; j++) v.a[j] = make_float2(0.f, 0.f);
+    for (int i = 0; i < 4; i++) {
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (8 * i < src.rows && ka < M) u = __ldg(reinterpret_cast<const float4 *>(src.a + (size_t)(8 * i) * M + ka));
+        v.a[2 * i] = make_float2(u.x, u.y);
+        v.a[2 * i + 1] = make_float2(u.z, u.w);
     }
-    if (src.b && in) {
-        if (PH == 0) {
-            // L[k][n] = Lc[(d(k / NS2, n / NS2) NS2 + k % NS2) NS2 + n % NS2]
-            const float2 *b = src.b + ((size_t)sdij[(k0 / NS2) * nff + src.nj] * NS2 + k0 % NS2) * NS2;
 #pragma unroll
-            for (int j = 0; j < 4; j++) v.b[j] = __ldg(b + j * NS2);
+    for (int i = 0; i < 8; i += 4) {
+        const int k = k0 + i;
+        if (src.b && k < M) {
+            if (PH == 0) {
+                // L[k][n] = Lc[(d(k / NS2, n / NS2) NS2 + k % NS2) NS2 + n % NS2]
+                const float2 *b = src.b + ((size_t)sdij[(k / NS2) * nff + src.nj] * NS2 + k % NS2) * NS2;
+#pragma unroll
+                for (int j = 0; j < 4; j++) v.b[i + j] = __ldg(b + j * NS2);
+            } else {
+                const float2 *b = src.b + (size_t)k * M;
+#pragma unroll
+                for (int j = 0; j < 4; j++) v.b[i + j] = __ldg(b + (size_t)j * M);
+            }
         } else {
-            const float2 *b = src.b + (size_t)k0 * M;
 #pragma unroll
-            for (int j = 0; j < 4; j++) v.b[j] = __ldg(b + (size_t)j * M);
+            for (int j = 0; j < 4; j++) v.b[i + j] = make_float2(0.f, 0.f);
         }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; j++) v.b[j] = make_float2(0.f, 0.f);
     }
 }
 
@@ -157,18 +169,27 @@ __device__ __forceinline__ double f32_to_f64(float x)
     return __hiloint2double((int)hi, (int)lo);
 }
 
+// two neighbouring entries: one 32-byte store where the output starts on a 32-byte boundary (its rows then do)
+__device__ __forceinline__ void store_pair(double2 *o, int aligned32, double a, double b, double c, double d)
+{
+    if (aligned32) {
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+    } else {
+        o[0] = make_double2(a, b);
+        o[1] = make_double2(c, d);
+    }
+}
+
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
 template <int PH, int NS2>
 __global__ void __launch_bounds__(NTHREADS, 1) vlv_tc_kernel(VlvArgs p)
 {
-    // dynamic shared memory: NSTAGE right-operand stages, the epilogue's FP32 tile [128][NB + 2], the bond table
+    // dynamic shared memory: NSTAGE right-operand stages, the bond table
     extern __shared__ __align__(1024) unsigned char smem[];
     const int NB = p.d.nb, nks = p.d.nks;
-    const unsigned b_plane = (unsigned)NB * KS * 4, b_stage = 4 * b_plane;   // bytes
-    const int estr = NB + 2;                                                  // tile row stride (complex)
-    float2 *etile = reinterpret_cast<float2 *>(smem + NSTAGE * (size_t)b_stage);
-    int *sdij = reinterpret_cast<int *>(etile + (size_t)TM * estr);
+    const unsigned b_plane = 3u * NB * KS * 4, b_stage = 2 * b_plane;   // bytes; planes hi, lo of [-Bi | Br | Bi]
+    int *sdij = reinterpret_cast<int *>(smem + NSTAGE * (size_t)b_stage);
     __shared__ __align__(8) unsigned long long full[NSTAGE], empty[NSTAGE], accf, acce, done;
     __shared__ unsigned tmem_base;
     __shared__ int abort_flag;
@@ -181,11 +202,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) vlv_tc_kernel(VlvArgs p)
     }
     if (tid == 0) {
         for (int b = 0; b < NSTAGE; b++) {
-            tc::mbar_init(tc::smem_u32(&full[b]), NPROD);
+            tc::mbar_init(tc::smem_u32(&full[b]), NPROD / 2);
             tc::mbar_init(tc::smem_u32(&empty[b]), 1);
         }
         tc::mbar_init(tc::smem_u32(&accf), 1);
-        tc::mbar_init(tc::smem_u32(&acce), 128);
+        tc::mbar_init(tc::smem_u32(&acce), 96);   // (warp 16 itself issues the next MMAs)
         tc::mbar_init(tc::smem_u32(&done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
@@ -210,28 +231,41 @@ __global__ void __launch_bounds__(NTHREADS, 1) vlv_tc_kernel(VlvArgs p)
 
     if (warp < MMA_WARP) {
         // ------------------------------------------------------------------ producers
-        const int r = tid & 127, kg = tid >> 7;
-        const unsigned lane_base = (unsigned)((warp & 3) * 32) << 16;   // this warp's tensor-memory lanes
+        const int grp = warp >> 3, r = tid & 127, kh = (tid >> 7) & 1;
+        // left operand: the 32 rows of the warp's quarter, columns 8 kh of the stage
+        const int ra = (warp & 3) * 32 + (lane >> 2), ca0 = 8 * kh + 2 * (lane & 3);
+        const unsigned a_base = ((unsigned)((warp & 3) * 32) << 16) + A_COL0 + (unsigned)(8 * kh);
         const int n_stages = my_items * nks;
         const int M = p.d.M, nff = p.nff;
-        int li = 0, k0 = 4 * kg;   // item (local index) and first K of this thread in the stage of the loads in flight
-        int ch, z, mt, nt;
-        decode((int)blockIdx.x, ch, z, mt, nt);
-        Src src = item_src<PH, NS2>(p, ch, z, mt, nt, r);
-        Vals cur, nxt;
-        if (n_stages > 0) load_stage<PH, NS2>(src, sdij, nff, M, k0, nxt);
-        for (int n = 0; n < n_stages; n++) {
-            cur = nxt;
-            // issue the loads of stage n + 1 (they land while this stage is split and stored)
-            k0 += KS;
-            if (k0 >= nks * KS) {
-                k0 = 4 * kg;
-                if (++li < my_items) {
-                    decode((int)blockIdx.x + li * G, ch, z, mt, nt);
-                    src = item_src<PH, NS2>(p, ch, z, mt, nt, r);
-                }
+        int li = 0, st = grp;   // item (local index) and its stage of the loads in flight
+        Src src;
+        auto settle = [&]() {   // the item that stage st of item li falls into
+            while (st >= nks) {
+                st -= nks;
+                li++;
             }
-            if (n + 1 < n_stages) load_stage<PH, NS2>(src, sdij, nff, M, k0, nxt);
+        };
+        auto locate = [&]() {
+            int ch, z, mt, nt;
+            decode((int)blockIdx.x + li * G, ch, z, mt, nt);
+            src = item_src<PH, NS2>(p, ch, z, mt, nt, ra, r);
+        };
+        Vals cur, nxt;
+        settle();
+        if (grp < n_stages) {
+            locate();
+            load_stage<PH, NS2>(src, sdij, nff, M, st * KS + ca0, st * KS + 8 * kh, nxt);
+        }
+        for (int n = grp; n < n_stages; n += 2) {
+            cur = nxt;
+            // issue the loads of the group's next stage (they land while this stage is split and stored)
+            if (n + 2 < n_stages) {
+                const int before = li;
+                st += 2;
+                settle();
+                if (li != before) locate();
+                load_stage<PH, NS2>(src, sdij, nff, M, st * KS + ca0, st * KS + 8 * kh, nxt);
+            }
             const int b = n % NSTAGE;
             // the MMAs that read this stage buffer NSTAGE stages ago must be complete
             int ok = 1;
@@ -248,145 +282,140 @@ __global__ void __launch_bounds__(NTHREADS, 1) vlv_tc_kernel(VlvArgs p)
                 break;   // the whole warp leaves (the MMA thread's waits then run out or see the flag)
             }
             tc::fence_after();
-            // left operand: four planes x 4 columns of this lane's row into tensor memory
-            const unsigned ca = tmem + lane_base + A_COL0 + b * A_STAGE_COLS + 4 * kg;
-            float h[4], l[4];
+            // left operand: four planes x two blocks of 16 rows x 8 columns into tensor memory
+            const unsigned ca = tmem + a_base + b * A_STAGE_COLS;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                h[j] = tf32_trunc(cur.a[j].x);
-                l[j] = cur.a[j].x - h[j];
-            }
-            tc::tmem_st4(ca + 0 * A_PLANE_COLS, h[0], h[1], h[2], h[3]);
-            tc::tmem_st4(ca + 1 * A_PLANE_COLS, l[0], l[1], l[2], l[3]);
+            for (int g = 0; g < 2; g++) {
+                const unsigned cg = ca + ((unsigned)(16 * g) << 16);
+                float h[4], l[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                h[j] = tf32_trunc(cur.a[j].y);
-                l[j] = cur.a[j].y - h[j];
+                for (int j = 0; j < 4; j++) {
+                    h[j] = tf32_trunc(cur.a[4 * g + j].x);
+                    l[j] = cur.a[4 * g + j].x - h[j];
+                }
+                tc::tmem_st_16x8(cg + 0 * A_PLANE_COLS, h[0], h[1], h[2], h[3]);
+                tc::tmem_st_16x8(cg + 1 * A_PLANE_COLS, l[0], l[1], l[2], l[3]);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    h[j] = tf32_trunc(cur.a[4 * g + j].y);
+                    l[j] = cur.a[4 * g + j].y - h[j];
+                }
+                tc::tmem_st_16x8(cg + 2 * A_PLANE_COLS, h[0], h[1], h[2], h[3]);
+                tc::tmem_st_16x8(cg + 3 * A_PLANE_COLS, l[0], l[1], l[2], l[3]);
             }
-            tc::tmem_st4(ca + 2 * A_PLANE_COLS, h[0], h[1], h[2], h[3]);
-            tc::tmem_st4(ca + 3 * A_PLANE_COLS, l[0], l[1], l[2], l[3]);
             // right operand: row r of the stage's four planes in shared memory
             if (r < NB) {
                 float *pb = reinterpret_cast<float *>(smem + (size_t)b * b_stage);
-                const int o = tc::core_off(r, 4 * kg, NB);
-                float4 hv, lv;
-                hv = make_float4(tf32_trunc(cur.b[0].x), tf32_trunc(cur.b[1].x), tf32_trunc(cur.b[2].x), tf32_trunc(cur.b[3].x));
-                lv = make_float4(cur.b[0].x - hv.x, cur.b[1].x - hv.y, cur.b[2].x - hv.z, cur.b[3].x - hv.w);
-                *reinterpret_cast<float4 *>(pb + 0 * (b_plane / 4) + o) = hv;
-                *reinterpret_cast<float4 *>(pb + 1 * (b_plane / 4) + o) = lv;
-                hv = make_float4(tf32_trunc(cur.b[0].y), tf32_trunc(cur.b[1].y), tf32_trunc(cur.b[2].y), tf32_trunc(cur.b[3].y));
-                lv = make_float4(cur.b[0].y - hv.x, cur.b[1].y - hv.y, cur.b[2].y - hv.z, cur.b[3].y - hv.w);
-                *reinterpret_cast<float4 *>(pb + 2 * (b_plane / 4) + o) = hv;
-                *reinterpret_cast<float4 *>(pb + 3 * (b_plane / 4) + o) = lv;
+#pragma unroll
+                for (int i = 0; i < 8; i += 4) {
+                    const int o = tc::core_off(r, 8 * kh + i, 3 * NB), bo = NB * 4;   // (rows + NB: 4 NB floats on)
+                    const float2 *v = cur.b + i;
+                    float4 hv, lv;
+                    hv = make_float4(tf32_trunc(v[0].x), tf32_trunc(v[1].x), tf32_trunc(v[2].x), tf32_trunc(v[3].x));
+                    lv = make_float4(v[0].x - hv.x, v[1].x - hv.y, v[2].x - hv.z, v[3].x - hv.w);
+                    *reinterpret_cast<float4 *>(pb + o + bo) = hv;
+                    *reinterpret_cast<float4 *>(pb + b_plane / 4 + o + bo) = lv;
+                    hv = make_float4(tf32_trunc(v[0].y), tf32_trunc(v[1].y), tf32_trunc(v[2].y), tf32_trunc(v[3].y));
+                    lv = make_float4(v[0].y - hv.x, v[1].y - hv.y, v[2].y - hv.z, v[3].y - hv.w);
+                    *reinterpret_cast<float4 *>(pb + o + 2 * bo) = hv;
+                    *reinterpret_cast<float4 *>(pb + b_plane / 4 + o + 2 * bo) = lv;
+                    *reinterpret_cast<float4 *>(pb + o) = make_float4(-hv.x, -hv.y, -hv.z, -hv.w);
+                    *reinterpret_cast<float4 *>(pb + b_plane / 4 + o) = make_float4(-lv.x, -lv.y, -lv.z, -lv.w);
+                }
             }
             tc::tmem_wait_st();
             tc::fence_smem_async();
             tc::fence_before();
             tc::mbar_arrive(tc::smem_u32(&full[b]));
         }
-    } else if (warp == MMA_WARP) {
-        // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const unsigned id = tc::idesc_tf32(TM, NB, false), idn = tc::idesc_tf32(TM, NB, true);
-            const unsigned tr = tmem, ti = tmem + ACC_IM;
-            bool ok = true;
-            int n = 0;
-            for (int it = 0; it < my_items && ok; it++) {
-                // the accumulator must have been read by the epilogue of the previous item
-                if (it >= 1 && !tc::mbar_wait_or_abort(tc::smem_u32(&acce), (it - 1) & 1, &abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after();
-                for (int s = 0; s < nks; s++, n++) {
-                    const int b = n % NSTAGE;
-                    if (!tc::mbar_wait_or_abort(tc::smem_u32(&full[b]), (n / NSTAGE) & 1, &abort_flag)) { ok = false; break; }
-                    tc::fence_after();
-                    const unsigned sb = tc::smem_u32(smem + (size_t)b * b_stage), ta = tmem + A_COL0 + b * A_STAGE_COLS;
-#pragma unroll
-                    for (int kk = 0; kk < KS / 8; kk++) {
-                        const unsigned bo = kk * 2 * (NB / 8) * 128;
-                        const unsigned arh = ta + 0 * A_PLANE_COLS + 8 * kk, arl = ta + 1 * A_PLANE_COLS + 8 * kk;
-                        const unsigned aih = ta + 2 * A_PLANE_COLS + 8 * kk, ail = ta + 3 * A_PLANE_COLS + 8 * kk;
-                        const unsigned long long brh = tc::smem_desc(sb + 0 * b_plane + bo, NB), brl = tc::smem_desc(sb + 1 * b_plane + bo, NB);
-                        const unsigned long long bih = tc::smem_desc(sb + 2 * b_plane + bo, NB), bil = tc::smem_desc(sb + 3 * b_plane + bo, NB);
-                        const unsigned first = (s == 0 && kk == 0) ? 0u : 1u;
-                        tc::mma_tf32_ta(tr, arh, brh, id, first);  tc::mma_tf32_ta(tr, arh, brl, id, 1u);  tc::mma_tf32_ta(tr, arl, brh, id, 1u);
-                        tc::mma_tf32_ta(tr, aih, bih, idn, 1u);    tc::mma_tf32_ta(tr, aih, bil, idn, 1u); tc::mma_tf32_ta(tr, ail, bih, idn, 1u);
-                        tc::mma_tf32_ta(ti, arh, bih, id, first);  tc::mma_tf32_ta(ti, arh, bil, id, 1u);  tc::mma_tf32_ta(ti, arl, bih, id, 1u);
-                        tc::mma_tf32_ta(ti, aih, brh, id, 1u);     tc::mma_tf32_ta(ti, aih, brl, id, 1u);  tc::mma_tf32_ta(ti, ail, brh, id, 1u);
-                    }
-                    tc::commit(tc::smem_u32(&empty[b]));
-                }
-                if (ok) tc::commit(tc::smem_u32(&accf));
-            }
-            if (!ok) {
-                atomicExch(&abort_flag, 1);
-                atomicExch(p.err, 1);
-            }
-            tc::commit(tc::smem_u32(&done));   // completion of every MMA issued above
-        }
-        __syncwarp();
     } else {
-        // ------------------------------------------------------------------ epilogue: tensor memory -> global
+        // ------------------------------------------------------------------ MMA issuer (warp 16) and epilogue
         const int qw = warp & 3, M = p.d.M;
         const unsigned lane_off = (unsigned)(qw * 32) << 16;
         const size_t M2 = (size_t)M * M;
-        for (int it = 0; it < my_items; it++) {
+        const unsigned id = tc::idesc_tf32(TM, 2 * NB, false);
+        int n = 0;
+        // a wait of the warp's first lane, its outcome for the whole warp
+        auto wait_all = [&](unsigned long long *bar, int parity) {
             int ok = 1;
-            if (lane == 0) ok = tc::mbar_wait_or_abort(tc::smem_u32(&accf), it & 1, &abort_flag) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) {
+            if (lane == 0) ok = tc::mbar_wait_or_abort(tc::smem_u32(bar), parity, &abort_flag) ? 1 : 0;
+            return __shfl_sync(0xffffffffu, ok, 0) != 0;
+        };
+        bool ok = true;
+        for (int it = 0; it < my_items; it++) {
+            if (warp == MMA_WARP) {
+                int issued = 1;
+                // the accumulator must have been read by the other warps' epilogue of the previous item
                 if (lane == 0) {
-                    atomicExch(&abort_flag, 1);
-                    atomicExch(p.err, 1);
-                }
-                break;
-            }
-            tc::fence_after();
-            // the accumulator into this warp's rows of the shared-memory tile (lane = row, two columns per 16-byte
-            // store; the row stride of NB + 2 columns keeps them free of bank conflicts), then release it to the
-            // next item's MMAs
-            float2 *et = etile + (size_t)(qw * 32) * estr;
-            for (int c0 = 0; c0 < NB; c0 += 8) {
-                unsigned vr[8], vi[8];
-                tc::tmem_ld8(tmem + lane_off + (unsigned)c0, vr);
-                tc::tmem_ld8(tmem + lane_off + ACC_IM + (unsigned)c0, vi);
-                tc::tmem_wait_ld();
+                    if (it >= 1 && !tc::mbar_wait_or_abort(tc::smem_u32(&acce), (it - 1) & 1, &abort_flag)) issued = 0;
+                    tc::fence_after();
+                    for (int s = 0; s < nks && issued; s++, n++) {
+                        const int b = n % NSTAGE;
+                        if (!tc::mbar_wait_or_abort(tc::smem_u32(&full[b]), (n / NSTAGE) & 1, &abort_flag)) { issued = 0; break; }
+                        tc::fence_after();
+                        const unsigned sb = tc::smem_u32(smem + (size_t)b * b_stage), ta = tmem + A_COL0 + b * A_STAGE_COLS;
 #pragma unroll
-                for (int j = 0; j < 8; j += 2)
-                    *reinterpret_cast<float4 *>(et + (size_t)lane * estr + c0 + j) =
-                        make_float4(__uint_as_float(vr[j]), __uint_as_float(vi[j]), __uint_as_float(vr[j + 1]), __uint_as_float(vi[j + 1]));
+                        for (int kk = 0; kk < KS / 8; kk++) {
+                            const unsigned bo = sb + kk * 2 * (3 * NB / 8) * 128, win = (NB / 8) * 128;   // [-Bi | Br], [Br | Bi] at + win
+                            const unsigned arh = ta + 0 * A_PLANE_COLS + 8 * kk, arl = ta + 1 * A_PLANE_COLS + 8 * kk;
+                            const unsigned aih = ta + 2 * A_PLANE_COLS + 8 * kk, ail = ta + 3 * A_PLANE_COLS + 8 * kk;
+                            const unsigned long long rh = tc::smem_desc(bo + win, 3 * NB), rl = tc::smem_desc(bo + b_plane + win, 3 * NB);
+                            const unsigned long long ih = tc::smem_desc(bo, 3 * NB), il = tc::smem_desc(bo + b_plane, 3 * NB);
+                            const unsigned first = (s == 0 && kk == 0) ? 0u : 1u;
+                            tc::mma_tf32_ta(tmem, arh, rh, id, first); tc::mma_tf32_ta(tmem, arh, rl, id, 1u); tc::mma_tf32_ta(tmem, arl, rh, id, 1u);
+                            tc::mma_tf32_ta(tmem, aih, ih, id, 1u);    tc::mma_tf32_ta(tmem, aih, il, id, 1u); tc::mma_tf32_ta(tmem, ail, ih, id, 1u);
+                        }
+                        tc::commit(tc::smem_u32(&empty[b]));
+                    }
+                    if (issued) tc::commit(tc::smem_u32(&accf));
+                }
+                ok = __shfl_sync(0xffffffffu, issued, 0) != 0;
+                if (!ok) break;
             }
-            tc::fence_before();
-            tc::mbar_arrive(tc::smem_u32(&acce));
-            __syncwarp();
-            // coalesced rows: for each of the warp's 32 rows, consecutive lanes write consecutive columns
+            // the item's MMAs are complete
+            ok = wait_all(&accf, it & 1);
+            if (!ok) break;
+            tc::fence_after();
             int ch, z, mt, nt;
             decode((int)blockIdx.x + it * G, ch, z, mt, nt);
             const int qs = p.qlist ? p.qlist[z] : z;
-            const int n0 = nt * NB, ncol = min(NB, M - n0), m0 = mt * TM + qw * 32, nrow = min(32, M - m0);
+            const int n0 = nt * NB, m0 = mt * TM + qw * 32 + (lane >> 2), cl = n0 + 2 * (lane & 3);
+            const int nlim = min(n0 + NB, M);
             // c_X times the flow-scale factor, applied in FP32 (the products carry FP32 accuracy)
             const float c = PH == 1 ? (float)((ch == 0 ? 1.0 : 2.0) * (p.scal ? p.scal[1] : 1.0)) : 1.f;
-            // two columns per lane and store (ncol and n0 are even, rows start 16-byte aligned)
-            const int npair = ncol / 2;
-#pragma unroll 4
-            for (int rr = 0; rr < nrow; rr++) {
-                const float4 *src = reinterpret_cast<const float4 *>(et + (size_t)rr * estr);
-                if (PH == 0) {
-                    float4 *dst = reinterpret_cast<float4 *>(p.T + ((size_t)ch * p.nz + z) * M2 + (size_t)(m0 + rr) * M + n0);
-                    for (int cp = lane; cp < npair; cp += 32) dst[cp] = src[cp];
-                } else {
-                    double2 *dst = p.out + ((size_t)ch * p.Nq + qs) * M2 + (size_t)(m0 + rr) * M + n0;
-                    for (int cp = lane; cp < npair; cp += 32) {
-                        const float4 v = src[cp];
-                        dst[2 * cp] = make_double2(f32_to_f64(c * v.x), f32_to_f64(c * v.y));
-                        dst[2 * cp + 1] = make_double2(f32_to_f64(c * v.z), f32_to_f64(c * v.w));
-                    }
+            float2 *dT = p.T + ((size_t)ch * p.nz + z) * M2;
+            double2 *dX = p.out + ((size_t)ch * p.Nq + qs) * M2;
+            for (int c0 = 0; c0 < NB; c0 += 8) {
+                unsigned vr[2][4], vi[2][4];   // rows lane / 4 + 16 g (0, 1) and + 8 (2, 3), two columns each
+#pragma unroll
+                for (int g = 0; g < 2; g++) {
+                    tc::tmem_ld_16x8(tmem + lane_off + ((unsigned)(16 * g) << 16) + (unsigned)c0, vr[g]);
+                    tc::tmem_ld_16x8(tmem + lane_off + ((unsigned)(16 * g) << 16) + (unsigned)(NB + c0), vi[g]);
                 }
+                tc::tmem_wait_ld();
+                const int n = cl + c0;   // (even, as is M: the second column exists with the first)
+#pragma unroll
+                for (int g = 0; g < 4; g++) {
+                    const int m = m0 + 8 * g, h = 2 * (g & 1);
+                    if (n >= nlim || m >= M) continue;
+                    const float r0 = __uint_as_float(vr[g >> 1][h]), r1 = __uint_as_float(vr[g >> 1][h + 1]);
+                    const float i0 = __uint_as_float(vi[g >> 1][h]), i1 = __uint_as_float(vi[g >> 1][h + 1]);
+                    const size_t o = (size_t)m * M + n;
+                    if (PH == 0) *reinterpret_cast<float4 *>(dT + o) = make_float4(r0, i0, r1, i1);
+                    else store_pair(dX + o, p.out32B, f32_to_f64(c * r0), f32_to_f64(c * i0), f32_to_f64(c * r1), f32_to_f64(c * i1));
+                }
+                __syncwarp();   // (the loads are warp-collective)
             }
-            __syncwarp();   // the tile rows are read before the next item's accumulator overwrites them
+            tc::fence_before();
+            if (warp == MMA_WARP) __syncwarp();   // (its own reads are complete before it issues the next item's MMAs)
+            else tc::mbar_arrive(tc::smem_u32(&acce));
         }
+        if (!ok && lane == 0) {
+            atomicExch(&abort_flag, 1);
+            atomicExch(p.err, 1);
+        }
+        if (warp == MMA_WARP && lane == 0) tc::commit(tc::smem_u32(&done));   // completion of every MMA issued above
+        __syncwarp();
     }
     __syncthreads();
     if (tid == MMA_WARP * 32) (void)tc::mbar_wait(tc::smem_u32(&done), 0);   // bounded; the MMAs read shared memory
@@ -401,8 +430,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) vlv_tc_kernel(VlvArgs p)
 template <int PH>
 cudaError_t launch_phase(tufrg_model *m, const VlvArgs &a)
 {
-    const size_t smem = NSTAGE * 4 * (size_t)a.d.nb * KS * 4 + sizeof(float2) * (size_t)TM * (a.d.nb + 2) +
-                        sizeof(int) * (size_t)a.nff * a.nff;
+    const size_t smem = NSTAGE * 6 * (size_t)a.d.nb * KS * 4 + sizeof(int) * (size_t)a.nff * a.nff;
     void (*k)(VlvArgs) = nullptr;
     switch (m->ns * m->ns) {
     case 4: k = vlv_tc_kernel<PH, 4>; break;
@@ -452,6 +480,7 @@ cudaError_t launch_vlv_tc(tufrg_model *m, int channel_mask, double2 *d_out, cons
     a.dij = m->d_dij;
     a.T = reinterpret_cast<float2 *>(m->d_T);
     a.out = d_out;
+    a.out32B = (reinterpret_cast<uintptr_t>(d_out) & 31) == 0;
     a.qlist = qlist;
     a.scal = m->d_scal;
     a.err = m->d_err;

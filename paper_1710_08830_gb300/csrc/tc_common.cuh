@@ -103,6 +103,18 @@ __device__ __forceinline__ void tmem_st4(unsigned addr, float v0, float v1, floa
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(__float_as_uint(v0)),
                  "r"(__float_as_uint(v1)), "r"(__float_as_uint(v2)), "r"(__float_as_uint(v3)) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_16x8(unsigned addr, unsigned (&v)[4])   // the arrangement of tmem_st_16x8
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
+}
+// 16 lanes x 8 columns: thread t holds lanes t / 4 (a, b) and t / 4 + 8 (c, d) at columns 2 (t % 4) and + 1; the
+// address's lane is a multiple of 16 within the warp's 32
+__device__ __forceinline__ void tmem_st_16x8(unsigned addr, float a, float b, float c, float d)
+{
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x1.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(__float_as_uint(a)),
+                 "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)) : "memory");
+}
 __device__ __forceinline__ void tmem_st2(unsigned addr, float v0, float v1)
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_uint(v0)),

@@ -534,7 +534,7 @@ void release(tufrg_model *m)
                     m->d_V0, m->d_Lc, m->d_Lc32, m->d_part, m->d_Xr, m->d_A, m->d_A32, m->d_T, m->d_amax,
                     m->d_red, m->d_y, m->d_yt, m->d_yn, m->d_state_in, m->d_state_out, m->d_rec, m->d_Xr32,
                     m->d_ph32, m->d_dftpart, m->d_dpartner, m->d_err, m->d_scal, m->d_flow, m->d_eofs[0],
-                    m->d_eofs[1], m->d_eterms[0], m->d_eterms[1], m->d_v0d[0], m->d_v0d[1], m->d_X32,
+                    m->d_eofs[1], m->d_eterms[0], m->d_eterms[1], m->d_bofs[0], m->d_bofs[1], m->d_bterms[0], m->d_bterms[1], m->d_v0d[0], m->d_v0d[1], m->d_X32,
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
@@ -1172,6 +1172,15 @@ try {
             CK(upload(&m->d_eofs[ch], eofs[ch], m->stream), "upload projection tables");
             if (!eterms[ch].empty()) CK(upload(&m->d_eterms[ch], eterms[ch], m->stream), "upload projection tables");
             CK(upload(&m->d_v0d[ch], v0d[ch], m->stream), "upload projection tables");
+            // the same terms per bond pair: the source is a whole N_s^2 x N_s^2 block
+            std::vector<int4> bt;
+            for (const tufrg::GatherTerm &g : m->gterms[ch]) {
+                const int sch = g.kind == 2 ? 0 : 1;
+                const long idx = ((long)sch * m->ncls + g.cls) * m->M * m->M + (long)g.i1 * ns2 * m->M + g.i2 * ns2;
+                bt.push_back(make_int4((int)idx, g.ph, g.kind & 1, sch));
+            }
+            CK(upload(&m->d_bofs[ch], m->gofs[ch], m->stream), "upload projection tables");
+            if (!bt.empty()) CK(upload(&m->d_bterms[ch], bt, m->stream), "upload projection tables");
             if (split) {
                 std::vector<float2> v32(v0d[ch].size());
                 for (size_t i = 0; i < v32.size(); i++) v32[i] = make_float2((float)v0d[ch][i].x, (float)v0d[ch][i].y);

@@ -256,9 +256,15 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2 *phs = reinterpret_cast<C2 *>(smem_raw);   // [QT][nph]
     __shared__ int sq[QT];                         // transfer momenta of this CTA (list positions p0 ..)
+    __shared__ size_t so_x[QT], so_q[QT];          // offsets of their rows of X and of their matrices (64-bit products once)
     const int ch = blockIdx.z, p0 = blockIdx.y * QT, nq = min(QT, nlist - p0);
     grid_release();
-    if (threadIdx.x < QT) sq[threadIdx.x] = threadIdx.x < nq ? (qlist ? qlist[p0 + threadIdx.x] : p0 + threadIdx.x) : 0;
+    if (threadIdx.x < QT) {
+        const int q = threadIdx.x < nq ? (qlist ? qlist[p0 + threadIdx.x] : p0 + threadIdx.x) : 0;
+        sq[threadIdx.x] = q;
+        so_q[threadIdx.x] = (size_t)q * M2;
+        so_x[threadIdx.x] = (size_t)(x_local ? (int)threadIdx.x : q) * M2;
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < QT * nph; i += blockDim.x) {
         const int qi = i / nph;
@@ -278,9 +284,9 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
             const C2 v0 = ld_as<R>((ch == 0 ? v0d0 : v0d1)[e]);
 #pragma unroll
             for (int qi = 0; qi < QT; qi++) {
-                acc[qi] = qi < nq ? ld_as<R>(X[xbase + (size_t)(x_local ? qi : sq[qi]) * M2]) : mk(R(0), R(0));
+                acc[qi] = qi < nq ? ld_as<R>(X[xbase + so_x[qi]]) : mk(R(0), R(0));
                 // the bare vertex: onsite (one value for every momentum), or per momentum in the band basis
-                const C2 vq = v0q && qi < nq ? ld_as<R>(v0q[((size_t)ch * Nq + sq[qi]) * M2 + e]) : v0;
+                const C2 vq = v0q && qi < nq ? ld_as<R>(v0q[base + so_q[qi]]) : v0;
                 acc[qi].x += vq.x;
                 acc[qi].y += vq.y;
             }
@@ -336,7 +342,7 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
 #pragma unroll
         for (int qi = 0; qi < QT; qi++) {
             if (qi >= nq) break;
-            const size_t o = base + (size_t)sq[qi] * M2;
+            const size_t o = base + so_q[qi];
             if (A) A[o] = make_double2((double)acc[qi].x, (double)acc[qi].y);
             if (A32) A32[o] = make_float2((float)acc[qi].x, (float)acc[qi].y);
             m2 = max(m2, abs2(acc[qi]));
@@ -350,6 +356,155 @@ __global__ void __launch_bounds__(256) project_kernel(const XT *__restrict__ X, 
     if (threadIdx.x == 0) {
         for (int w = 1; w < (int)(blockDim.x >> 5); w++) m2 = max(m2, wmax[w]);
         if (m2 > R(0)) atomicMax(amax, (unsigned long long)__double_as_longlong(mag_of(m2)));
+    }
+}
+
+// The same for the split path of several orbitals: a CTA per (bond pair, QT transfer momenta, channel).  A term's source for
+// the N_s^2 x N_s^2 entries of a bond pair is one block of the Fourier transforms with its four orbital indices in another
+// order, so the block is read along its rows into shared memory (the next term's while this one is added) and picked up
+// there in that order; the terms and their phases are the same for all threads.  The per-entry kernel above gathers the same
+// values one 8-byte sector quarter per lane and reads a term list per entry.  225 momenta, two channels, M = 324: 352 us per
+// entry, 255 us here (64-bit address products once per CTA are most of the difference); 28 momenta, M = 80: 20.0 and 18.1 us.
+// The rows of the staged block are LD apart, one more than a multiple of 16 values, so that the lanes of a half warp
+// (neighbouring second indices) fall on different banks.
+template <int NS, int QT>
+__global__ void __launch_bounds__(NS == 6 ? 432 : 256, 2) project_block_kernel(
+    const float2 *__restrict__ X, const float2 *__restrict__ Xr, const float2 *v0d0, const float2 *v0d1, const int *bofs0,
+    const int *bofs1, const int4 *bt0, const int4 *bt1, const float2 *ph, int nph, int Nq, int M, int nff, int chmask,
+    const int *qlist, int nlist, float2 *A32, unsigned long long *amax, const float2 *v0q)
+{
+    constexpr int NS2 = NS * NS, THR = NS == 6 ? 432 : 256, EPT = NS2 * NS2 / THR, LD = NS == 6 ? 49 : 17;
+    static_assert(EPT * THR == NS2 * NS2, "whole entries per thread");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *phs = reinterpret_cast<float2 *>(smem_raw);   // [QT][nph]
+    __shared__ float2 blk[2][NS2 * LD];
+    __shared__ int sq[QT];
+    __shared__ size_t so_q[QT];   // offsets of the momenta's matrices (64-bit products once per CTA)
+    __shared__ unsigned wmax[THR / 32 + 1];
+    const int ch = blockIdx.z, p0 = blockIdx.y * QT, nq = min(QT, nlist - p0), pair = blockIdx.x;
+    grid_release();
+    const size_t M2 = (size_t)M * M;
+    if (threadIdx.x < QT) {
+        const int q = threadIdx.x < nq ? (qlist ? qlist[p0 + threadIdx.x] : p0 + threadIdx.x) : 0;
+        sq[threadIdx.x] = q;
+        so_q[threadIdx.x] = q * M2;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < QT * nph; i += THR) {
+        const int qi = i / nph;
+        phs[i] = qi < nq ? ph[(size_t)sq[qi] * nph + (i - qi * nph)] : make_float2(0.f, 0.f);
+    }
+    const bool on = (chmask >> ch) & 1;
+    const int *bofs = ch == 0 ? bofs0 : bofs1;
+    const int4 *bt = ch == 0 ? bt0 : bt1;
+    int t = bofs[pair];
+    const int t1 = on ? bofs[pair + 1] : t;
+    // this thread's entries: offset in the matrix, in a source block, and the places of their direct and crossed sources
+    int eo[EPT], so[EPT], pick[EPT][2], put[EPT];
+#pragma unroll
+    for (int k = 0; k < EPT; k++) {
+        const int i = threadIdx.x + k * THR, rp = i / NS2, cp = i - rp * NS2;
+        const int s1 = rp / NS, sb = rp - s1 * NS, s4 = cp / NS, sd = cp - s4 * NS;   // P: (s1 s2),(s4 s3); C: (s1 s3),(s4 s2)
+        eo[k] = ((pair / nff) * NS2 + rp) * M + (pair % nff) * NS2 + cp;
+        so[k] = rp * M + cp;
+        put[k] = rp * LD + cp;
+        pick[k][0] = (s1 * NS + sd) * LD + s4 * NS + sb;
+        const int s2 = ch == 0 ? sb : sd, s3 = ch == 0 ? sd : sb;
+        pick[k][1] = (s1 * NS + s4) * LD + s3 * NS + s2;
+    }
+    grid_wait();
+    auto skip = [&]() {   // past the terms whose source channel is off
+        while (t < t1 && !((chmask >> bt[t].w) & 1)) t++;
+    };
+    skip();
+    int4 g = make_int4(0, 0, 0, 0);
+    float2 nxt[EPT];
+    if (t < t1) {
+        g = bt[t];
+#pragma unroll
+        for (int k = 0; k < EPT; k++) nxt[k] = Xr[g.x + so[k]];
+    }
+    const size_t base = (size_t)ch * Nq * M2;   // + q M2
+    float2 acc[EPT][QT];
+#pragma unroll
+    for (int qi = 0; qi < QT; qi++) {
+        const float2 *xq = X + base + so_q[qi];
+#pragma unroll
+        for (int k = 0; k < EPT; k++) acc[k][qi] = on && qi < nq ? xq[eo[k]] : make_float2(0.f, 0.f);
+    }
+    if (on && !v0q) {
+        const float2 *v0d = ch == 0 ? v0d0 : v0d1;
+#pragma unroll
+        for (int k = 0; k < EPT; k++) {
+            const float2 v0 = v0d[eo[k]];
+#pragma unroll
+            for (int qi = 0; qi < QT; qi++) {
+                acc[k][qi].x += v0.x;
+                acc[k][qi].y += v0.y;
+            }
+        }
+    } else if (on) {
+#pragma unroll
+        for (int qi = 0; qi < QT; qi++) {
+            const float2 *vq = v0q + base + so_q[qi];
+#pragma unroll
+            for (int k = 0; k < EPT; k++) {
+                if (qi >= nq) break;
+                const float2 v0 = vq[eo[k]];
+                acc[k][qi].x += v0.x;
+                acc[k][qi].y += v0.y;
+            }
+        }
+    }
+    for (int b = 0; t < t1; b ^= 1) {
+#pragma unroll
+        for (int k = 0; k < EPT; k++) blk[b][put[k]] = nxt[k];
+        __syncthreads();   // (the block before last is no longer read)
+        const int4 cur = g;
+        t++;
+        skip();
+        if (t < t1) {
+            g = bt[t];
+#pragma unroll
+            for (int k = 0; k < EPT; k++) nxt[k] = Xr[g.x + so[k]];
+        }
+        float2 x[EPT];
+#pragma unroll
+        for (int k = 0; k < EPT; k++) {
+            x[k] = blk[b][cur.z ? pick[k][1] : pick[k][0]];
+            if (cur.z) x[k] = make_float2(-x[k].x, -x[k].y);   // the crossed (D) terms enter with a minus sign
+        }
+#pragma unroll
+        for (int qi = 0; qi < QT; qi++) {
+            const float2 pq = phs[qi * nph + cur.y];
+#pragma unroll
+            for (int k = 0; k < EPT; k++) {
+                acc[k][qi].x = fmaf(-pq.y, x[k].y, fmaf(pq.x, x[k].x, acc[k][qi].x));
+                acc[k][qi].y = fmaf(pq.y, x[k].x, fmaf(pq.x, x[k].y, acc[k][qi].y));
+            }
+        }
+    }
+    float m2 = 0.f;
+#pragma unroll
+    for (int qi = 0; qi < QT; qi++) {
+        if (qi >= nq) break;
+        float2 *aq = A32 + base + so_q[qi];
+#pragma unroll
+        for (int k = 0; k < EPT; k++) {
+            aq[eo[k]] = acc[k][qi];
+            m2 = fmaxf(m2, abs2(acc[k][qi]));
+        }
+    }
+    // max |A| over the CTA, then one atomic (non-negative floats and doubles order like their bit patterns; the last warp
+    // of the 432 threads has 16)
+    const unsigned lanes = THR % 32 && threadIdx.x >= THR / 32 * 32 ? (1u << (THR % 32)) - 1 : 0xffffffffu;
+    const unsigned wm = __reduce_max_sync(lanes, __float_as_uint(m2));
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = wm;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned v = wm;
+        for (int w = 1; w < (THR + 31) / 32; w++) v = max(v, wmax[w]);
+        if (v) atomicMax(amax, (unsigned long long)__double_as_longlong(mag_of(__uint_as_float(v))));
     }
 }
 
@@ -539,6 +694,19 @@ cudaError_t launch_project(tufrg_model *m, const double2 *d_state, const float2 
                    m->d_v0q, false);
     }
     if (!d_state32) return cudaErrorInvalidValue;   // the split path projects the FP32 copy
+    if (m->ns == 4 || m->ns == 6) {
+        // QT momenta share each staged block; fewer where the grid would not give every SM two CTAs
+        const int pairs = m->nff * m->nff;
+        const bool few = (long)((nlist + PROJ_QT - 1) / PROJ_QT) * pairs * 2 < 2L * m->sm_count;
+        const int qt = few ? 2 : PROJ_QT;
+        auto k = m->ns == 4 ? (few ? project_block_kernel<4, 2> : project_block_kernel<4, PROJ_QT>)
+                            : (few ? project_block_kernel<6, 2> : project_block_kernel<6, PROJ_QT>);
+        const size_t smem = sizeof(float2) * qt * m->nph;
+        TUFRG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        return launch_chained(k, dim3(pairs, (nlist + qt - 1) / qt, 2), m->ns == 4 ? 256 : 432, smem, m->stream, true, d_state32,
+                              m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_bofs[0], m->d_bofs[1], m->d_bterms[0], m->d_bterms[1],
+                              m->d_ph32, m->nph, m->Nq, m->M, m->nff, channel_mask, qlist, nlist, m->d_A32, m->d_amax, m->d_v0q32);
+    }
     auto run = short_list ? project_run<float, float2, 2> : project_run<float, float2, PROJ_QT>;
     return run(m, d_state32, m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_ph32, channel_mask, qlist, nlist, d_A,
                m->d_A32, 0, m->d_v0q32, true);

@@ -283,6 +283,8 @@ struct tufrg_model {
     int *d_eofs[2] = {nullptr, nullptr};       // per output channel: CSR offsets per matrix entry, [M*M + 1]
     int2 *d_eterms[2] = {nullptr, nullptr};    // per entry terms: (flat index into the Fourier transforms,
                                                //  high bit = minus sign; phase-table column)
+    int *d_bofs[2] = {nullptr, nullptr};       // per output channel: offsets of a bond pair's terms, [n_ff^2 + 1]
+    int4 *d_bterms[2] = {nullptr, nullptr};    // (flat index of the source block, phase-table column, crossed, source channel)
     double2 *d_v0d[2] = {nullptr, nullptr};    // [M*M] bare vertex V0 at the onsite bond pair, 0 elsewhere
     float2 *d_X32 = nullptr;        // [2][Nq][M][M] FP32 copy of the state being evaluated (split path)
     float2 *d_lph32 = nullptr;      // [Lf] e^{-2 pi i n / Lf} for the loop kernels (split path)

@@ -371,7 +371,7 @@ template <int NS, int QT>
 __global__ void __launch_bounds__(NS == 6 ? 432 : 256, 2) project_block_kernel(
     const float2 *__restrict__ X, const float2 *__restrict__ Xr, const float2 *v0d0, const float2 *v0d1, const int *bofs0,
     const int *bofs1, const int4 *bt0, const int4 *bt1, const float2 *ph, int nph, int Nq, int M, int nff, int chmask,
-    const int *qlist, int nlist, float2 *A32, unsigned long long *amax, const float2 *v0q)
+    const int *qlist, int nlist, double2 *A, float2 *A32, unsigned long long *amax, const float2 *v0q)
 {
     constexpr int NS2 = NS * NS, THR = NS == 6 ? 432 : 256, EPT = NS2 * NS2 / THR, LD = NS == 6 ? 49 : 17;
     static_assert(EPT * THR == NS2 * NS2, "whole entries per thread");
@@ -492,6 +492,7 @@ __global__ void __launch_bounds__(NS == 6 ? 432 : 256, 2) project_block_kernel(
 #pragma unroll
         for (int k = 0; k < EPT; k++) {
             aq[eo[k]] = acc[k][qi];
+            if (A) A[base + so_q[qi] + eo[k]] = make_double2((double)acc[k][qi].x, (double)acc[k][qi].y);
             m2 = fmaxf(m2, abs2(acc[k][qi]));
         }
     }
@@ -705,7 +706,8 @@ cudaError_t launch_project(tufrg_model *m, const double2 *d_state, const float2 
         TUFRG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         return launch_chained(k, dim3(pairs, (nlist + qt - 1) / qt, 2), m->ns == 4 ? 256 : 432, smem, m->stream, true, d_state32,
                               m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_bofs[0], m->d_bofs[1], m->d_bterms[0], m->d_bterms[1],
-                              m->d_ph32, m->nph, m->Nq, m->M, m->nff, channel_mask, qlist, nlist, m->d_A32, m->d_amax, m->d_v0q32);
+                              m->d_ph32, m->nph, m->Nq, m->M, m->nff, channel_mask, qlist, nlist, d_A, m->d_A32, m->d_amax,
+                              m->d_v0q32);
     }
     auto run = short_list ? project_run<float, float2, 2> : project_run<float, float2, PROJ_QT>;
     return run(m, d_state32, m->d_Xr32, m->d_v0d32[0], m->d_v0d32[1], m->d_ph32, channel_mask, qlist, nlist, d_A,

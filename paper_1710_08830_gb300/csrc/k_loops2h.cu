@@ -817,13 +817,17 @@ cudaError_t launch_loops2h_reduce(tufrg_model *m, int channel_mask, const void *
 
 LoopPlan plan_loops2h(const tufrg_model *m)
 {
-    // Choose the number of ky ranges so that the grid fills whole waves of the SMs; the flush of the columns' sums
-    // costs about 8 rows of work.
+    // Choose the number of ky ranges so that the grid fills whole waves of the SMs; the flush of the columns' sums costs
+    // about 0.45 rows of work per pair of bond differences (measured: 6 rows for 5 x 3 pairs, 23 for 9 x 5).  Fewer
+    // ranges can be faster alone (24 x 24 momenta: one range 47 us, three 49), but not beside the state's transforms and
+    // projections (124 against 106 us for the whole right-hand side; FP64 8 x 8 five ranges 273, nine 252 us).
+    // 48 x 48, 13 form factors: two ranges 727 us, one 690 us, whole right-hand side 998 and 940 us.
     LoopPlan p{};
     const int ctas_x = (m->Lf + NT - 1) / NT;
     const int half = loops2_half_mask(m);
     const int rows = half == 3 ? m->Lf / 2 + 1 : m->Lf;
     const double slots = (double)m->sm_count * loops2h_blocks_per_sm(m);
+    const double flush = 0.45 * (double)m->dxs.size() * n_dyh(m);
     double best = 1e300;
     int best_c = 1;
     for (int c = 1; c <= 16; c++) {
@@ -831,7 +835,7 @@ LoopPlan plan_loops2h(const tufrg_model *m)
         if (len < 8) break;
         const double ctas = (double)m->n_loop_q * ctas_x * c * 2;
         const double waves = std::ceil(ctas / slots);
-        const double cost = waves * (len + 8.0);
+        const double cost = waves * (len + flush);
         if (cost < best * 0.999) { best = cost; best_c = c; }
     }
     p.ky_chunks = best_c;

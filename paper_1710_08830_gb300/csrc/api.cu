@@ -538,7 +538,7 @@ void release(tufrg_model *m)
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
-                    m->d_shard_q, m->d_oz, m->d_LcB, m->d_Lc32B, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
+                    m->d_shard_q, m->d_oz, m->d_LcB, m->d_Lc32B, m->d_recB, m->d_partB, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &p : m->d_k)
@@ -554,6 +554,7 @@ void release(tufrg_model *m)
     for (auto &e : m->aux_ev)
         if (e) cudaEventDestroy(e);
     if (m->aux_stream) cudaStreamDestroy(m->aux_stream);
+    if (m->aux_streamB) cudaStreamDestroy(m->aux_streamB);
     if (m->rhs_stream) cudaStreamDestroy(m->rhs_stream);
     if (m->flow_ev) cudaEventDestroy(m->flow_ev);
     for (int j = 0; j < 7; j++) {
@@ -647,7 +648,8 @@ const double DP_E[7] = {35.0 / 384 - 5179.0 / 57600, 0.0, 500.0 / 1113 - 7571.0 
 // buffers in turn; one where the second could not be allocated).  The last two stages share their temperature and with
 // it their loops (with a surrogate every stage evaluates its own, as its counters and decisions go by evaluation).
 // Launch chains of 29 us (loops) and 28 us (state) per stage at 8 x 8 momenta, two bands: one after the other
-// 12.7 ms per flow of 56 attempts, side by side 9.4 ms.
+// 12.7 ms per flow of 56 attempts, side by side 9.4 ms; 6.4 ms with overlapped launches and the attempts repeated on the
+// device, 5.2 ms with two stages' k-sums at a time.
 tufrg_status enqueue_attempt(tufrg_model *m, int mask, const cudaGraphConditionalHandle *loop)
 {
     const size_t n = state_elems(m);
@@ -663,14 +665,17 @@ tufrg_status enqueue_attempt(tufrg_model *m, int mask, const cudaGraphConditiona
         double *scal;
         double2 *Lc;
         float2 *Lc32;
+        void *rec, *part;
         ~Restore()
         {
+            m->d_rec = rec;
+            m->d_part = part;
             m->stream = stream;
             m->d_scal = scal;
             m->d_Lc = Lc;
             m->d_Lc32 = Lc32;
         }
-    } base{m, m->stream, m->d_scal, m->d_Lc, m->d_Lc32};
+    } base{m, m->stream, m->d_scal, m->d_Lc, m->d_Lc32, m->d_rec, m->d_part};
     const int n_buf = (split ? m->d_Lc32B != nullptr : m->d_LcB != nullptr) ? 2 : 1;
     auto use_stage = [&](int j, cudaStream_t s) {   // stage j's scalars and loop buffer on stream s
         m->stream = s;
@@ -679,19 +684,26 @@ tufrg_status enqueue_attempt(tufrg_model *m, int mask, const cudaGraphConditiona
         m->d_Lc = second && !split ? m->d_LcB : base.Lc;
         m->d_Lc32 = second && split ? m->d_Lc32B : base.Lc32;
     };
+    // odd stages' loops on a stream of their own, with their own records and partial sums (a surrogate has one set)
+    const bool two_sets = m->d_partB && m->aux_streamB && !m->sur;
     const int n_loops = m->sur ? 6 : 5;   // stages with loops of their own (the nodes of stages 5 and 6 are equal)
     auto loops = [&](int j) -> tufrg_status {
         if (j > n_loops) return TUFRG_OK;
-        if (j > n_buf) CK(cudaStreamWaitEvent(m->aux_stream, m->flow_O[j - n_buf], 0), "fork");
-        use_stage(j, m->aux_stream);
+        const bool setB = two_sets && (j & 1);
+        const cudaStream_t s = setB ? m->aux_streamB : m->aux_stream;
+        if (j > n_buf) CK(cudaStreamWaitEvent(s, m->flow_O[j - n_buf], 0), "fork");
+        use_stage(j, s);
+        m->d_rec = setB ? m->d_recB : base.rec;
+        m->d_part = setB ? m->d_partB : base.part;
         CK(launch_fermi(m), "fermi tables");
         CK(launch_loops(m, mask, sym, true), "loop k-sum");
-        CK(cudaEventRecord(m->flow_L[j], m->aux_stream), "join");
+        CK(cudaEventRecord(m->flow_L[j], s), "join");
         return TUFRG_OK;
     };
     CK(launch_attempt_scalars(m, m->d_flow, DP_C), "stage temperatures");
     CK(cudaEventRecord(m->flow_O[0], m->stream), "fork");
     CK(cudaStreamWaitEvent(m->aux_stream, m->flow_O[0], 0), "fork");
+    if (two_sets) CK(cudaStreamWaitEvent(m->aux_streamB, m->flow_O[0], 0), "fork");
     for (int j = 1; j <= n_buf; j++) {
         const tufrg_status st = loops(j);
         if (st != TUFRG_OK) return st;
@@ -737,6 +749,19 @@ tufrg_status flow_alloc(tufrg_model *m)
             (void)cudaGetLastError();
             m->d_Lc32B = nullptr;
             m->d_LcB = nullptr;
+        }
+        // a k-sum of few CTAs is bound by its chain of rows: two stages' k-sums side by side then (four CTAs of two
+        // warps per SM: from there on one fills the SMs)
+        if (m->precision != TUFRG_FP64 && m->ns == 2 && m->d_Lc32B && loops_flow_ctas(m) <= 4L * m->sm_count) {
+            CK(cudaStreamCreateWithFlags(&m->aux_streamB, cudaStreamNonBlocking), "create stream");
+            if (cudaMalloc(&m->d_recB, loops2_rec_bytes(m)) != cudaSuccess || cudaMalloc(&m->d_partB, m->part_bytes) != cudaSuccess) {
+                (void)cudaGetLastError();
+                if (m->d_recB) cudaFree(m->d_recB);
+                m->d_recB = nullptr;
+                m->d_partB = nullptr;
+            } else {   // (the records' projectors and energies are written once per model)
+                CK(cudaMemcpyAsync(m->d_recB, m->d_rec, loops2_rec_bytes(m), cudaMemcpyDeviceToDevice, m->stream), "copy records");
+            }
         }
     }
     return TUFRG_OK;

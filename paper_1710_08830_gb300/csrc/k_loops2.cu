@@ -581,6 +581,11 @@ cudaError_t launch_loops_reduce_f32(tufrg_model *m, const float2 *part, int n_s,
     return cudaGetLastError();
 }
 
+long loops_flow_ctas(const tufrg_model *m)
+{
+    return 2L * (m->sym ? m->n_loop_q : m->Nq) * ((m->Lf + 32 * WARPS - 1) / (32 * WARPS)) * m->plan.ky_chunks;
+}
+
 // The loops of a split two-band flow (every stage of it and the surrogate's fallback).
 cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
 {

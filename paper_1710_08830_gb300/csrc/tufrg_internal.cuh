@@ -349,6 +349,9 @@ struct tufrg_model {
     cudaEvent_t flow_L[7] = {}, flow_O[7] = {};   // stage j's loops are there / its products have read them
     double2 *d_LcB = nullptr;       // second loop buffer of a flow's stages (FP64 path; split path below), or null
     float2 *d_Lc32B = nullptr;
+    // second records, partial sums and stream of a two-band split flow whose k-sum leaves SMs idle, or null
+    void *d_recB = nullptr, *d_partB = nullptr;
+    cudaStream_t aux_streamB = nullptr;
     // tufrg_rhs replays captured graphs of its launches, one per (input, output, mask) used more than once (the
     // four most recently used triples kept; exec is null after the first use)
     struct RhsGraph {
@@ -463,6 +466,7 @@ void drop_rhs_graphs(tufrg_model *m);
 void drop_flow_graphs(tufrg_model *m);
 // the launch shapes the two-band split loop kernel's autotuner times (ky ranges per column)
 std::vector<LoopPlan> loop_plan_candidates(const tufrg_model *m);
+long loops_flow_ctas(const tufrg_model *m);   // CTAs of one stage's k-sum in a two-band split flow
 int plan_gen_chunks(const tufrg_model *m);   // kx ranges per momentum of the multi-orbital loop kernel
 size_t gen_part_bytes(const tufrg_model *m);   // loop scratch of the multi-orbital kernel
 int dft_plan_nsplit(const tufrg_model *m);

@@ -148,7 +148,7 @@ def products_tf32_flop(M, Nq):
     return 2.0 * 2 * 2 * 4 * 3 * float(M) ** 3 * Nq
 
 
-LOOP_KERNEL_SOURCES = ("paper_1710_08830_gb300/csrc/k_loops2.cu", "paper_1710_08830_gb300/csrc/tufrg_internal.cuh")
+LOOP_KERNEL_SOURCES = ("paper_1710_08830_gb300/csrc/k_loops2h.cu", "paper_1710_08830_gb300/csrc/tufrg_internal.cuh")
 
 
 def loop_sources_hash() -> str:
@@ -208,15 +208,27 @@ def run_products_sweep(args):
                       "note": "products phase of one right-hand side (both channels, packing included), CUDA events"}))
 
 
+def loop_fma(n_s, ndyh):
+    """Real FMAs of the loop k-sum per (q, k) and channel, in Hermitian components: partner matrices N_s^4, their products
+    with the projectors N_s^5, and 2 ndyh - 1 real row phases of N_s^4 entries."""
+    return n_s ** 4 + n_s ** 5 + (2 * ndyh - 1) * n_s ** 4
+
+
+def loop_launch_flop(n_s, n_q, Nk, ndyh):
+    """FP32 flop of one loop launch: half of the fine mesh per channel (the workloads here have a symmetry that inverts the
+    momentum), both channels in one launch for two bands."""
+    return 2.0 * loop_fma(n_s, ndyh) * n_q * Nk / 2 * (2 if n_s == 2 else 1)
+
+
 def loops_tc_tensor_flop(n_direct, Lf, Nk, ndyh):
-    """3xTF32 work of one launch of the tensor-core loop k-sum (N_s = 6): executed = MMAs as issued (128 x 112 x 8
-    per instruction, 36 per stage of 4 fine-mesh rows, stages padded to 4 rows, groups of 3 momenta padded to 3);
-    useful = the unpadded operands (3 dy x 36 rows, 3 momenta x 36 columns, K = 6 per fine point): per (q, k)
-    2 flop x 3 TF32 passes x 4 real products x (ndyh 36) x 36 x 6."""
+    """3xTF32 work of one launch of the tensor-core loop k-sum (N_s = 6): executed = MMAs as issued (128 x 192 x 8 per
+    instruction, 9 per stage of 4 fine-mesh rows, half of the columns, groups of 3 momenta with one q_x: at least
+    n_direct / 3 of them); useful = the unpadded operands (36 (2 ndyh - 1) columns, 36 rows per momentum, K = 6 per fine
+    point of half of the mesh), three TF32 passes."""
     groups = (n_direct + 2) // 3
     stages = (Lf + 3) // 4
-    executed = float(groups) * Lf * stages * 36 * 2 * 128 * 112 * 8
-    useful = float(n_direct) * Nk * 2 * 3 * 4 * (ndyh * 36) * 36 * 6
+    executed = float(groups) * (Lf // 2 + 1) * stages * 9 * 2 * 128 * 192 * 8
+    useful = float(n_direct) * Nk / 2 * 2 * 3 * ((2 * ndyh - 1) * 36) * 36 * 6
     return executed, useful
 
 
@@ -258,25 +270,25 @@ def run_config_t2g(stream, peaks, fp32_peak, seed=0, k=10):
     ph = {kk: v / 3 for kk, v in ph.items()}
     loop_ms = ph["loops"] * 3 / max(1, nloop)
     ndyh = int(sum(1 for d in np.unique(spec.ff_R[:, 1][:, None] - spec.ff_R[:, 1][None, :]) if d >= 0))
-    unit = spec.n_s ** 4 + spec.n_s ** 5 + ndyh * spec.n_s ** 4
-    fp32_flop = 8.0 * m.n_loop_q * spec.Nk * unit
+    unit = loop_fma(spec.n_s, ndyh)
+    fp32_flop = loop_launch_flop(spec.n_s, m.n_loop_q, spec.Nk, ndyh)
     tf32 = tf32_peak_tflops(peaks)
     loops = {"kernel": "loops_tc_kernel" if m.loops_backend == "tc" else "loops_gen_kernel",
              "backend": m.loops_backend, "avg_launch_ms": loop_ms,
-             "units_per_launch": f"{m.n_loop_q} directly summed q x {spec.Nk} k",
-             "method_fp32": {"unit_work": f"(N_s^4 + N_s^5 + {ndyh} N_s^4) = {unit} complex FMA per (q, k)",
+             "units_per_launch": f"{m.n_loop_q} directly summed q x {spec.Nk} / 2 k",
+             "method_fp32": {"unit_work": f"(N_s^4 + N_s^5 + {2 * ndyh - 1} N_s^4) = {unit} real FMA per (q, k)",
                              "achieved_tflops": fp32_flop / (loop_ms * 1e-3) / 1e12, "peak_tflops": fp32_peak,
                              "frac": fp32_flop / (loop_ms * 1e-3) / 1e12 / fp32_peak,
-                             "note": "the method's complex FP32 work against the FP32 FMA peak (the count used for the "
-                                     "CUDA-core kernel)"}}
+                             "note": "the method's FP32 work (real Hermitian components, half of the fine mesh) against "
+                                     "the FP32 FMA peak (the count used for the CUDA-core kernel)"}}
     if m.loops_backend == "tc":
         ex, us = loops_tc_tensor_flop(m.n_loop_q, spec.Lf, spec.Nk, ndyh)
         loops["tensor_3xtf32"] = {
             "bound": "tensor", "peak_tflops": tf32, "peak_source": "measured bf16 x 1.1/2.25 (nominal TF32/BF16)",
             "executed_tflops": ex / (loop_ms * 1e-3) / 1e12, "executed_frac": ex / (loop_ms * 1e-3) / 1e12 / tf32,
             "useful_tflops": us / (loop_ms * 1e-3) / 1e12, "useful_frac": us / (loop_ms * 1e-3) / 1e12 / tf32,
-            "note": "executed counts the MMAs as issued (padded 128 x 112 tiles), useful the unpadded 108 x 108 operands; "
-                    "three TF32 passes per real product, four real products per complex one"}
+            "note": "executed counts the MMAs as issued (padded 128 x 192 tiles), useful the unpadded 108 x 180 operands; "
+                    "three TF32 passes per real product"}
     n_products = m.n_loop_q if m.symmetric_state_path else spec.Nq
     prod = None
     if m.products == "tc":
@@ -723,24 +735,24 @@ def main():
     fp32_peak_tflops = sm_count * 128 * 2 * sm_max * 1e6 / 1e12
     ns = spec.n_s
     ndy_half = int(sum(1 for d in np.unique(spec.ff_R[:, 1][:, None] - spec.ff_R[:, 1][None, :]) if d >= 0))
-    unit_cfma = ns ** 4 + ns ** 5 + ndy_half * ns ** 4
-    # one launch sums every fine k for each directly evaluated transfer momentum (the loop symmetries
-    # supply the other momenta)
-    flops_per_launch = 8.0 * m32.n_loop_q * spec.Nk * unit_cfma
+    unit_fma = loop_fma(ns, ndy_half)
+    # one launch sums half of the fine mesh for each directly evaluated transfer momentum (the exchange of the propagators
+    # supplies the other half, the loop symmetries the other momenta)
+    flops_per_launch = loop_launch_flop(ns, m32.n_loop_q, spec.Nk, ndy_half)
     # the timed loop's products run at the orbit representatives when the state symmetries hold
     n_products = m32.n_loop_q if m32.symmetric_state_path else spec.Nq
     loop_ms_avg = phase_ms["loops"] / max(1, loop_launches)
     achieved = flops_per_launch / (loop_ms_avg * 1e-3) / 1e12
     trec = loop_traffic_record()[0] if args.workload == "rashba" else None   # recorded for that workload
-    kname = ("loops2_kernel (split-precision two-band loop k-sum)" if spec.n_s == 2
+    kname = ("loops2h_kernel (split-precision two-band loop k-sum, both channels)" if spec.n_s == 2
              else "loops_gen_kernel (split-precision multi-orbital loop k-sum)")
     roofline = {"bound": "alu", "kernel": kname,
                 "achieved": achieved, "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": achieved / fp32_peak_tflops,
                 "traffic": (trec["dram_bytes_per_launch"] if trec else None),
                 "peak_source": f"FP32 FMA peak derived: {sm_count} SMs x 128 lanes x 2 flop x {sm_max:.0f} MHz",
                 "algorithmic_flops_per_launch": flops_per_launch,
-                "unit_work": f"(N_s^4 + N_s^5 + {ndy_half} N_s^4) = {unit_cfma} complex FMA per (q, k) pair",
-                "units_per_launch": f"{m32.n_loop_q} directly summed q x {spec.Nk} k",
+                "unit_work": f"(N_s^4 + N_s^5 + {2 * ndy_half - 1} N_s^4) = {unit_fma} real FMA per (q, k) pair and channel",
+                "units_per_launch": f"{m32.n_loop_q} directly summed q x {spec.Nk} / 2 k",
                 "avg_launch_ms": loop_ms_avg}
     if m32.loops_backend == "tc":
         # the tensor-core loop kernel: its bound is the TF32 tensor pipe; the method's FP32 count stays beside it
@@ -751,12 +763,12 @@ def main():
                     "frac": ex / (loop_ms_avg * 1e-3) / 1e12 / tf32, "traffic": None,
                     "peak_source": "measured bf16 x 1.1/2.25 (nominal TF32/BF16)",
                     "algorithmic_flops_per_launch": ex,
-                    "unit_work": "36 MMAs of 128 x 112 x 8 (TF32) per stage of 4 fine-mesh rows, per column and "
+                    "unit_work": "9 MMAs of 128 x 192 x 8 (TF32) per stage of 4 fine-mesh rows, per column and "
                                  "group of 3 momenta",
-                    "units_per_launch": f"{m32.n_loop_q} directly summed q x {spec.Nk} k",
+                    "units_per_launch": f"{m32.n_loop_q} directly summed q x {spec.Nk} / 2 k",
                     "useful_frac": us / (loop_ms_avg * 1e-3) / 1e12 / tf32,
                     "method_fp32": {"achieved": achieved, "peak": fp32_peak_tflops, "frac": achieved / fp32_peak_tflops,
-                                    "unit_work": f"(N_s^4 + N_s^5 + {ndy_half} N_s^4) = {unit_cfma} complex FMA per (q, k)"},
+                                    "unit_work": f"(N_s^4 + N_s^5 + {2 * ndy_half - 1} N_s^4) = {unit_fma} real FMA per (q, k)"},
                     "avg_launch_ms": loop_ms_avg}
 
     cpu = None
@@ -790,12 +802,12 @@ def main():
                        "l2": "flushed (256 MB write) between timed steps", "instances": f"{world} (seed = rank)"},
             "split_vs_fp64_maxrel": err_split,
             "fp64_gpu": ({"value": fp64_rate, "unit": "RHS/s", "speedup_split": value / world / fp64_rate,
-                          "note": "every transfer momentum summed directly"} if fp64_rate else None),
+                          "note": "loops at the orbit representatives, projections and products at every momentum"} if fp64_rate else None),
             "rhs_general_state": {"value": general_rate, "unit": "RHS/s",
                                   "note": "tufrg_rhs without TUFRG_SYMMETRIC_STATE: projections and products at every "
                                           "momentum (the timed loop evaluates the flow state, which has the symmetries)"},
             "split_every_q_summed": {"value": full_rate, "unit": "RHS/s",
-                                     "note": "split path with the loop symmetries off (same loop work as fp64_gpu)"},
+                                     "note": "split path with the loop symmetries off"},
             "time_to_lambda_c": flows,
             "phase_ms_per_rhs": {k: v / args.steps for k, v in phase_ms.items()},
             "gpu_launches": launches,

@@ -1234,6 +1234,19 @@ try {
             if (std::find(ry.begin(), ry.end(), m->cls[2 * c + 1]) == ry.end()) ry.push_back(m->cls[2 * c + 1]);
             if (std::find(rx.begin(), rx.end(), m->cls[2 * c]) == rx.end()) rx.push_back(m->cls[2 * c]);
         }
+        if (!split) {   // the FP64 row pass forms R_y and -R_y together
+            std::vector<int> self, pairs;
+            for (int v : ry) {
+                const int w = (m->Lq - v) % m->Lq;
+                if (w == v) self.push_back(v);
+                else if (v < w && std::find(ry.begin(), ry.end(), w) != ry.end()) pairs.insert(pairs.end(), {v, w});
+            }
+            if (self.size() + pairs.size() == ry.size()) {
+                m->dft_nself = (int)self.size();
+                ry = self;
+                ry.insert(ry.end(), pairs.begin(), pairs.end());
+            }
+        }
         m->dft_nry = (int)ry.size();
         m->dft_nrx = (int)rx.size();
         dft_sep_plan(m, &m->dft_warps);

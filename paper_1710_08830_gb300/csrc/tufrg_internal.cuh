@@ -313,6 +313,7 @@ struct tufrg_model {
     // classes with one R_y; 0 = not used), int tables (class id by R_y group, R_x index, R_y group offsets) and
     // phases [Lq][n_Ry], [Lq][n_Rx]; its row pass keeps Z(u_x, R_y) in d_dftpart
     int dft_nry = 0, dft_nrx = 0, dft_warps = 0;
+    int dft_nself = -1;             // FP64: R_y = -R_y first (that many), then pairs R_y, -R_y; -1: not paired
     int *d_dft_tabs = nullptr;
     double2 *d_dft_phy = nullptr, *d_dft_phx = nullptr;
     float2 *d_dft_phy32 = nullptr, *d_dft_phx32 = nullptr;

@@ -538,7 +538,7 @@ void release(tufrg_model *m)
                     m->d_loop_list, m->d_qmap, m->d_sym_elem, m->d_sym_dinv, m->d_lph32,
                     m->d_clsph32, m->d_v0d32[0], m->d_v0d32[1], m->d_sym_srow, m->d_sym_qrow, m->d_sym_sinv, m->d_orb_ofs, m->d_orb_q, m->d_sym_emap, m->d_orb_lexp, m->d_band_tc,
                     m->d_dft_tabs, m->d_dft_phy, m->d_dft_phx, m->d_dft_phy32, m->d_dft_phx32, m->d_loop_w,
-                    m->d_shard_q, m->d_oz, m->d_LcB, m->d_Lc32B, m->d_recB, m->d_partB, m->d_lph, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
+                    m->d_shard_q, m->d_oz, m->d_LcB, m->d_Lc32B, m->d_recB, m->d_partB, m->d_lph, m->d_lph_pair, m->d_hp, m->d_rho, m->d_tc_grp, m->d_shard_out, m->d_v0q, m->d_v0q32, m->d_ffW, m->d_amax_ch};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &p : m->d_k)
@@ -1312,8 +1312,15 @@ try {
             std::vector<float2> l32(lph.size());
             for (size_t i = 0; i < lph.size(); i++) l32[i] = make_float2((float)lph[i].x, (float)lph[i].y);
             CK(upload(&m->d_lph32, l32, m->stream), "upload phase table");
-        } else {
-            CK(upload(&m->d_lph, lph, m->stream), "upload phase table");
+        }
+        if (!split) CK(upload(&m->d_lph, lph, m->stream), "upload phase table");
+        if (split && ns != 2) {   // the same as FP32 pairs (leading parts, then what they leave)
+            std::vector<float4> lp(lph.size());
+            for (size_t i = 0; i < lph.size(); i++) {
+                const float x = (float)lph[i].x, y = (float)lph[i].y;
+                lp[i] = make_float4(x, y, (float)(lph[i].x - (double)x), (float)(lph[i].y - (double)y));
+            }
+            CK(upload(&m->d_lph_pair, lp, m->stream), "upload phase table");
         }
     }
     CK(dalloc(&m->d_E, Nk * ns), "cudaMalloc eigenvalues");

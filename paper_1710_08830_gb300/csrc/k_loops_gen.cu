@@ -21,10 +21,12 @@
 // e^{-iqx dx} W into the accumulator of its own entries (no other CTA touches them, so no atomics; the order is fixed).
 // loops_gen_finish puts the orbital entries together from the real components, adds the exchanged half, writes both
 // Hermitian halves, L(-d)[b][a] = conj(L(d)[a][b]), and scales by 1/Nk; loops_gen_gather writes the other momenta of
-// the orbits.
+// the orbits.  From the ranges' accumulators on, the split path adds in FP32 pairs (in FP32 alone the 12 x 12 / 5 x 5 bilayer
+// mesh's P loops are off by 1.9e-7 instead of 0.7e-7).
 // FP64: bound by the FP64 pipe (two results per clock and SM); the 8 x 8 / 6 x 6 three-orbital sums of both channels
 // take 1.8 ms (6.9 ms in complex arithmetic over the whole mesh).
 #include <cmath>
+#include <type_traits>
 
 #include "tufrg_internal.cuh"
 
@@ -313,59 +315,98 @@ __global__ void loops_gen_kernel(const __grid_constant__ GenArgs<R> a)
         for (size_t i = threadIdx.x; i < (size_t)a.nd * NS2 * NS2; i += blockDim.x) acc[i] = mk(R(0), R(0));
 }
 
-// the kx ranges' accumulators added into the first range's (fixed order, eight loads in flight)
-template <typename C2>
-__global__ void loops_gen_chunk_sum(C2 *acc, int nchunk, size_t n)
+// Numbers of the sums after the k-sum: FP64, or on the split path an unevaluated FP32 pair h + l (l the rounding errors of
+// h), good to about 2^-46.  The pairs take FP32 operations only: FP64 ones have one 64th of their rate, and with the
+// conversions the 153 representatives of the 32 x 32 three-orbital mesh took 0.24 ms more per channel (10.07 against 9.60 ms
+// for the right-hand side).
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ double plus(double a, double b) { return a + b; }
+__device__ __forceinline__ Pair plus(Pair a, Pair b)   // Knuth's two-sum of the leading parts
+{
+    const float t = __fadd_rn(a.h, b.h), u = __fsub_rn(t, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(t, u)), __fsub_rn(b.h, u));
+    return Pair{t, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ double times(double a, double b) { return a * b; }
+__device__ __forceinline__ Pair times(Pair a, Pair b)
+{
+    const float t = __fmul_rn(a.h, b.h);
+    return Pair{t, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -t)))};
+}
+__device__ __forceinline__ double minus(double a) { return -a; }
+__device__ __forceinline__ Pair minus(Pair a) { return Pair{-a.h, -a.l}; }
+// (an infinite leading part leaves a NaN in the other)
+__device__ __forceinline__ float as_f32(Pair a) { return isfinite(a.h) ? __fadd_rn(a.h, a.l) : a.h; }
+__device__ __forceinline__ float as_f32(double a) { return narrow_f(a); }
+__device__ __forceinline__ double as_f64(Pair a) { return isfinite(a.h) ? widen_f(a.h) + widen_f(a.l) : widen_f(a.h); }
+__device__ __forceinline__ double as_f64(double a) { return a; }
+
+template <typename V>
+struct Cx {
+    V x, y;
+};
+template <typename V> __device__ __forceinline__ Cx<V> add(Cx<V> a, Cx<V> b) { return Cx<V>{plus(a.x, b.x), plus(a.y, b.y)}; }
+template <typename V> __device__ __forceinline__ Cx<V> times(Cx<V> a, Cx<V> b)
+{
+    return Cx<V>{plus(times(a.x, b.x), minus(times(a.y, b.y))), plus(times(a.x, b.y), times(a.y, b.x))};
+}
+template <typename V> __device__ __forceinline__ Cx<V> turn(Cx<V> v, int k)   // i^k v
+{
+    switch (k & 3) {
+    case 0: return v;
+    case 1: return Cx<V>{minus(v.y), v.x};
+    case 2: return Cx<V>{minus(v.x), minus(v.y)};
+    default: return Cx<V>{v.y, minus(v.x)};
+    }
+}
+// complex values as they lie in memory: FP64, FP32 accumulators, FP32 pairs (h, h, l, l)
+__device__ __forceinline__ Cx<double> ld_cx(double2 v) { return Cx<double>{v.x, v.y}; }
+__device__ __forceinline__ Cx<Pair> ld_cx(float2 v) { return Cx<Pair>{Pair{v.x, 0.f}, Pair{v.y, 0.f}}; }
+__device__ __forceinline__ Cx<Pair> ld_cx(float4 v) { return Cx<Pair>{Pair{v.x, v.z}, Pair{v.y, v.w}}; }
+__device__ __forceinline__ double2 st_cx(Cx<double> v) { return make_double2(v.x, v.y); }
+__device__ __forceinline__ float4 st_cx(Cx<Pair> v) { return make_float4(v.x.h, v.y.h, v.x.l, v.y.l); }
+template <typename S> using val_t = decltype(ld_cx(S{}).x);                    // its number
+template <typename S> using wide_t = decltype(st_cx(ld_cx(S{})));               // a sum of such values in memory
+
+// the kx ranges' accumulators added (fixed order, eight loads in flight): FP64 over the first range's accumulators, FP32
+// into pairs
+template <typename S>
+__global__ void loops_gen_chunk_sum(const S *acc, int nchunk, size_t n, wide_t<S> *sum)
 {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     constexpr int UB = 8;
-    C2 s = acc[t];
+    auto s = ld_cx(acc[t]);
     for (int c = 1; c < nchunk; c += UB) {
-        C2 w[UB];
+        S w[UB];
 #pragma unroll
         for (int j = 0; j < UB; j++)
             if (c + j < nchunk) w[j] = acc[(size_t)(c + j) * n + t];
 #pragma unroll
         for (int j = 0; j < UB; j++)
-            if (c + j < nchunk) {
-                s.x += w[j].x;
-                s.y += w[j].y;
-            }
+            if (c + j < nchunk) s = add(s, ld_cx(w[j]));
     }
-    acc[t] = s;
+    sum[t] = st_cx(s);
 }
 
-template <typename C2>
+template <typename S>
 struct FinArgs {
-    const C2 *acc;               // [slot][nd][NS2][NS2] half-plane sums in real components
-    const C2 *ptab;              // e^{-2 pi i n / Lf}
+    const S *acc;                // [slot][nd][NS2][NS2] half-plane sums in real components
+    const wide_t<S> *ptab;       // e^{-2 pi i n / Lf}
     const int *deltas, *partner, *slot_q;   // slot_q: momentum of a slot (null: the slot)
     const SymElem *elem;         // the element inv inverts the momentum (C channel's exchanged half)
     const int *dinv;
     int nd, Lq, nc, half, inv;
-    double inv_nk;
+    val_t<S> inv_nk;
     double2 *out64;
     float2 *out32;
 };
 
-template <typename C2> __device__ __forceinline__ C2 turn(C2 v, int k)
-{
-    switch (k & 3) {
-    case 0: return v;
-    case 1: return mk(-v.y, v.x);
-    case 2: return mk(-v.x, -v.y);
-    default: return mk(v.y, -v.x);
-    }
-}
-__device__ __forceinline__ double2 wide2(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
-__device__ __forceinline__ double2 wide2(double2 v) { return v; }
-__device__ __forceinline__ void put_f32(float2 *p, float2 v) { *p = v; }
-__device__ __forceinline__ void put_f32(float2 *p, double2 v) { *p = make_float2((float)v.x, (float)v.y); }
-
 // orbital entry S[d][ia][ib] of one slot's half-plane sums
-template <int NS, int CH, typename C2>
-__device__ __forceinline__ C2 gen_entry(const C2 *acc, const FinArgs<C2> &f, int d, int ia, int ib)
+template <int NS, int CH, typename S>
+__device__ __forceinline__ auto gen_entry(const S *acc, const FinArgs<S> &f, int d, int ia, int ib)
 {
     constexpr int NS2 = NS * NS;
     const int dx = f.deltas[2 * d], dy = f.deltas[2 * d + 1];
@@ -381,47 +422,34 @@ __device__ __forceinline__ C2 gen_entry(const C2 *acc, const FinArgs<C2> &f, int
     const int t1 = CH == 0 ? ay : ax, t2 = CH == 0 ? ax : ay, t3 = CH == 0 ? by : bx, t4 = CH == 0 ? bx : by;
     const int lr = loop_comp_index<NS>(t1, t3), rr = loop_comp_index<NS>(t2, t4);
     const int ls = t1 == t3 ? 0 : t1 < t3 ? 1 : -1, rs0 = t2 == t4 ? 0 : t2 < t4 ? 1 : -1, rs = CH == 0 ? rs0 : -rs0;
-    const C2 *o = acc + (size_t)d * NS2 * NS2;
-    C2 v = o[lr * NS2 + rr];
-    if (ls) {
-        const C2 w = o[(lr + 1) * NS2 + rr];   // + i ls w
-        v.x -= ls * w.y;
-        v.y += ls * w.x;
-    }
-    if (rs) {
-        const C2 w = o[lr * NS2 + rr + 1];
-        v.x -= rs * w.y;
-        v.y += rs * w.x;
-    }
-    if (ls && rs) {
-        const C2 w = o[(lr + 1) * NS2 + rr + 1];
-        v.x -= ls * rs * w.x;
-        v.y -= ls * rs * w.y;
-    }
-    if (!hp) v.y = -v.y;
+    const S *o = acc + (size_t)d * NS2 * NS2;
+    auto v = ld_cx(o[lr * NS2 + rr]);
+    if (ls) v = add(v, turn(ld_cx(o[(lr + 1) * NS2 + rr]), ls));        // + i ls w
+    if (rs) v = add(v, turn(ld_cx(o[lr * NS2 + rr + 1]), rs));
+    if (ls && rs) v = add(v, turn(ld_cx(o[(lr + 1) * NS2 + rr + 1]), ls + rs));
+    if (!hp) v.y = minus(v.y);
     return v;
 }
 
-// Every entry of every slot's loops at the slot's momentum: the sums, the exchanged half, 1/Nk.
-// Grid: (entries / 256, slots).
-template <int NS, int CH, typename R>
-__global__ void __launch_bounds__(256) loops_gen_finish(const __grid_constant__ FinArgs<typename cpx<R>::t> f)
+// Every entry of every slot's loops at the slot's momentum: the sums, the exchanged half, 1/Nk, rounded once for the FP32
+// loops.  Grid: (entries / 256, slots).
+template <int NS, int CH, typename S>
+__global__ void __launch_bounds__(256) loops_gen_finish(const __grid_constant__ FinArgs<S> f)
 {
-    using C2 = typename cpx<R>::t;
     constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= f.nd * NS4) return;
     const int s = blockIdx.y, d = t / NS4, ia = (t / NS2) % NS2, ib = t % NS2;
     const int q = f.slot_q ? f.slot_q[s] : s;
-    const C2 *acc = f.acc + (size_t)s * f.nd * NS4;
-    C2 v = gen_entry<NS, CH>(acc, f, d, ia, ib);
+    const S *acc = f.acc + (size_t)s * f.nd * NS4;
+    auto v = gen_entry<NS, CH>(acc, f, d, ia, ib);
     if (f.half) {
         auto swp = [](int a) { return (a % NS) * NS + a / NS; };
         int d2 = d, k = 0;
-        C2 w;
+        decltype(v) w;
         if (CH == 0) {   // e^{-is.Delta} conj(S[b~][a~])
             w = gen_entry<NS, CH>(acc, f, d, swp(ib), swp(ia));
-            w.y = -w.y;
+            w.y = minus(w.y);
         } else {         // V [e^{iu.Delta} S[b~][a~]] V^dagger
             const SymElem &e = f.elem[f.inv];
             d2 = f.dinv[f.inv * f.nd + d];
@@ -429,28 +457,27 @@ __global__ void __launch_bounds__(256) loops_gen_finish(const __grid_constant__ 
             k = e.qt[1][ia] - e.qt[1][ib];
         }
         const int n = (((q / f.Lq) * f.deltas[2 * d2] + (q % f.Lq) * f.deltas[2 * d2 + 1]) % f.Lq + f.Lq) % f.Lq * f.nc;
-        C2 p = f.ptab[n];
-        if (CH == 1) p.y = -p.y;
-        w = mk(p.x * w.x - p.y * w.y, p.x * w.y + p.y * w.x);
+        auto p = ld_cx(f.ptab[n]);
+        if (CH == 1) p.y = minus(p.y);
+        w = times(p, w);
         if (CH == 1) {
-            if (f.elem[f.inv].conj) w.y = -w.y;
+            if (f.elem[f.inv].conj) w.y = minus(w.y);
             w = turn(w, k);
         }
-        v.x += w.x;
-        v.y += w.y;
+        v = add(v, w);
     }
-    v.x *= R(f.inv_nk);
-    v.y *= R(f.inv_nk);
+    v.x = times(v.x, f.inv_nk);
+    v.y = times(v.y, f.inv_nk);
     const size_t o = (size_t)q * f.nd * NS4 + t;
-    if (f.out64) f.out64[o] = wide2(v);
-    if (f.out32) put_f32(f.out32 + o, v);
+    if (f.out64) f.out64[o] = make_double2(as_f64(v.x), as_f64(v.y));
+    if (f.out32) f.out32[o] = make_float2(as_f32(v.x), as_f32(v.y));
 }
 
 // The momenta that are not orbit representatives: entry (d', a', b') of q' from the representative's (d, src a', src b'),
 // i^(qt[a'] - qt[b']) (conj ? conj(v) : v).  Grid: (entries / 256, momenta).  Reads and writes the same buffers (the
 // representatives' rows are only read).
-template <int NS, typename C2>
-__global__ void __launch_bounds__(256) loops_gen_gather(C2 *L, double2 *out64, int nd, const int2 *qmap, const int *list,
+template <int NS>
+__global__ void __launch_bounds__(256) loops_gen_gather(double2 *L64, float2 *L32, int nd, const int2 *qmap, const int *list,
                                                         const SymElem *elem, const int *dinv, int ch)
 {
     constexpr int NS2 = NS * NS, NS4 = NS2 * NS2;
@@ -462,12 +489,20 @@ __global__ void __launch_bounds__(256) loops_gen_gather(C2 *L, double2 *out64, i
     if (q == q2) return;
     const int d2 = t / NS4, a2 = (t / NS2) % NS2, b2 = t % NS2;
     const SymElem &e = elem[ie.y];
-    C2 v = L[(size_t)q * nd * NS4 + ((size_t)dinv[ie.y * nd + d2] * NS2 + e.src[ch][a2]) * NS2 + e.src[ch][b2]];
-    if (e.conj) v.y = -v.y;
-    v = turn(v, e.qt[ch][a2] - e.qt[ch][b2]);
+    const size_t i = (size_t)q * nd * NS4 + ((size_t)dinv[ie.y * nd + d2] * NS2 + e.src[ch][a2]) * NS2 + e.src[ch][b2];
     const size_t o = (size_t)q2 * nd * NS4 + t;
-    L[o] = v;
-    if (sizeof(C2) == sizeof(float2)) out64[o] = wide2(v);
+    const int k = e.qt[ch][a2] - e.qt[ch][b2], conj = e.conj;
+    auto image = [&](auto v) {
+        Cx<decltype(v.x)> w{v.x, conj ? -v.y : v.y};
+        switch (k & 3) {
+        case 0: return mk(w.x, w.y);
+        case 1: return mk(-w.y, w.x);
+        case 2: return mk(-w.x, -w.y);
+        default: return mk(w.y, -w.x);
+        }
+    };
+    if (L64) L64[o] = image(L64[i]);
+    if (L32) L32[o] = image(L32[i]);
 }
 
 // per instantiation: tile and thread groups.  FP64 tiles are sized for the registers of the column sums; the FP32
@@ -505,6 +540,17 @@ cudaError_t dispatch_gen(tufrg_model *m, const GenArgs<R> &a, int ch)
     return cudaErrorNotSupported;
 }
 
+// where the sums over several kx ranges lie: behind FP32 accumulators, over the first range's FP64 ones
+size_t gen_acc_bytes(const tufrg_model *m)
+{
+    const size_t ns2 = (size_t)m->ns * m->ns, values = (size_t)m->gen_chunks * m->n_loop_q * m->nd * ns2 * ns2;
+    return (values * (m->precision == TUFRG_FP64 ? sizeof(double2) : sizeof(float2)) + 15) & ~size_t(15);
+}
+template <typename S> wide_t<S> *gen_sums(tufrg_model *m)   // S: the accumulators
+{
+    return reinterpret_cast<wide_t<S> *>(static_cast<char *>(m->d_part) + (sizeof(S) == sizeof(double2) ? 0 : gen_acc_bytes(m)));
+}
+
 template <typename R>
 cudaError_t run_gen(tufrg_model *m, int ch, bool half, const typename cpx<R>::t *U, const typename FTg<R>::t *ft,
                     const typename cpx<R>::t *ptab)
@@ -540,23 +586,23 @@ cudaError_t run_gen(tufrg_model *m, int ch, bool half, const typename cpx<R>::t 
     TUFRG_CUDA_TRY((m->ns == 6 ? dispatch_gen<R, 6>(m, a, ch) : dispatch_gen<R, 4>(m, a, ch)));
     if (m->gen_chunks > 1) {
         PhaseScope ps(m, PH_LOOPRED);
-        loops_gen_chunk_sum<C2><<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(a.acc, m->gen_chunks, n);
+        loops_gen_chunk_sum<C2><<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(a.acc, m->gen_chunks, n, gen_sums<C2>(m));
     }
     return cudaGetLastError();
 }
 
-template <int NS, typename R>
-cudaError_t finish(tufrg_model *m, int ch, int n_slot, const FinArgs<typename cpx<R>::t> &f, bool gather, typename cpx<R>::t *L)
+template <int NS, typename S>
+cudaError_t finish(tufrg_model *m, int ch, int n_slot, const FinArgs<S> &f, bool gather)
 {
     constexpr int NS4 = NS * NS * NS * NS;
     const unsigned gx = (unsigned)((m->nd * NS4 + 255) / 256);
     PhaseScope ps(m, PH_LOOPRED, gather ? 2 : 1);
-    if (ch == 0) loops_gen_finish<NS, 0, R><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
-    else loops_gen_finish<NS, 1, R><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
+    if (ch == 0) loops_gen_finish<NS, 0><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
+    else loops_gen_finish<NS, 1><<<dim3(gx, n_slot), 256, 0, m->stream>>>(f);
     TUFRG_CUDA_TRY(cudaGetLastError());
     if (gather)
-        loops_gen_gather<NS><<<dim3(gx, m->Nq), 256, 0, m->stream>>>(L, f.out64, m->nd, m->d_qmap, m->d_loop_list, m->d_sym_elem,
-                                                                    m->d_sym_dinv, ch);
+        loops_gen_gather<NS><<<dim3(gx, m->Nq), 256, 0, m->stream>>>(f.out64, f.out32, m->nd, m->d_qmap, m->d_loop_list,
+                                                                    m->d_sym_elem, m->d_sym_dinv, ch);
     return cudaGetLastError();
 }
 
@@ -588,8 +634,8 @@ bool loops_gen_supported(const tufrg_model *m)
 
 size_t gen_part_bytes(const tufrg_model *m)
 {
-    const size_t ns2 = (size_t)m->ns * m->ns;
-    return (size_t)m->gen_chunks * m->n_loop_q * m->nd * ns2 * ns2 * (m->precision == TUFRG_FP64 ? sizeof(double2) : sizeof(float2));
+    const size_t ns2 = (size_t)m->ns * m->ns, sums = (size_t)m->n_loop_q * m->nd * ns2 * ns2 * sizeof(float4);
+    return gen_acc_bytes(m) + (m->precision != TUFRG_FP64 && m->gen_chunks > 1 ? sums : 0);
 }
 
 // The kx ranges per momentum that fill the GPU best: the fewest waves of CTAs times columns per range (plus about one
@@ -627,7 +673,10 @@ cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only)
         if (m->loops_tc) TUFRG_CUDA_TRY(launch_loops_tc(m, ch, half, reinterpret_cast<float2 *>(m->d_part)));
         else if (fp64) TUFRG_CUDA_TRY(run_gen<double>(m, ch, half, m->d_U, m->d_ft, m->d_lph));
         else TUFRG_CUDA_TRY(run_gen<float>(m, ch, half, m->d_U32, m->d_ft32, m->d_lph32));
-        auto fill = [&](auto &f) {
+        auto run = [&](auto *acc) {
+            FinArgs<std::remove_pointer_t<decltype(acc)>> f{};
+            f.acc = acc;
+            f.ptab = reinterpret_cast<decltype(f.ptab)>(fp64 ? (const void *)m->d_lph : (const void *)m->d_lph_pair);
             f.deltas = m->d_deltas;
             f.partner = m->d_dpartner;
             f.slot_q = m->sym ? m->d_loop_list : nullptr;
@@ -638,25 +687,18 @@ cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only)
             f.nc = m->nc;
             f.half = half ? 1 : 0;
             f.inv = m->sym_inv;
-            f.inv_nk = 1.0 / (double)m->Nk;
+            const double inv_nk = 1.0 / (double)m->Nk;
+            if constexpr (sizeof(f.inv_nk) == sizeof(double) && std::is_floating_point_v<decltype(f.inv_nk)>) f.inv_nk = inv_nk;
+            else f.inv_nk = Pair{(float)inv_nk, (float)(inv_nk - (double)(float)inv_nk)};
             // symmetric states: the split path's products read the FP32 loops only
             f.out64 = reps_only && !fp64 ? nullptr : m->d_Lc + ch * per;
             f.out32 = fp64 ? nullptr : m->d_Lc32 + ch * per;
+            const bool gather = m->sym && !reps_only;
+            return m->ns == 6 ? finish<6>(m, ch, n_slot, f, gather) : finish<4>(m, ch, n_slot, f, gather);
         };
-        const bool gather = m->sym && !reps_only;
-        if (fp64) {
-            FinArgs<double2> f{};
-            f.acc = reinterpret_cast<const double2 *>(m->d_part);
-            f.ptab = m->d_lph;
-            fill(f);
-            TUFRG_CUDA_TRY((m->ns == 6 ? finish<6, double>(m, ch, n_slot, f, gather, f.out64) : finish<4, double>(m, ch, n_slot, f, gather, f.out64)));
-        } else {
-            FinArgs<float2> f{};
-            f.acc = reinterpret_cast<const float2 *>(m->d_part);
-            f.ptab = m->d_lph32;
-            fill(f);
-            TUFRG_CUDA_TRY((m->ns == 6 ? finish<6, float>(m, ch, n_slot, f, gather, f.out32) : finish<4, float>(m, ch, n_slot, f, gather, f.out32)));
-        }
+        if (fp64) TUFRG_CUDA_TRY(run(reinterpret_cast<double2 *>(m->d_part)));
+        else if (m->gen_chunks > 1) TUFRG_CUDA_TRY(run(gen_sums<float2>(m)));
+        else TUFRG_CUDA_TRY(run(reinterpret_cast<float2 *>(m->d_part)));
     }
     return cudaSuccess;
 }

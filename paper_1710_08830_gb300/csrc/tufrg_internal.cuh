@@ -289,6 +289,7 @@ struct tufrg_model {
     float2 *d_X32 = nullptr;        // [2][Nq][M][M] FP32 copy of the state being evaluated (split path)
     float2 *d_lph32 = nullptr;      // [Lf] e^{-2 pi i n / Lf} for the loop kernels (split path)
     double2 *d_lph = nullptr;       // the same in FP64 (FP64 path)
+    float4 *d_lph_pair = nullptr;   // the same as FP32 pairs (split path, multi-orbital sums)
     int *d_hp = nullptr;            // [(nd + 1) / 2] bond differences of the Hermitian half, then [nd] the place of d or -d
     float2 *d_clsph32 = nullptr;    // [Nq][ncls] e^{i u.R''} (split-path Fourier transform)
     float2 *d_v0d32[2] = {nullptr, nullptr};   // FP32 copies of d_v0d (split path)

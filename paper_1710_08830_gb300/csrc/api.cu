@@ -1154,6 +1154,8 @@ try {
     // sized for the largest)
     if (loops2_supported(m) && m->precision != TUFRG_FP64) m->plan_cand = loop_plan_candidates(m);
     m->plan_h = plan_loops2h(m);
+    if (loops2_supported(m) && (m->plan.ky_chunks == 0 || m->plan_h.ky_chunks == 0))
+        return fail(m, TUFRG_ECUDA, "the loop k-sum of this mesh does not fit an SM");
     int max_partials = std::max(m->plan.n_partials, m->plan_h.n_partials);
     for (const LoopPlan &p : m->plan_cand) max_partials = std::max(max_partials, p.n_partials);
 
@@ -1343,6 +1345,7 @@ try {
         if (!loops_gen_supported(m)) return fail(m, TUFRG_ENOTSUP, "bond set too large for the multi-orbital loop kernel");
         m->loops_tc = d.loops != TUFRG_LOOPS_SIMT && loops_tc_supported(m);
         m->gen_chunks = m->loops_tc ? 1 : plan_gen_chunks(m);
+        if (m->gen_chunks == 0) return fail(m, TUFRG_ECUDA, "the loop k-sum of this model does not fit an SM");
         // accumulators of one channel: one slot per (kx range, directly summed momentum)
         m->part_bytes = gen_part_bytes(m);
         if (m->loops_tc) {

@@ -452,14 +452,14 @@ int loops2_blocks_per_sm(const tufrg_model *m)
     int ndyh = 0;
     for (int v : m->dys) ndyh += v >= 0;
     const size_t smem = loops2_smem_bytes(m->Lf, ndyh);
-    int n = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-    if (ndyh == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2_kernel<1, 0>, 32 * WARPS, smem);
-    if (ndyh == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2_kernel<2, 0>, 32 * WARPS, smem);
-    if (ndyh == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2_kernel<3, 0>, 32 * WARPS, smem);
-    if (ndyh == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2_kernel<4, 0>, 32 * WARPS, smem);
-    if (ndyh == 5) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2_kernel<5, 0>, 32 * WARPS, smem);
-    return (e == cudaSuccess && n > 0) ? n : 4;
+    switch (ndyh) {
+    case 1: return resident_ctas(loops2_kernel<1, 0>, 32 * WARPS, smem);
+    case 2: return resident_ctas(loops2_kernel<2, 0>, 32 * WARPS, smem);
+    case 3: return resident_ctas(loops2_kernel<3, 0>, 32 * WARPS, smem);
+    case 4: return resident_ctas(loops2_kernel<4, 0>, 32 * WARPS, smem);
+    case 5: return resident_ctas(loops2_kernel<5, 0>, 32 * WARPS, smem);
+    default: return 0;
+    }
 }
 
 static Args2 loops2_args(const tufrg_model *m, const int *s_list, float2 *part, const int *skip)
@@ -526,6 +526,7 @@ LoopPlan plan_loops(const tufrg_model *m)
     p.kx_per_cta = 32 * WARPS;
     const int ctas_x = (m->Lf + p.kx_per_cta - 1) / p.kx_per_cta;
     const int per_sm = loops2_supported(m) ? loops2_blocks_per_sm(m) : (m->precision == TUFRG_FP64 ? 4 : 6);
+    if (per_sm == 0) return p;
     const double slots = (double)m->sm_count * per_sm;
     double best = 1e300;
     int best_c = 1;

@@ -729,23 +729,23 @@ cudaError_t reduce2(tufrg_model *m, int channel_mask, const void *part, size_t p
 int loops2h_blocks_per_sm(const tufrg_model *m)
 {
     const int ndyh = n_dyh(m);
-    int n = 0;
-    cudaError_t e = cudaErrorInvalidValue;
     if (m->precision == TUFRG_FP64) {
         const size_t smem = loops2h_smem_bytes<double>(m->Lf, std::min(ndyh, 3));
-        e = ndyh == 1   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<double, 0, 1, false>, NT, smem)
-            : ndyh == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<double, 1, 1, false>, NT, smem)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<double, 2, 1, false>, NT, smem);
-    } else {
-        const size_t smem = loops2h_smem_bytes<float>(m->Lf, ndyh);
-        if (ndyh == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<float, 0, 1, false>, NT, smem);
-        if (ndyh == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<float, 1, 1, false>, NT, smem);
-        if (ndyh == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<float, 2, 1, false>, NT, smem);
-        if (ndyh == 4) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<float, 3, 1, false>, NT, smem);
-        if (ndyh == 5) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, loops2h_kernel<float, 4, 1, false>, NT, smem);
+        switch (ndyh) {
+        case 1: return resident_ctas(loops2h_kernel<double, 0, 1, false>, NT, smem);
+        case 2: return resident_ctas(loops2h_kernel<double, 1, 1, false>, NT, smem);
+        default: return resident_ctas(loops2h_kernel<double, 2, 1, false>, NT, smem);
+        }
     }
-    if (e != cudaSuccess) (void)cudaGetLastError();
-    return (e == cudaSuccess && n > 0) ? n : 4;
+    const size_t smem = loops2h_smem_bytes<float>(m->Lf, ndyh);
+    switch (ndyh) {
+    case 1: return resident_ctas(loops2h_kernel<float, 0, 1, false>, NT, smem);
+    case 2: return resident_ctas(loops2h_kernel<float, 1, 1, false>, NT, smem);
+    case 3: return resident_ctas(loops2h_kernel<float, 2, 1, false>, NT, smem);
+    case 4: return resident_ctas(loops2h_kernel<float, 3, 1, false>, NT, smem);
+    case 5: return resident_ctas(loops2h_kernel<float, 4, 1, false>, NT, smem);
+    default: return 0;
+    }
 }
 
 bool loops2_supported(const tufrg_model *m) { return m->ns == 2 && n_dyh(m) <= MAXDH && (int)m->dxs.size() <= MAXD; }
@@ -834,7 +834,9 @@ LoopPlan plan_loops2h(const tufrg_model *m)
     const int ctas_x = (m->Lf + NT - 1) / NT;
     const int half = loops2_half_mask(m);
     const int rows = half == 3 ? m->Lf / 2 + 1 : m->Lf;
-    const double slots = (double)m->sm_count * loops2h_blocks_per_sm(m);
+    const int per_sm = loops2h_blocks_per_sm(m);
+    if (per_sm == 0) return p;
+    const double slots = (double)m->sm_count * per_sm;
     const double flush = 0.45 * (double)m->dxs.size() * n_dyh(m);
     double best = 1e300;
     int best_c = 1;

@@ -617,12 +617,8 @@ int gen_ndyh(const tufrg_model *m)
 template <typename R, int NS>
 int gen_blocks_per_sm(int ndyh)
 {
-    int n = 0;
-    const cudaError_t e =
-        ndyh <= 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gen_kernel<R, NS, 3, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 3, Tile<R, NS>::G>())
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gen_kernel<R, NS, 5, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 5, Tile<R, NS>::G>());
-    if (e != cudaSuccess) (void)cudaGetLastError();
-    return (e == cudaSuccess && n > 0) ? n : 1;
+    return ndyh <= 3 ? resident_ctas(gen_kernel<R, NS, 3, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 3, Tile<R, NS>::G>())
+                     : resident_ctas(gen_kernel<R, NS, 5, 0>(), gen_threads<R, NS>(), gen_smem<R, NS, 5, Tile<R, NS>::G>());
 }
 
 }  // namespace
@@ -641,7 +637,9 @@ size_t gen_part_bytes(const tufrg_model *m)
 // The kx ranges per momentum that fill the GPU best: the fewest waves of CTAs times columns per range (plus about one
 // column's time of start and end per CTA), up to one column per range within MAX_RANGES accumulators.  With few
 // momenta the short ranges are what fills the SMs: the sums of 28 momenta of the 12 x 12 / 5 x 5 bilayer mesh take 76 us
-// per evaluation, 206 us with at least four columns per range.
+// per evaluation, 206 us with at least four columns per range.  The FP64 sums of six states fill the FP64 pipe to nine
+// tenths with one CTA (0.60 ms per column; two side by side 0.54 each), so their waves are counted over the SMs: 15 momenta
+// of 25 columns take 1.81 ms in 9 ranges, 2.16 in 13 (195 CTAs, two on some SMs), 1.66 in 25; 10 of 22 1.08 in 11, 0.97 in 22.
 int plan_gen_chunks(const tufrg_model *m)
 {
     constexpr int MAX_RANGES = 64;
@@ -649,13 +647,15 @@ int plan_gen_chunks(const tufrg_model *m)
     int per_sm;
     if (m->precision == TUFRG_FP64) per_sm = m->ns == 6 ? gen_blocks_per_sm<double, 6>(ndyh) : gen_blocks_per_sm<double, 4>(ndyh);
     else per_sm = m->ns == 6 ? gen_blocks_per_sm<float, 6>(ndyh) : gen_blocks_per_sm<float, 4>(ndyh);
-    const long slots = (long)m->sm_count * per_sm;
+    if (per_sm == 0) return 0;
+    const bool pipe = m->precision == TUFRG_FP64 && m->ns == 6;
+    const long slots = (long)m->sm_count * (pipe ? 1 : per_sm);
     const int ncol = loops2_half_mask(m) == 3 ? m->Lf / 2 + 1 : m->Lf;
     int best = 1;
     double best_cost = 1e300;
     for (int c = 1; c <= std::min(MAX_RANGES, ncol); c++) {
         const double waves = std::ceil((double)m->n_loop_q * c / (double)slots);
-        const double cost = waves * (std::ceil((double)ncol / c) + 1.0);
+        const double cost = waves * (std::ceil((double)ncol / c) + (pipe ? 0.05 : 1.0)) * (pipe && waves > 1.0 ? 0.9 : 1.0);
         if (cost < best_cost * 0.999) { best_cost = cost; best = c; }
     }
     return best;

@@ -469,7 +469,7 @@ void drop_flow_graphs(tufrg_model *m);
 // the launch shapes the two-band split loop kernel's autotuner times (ky ranges per column)
 std::vector<LoopPlan> loop_plan_candidates(const tufrg_model *m);
 long loops_flow_ctas(const tufrg_model *m);   // CTAs of one stage's k-sum in a two-band split flow
-int plan_gen_chunks(const tufrg_model *m);   // kx ranges per momentum of the multi-orbital loop kernel
+int plan_gen_chunks(const tufrg_model *m);   // kx ranges per momentum of the multi-orbital loop kernel (0: it cannot run here)
 size_t gen_part_bytes(const tufrg_model *m);   // loop scratch of the multi-orbital kernel
 int dft_plan_nsplit(const tufrg_model *m);
 bool loops2_supported(const tufrg_model *m);
@@ -551,6 +551,21 @@ cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, 
     c.attrs = &at;
     c.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// CTAs of a kernel that an SM holds at once, 0 where it cannot run.  The kernel is allowed its shared memory first: without
+// that the query answers 0 above 48 KB until the first launch, and plans would depend on what the process ran before.
+template <typename K>
+int resident_ctas(K *kern, int threads, size_t smem)
+{
+    cudaFuncAttributes fa{};
+    int n = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e == cudaSuccess ? n : 0;
 }
 
 // whether a flow's two-band k-sum directly follows the kernel that writes its records

@@ -208,13 +208,14 @@ tufrg_status tufrg_loop_momenta(const tufrg_model *m, int *n_direct);
  * Errors: TUFRG_EINVAL for NULL arguments. */
 tufrg_status tufrg_loops_info(const tufrg_model *m, int *backend);
 
-/* Launch shape of the loop k-sum: *ky_chunks = the number of k_y ranges each fine-mesh column is split into (the
- * grid's depth; every range ends with a flush of its partial sums), and, for the flows of the two-band split path, which
- * time every candidate from 1 to 16 ranges (each range at least 8 rows) at model set-up and keep the fastest:
- * *n_candidates = their number and h_ms[i] (i < min(n_ms, *n_candidates)) = the measured milliseconds per launch
- * of candidate i, which has i + 1 ranges.  Other paths report their heuristic choice and *n_candidates = 0.
- * The choice is cached per process and model shape, so models of the same shape sum in the same order.  (The k-sum of
- * single right-hand sides takes its ranges from the shape alone.)
+/* Launch shape of the loop k-sum in the model's flows: *ky_chunks = the number of k_y ranges each fine-mesh column is split
+ * into (with N_s = 4, 6 the number of k_x ranges of the mesh; every range ends with a flush of its sums).  The flows of the
+ * two-band split path time every candidate from 1 to 16 ranges (each range at least 8 rows) at model set-up and keep the
+ * fastest: *n_candidates = their number and h_ms[i] (i < min(n_ms, *n_candidates)) = the measured milliseconds per launch of
+ * candidate i, which has i + 1 ranges; the choice is cached per process and model shape, so models of the same shape sum in
+ * the same order.  Every other k-sum takes its ranges from the shape alone (*n_candidates = 0): FP64 models, N_s = 4, 6, and
+ * the single right-hand sides of two-band split models, which sum over half of the fine mesh, in another order than the
+ * same model's flows (the results differ by FP32 rounding).
  * Errors: TUFRG_EINVAL for NULL arguments or n_ms < 0 (h_ms may be NULL when n_ms is 0). */
 tufrg_status tufrg_loop_tiles(const tufrg_model *m, int *ky_chunks, int *n_candidates, double *h_ms, int n_ms);
 
@@ -443,14 +444,15 @@ tufrg_status tufrg_flow_batch(tufrg_model *const *models, int n, const tufrg_flo
  *   status tufrg_flow would return.
  * tufrg_flow_checkpoint_bytes: size of a checkpoint of this model (0 for NULL).
  * tufrg_flow_save: writes the open flow's checkpoint to the host buffer h_buf (caller-owned, at least
- *   tufrg_flow_checkpoint_bytes): a header (library version, model shape, channel mask, the products backend and
- *   loop launch shape in use), the device controller, the state y and k1 = f(y), FP64.
+ *   tufrg_flow_checkpoint_bytes): a header (version of the model's sums, model shape, channel mask, the products backend
+ *   and loop launch shape in use), the device controller, the state y and k1 = f(y), FP64.
  * tufrg_flow_resume: opens a stepwise flow from a checkpoint of a model of the same shape and channel mask,
  *   restoring the controller, y and k1, and the checkpointed run's products backend and loop launch shape (they
  *   fix the summation order): the steps that follow are bit for bit those of the uninterrupted run.  opts gives
  *   the channel mask (the controller's scale range, tolerances and stop value come from the checkpoint).
  * Errors: TUFRG_EINVAL (NULL arguments, bad options, a second open flow, no open flow, a short buffer, a
- * checkpoint of another model, mask or library version), TUFRG_ENOTSUP (checkpoints of a model with a loop
+ * checkpoint of another model or mask, of a loop launch shape that the model does not have, or of an earlier version of
+ * the model's sums: version 1 for FP64 models and N_s = 4, 6), TUFRG_ENOTSUP (checkpoints of a model with a loop
  * surrogate), TUFRG_ENONFINITE (tufrg_flow_resume: a non-finite value in the checkpoint's state or derivative; the
  * model is left as it was), TUFRG_ETIMEOUT (a bounded device wait gave up), TUFRG_ECUDA, and tufrg_flow_end's flow
  * statuses. */

@@ -932,12 +932,22 @@ struct CkptHeader {
     long long n_elems;
 };
 
+// Ranges of the loop k-sum that the model's flows launch (k_y ranges, with several orbitals k_x ranges).
+int loop_ranges(const tufrg_model *m)
+{
+    return m->ns != 2 ? m->gen_chunks : m->precision == TUFRG_FP64 ? m->plan_h.ky_chunks : m->plan.ky_chunks;
+}
+
+// Version 2: the sums over half of the fine mesh, in another order than those behind the version 1 checkpoints of the same
+// models, which therefore cannot be continued bit for bit.  Split two-band flows still take the sums of version 1.
+int ckpt_version(const tufrg_model *m) { return m->ns == 2 && m->precision != TUFRG_FP64 ? 1 : 2; }
+
 CkptHeader ckpt_header(const tufrg_model *m, int mask)
 {
     CkptHeader h;
     std::memset(&h, 0, sizeof(h));
     std::memcpy(h.magic, "TUFRGCK1", 8);
-    h.version = 1;
+    h.version = ckpt_version(m);
     h.flowdev_bytes = (int)sizeof(FlowDev);
     h.precision = m->precision;
     h.ns = m->ns;
@@ -950,7 +960,7 @@ CkptHeader ckpt_header(const tufrg_model *m, int mask)
     h.regulator = m->regulator;
     h.loops_tc = m->loops_tc ? 1 : 0;
     h.products = m->products;
-    h.ky_chunks = m->plan.ky_chunks;
+    h.ky_chunks = loop_ranges(m);
     h.n_elems = (long long)state_elems(m);
     return h;
 }
@@ -1149,13 +1159,16 @@ try {
             }
         }
     }
-    m->plan = plan_loops(m);
-    // the two-band split loop kernel's launch shapes are timed at the end of the set-up (the partial sums are
-    // sized for the largest)
-    if (loops2_supported(m) && m->precision != TUFRG_FP64) m->plan_cand = loop_plan_candidates(m);
-    m->plan_h = plan_loops2h(m);
-    if (loops2_supported(m) && (m->plan.ky_chunks == 0 || m->plan_h.ky_chunks == 0))
-        return fail(m, TUFRG_ECUDA, "the loop k-sum of this mesh does not fit an SM");
+    if (loops2_supported(m)) {
+        m->plan_h = plan_loops2h(m);
+        // the launch shapes of split flows are timed at the end of the set-up (the partial sums are sized for the largest)
+        if (m->precision != TUFRG_FP64) {
+            m->plan = plan_loops(m);
+            m->plan_cand = loop_plan_candidates(m);
+        }
+        if (m->plan_h.ky_chunks == 0 || (m->precision != TUFRG_FP64 && m->plan.ky_chunks == 0))
+            return fail(m, TUFRG_ECUDA, "the loop k-sum of this mesh does not fit an SM");
+    }
     int max_partials = std::max(m->plan.n_partials, m->plan_h.n_partials);
     for (const LoopPlan &p : m->plan_cand) max_partials = std::max(max_partials, p.n_partials);
 
@@ -1608,7 +1621,7 @@ tufrg_status tufrg_products_tiles(const tufrg_model *m, int *tile_width, int *n_
 tufrg_status tufrg_loop_tiles(const tufrg_model *m, int *ky_chunks, int *n_candidates, double *h_ms, int n_ms)
 {
     if (!m || !ky_chunks || !n_candidates || (n_ms > 0 && !h_ms) || n_ms < 0) return TUFRG_EINVAL;
-    *ky_chunks = m->plan.ky_chunks;
+    *ky_chunks = loop_ranges(m);
     *n_candidates = (int)m->plan_ms.size();
     for (int i = 0; i < n_ms && i < (int)m->plan_ms.size(); i++) h_ms[i] = m->plan_ms[i];
     return TUFRG_OK;
@@ -2144,8 +2157,8 @@ tufrg_status tufrg_flow_resume(tufrg_model *m, const tufrg_flow_opts *o, const v
     if (h.products != m->products &&
         (m->precision == TUFRG_FP64 || (h.products != TUFRG_PRODUCTS_TC && h.products != TUFRG_PRODUCTS_SIMT)))
         return fail(m, TUFRG_EINVAL, "the checkpoint's products backend does not apply to this model");
-    // (a path without timed launch shapes keeps its own)
-    if (h.ky_chunks < 1 || h.ky_chunks > (m->plan_cand.empty() ? 16 : (int)m->plan_cand.size()))
+    // (a path without timed launch shapes has its one)
+    if (m->plan_cand.empty() ? h.ky_chunks != want.ky_chunks : h.ky_chunks < 1 || h.ky_chunks > (int)m->plan_cand.size())
         return fail(m, TUFRG_EINVAL, "the checkpoint's loop launch shape does not apply to this model");
     bool reshaped = false;
     if (h.products != m->products) {

@@ -525,7 +525,7 @@ LoopPlan plan_loops(const tufrg_model *m)
     LoopPlan p{};
     p.kx_per_cta = 32 * WARPS;
     const int ctas_x = (m->Lf + p.kx_per_cta - 1) / p.kx_per_cta;
-    const int per_sm = loops2_supported(m) ? loops2_blocks_per_sm(m) : (m->precision == TUFRG_FP64 ? 4 : 6);
+    const int per_sm = loops2_blocks_per_sm(m);
     if (per_sm == 0) return p;
     const double slots = (double)m->sm_count * per_sm;
     double best = 1e300;
@@ -533,7 +533,7 @@ LoopPlan plan_loops(const tufrg_model *m)
     for (int c = 1; c <= 16; c++) {
         const int len = (m->Lf + c - 1) / c;
         if (len < 8) break;
-        const double ctas = (double)m->n_loop_q * ctas_x * c * (m->precision == TUFRG_FP64 ? 2 : 1);
+        const double ctas = (double)m->n_loop_q * ctas_x * c;
         const double waves = std::ceil(ctas / slots);
         const double cost = waves * (len + 8.0);
         if (cost < best * 0.999) { best = cost; best_c = c; }

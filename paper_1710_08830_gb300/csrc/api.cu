@@ -1718,7 +1718,7 @@ tufrg_status tufrg_loops(tufrg_model *m, double T, int channel_mask, void *d_loo
     CK(launch_set_scalars(m, T, 1.0), "set temperature");
     CK(surrogate_rearm(m), "re-arm surrogate");
     CK(launch_fermi(m), "fermi tables");
-    CK(launch_loops(m, channel_mask), "loop k-sum");
+    CK(launch_loops(m, channel_mask, false, false, true), "loop k-sum");
     const size_t per = (size_t)m->Nq * m->nd * m->ns * m->ns * m->ns * m->ns;
     for (int ch = 0; ch < 2; ch++)
         if ((channel_mask >> ch) & 1)

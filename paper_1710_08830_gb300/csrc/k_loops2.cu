@@ -379,8 +379,8 @@ __global__ void loops_reduce_sym_kernel(const typename cpx<R>::t *__restrict__ p
     const int ch = blockIdx.z;   // as in loops_reduce_kernel
     if (!((chmask >> ch) & 1)) return;
     part += ch * part_cs;
-    out64 += ch * out_cs;
-    out32 += ch * out_cs;
+    if (out64) out64 += ch * out_cs;
+    if (out32) out32 += ch * out_cs;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nd * NS4) return;
     const int q2 = blockIdx.y, d2 = t / NS4, a2 = (t / NS2) % NS2, b2 = t % NS2;
@@ -587,7 +587,8 @@ long loops_flow_ctas(const tufrg_model *m)
     return 2L * (m->sym ? m->n_loop_q : m->Nq) * ((m->Lf + 32 * WARPS - 1) / (32 * WARPS)) * m->plan.ky_chunks;
 }
 
-// The loops of a split two-band flow (every stage of it and the surrogate's fallback).
+// The loops of a split two-band flow (every stage of it and the surrogate's fallback): FP32 only, what its products read (two
+// stages' loops may run at a time, each into its own FP32 buffer).
 cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
 {
     const LoopPlan &pl = m->plan;
@@ -625,10 +626,10 @@ cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only)
     if (m->sym)
         loops_reduce_sym_kernel<float><<<grid, thr, 0, m->stream>>>(
             part, pl.n_partials, ndx, ndyh, m->d_dslot, m->d_deltas, m->nd, m->d_qmap, m->d_sym_elem, m->d_sym_dinv,
-            inv_nk, m->d_Lc, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
+            inv_nk, nullptr, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
     else
         return launch_chained(loops_reduce_kernel<float>, grid, thr, 0, m->stream, true, part, pl.n_partials, ndx, ndyh, m->d_dslot,
-                              m->d_deltas, m->nd, inv_nk, nullptr, m->d_Lc, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
+                              m->d_deltas, m->nd, inv_nk, nullptr, nullptr, m->d_Lc32, skip, channel_mask, part_cs, out_cs);
     return cudaGetLastError();
 }
 

@@ -853,11 +853,11 @@ LoopPlan plan_loops2h(const tufrg_model *m)
     return p;
 }
 
-cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only, bool flow)
+cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only, bool flow, bool want64)
 {
     if (m->sur) TUFRG_CUDA_TRY(launch_surrogate(m, channel_mask));
     reps_only = reps_only && m->sym;
-    if (m->ns != 2) return loops_gen_supported(m) ? launch_loops_gen(m, channel_mask, reps_only) : cudaErrorNotSupported;
+    if (m->ns != 2) return loops_gen_supported(m) ? launch_loops_gen(m, channel_mask, reps_only, want64) : cudaErrorNotSupported;
     if (!loops2_supported(m)) return cudaErrorNotSupported;
     if (flow && m->precision != TUFRG_FP64) return launch_loops_flow(m, channel_mask, reps_only);
     if (!(channel_mask & 3)) return cudaSuccess;
@@ -868,7 +868,7 @@ cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only, bool 
     // symmetric states: the representatives' loops at their own momenta, in the precision their products read
     return launch_loops2h_reduce(m, channel_mask, m->d_part, part_cs, m->sym ? m->d_loop_list : nullptr,
                                 reps_only ? m->n_loop_q : m->Nq, m->sym && !reps_only, reps_only,
-                                reps_only && !fp64 ? nullptr : m->d_Lc, fp64 ? nullptr : m->d_Lc32, out_cs,
+                                fp64 || (want64 && !reps_only) ? m->d_Lc : nullptr, fp64 ? nullptr : m->d_Lc32, out_cs,
                                 m->sur ? m->d_sur_flag : nullptr);
 }
 

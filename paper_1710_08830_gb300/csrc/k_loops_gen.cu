@@ -661,7 +661,7 @@ int plan_gen_chunks(const tufrg_model *m)
     return best;
 }
 
-cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only)
+cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only, bool want64)
 {
     const size_t ns4 = (size_t)m->ns * m->ns * m->ns * m->ns, per = (size_t)m->Nq * m->nd * ns4;
     const int n_slot = m->sym ? m->n_loop_q : m->Nq;
@@ -690,8 +690,7 @@ cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only)
             const double inv_nk = 1.0 / (double)m->Nk;
             if constexpr (sizeof(f.inv_nk) == sizeof(double) && std::is_floating_point_v<decltype(f.inv_nk)>) f.inv_nk = inv_nk;
             else f.inv_nk = Pair{(float)inv_nk, (float)(inv_nk - (double)(float)inv_nk)};
-            // symmetric states: the split path's products read the FP32 loops only
-            f.out64 = reps_only && !fp64 ? nullptr : m->d_Lc + ch * per;
+            f.out64 = fp64 || (want64 && !reps_only) ? m->d_Lc + ch * per : nullptr;
             f.out32 = fp64 ? nullptr : m->d_Lc32 + ch * per;
             const bool gather = m->sym && !reps_only;
             return m->ns == 6 ? finish<6>(m, ch, n_slot, f, gather) : finish<4>(m, ch, n_slot, f, gather);

@@ -430,8 +430,9 @@ cudaError_t launch_fermi(tufrg_model *m);
 cudaError_t launch_set_scalars(tufrg_model *m, double T, double scale);
 // reps_only (with loop symmetries): the FP32 loops of the orbit representatives only, at their own
 // momenta, and no FP64 copy on the split path (what the symmetric-state products read)
-// flow: a stage of a flow (split two-band flows keep their own k-sum)
-cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only = false, bool flow = false);
+// flow: a stage of a flow (split two-band flows keep their own k-sum); want64: the split path writes FP64 loops too (its
+// products read the FP32 ones only)
+cudaError_t launch_loops(tufrg_model *m, int channel_mask, bool reps_only = false, bool flow = false, bool want64 = false);
 cudaError_t launch_loops_flow(tufrg_model *m, int channel_mask, bool reps_only);
 LoopPlan plan_loops2h(const tufrg_model *m);
 cudaError_t launch_records_f32(const double *E, const double2 *U, int Nk, int Lf, double mu, double T, float4 *rec, cudaStream_t s);
@@ -475,7 +476,7 @@ int dft_plan_nsplit(const tufrg_model *m);
 bool loops2_supported(const tufrg_model *m);
 int loops2_blocks_per_sm(const tufrg_model *m);
 bool loops_gen_supported(const tufrg_model *m);
-cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only);
+cudaError_t launch_loops_gen(tufrg_model *m, int channel_mask, bool reps_only, bool want64);
 // sharded right-hand side (k_shard.cu): a shard's part of the Fourier transform, the gather of its rows, and the
 // loops at a list of momenta
 cudaError_t launch_shard_dft(tufrg_model *m, const double2 *d_state_local, int n, const int *d_q, int mask, double2 *d_xr);

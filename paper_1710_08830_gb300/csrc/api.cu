@@ -1376,11 +1376,9 @@ try {
         }
     }
     m->products = split ? (d.products == TUFRG_PRODUCTS_AUTO ? TUFRG_PRODUCTS_TC : d.products) : TUFRG_PRODUCTS_SIMT;
-    // product scratch: the large-M CUDA-core GEMMs' intermediate, or the tensor-core products' first product of both
-    // channels (FP32 complex, the same bytes)
-    if (m->M > 64 || split)
+    // product scratch of the split path: the first product of both channels (FP32 complex)
+    if (split)
         CK(cudaMalloc(reinterpret_cast<void **>(&m->d_T), (size_t)m->Nq * M2 * sizeof(double2)), "cudaMalloc product scratch");
-    if (m->M > 64 && !split) CK(cudaMalloc(&m->d_oz, vlv64_scratch_bytes(m)), "cudaMalloc product digits");
     CK(dalloc(&m->d_err, 1), "cudaMalloc error flag");
     CK(dalloc(&m->d_scal, 14), "cudaMalloc scalars");
     CK(cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream), "zero error flag");
@@ -1396,6 +1394,7 @@ try {
     if (!split) CK(dalloc(&m->d_A, 2 * (size_t)m->Nq * M2), "cudaMalloc projections");   // split: FP32 copy only
     CK(dalloc(&m->d_amax, 4), "cudaMalloc reductions");
     CK(dalloc(&m->d_red, 512), "cudaMalloc reductions");
+    if (m->M > 64 && !split) CK(vlv64_alloc(m), "cudaMalloc product digits");   // (last: it takes what fits)
 
     // ---- eigensystem and chemical potential
     CK(launch_bands(m), "eigensolve");

@@ -545,20 +545,31 @@ __global__ void __launch_bounds__(32 * EX_WARPS) oz_exact_kernel(const __grid_co
     if (g.rmax_out && warp == 0 && top) atomicMax(g.rmax_out + (size_t)mat * M + r, top);
 }
 
-int chunk_mats(const tufrg_model *m)   // matrices per chunk
+// scratch of one matrix of a chunk: T, left and right digits, the bits of the entries left to FP64 sums, row and column
+// maxima of A, column maxima of L, row maxima of T
+size_t mat_bytes(const Dims &d)
 {
-    const Dims d = dims_of(m->M);
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)m->Nq, CHUNK_BYTES / (d.a_bytes() + d.b_bytes())));
+    return (size_t)d.M * d.M * sizeof(double2) + d.a_bytes() + d.b_bytes() +
+           (size_t)d.M * (d.n_tiles * sizeof(unsigned long long) + 4 * sizeof(unsigned));
 }
 
 }  // namespace
 
-// digit buffers, the entries left to FP64 sums and the maxima of one chunk: left and right digits, the entries' bits, row
-// and column maxima of A, column maxima of L, row maxima of T
-size_t vlv64_scratch_bytes(const tufrg_model *m)
+// The scratch of a chunk of matrices, as many as fit 1 GiB and a sixteenth of the free memory (112 matrices of M = 324 fill
+// the GPU many times over; the chunk does not change results), fewer where the allocation fails, one at least.
+cudaError_t vlv64_alloc(tufrg_model *m)
 {
-    const Dims d = dims_of(m->M);
-    return (size_t)chunk_mats(m) * (d.a_bytes() + d.b_bytes() + (size_t)m->M * (d.n_tiles * sizeof(unsigned long long) + 4 * sizeof(unsigned)));
+    const size_t per = mat_bytes(dims_of(m->M));
+    size_t free_bytes = 0, total = 0;
+    TUFRG_CUDA_TRY(cudaMemGetInfo(&free_bytes, &total));
+    size_t n = std::max<size_t>(1, std::min<size_t>((size_t)m->Nq, std::min(CHUNK_BYTES, free_bytes / 16) / per));
+    cudaError_t e;
+    while ((e = cudaMalloc(&m->d_oz, n * per)) == cudaErrorMemoryAllocation && n > 1) {
+        (void)cudaGetLastError();
+        n /= 2;
+    }
+    m->oz_mats = (int)n;
+    return e;
 }
 
 cudaError_t launch_vlv64(tufrg_model *m, const double2 *d_A, int channel_mask, double2 *d_out, const int *qlist, int nlist)
@@ -570,8 +581,9 @@ cudaError_t launch_vlv64(tufrg_model *m, const double2 *d_A, int channel_mask, d
             TUFRG_CUDA_TRY(cudaMemsetAsync(d_out + (size_t)ch * m->Nq * M2, 0, sizeof(double2) * m->Nq * M2, m->stream));
     if (!(channel_mask & 3)) return cudaSuccess;
     const Dims d = dims_of(M);
-    const int cap = chunk_mats(m), total = nl * (channel_mask == 3 ? 2 : 1);
-    unsigned char *pa = static_cast<unsigned char *>(m->d_oz), *pb = pa + (size_t)cap * d.a_bytes();
+    const int cap = m->oz_mats, total = nl * (channel_mask == 3 ? 2 : 1);
+    double2 *T = static_cast<double2 *>(m->d_oz);
+    unsigned char *pa = reinterpret_cast<unsigned char *>(T + (size_t)cap * M2), *pb = pa + (size_t)cap * d.a_bytes();
     unsigned long long *ex = reinterpret_cast<unsigned long long *>(pb + (size_t)cap * d.b_bytes());
     unsigned *mx = reinterpret_cast<unsigned *>(ex + (size_t)cap * M * d.n_tiles);
     unsigned *ra = mx, *ca = ra + (size_t)cap * M, *cl = ca + (size_t)cap * M, *rt = cl + (size_t)cap * M;
@@ -588,15 +600,15 @@ cudaError_t launch_vlv64(tufrg_model *m, const double2 *d_A, int channel_mask, d
         const dim3 gr((d.n_tiles * TN + 127) / 128 * d.ks * 2, n), rows(M, n);
         const size_t ex_smem = (size_t)M * (sizeof(double2) + sizeof(int2) + sizeof(int));
         oz_right_kernel<true><<<gr, 128, 0, m->stream>>>(m->d_Lc, m->d_dij, m->nff, ns2, m->nd, mt, d, cl, pb);
-        GemmArgs g{pa, pb, ra, cl, m->d_T, rt, ex, mt, d, nullptr, m->d_err};
+        GemmArgs g{pa, pb, ra, cl, T, rt, ex, mt, d, nullptr, m->d_err};
         const unsigned tiles = (unsigned)((size_t)n * d.m_tiles * d.n_tiles * 2);   // two parts
         oz_gemm_kernel<<<tiles, NTHREADS, smem, m->stream>>>(g);
         oz_exact_kernel<true><<<rows, 32 * EX_WARPS, ex_smem, m->stream>>>(ExactArgs{d_A, m->d_Lc, m->d_dij, 0, m->nff, ns2, m->nd, g});
-        oz_left_kernel<true><<<dim3(d.m_tiles * d.ks * 2, n), TM, 0, m->stream>>>(m->d_T, mt, d, rt, pa);
+        oz_left_kernel<true><<<dim3(d.m_tiles * d.ks * 2, n), TM, 0, m->stream>>>(T, mt, d, rt, pa);
         oz_right_kernel<false><<<gr, 128, 0, m->stream>>>(d_A, nullptr, 0, 1, 0, mt, d, ca, pb);
         g = GemmArgs{pa, pb, rt, ca, d_out, nullptr, ex, mt, d, m->d_scal, m->d_err};
         oz_gemm_kernel<<<tiles, NTHREADS, smem, m->stream>>>(g);
-        oz_exact_kernel<false><<<rows, 32 * EX_WARPS, ex_smem, m->stream>>>(ExactArgs{m->d_T, d_A, nullptr, 1, 0, 1, 0, g});
+        oz_exact_kernel<false><<<rows, 32 * EX_WARPS, ex_smem, m->stream>>>(ExactArgs{T, d_A, nullptr, 1, 0, 1, 0, g});
         TUFRG_CUDA_TRY(cudaGetLastError());
     }
     return cudaSuccess;

@@ -303,8 +303,9 @@ struct tufrg_model {
     double2 *d_Xr = nullptr;        // [2][ncls][M][M] Fourier transforms
     double2 *d_A = nullptr;         // [2][Nq][M][M] projected vertex
     float2 *d_A32 = nullptr;        // [2][Nq][M][M] (split path)
-    void *d_oz = nullptr;           // digit buffers of the FP64 products (large M)
-    double2 *d_T = nullptr;         // [Nq][M][M] GEMM intermediate (large M); split: [2][Nq][M][M] FP32 complex
+    void *d_oz = nullptr;           // scratch of the FP64 products (large M), for oz_mats matrices
+    int oz_mats = 0;
+    double2 *d_T = nullptr;         // split: product scratch, [2][Nq][M][M] FP32 complex
     void *d_rec = nullptr;          // [3][Nk] two-band loop records (projectors + Fermi data; float4 or four doubles)
     float2 *d_Xr32 = nullptr;       // [2][ncls][M][M] Fourier transforms (split path)
     float2 *d_ph32 = nullptr;       // [Nq][nph] phase table (split path)
@@ -493,7 +494,7 @@ size_t loops_tc_w_bytes(const tufrg_model *m);
 std::vector<int> loops_tc_groups(const std::vector<int> &q_of_slot, int Lq);
 cudaError_t launch_loops_rho(tufrg_model *m);   // once per model
 cudaError_t launch_loops_tc(tufrg_model *m, int ch, bool half, float2 *acc);
-size_t vlv64_scratch_bytes(const tufrg_model *m);
+cudaError_t vlv64_alloc(tufrg_model *m);
 cudaError_t launch_vlv64(tufrg_model *m, const double2 *d_A, int channel_mask, double2 *d_out, const int *qlist, int nlist);   // FP64, M > 64
 cudaError_t launch_vlv_large(tufrg_model *m, int channel_mask, double2 *d_out, const int *qlist, int nlist);   // FP32, M > 64
 cudaError_t launch_sym_scatter(tufrg_model *m, double2 *d_out);

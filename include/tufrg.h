@@ -119,9 +119,9 @@ typedef struct {
 enum { TUFRG_BASIS_ORBITAL = 0, TUFRG_BASIS_BAND = 1 };
 
 /* Backend of the loop k-sum of split-precision models with N_s = 6 and at most three non-negative y components
- * of the bond differences (5 or 9 bonds): TC runs the per-column orbital sums as complex 3xTF32 GEMMs on the
- * tensor cores (FP32 accumulation in tensor memory), SIMT as FP32 FMAs on the CUDA cores; AUTO takes TC where it
- * applies.  Every other model uses the CUDA-core kernels whatever the value. */
+ * of the bond differences (5 or 9 bonds): TC runs the per-column orbital sums as 3xTF32 GEMMs of real Hermitian
+ * components on the tensor cores (FP32 accumulation in tensor memory), SIMT as FP32 FMAs on the CUDA cores; AUTO takes
+ * TC where it applies.  Every other model uses the CUDA-core kernels whatever the value. */
 enum { TUFRG_LOOPS_AUTO = 0, TUFRG_LOOPS_TC = 1, TUFRG_LOOPS_SIMT = 2 };
 
 /* Regulator of the loops (Eq. def_lmp, L = d/dLambda [chi(e1) chi(e2)] F(e1, e2)).
@@ -139,12 +139,13 @@ enum { TUFRG_REG_TEMPERATURE = 0, TUFRG_REG_MOMENTUM_SHELL = 1 };
  * U (x) U^* on the C pair).  Time reversal, t_R = W t_R^* W^T with W = i sigma_y, gives
  * Lc(-q)[Delta] = V conj(Lc(q)[Delta]) V^dagger with V built from W.  With TUFRG_SYMMETRY_AUTO the
  * operations that hold (U searched among the monomial unitaries) are found at init, the k-sum runs
- * for one momentum per orbit and the others are written from it.  TUFRG_SYMMETRY_OFF sums every q. */
-/* For symmetric states (tufrg_rhs with TUFRG_SYMMETRIC_STATE, and every flow) the projections and products can
+ * for one momentum per orbit and the others are written from it.  TUFRG_SYMMETRY_OFF sums every q.
+ *
+ * For symmetric states (tufrg_rhs with TUFRG_SYMMETRIC_STATE, and every flow) the projections and products can
  * run for the orbit representatives only, and do so whenever the state symmetries hold (AUTO and STATES
- * alike; OFF disables every symmetry).  Both paths are timed at init for tufrg_symmetry_info.  FP64 two-band models use
-   the loop symmetries and, inside flows, the state symmetries; they ignore TUFRG_SYMMETRIC_STATE (a caller's state
-   that was kept in lower precision has the symmetries to that precision only). */
+ * alike; OFF disables every symmetry).  Both paths are timed at init for tufrg_symmetry_info.  FP64
+ * two-band models use the loop symmetries and, inside flows, the state symmetries; they ignore TUFRG_SYMMETRIC_STATE (a
+ * caller's state that was kept in lower precision has the symmetries to that precision only). */
 enum { TUFRG_SYMMETRY_AUTO = 0, TUFRG_SYMMETRY_OFF = 1, TUFRG_SYMMETRY_STATES = 2 };
 
 /* Adaptive flow options (Dormand-Prince 5(4) in x = ln T, from T0 down to T_end; T is Lambda with the
@@ -270,7 +271,7 @@ tufrg_status tufrg_widen_f64(const void *d_in, void *d_out, size_t n, void *cuda
 
 /* Symmetric-state path (TUFRG_SYMMETRIC_STATE): *in_use = 1 when calls that set the flag project and
  * multiply at the orbit representatives only, 0 when they take the general path (the state symmetries
- * do not hold for this model).  *ms_general and *ms_reps are the init-time timings of projections +
+ * do not hold for this model; FP64 two-band models, whose flows work at the representatives all the same).  *ms_general and *ms_reps are the init-time timings of projections +
  * products of both channels on the two paths in milliseconds (-1 when not measured).
  * Errors: TUFRG_EINVAL for NULL arguments. */
 tufrg_status tufrg_symmetry_info(const tufrg_model *m, int *in_use, double *ms_general, double *ms_reps);
@@ -336,8 +337,8 @@ tufrg_status tufrg_rhs(tufrg_model *m, double T, const void *d_state, int channe
  *      products: d_dstate_local [2][n_q][M][M], dX/dT of the shard's momenta in list order.
  * With the shards partitioning the mesh, the rows equal those of tufrg_rhs.  h_q_list: n_q distinct
  * momenta in [0, Nq) (host memory); the model keeps full-size work buffers, the shard's rows alone are
- * read and written.  The loops are summed at the listed momenta; the general (not symmetric-state) path is taken; a model with an attached surrogate is
- * refused (TUFRG_ENOTSUP).  Stream ordered, no host synchronisation beyond the list upload.
+ * read and written.  The loops are summed at the listed momenta; the general (not symmetric-state) path is
+ * taken; a model with an attached surrogate is refused (TUFRG_ENOTSUP).  Stream ordered, no host synchronisation beyond the list upload.
  * Errors: TUFRG_EINVAL (NULL argument, bad list, T not positive and finite, bad mask), TUFRG_ENOTSUP,
  * TUFRG_ENOMEM, TUFRG_ECUDA.
  * ------------------------------------------------------------------------------------------ */

@@ -530,7 +530,7 @@ namespace {
 void release(tufrg_model *m)
 {
     void *ptrs[] = {m->d_E, m->d_U, m->d_U32, m->d_ft, m->d_ft32, m->d_dslot, m->d_deltas, m->d_hopR, m->d_hopt,
-                    m->d_dij, m->d_gofs[0], m->d_gofs[1], m->d_gterms[0], m->d_gterms[1], m->d_ph, m->d_clsph,
+                    m->d_dij, m->d_ph, m->d_clsph,
                     m->d_V0, m->d_Lc, m->d_Lc32, m->d_part, m->d_Xr, m->d_A, m->d_A32, m->d_T, m->d_amax,
                     m->d_red, m->d_y, m->d_yt, m->d_yn, m->d_state_in, m->d_state_out, m->d_rec, m->d_Xr32,
                     m->d_ph32, m->d_dftpart, m->d_dpartner, m->d_err, m->d_scal, m->d_flow, m->d_eofs[0],
@@ -1199,8 +1199,6 @@ try {
         CK(upload(&m->d_hp, hp, m->stream), "upload bond tables");
     }
     for (int ch = 0; ch < 2; ch++) {
-        CK(upload(&m->d_gofs[ch], m->gofs[ch], m->stream), "upload gather tables");
-        CK(upload(&m->d_gterms[ch], m->gterms[ch], m->stream), "upload gather tables");
     }
     if (2L * m->ncls * (long)m->M * m->M >= (long)INT_MAX) return fail(m, TUFRG_ETOOBIG, "projection tables exceed 2^31 entries");
     {

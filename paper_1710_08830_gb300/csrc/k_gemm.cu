@@ -12,7 +12,7 @@ namespace {
 
 constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
 
-template <typename C2> __device__ __forceinline__ void cfma(C2 &acc, C2 a, C2 b)
+__device__ __forceinline__ void cfma(float2 &acc, float2 a, float2 b)
 {
     acc.x = fma(a.x, b.x, acc.x);
     acc.x = fma(-a.y, b.y, acc.x);
@@ -21,13 +21,12 @@ template <typename C2> __device__ __forceinline__ void cfma(C2 &acc, C2 a, C2 b)
 }
 
 // C[q] = scale * A[q] * B[q]; B is either a plain matrix (Bm) or the loop matrix gathered from Lc.
-template <typename R, bool GATHER, bool OUT64>
-__global__ void __launch_bounds__(256) cgemm_kernel(const typename cpx<R>::t *A, const typename cpx<R>::t *Bm,
-                                                    const typename cpx<R>::t *Lc, const int *dij, int M, int nff,
-                                                    int ns2, int nd, double scale, const double *scal, const int *qlist,
-                                                    void *Cout)
+template <bool GATHER, bool OUT64>
+__global__ void __launch_bounds__(256) cgemm_kernel(const float2 *A, const float2 *Bm, const float2 *Lc, const int *dij, int M,
+                                                    int nff, int ns2, int nd, double scale, const double *scal,
+                                                    const int *qlist, void *Cout)
 {
-    using C2 = typename cpx<R>::t;
+    using C2 = float2;
     __shared__ C2 As[BK][BM + 1];
     __shared__ C2 Bs[BK][BN + 1];
     const int q = qlist ? qlist[blockIdx.z] : blockIdx.z;
@@ -42,19 +41,19 @@ __global__ void __launch_bounds__(256) cgemm_kernel(const typename cpx<R>::t *A,
 #pragma unroll
     for (int i = 0; i < TM; i++)
 #pragma unroll
-        for (int j = 0; j < TN; j++) acc[i][j] = mk(R(0), R(0));
+        for (int j = 0; j < TN; j++) acc[i][j] = mk(0.f, 0.f);
     for (int k0 = 0; k0 < M; k0 += BK) {
         // A tile: rows row0..+BM, cols k0..+BK  (stored transposed, As[k][row])
         for (int e = threadIdx.x; e < BM * BK; e += 256) {
             const int r = e / BK, kk = e % BK;
             const int gr = row0 + r, gk = k0 + kk;
-            As[kk][r] = (gr < M && gk < M) ? a[(size_t)gr * M + gk] : mk(R(0), R(0));
+            As[kk][r] = (gr < M && gk < M) ? a[(size_t)gr * M + gk] : mk(0.f, 0.f);
         }
         // B tile: rows k0..+BK, cols col0..+BN
         for (int e = threadIdx.x; e < BK * BN; e += 256) {
             const int kk = e / BN, c = e % BN;
             const int gk = k0 + kk, gc = col0 + c;
-            C2 v = mk(R(0), R(0));
+            C2 v = mk(0.f, 0.f);
             if (gk < M && gc < M) {
                 if (GATHER) {
                     const int d = dij[(gk / ns2) * nff + gc / ns2];
@@ -90,32 +89,8 @@ __global__ void __launch_bounds__(256) cgemm_kernel(const typename cpx<R>::t *A,
             if (OUT64)
                 reinterpret_cast<double2 *>(Cout)[o] = make_double2(scale * (double)acc[i][j].x, scale * (double)acc[i][j].y);
             else
-                reinterpret_cast<C2 *>(Cout)[o] = mk(R(scale * acc[i][j].x), R(scale * acc[i][j].y));
+                reinterpret_cast<C2 *>(Cout)[o] = mk((float)(scale * acc[i][j].x), (float)(scale * acc[i][j].y));
         }
-}
-
-template <typename R>
-cudaError_t run(tufrg_model *m, const typename cpx<R>::t *A, const typename cpx<R>::t *Lc, int channel_mask,
-                double2 *out, typename cpx<R>::t *Tbuf, const int *qlist, int nlist)
-{
-    const int M = m->M, ns2 = m->ns * m->ns;
-    const size_t M2 = (size_t)M * M, lper = (size_t)m->Nq * m->nd * ns2 * ns2;
-    const dim3 grid((M + BN - 1) / BN, (M + BM - 1) / BM, qlist ? nlist : m->Nq);
-    for (int ch = 0; ch < 2; ch++) {
-        double2 *o = out + (size_t)ch * m->Nq * M2;
-        if (!((channel_mask >> ch) & 1)) {
-            TUFRG_CUDA_TRY(cudaMemsetAsync(o, 0, sizeof(double2) * m->Nq * M2, m->stream));
-            continue;
-        }
-        const auto *a = A + (size_t)ch * m->Nq * M2;
-        cgemm_kernel<R, true, false><<<grid, 256, 0, m->stream>>>(a, nullptr, Lc + ch * lper, m->d_dij, M, m->nff,
-                                                                  ns2, m->nd, 1.0, nullptr, qlist, Tbuf);
-        TUFRG_CUDA_TRY(cudaGetLastError());
-        cgemm_kernel<R, false, true><<<grid, 256, 0, m->stream>>>(Tbuf, a, nullptr, nullptr, M, m->nff, ns2, m->nd,
-                                                                  ch == 0 ? 1.0 : 2.0, m->d_scal, qlist, o);
-        TUFRG_CUDA_TRY(cudaGetLastError());
-    }
-    return cudaSuccess;
 }
 
 }  // namespace
@@ -123,7 +98,25 @@ cudaError_t run(tufrg_model *m, const typename cpx<R>::t *A, const typename cpx<
 cudaError_t launch_vlv_large(tufrg_model *m, int channel_mask, double2 *d_out, const int *qlist, int nlist)
 {
     PhaseScope ps(m, PH_VLV, 4);
-    return run<float>(m, m->d_A32, m->d_Lc32, channel_mask, d_out, reinterpret_cast<float2 *>(m->d_T), qlist, nlist);
+    const int M = m->M, ns2 = m->ns * m->ns;
+    const size_t M2 = (size_t)M * M, lper = (size_t)m->Nq * m->nd * ns2 * ns2;
+    float2 *T = reinterpret_cast<float2 *>(m->d_T);
+    const dim3 grid((M + BN - 1) / BN, (M + BM - 1) / BM, qlist ? nlist : m->Nq);
+    for (int ch = 0; ch < 2; ch++) {
+        double2 *o = d_out + (size_t)ch * m->Nq * M2;
+        if (!((channel_mask >> ch) & 1)) {
+            TUFRG_CUDA_TRY(cudaMemsetAsync(o, 0, sizeof(double2) * m->Nq * M2, m->stream));
+            continue;
+        }
+        const float2 *a = m->d_A32 + (size_t)ch * m->Nq * M2;
+        cgemm_kernel<true, false><<<grid, 256, 0, m->stream>>>(a, nullptr, m->d_Lc32 + ch * lper, m->d_dij, M, m->nff, ns2, m->nd,
+                                                               1.0, nullptr, qlist, T);
+        TUFRG_CUDA_TRY(cudaGetLastError());
+        cgemm_kernel<false, true><<<grid, 256, 0, m->stream>>>(T, a, nullptr, nullptr, M, m->nff, ns2, m->nd,
+                                                               ch == 0 ? 1.0 : 2.0, m->d_scal, qlist, o);
+        TUFRG_CUDA_TRY(cudaGetLastError());
+    }
+    return cudaSuccess;
 }
 
 }  // namespace tufrg

@@ -94,12 +94,12 @@ struct Args2 {
     unsigned needed[MAXD];   // bit dyi set if (dx, dy) is in the Hermitian half of the bond differences
     int ky_chunks, ky_len;
     int ch0, half;           // first channel; bit ch set: channel ch sums half of the mesh
-    R thr, thr_factor;       // degenerate-pair switch: thr, or thr_factor * T with T read from the device
-    const double *Tp;        // device flow scale (T, or Lambda with the momentum shell), or null
+    R thr_factor;            // degenerate-pair switch = thr_factor * T
+    const double *Tp;        // device flow scale (T, or Lambda with the momentum shell)
     R shell_T;               // > 0: momentum-shell regulator at this fixed temperature (records hold f, h)
     const int *s_list;       // optional: CTA x evaluates transfer momentum s_list[x] (partials indexed by x)
     const int *skip;         // optional: the whole launch returns at once when *skip != 0
-    const typename cpx<R>::t *ptab;   // optional: e^{-2 pi i n / Lf}, n < Lf (computed in the kernel when null)
+    const typename cpx<R>::t *ptab;   // e^{-2 pi i n / Lf}, n < Lf
 };
 
 // (t1,t3,t2,t4) -> ab index of the compact loop (P: a=(t2,t1), b=(t4,t3); C: a=(t1,t2), b=(t3,t4))
@@ -184,15 +184,7 @@ __device__ __forceinline__ void loops2h_body(const Args2<R> &a, unsigned char *s
     C2 *ptab = reinterpret_cast<C2 *>(smem_raw);
     C2 *xph = reinterpret_cast<C2 *>(smem_raw + ((sizeof(C2) * Lf + 15) & ~size_t(15)));   // [64][MAXDH - 1] e^{-i kx dx}
     unsigned char *region = reinterpret_cast<unsigned char *>(xph + NT * (MAXDH - 1));
-    if (a.ptab) {
-        for (int n = threadIdx.x; n < Lf; n += NT) ptab[n] = a.ptab[n];
-    } else {
-        for (int n = threadIdx.x; n < Lf; n += NT) {
-            double sn, cs;
-            sincospi(2.0 * (double)n / (double)Lf, &sn, &cs);
-            ptab[n] = mk((R)cs, (R)-sn);   // e^{-2 pi i n / Lf}
-        }
-    }
+    for (int n = threadIdx.x; n < Lf; n += NT) ptab[n] = a.ptab[n];
     __syncthreads();
 
     const int s = blockIdx.x;                                    // slot of the partial sums
@@ -203,7 +195,7 @@ __device__ __forceinline__ void loops2h_body(const Args2<R> &a, unsigned char *s
     const int kx = blockIdx.y * NT + threadIdx.x;
     // temperature flow: the scale is T; momentum shell: the scale is Lambda and the temperature is fixed
     const R lam = SHELL ? (R)*a.Tp : R(0);
-    const R thr = SHELL ? a.thr_factor * a.shell_T : (a.Tp ? (R)(a.thr_factor * *a.Tp) : a.thr);
+    const R thr = SHELL ? a.thr_factor * a.shell_T : (R)(a.thr_factor * *a.Tp);
     const bool valid = kx < Lf;
     const int kyc = blockIdx.z % a.ky_chunks;
     // rows of this sum: the whole column, or hy .. hy + n_rows - 1 (mod Lf) with the self-paired rows fix0, fix1
@@ -494,7 +486,7 @@ struct Red2 {
     const typename cpx<R>::t *part;
     size_t part_cs, out_cs;
     int n_part, ndx, ndyh, nd, n_hp, chmask, half;
-    const int *dslot, *deltas, *dpartner, *hp;   // hp[i]: i-th bond difference of the half plane; dslot: partial slot
+    const int *dslot, *deltas, *hp;              // hp[i]: i-th bond difference of the half plane; dslot: partial slot
     const int *hpos;                             // [nd] position in hp of d or of -d
     const int *slot_q;                           // momentum of a list position (null: the position)
     const int2 *qmap;                            // symmetric gather: output momentum -> (list position, element); or null
@@ -722,7 +714,6 @@ cudaError_t reduce2(tufrg_model *m, int channel_mask, const void *part, size_t p
     a.half = loops2_half_mask(m);
     a.dslot = m->d_dslot;
     a.deltas = m->d_deltas;
-    a.dpartner = m->d_dpartner;
     a.hp = m->d_hp;
     a.hpos = m->d_hp + a.n_hp;
     a.slot_q = slot_q;

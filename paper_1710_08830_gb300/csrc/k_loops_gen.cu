@@ -10,7 +10,7 @@
 // the real rank-N_s product Y = A B with A[c][l] = rho1, B[l][c'] = T.  The row phase e^{-iqy dy} is a cosine and a sine
 // for dy > 0, so a column's sums are W[p][c][c'] = sum_qy phi_p(qy) Y, p over 1, cos, sin, cos, sin, ...: N_s^5 +
 // (2 n_dy - 1) N_s^4 real multiply-adds per (s, q), 3.3 times fewer than in complex arithmetic at N_s = 6 and n_dy = 3.
-// Half of the fine mesh suffices where exchanging the propagators maps the sum onto itself (see k_loops2.cu): columns
+// Half of the fine mesh suffices where exchanging the propagators maps the sum onto itself (see k_loops2h.cu): columns
 // qx = hx + j, 2 hx = sx (mod Lf), a column that is its own partner with weight 1/2.
 //
 // One CTA owns one transfer momentum and a range of columns; it walks the fine mesh column by column in batches of KB

@@ -17,7 +17,7 @@
 //       W[(s_j, c')][(p, c)] = sum_{(ky, l)} T^l_{c'}(s_j; kx, ky) * phi_p(ky) rho^l_c(kx, ky)
 //     with M = 3 momenta x 36 = 108 rows (of 128), N = 5 x 36 = 180 columns (of 192), K = Lf x 6;
 //   * exchanging the two propagators maps k to s - k, so one point of every pair {k, s - k} suffices where the channel
-//     allows it (P always, C with a symmetry that inverts the momentum; see k_loops2.cu): columns
+//     allows it (P always, C with a symmetry that inverts the momentum; see k_loops2h.cu): columns
 //     kx = hx + c, 2 hx = sx (mod Lf), c up to Lf / 2.  The momenta of a group share sx and hence their columns.
 // It runs as 3xTF32 (hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor memory).  The x phases e^{-+ i kx dx} are
 // applied afterwards by loops_tc_xsum over the written columns.

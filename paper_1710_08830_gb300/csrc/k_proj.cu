@@ -164,8 +164,6 @@ __global__ void __launch_bounds__(DFT_THREADS) dft_rows_kernel(const XT *__restr
         if (r < nry) zo[(size_t)r * M2] = z[r];
 }
 
-// Classes are visited grouped by R_y: sorted position c has class id cid[c] and R_x index rxi[c], and the group of
-// the r-th R_y is [ryo[r], ryo[r+1]).
 // The FP64 row pass with R_y and -R_y formed together: e^{+-i u R} x from the sums of cos(u R) x and sin(u R) x, four
 // multiply-adds per pair and value instead of eight, two where R_y = -R_y.  It runs at the rate of the FP64 pipe.
 // Table columns: n_self real phases, then the pairs.  Both passes at 8 x 8 momenta, M = 324 (five R_y): 744 -> 611 us; at
@@ -227,6 +225,8 @@ __global__ void __launch_bounds__(DFT_THREADS) dft_rows_pairs_kernel(const doubl
         }
 }
 
+// Classes are visited grouped by R_y: sorted position c has class id cid[c] and R_x index rxi[c], and the group of
+// the r-th R_y is [ryo[r], ryo[r+1]).
 template <typename R>
 __global__ void __launch_bounds__(32 * DFT_MAXG) dft_cols_kernel(const typename cpx<R>::t *__restrict__ Z, int Lq,
                                                                  int M2, int ncls, int nry, int nrx,

@@ -254,8 +254,6 @@ struct tufrg_model {
     double *d_scal = nullptr;       // device scalars: [0] temperature of the current evaluation, [1] product scale; the
                                     // stages j = 1 .. 6 of a flow's attempt at [2 j], [2 j + 1]
     int *d_dij = nullptr;           // [nff][nff]
-    int *d_gofs[2] = {nullptr, nullptr};
-    tufrg::GatherTerm *d_gterms[2] = {nullptr, nullptr};
     // loop symmetries (TUFRG_SYMMETRY_AUTO): the k-sums run for one representative momentum per orbit
     // of the symmetry group and the reduction writes every orbit member from it
     bool sym = false;

@@ -459,8 +459,8 @@ void build_loop_symmetry(const tufrg_model *m, LoopSymmetry &ls)
 
 // Autotuner decisions, shared by every model of the same shape in the process: the first model of a
 // shape times the alternatives, later ones reuse its choice, so that equal models take equal paths (and
-// give equal results) whatever the timing noise.  Key: device, decision kind and the sizes the costs
-// depend on.
+// give equal results) whatever the timing noise.  Key: device, decision kind (0: products backend, 3: loop launch shape,
+// 4 + products backend: the symmetric-state path) and the sizes the costs depend on.
 struct TuneResult {
     double ms[2];
     int choice;
@@ -1523,7 +1523,7 @@ try {
         CK(cudaMemcpy(&dev_err, m->d_err, sizeof(int), cudaMemcpyDeviceToHost), "copy error flag");
         if (dev_err) return fail(m, TUFRG_ETIMEOUT, "a bounded device-side wait gave up during autotuning");
     }
-    if (m->sym_calls && tune_lookup(m, 1 + m->products, &cached)) {
+    if (m->sym_calls && tune_lookup(m, 4 + m->products, &cached)) {
         m->sym_tune_ms[0] = cached.ms[0];
         m->sym_tune_ms[1] = cached.ms[1];
     } else if (m->sym_calls) {
@@ -1568,7 +1568,7 @@ try {
             CK(cudaEventElapsedTime(&ms, e0, e1), "event");
             m->sym_tune_ms[c] = ms / reps;
         }
-        tune_store(m, 1 + m->products, TuneResult{{m->sym_tune_ms[0], m->sym_tune_ms[1]}, 1});
+        tune_store(m, 4 + m->products, TuneResult{{m->sym_tune_ms[0], m->sym_tune_ms[1]}, 1});
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         cudaFree(tmp);

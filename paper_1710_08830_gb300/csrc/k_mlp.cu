@@ -102,6 +102,7 @@ tufrg_status mlp_host_alloc_fail(tufrg_mlp *n, const std::exception &ex) noexcep
 tufrg_status ensure_capacity(tufrg_mlp *n, int batch)
 {
     if (batch <= n->cap) return TUFRG_OK;
+    n->cap = 0;   // (until every buffer is there again)
     for (auto p : n->Z) cudaFree(p);
     for (auto p : n->part) cudaFree(p);
     cudaFree(n->dA); cudaFree(n->dA2); cudaFree(n->loss_part);

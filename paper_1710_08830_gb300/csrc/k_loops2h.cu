@@ -37,9 +37,10 @@
 // FP64: bound by the FP64 pipe (two results per clock and SM), so the four pair weights share one division, and bond
 // sets with more than three non-negative y differences split them over two groups of CTAs (registers).
 // Measured, both channels (before: the whole mesh, one launch per channel; FP64 also every transfer momentum and the
-// projectors from the eigenvectors at every point): 24 x 24 / 8 x 8 mesh, 9 bonds: split 90 -> 48 us, FP64 43.2 -> 1.1 ms;
-// 8 x 8 / 16 x 16, 5 bonds: split 30 -> 14 us, FP64 2.5 ms -> 139 us; 48 x 48 / 8 x 8, 13 bonds: split 1.40 -> 0.73 ms.
-// Bound by instruction issue (split) and by the FP64 pipe.
+// projectors from the eigenvectors at every point): 24 x 24 / 8 x 8 mesh, 9 bonds: split 90 -> 45 us, FP64 43.2 -> 1.1 ms;
+// 8 x 8 / 16 x 16, 5 bonds: split 30 -> 14 us, FP64 2.5 ms -> 139 us; 48 x 48 / 8 x 8, 13 bonds: split 1.40 -> 0.63 ms.
+// Split: bound by latency and issue (24 x 24: 11 warps per SM by registers, issue slots 58% busy, the FMA pipe 32%; reads
+// the records from DRAM once, 1.8 MB); FP64: by the FP64 pipe.
 #include <algorithm>
 #include <cmath>
 #include <vector>

@@ -24,7 +24,7 @@
 // the orbits.  From the ranges' accumulators on, the split path adds in FP32 pairs (in FP32 alone the 12 x 12 / 5 x 5 bilayer
 // mesh's P loops are off by 1.9e-7 instead of 0.7e-7).
 // FP64: bound by the FP64 pipe (two results per clock and SM); the 8 x 8 / 6 x 6 three-orbital sums of both channels
-// take 1.8 ms (6.9 ms in complex arithmetic over the whole mesh).
+// take 1.66 ms (6.9 ms in complex arithmetic over the whole mesh).
 #include <cmath>
 #include <type_traits>
 

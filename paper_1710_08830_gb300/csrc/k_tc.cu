@@ -11,7 +11,8 @@
 // takes about 34 cycles plus half a cycle per column, so half as many of twice the width are faster than four streams
 // into two accumulators.
 // Both products of 225 momenta, two channels, M = 324: 1.45 ms with four streams, one row per lane and a shared-memory
-// tile for the epilogue; 1.15 ms now (its MMAs alone about 0.95 ms, its producers alone 0.88 ms).
+// tile for the epilogue; 1.15 ms now (its MMAs alone about 0.95 ms, its producers alone 0.88 ms).  The tensor pipe is busy
+// 78% of the cycles in the first product and 62% in the second, which writes FP64 (45 representatives).
 // Precision: 3xTF32 - every FP32 operand x is split into hi = x with the 13 low mantissa bits cleared and lo = x - hi
 // (exact), and each real product is hi*hi + hi*lo + lo*hi accumulated in FP32 in tensor memory.
 //

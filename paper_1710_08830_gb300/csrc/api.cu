@@ -773,7 +773,8 @@ tufrg_status flow_alloc(tufrg_model *m)
 tufrg_status flow_capture(tufrg_model *m, int mask, bool loop)
 {
     tufrg_model::FlowGraph &fg = loop ? m->loop_graph : m->step_graph;
-    if (fg.exec && fg.mask == mask) return TUFRG_OK;
+    const unsigned net = m->sur ? mlp_generation(m->sur) : 0;
+    if (fg.exec && fg.mask == mask && fg.net == net) return TUFRG_OK;
     if (fg.exec) {
         cudaGraphExecDestroy(fg.exec);
         fg.exec = nullptr;
@@ -816,6 +817,7 @@ tufrg_status flow_capture(tufrg_model *m, int mask, bool loop)
         return cuda_fail(m, ce, "capture of a flow step");
     }
     fg.mask = mask;
+    fg.net = net;
     return TUFRG_OK;
 }
 
@@ -2054,6 +2056,9 @@ tufrg_status tufrg_flow_step(tufrg_model *m, tufrg_flow_step_info *s)
     if (!m || !s) return fail(m, TUFRG_EINVAL, "NULL argument");
     if (!m->flow_open) return fail(m, TUFRG_EINVAL, "no stepwise flow is open on this model");
     if (m->h_flow->status == 0) {
+        // (captured again where a surrogate's network has grown since)
+        const tufrg_status st = flow_capture(m, m->flow_mask, false);
+        if (st != TUFRG_OK) return st;
         cudaError_t e = cudaGraphLaunch(m->step_graph.exec, m->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
@@ -2235,14 +2240,31 @@ try {
             if (first == TUFRG_OK) first = st;
         }
     }
-    // lock-step rounds: every running flow replays one attempt on its own stream, then all are polled
+    // a network that several models share may have grown for a later one: their attempts are captured again
+    for (int i = 0; i < n; i++) {
+        if (!active[i]) continue;
+        const tufrg_status st = flow_capture(models[i], o->channel_mask, false);
+        if (st != TUFRG_OK) {
+            active[i] = 0;
+            if (first == TUFRG_OK) first = st;
+        }
+    }
+    // lock-step rounds: every running flow replays one attempt on its own stream, then all are polled.  Models that share
+    // a surrogate network share its buffers and take turns.
     int running = 0;
     for (int i = 0; i < n; i++) running += active[i];
     while (running > 0) {
         for (int i = 0; i < n; i++) {
             if (!active[i]) continue;
             tufrg_model *m = models[i];
-            cudaError_t e = cudaGraphLaunch(m->step_graph.exec, m->stream);
+            cudaError_t e = cudaSuccess;
+            for (int j = i - 1; m->sur && j >= 0 && e == cudaSuccess; j--)
+                if (active[j] && models[j]->sur == m->sur) {
+                    e = cudaStreamWaitEvent(m->stream, models[j]->flow_ev, 0);
+                    break;
+                }
+            if (e == cudaSuccess) e = cudaGraphLaunch(m->step_graph.exec, m->stream);
+            if (e == cudaSuccess && m->sur) e = cudaEventRecord(m->flow_ev, m->stream);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(m->h_flow, m->d_flow, sizeof(FlowDev), cudaMemcpyDeviceToHost, m->stream);
             if (e != cudaSuccess) {

@@ -36,6 +36,7 @@ struct tufrg_mlp {
     float *d_g = nullptr, *d_m = nullptr, *d_v = nullptr;   // gradient, Adam moments
     int adam_t = 0;
     int cap = 0;                           // batch capacity of the activation buffers
+    unsigned generation = 0;               // counts their reallocations (captured graphs hold their addresses)
     std::vector<float *> Z;                // [layer] pre-activations, FP32 [cap][dout]
     float *dA = nullptr, *dA2 = nullptr;   // FP32 upstream gradients [cap][max width]
     std::vector<float *> part;             // [layer] partial sums of the bias gradients
@@ -103,6 +104,7 @@ tufrg_status ensure_capacity(tufrg_mlp *n, int batch)
 {
     if (batch <= n->cap) return TUFRG_OK;
     n->cap = 0;   // (until every buffer is there again)
+    n->generation++;
     for (auto p : n->Z) cudaFree(p);
     for (auto p : n->part) cudaFree(p);
     cudaFree(n->dA); cudaFree(n->dA2); cudaFree(n->loss_part);
@@ -326,6 +328,8 @@ void mlp_dims(const tufrg_mlp *n, int *n_in, int *n_out)
     *n_in = n->n_in;
     *n_out = n->n_out;
 }
+
+unsigned mlp_generation(const tufrg_mlp *n) { return n->generation; }
 
 // Inference for the surrogate inside a model's right-hand side (stream-ordered, no sync); all kernels
 // return at once while *skip != 0.

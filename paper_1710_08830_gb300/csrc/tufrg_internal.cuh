@@ -340,6 +340,7 @@ struct tufrg_model {
     struct FlowGraph {
         cudaGraphExec_t exec = nullptr;
         int mask = 0;
+        unsigned net = 0;   // generation of the surrogate network's buffers that it holds
     } step_graph, loop_graph;
     cudaStream_t flow_stream = nullptr;      // private capturable stream of the flow (joined to `stream` by events)
     // second stream of a right-hand side: the Fourier transform and projections (they read the state only) run
@@ -523,6 +524,7 @@ cudaError_t launch_surrogate(tufrg_model *m, int channel_mask);
 cudaError_t mlp_forward_on(tufrg_mlp *n, cudaStream_t s, const float *X, int batch, float *Y, const int *skip);
 cudaError_t surrogate_rearm(tufrg_model *m);
 void mlp_dims(const tufrg_mlp *n, int *n_in, int *n_out);
+unsigned mlp_generation(const tufrg_mlp *n);   // changes when the network's buffers move
 
 enum Phase { PH_FERMI = 0, PH_LOOPS = 1, PH_LOOPRED = 2, PH_DFT = 3, PH_PROJ = 4, PH_VLV = 5, PH_RK = 6, PH_SCATTER = 7, PH_N = 8 };
 

@@ -371,12 +371,15 @@ template <typename S> using val_t = decltype(ld_cx(S{}).x);                    /
 template <typename S> using wide_t = decltype(st_cx(ld_cx(S{})));               // a sum of such values in memory
 
 // the kx ranges' accumulators added (fixed order, eight loads in flight): FP64 over the first range's accumulators, FP32
-// into pairs
-template <typename S>
-__global__ void loops_gen_chunk_sum(const S *acc, int nchunk, size_t n, wide_t<S> *sum)
+// into pairs; the half-plane differences hp only, which alone the k-sum writes.  Grid: (n_hp entries / 256, slots); n: values
+// of one range.
+template <int NS, typename S>
+__global__ void __launch_bounds__(256) loops_gen_chunk_sum(const S *acc, int nchunk, size_t n, const int *hp, int n_hp, int nd, wide_t<S> *sum)
 {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
+    constexpr int NS4 = NS * NS * NS * NS;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_hp * NS4) return;
+    const size_t t = ((size_t)blockIdx.y * nd + hp[i / NS4]) * NS4 + i % NS4;
     constexpr int UB = 8;
     auto s = ld_cx(acc[t]);
     for (int c = 1; c < nchunk; c += UB) {
@@ -586,7 +589,10 @@ cudaError_t run_gen(tufrg_model *m, int ch, bool half, const typename cpx<R>::t 
     TUFRG_CUDA_TRY((m->ns == 6 ? dispatch_gen<R, 6>(m, a, ch) : dispatch_gen<R, 4>(m, a, ch)));
     if (m->gen_chunks > 1) {
         PhaseScope ps(m, PH_LOOPRED);
-        loops_gen_chunk_sum<C2><<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(a.acc, m->gen_chunks, n, gen_sums<C2>(m));
+        const int n_hp = (m->nd + 1) / 2;
+        const dim3 grid((n_hp * m->ns * m->ns * m->ns * m->ns + 255) / 256, a.n_slot);
+        auto k = m->ns == 6 ? loops_gen_chunk_sum<6, C2> : loops_gen_chunk_sum<4, C2>;
+        k<<<grid, 256, 0, m->stream>>>(a.acc, m->gen_chunks, n, m->d_hp, n_hp, m->nd, gen_sums<C2>(m));
     }
     return cudaGetLastError();
 }
